@@ -12,10 +12,28 @@
 #include <cuda_fp16.h>
 #include <string.h>
 
+#include <cmath>
+#include <type_traits>
+
 #include "iblb_internal.cuh"
 
 namespace iblb {
 namespace {
+
+// Coefficients of the collision (see collide below), formed on the host in double and rounded
+// once: la, ld (momentum), ba, bd, b0 (density and trace) and qa, qd (second order) of the axis,
+// diagonal and rest directions.
+template <typename real>
+struct CollideCoef {
+  real omc, nom;      // 1 - omega, -omega
+  real la, ld;        // 3 w omega
+  real ba, bd, b0;    // w omega
+  real qa, qd;        // 4.5 w omega
+  real m0, ma, md;    // weights of stored populations in the moments (16-bit storage)
+  real Fh[3];         // g/2:            u = (j + g/2)/rho
+  real Kc[3];         // (2 tau - 1/2) g: K = j + (2 tau - 1/2) g
+  real Lc[3];         // g/omega:        L = j + g/omega
+};
 
 template <typename real>
 struct LatParams {
@@ -28,7 +46,51 @@ struct LatParams {
   real g[3];         // uniform body force
   real wb[19];       // 6 w_i rho0 (c_i . u_bottom): moving-wall term, bottom wall
   real wt[19];       // same for the top wall
+  CollideCoef<real> cc;
 };
+
+// The collision's coefficients. Rounding them one by one would make the collision gain or lose
+// mass and momentum in proportion to the state, step after step; so the ones that are free are
+// taken from the ones already rounded, such that the sums over the 19 directions come out:
+//   sum of the momentum terms  2 la + 8 ld = om,   sum of the density terms 6 ba + 12 bd + b0 = om
+// exactly, with om the relaxation rate that the f term applies (FP32: f - om f with om as
+// rounded; FP64 and 16-bit storage: (1 - om) f, om = 1 - (1 - om as rounded)): ld and bd are
+// taken as multiples of an eighth of om's last place, which leaves la and b0 representable.
+// `scale` is 0 for plain storage, else K of the 16-bit units g_i = (f_i - w_i rho0) K / w_i,
+// where the weights cancel.
+template <typename real>
+CollideCoef<real> collide_coef(const Ctx &c, double scale) {
+  CollideCoef<real> k;
+  const double tau = c.tau;
+  k.nom = (real)(-1.0 / tau);
+  k.omc = (real)(1.0 - 1.0 / tau);
+  const bool delta = sizeof(real) == 4 && scale == 0.0;  // f - om f (see collide)
+  const double om = delta ? -(double)k.nom : 1.0 - (double)k.omc;
+  if (scale != 0.0) {
+    k.la = k.ld = (real)(3.0 * scale * om);
+    k.ba = k.bd = k.b0 = (real)(scale * om);
+    k.qa = k.qd = (real)(4.5 * scale * om);
+    k.m0 = (real)(1.0 / (3.0 * scale));
+    k.ma = (real)(1.0 / (18.0 * scale));
+    k.md = (real)(1.0 / (36.0 * scale));
+  } else {
+    const double step = std::ldexp(1.0, std::ilogb(om) - (sizeof(real) == 4 ? 23 : 52) - 3);
+    k.ld = (real)(std::rint(om / 12.0 / step) * step);
+    k.la = (real)((om - 8.0 * (double)k.ld) / 2.0);
+    k.bd = (real)(std::rint(om / 36.0 / step) * step);
+    k.ba = (real)(2.0 * (double)k.bd);
+    k.b0 = (real)(om - 24.0 * (double)k.bd);
+    k.qd = (real)(om / 8.0);
+    k.qa = (real)(2.0 * (double)k.qd);
+    k.m0 = k.ma = k.md = (real)1;
+  }
+  for (int a = 0; a < 3; a++) {
+    k.Fh[a] = (real)(0.5 * c.g[a]);
+    k.Kc[a] = (real)((2.0 * tau - 0.5) * c.g[a]);
+    k.Lc[a] = (real)(c.g[a] / om);
+  }
+  return k;
+}
 
 template <typename real>
 LatParams<real> lat_params(const Ctx &c) {
@@ -46,7 +108,44 @@ LatParams<real> lat_params(const Ctx &c) {
     p.wb[i] = (real)(6.0 * wgt(i) * c.rho0 * cb);
     p.wt[i] = (real)(6.0 * wgt(i) * c.rho0 * ct);
   }
+  p.cc = collide_coef<real>(c, c.precision == IBLB_FP16 ? 1024.0 : c.precision == IBLB_BF16 ? 1.0 : 0.0);
   return p;
+}
+
+// n / d for 0 <= n < 2^31 and a fixed d >= 1, by one multiplication (d >= 2): with 2^(l-1) < d <= 2^l and
+// m = floor(2^(31+l) / d) + 1 (below 2^32), m d exceeds 2^(31+l) by at most 2^l, which shifts
+// n m / 2^(31+l) from n / d by less than 1 / d: the floor is the same.
+struct FastDiv {
+  unsigned m;
+  int shift;
+  int d;
+  __device__ __forceinline__ int div(int n) const {
+    return d == 1 ? n : (int)(__umulhi((unsigned)n, m) >> shift);
+  }
+};
+FastDiv fast_div(int d) {
+  int l = 1;
+  while ((1ll << l) < d) l++;
+  FastDiv f;
+  f.m = (unsigned)(((1ull << (31 + l)) / (unsigned)d) + 1ull);
+  f.shift = l - 1;
+  f.d = d;
+  return f;
+}
+
+// Node groups of the fluid layers in memory order (a group: the nodes of one thread).
+struct FlatGroups {
+  FastDiv per_row, ny;  // groups per lattice row, rows per layer
+  int n;                // groups in all
+  __device__ __forceinline__ void at(int g, int &gx, int &y, int &z) const {
+    const int row = per_row.div(g);
+    gx = g - row * per_row.d;
+    z = ny.div(row);
+    y = row - z * ny.d;
+  }
+};
+FlatGroups flat_groups(int per_row, int ny, int layers) {
+  return FlatGroups{fast_div(per_row), fast_div(ny), per_row * ny * layers};
 }
 
 // Storage of the shifted populations. Population i is stored as g_i = (f_i - w_i rho0) k_i
@@ -245,83 +344,136 @@ __device__ __forceinline__ void tile_force(const int *__restrict__ tile_slot,
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 
-// n / (hi + lo) for |lo| << |hi| and r1 ~ 1/hi: q0 = n r1, then the residual
-// n - q0 hi - q0 lo (the first product exactly, by a fused multiply-add) corrects it once.
-template <typename real>
-__device__ __forceinline__ real quotient(real n, real hi, real lo, real r1) {
-  const real q0 = n * r1;
-  real e = fma_(-q0, hi, n);
-  e = fma_(-q0, lo, e);
-  return fma_(e, r1, q0);
+// Single roundings that the compiler does not fuse, so that every kernel that collides a node
+// gives the same bits.
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+
+// 1/a and 1/b of two nodes' densities. FP64 divides cost an order of magnitude more than an
+// FP64 multiply-add, so the two share one reciprocal, 1/(ab), by Newton's iteration
+// r <- r + r (1 - x r) from a float seed (relative error 2^-23, then 2^-46, then rounding);
+// outside the seed's range it is a plain division. u enters the collision only at second order.
+__device__ __forceinline__ void reciprocals(double a, double b, double &ra, double &rb) {
+  const double x = mul_(a, b);
+  const float s = (float)x;
+  double r;
+  if (s > 1e-30f && s < 1e30f) {
+    r = (double)(1.0f / s);
+    r = fma(r, fma(-x, r, 1.0), r);
+    r = fma(r, fma(-x, r, 1.0), r);
+  } else {
+    r = 1.0 / x;
+  }
+  ra = mul_(r, b);
+  rb = mul_(r, a);
 }
 
-// BGK collision with Guo forcing (Eqs. 9-10) of one node's shifted populations f, storing
-// the post-collision populations at node n of fout. Opposite directions i, i+1 (i odd) share
-// c.u and c.F up to sign, so each pair is computed from its symmetric and antisymmetric parts:
-//   f^eq - w rho0 = w [drho + rho (4.5 (c.u)^2 - 1.5 u^2)] +- w rho 3 (c.u)      (Eq. 10)
-//   S = w (1 - 1/2tau) [9 (c.F)(c.u) - 3 u.F] +- w (1 - 1/2tau) 3 (c.F)          (Eq. 9)
-// With FORCE false the force is zero and the Guo terms vanish.
-template <typename real, bool FORCE>
-__device__ __forceinline__ void collide(real f[Q], const real F[3], const LatParams<real> &P) {
-  // moments: rho = rho0 + sum f~, j = sum c f~ (the rest-state part carries no momentum)
-  real drho = f[0], jx = 0, jy = 0, jz = 0;
+// Density and momentum of a node's shifted populations: rho = rho0 + sum f, j = sum c f (the
+// rest-state part carries no momentum), from the sums and differences of opposite directions.
+template <typename real>
+__device__ __forceinline__ void node_moments(const real f[Q], real &drho, real j[3]) {
+  real s[9], d[9];
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    drho += f[i] + f[i + 1];
-    const real d = f[i] - f[i + 1];
-    if (cx(i)) jx += cx(i) > 0 ? d : -d;
-    if (cy(i)) jy += cy(i) > 0 ? d : -d;
-    if (cz(i)) jz += cz(i) > 0 ? d : -d;
+  for (int p = 0; p < 9; p++) {
+    s[p] = add_(f[2 * p + 1], f[2 * p + 2]);
+    d[p] = add_(f[2 * p + 1], -f[2 * p + 2]);
   }
-  // rho = rho0 + drho is never rounded as a whole: rho_lo carries the rounding remainder of
-  // the sum (Fast2Sum, |rho0| >= |drho|), and rho X is expanded as rho0 X + drho X
-  const real rho_hi = P.rho0 + drho;
-  const real rho_lo = (P.rho0 - rho_hi) + drho;
-  const real r1 = real(1) / rho_hi;
-  real ux = jx, uy = jy, uz = jz;
-  if (FORCE) {
-    ux += real(0.5) * F[0];
-    uy += real(0.5) * F[1];
-    uz += real(0.5) * F[2];
+  drho = add_(add_(f[0], add_(add_(s[0], s[1]), s[2])),
+              add_(add_(add_(s[3], s[4]), add_(s[5], s[6])), add_(s[7], s[8])));
+  j[0] = add_(d[0], add_(add_(d[3], d[4]), add_(d[5], d[6])));
+  j[1] = add_(d[1], add_(add_(d[3], -d[4]), add_(d[7], d[8])));
+  j[2] = add_(d[2], add_(add_(d[5], -d[6]), add_(d[7], -d[8])));
+}
+
+// One population after the collision: its relaxed value plus the equilibrium part P and the
+// momentum part l v. FP64: (1 - omega) f + P + l v; FP32: f + (P - omega f + l v), whose
+// rounding stays in proportion to omega at large tau.
+__device__ __forceinline__ double relaxed(double f, double P, double l, double v,
+                                          const CollideCoef<double> &k) {
+  return fma(l, v, fma(k.omc, f, P));
+}
+__device__ __forceinline__ float relaxed(float f, float P, float l, float v,
+                                         const CollideCoef<float> &k) {
+  return __fadd_rn(f, fmaf(l, v, fmaf(k.nom, f, P)));
+}
+// the rest population: no momentum part
+__device__ __forceinline__ double relaxed(double f, double P, const CollideCoef<double> &k) {
+  return fma(k.omc, f, P);
+}
+__device__ __forceinline__ float relaxed(float f, float P, const CollideCoef<float> &k) {
+  return __fadd_rn(f, fmaf(k.nom, f, P));
+}
+
+// BGK collision with Guo forcing (Eqs. 9-10) of one node's shifted populations f in place, with
+// the uniform force g (FORCE; without it the force terms vanish), given 1/rho. With
+// u = (j + g/2)/rho the momentum rho u is j + g/2 itself, so the equilibrium's linear term needs
+// no velocity and no density, and the linear parts of equilibrium and source join:
+//   omega 3 w c.(rho u) + (1 - omega/2) 3 w c.g           = omega 3 w c.L,  L = j + g/omega;
+// likewise the second-order parts, with K = j + (2 tau - 1/2) g:
+//   omega 4.5 w rho (c.u)^2 + (1 - omega/2) 9 w (c.g)(c.u)  = omega 4.5 w (c.u)(c.K),
+//   omega 1.5 w rho u^2 + (1 - omega/2) 3 w u.g             = omega 1.5 w u.K,
+// so f*_i = (1 - omega) f_i + w omega (drho - 1.5 u.K) + 4.5 w omega (c.u)(c.K) +- 3 w omega c.L,
+// where the directions of an axis or of a coordinate plane share their second-order term: about
+// 120 operations instead of 250. FP64 passes are bound by the FP64 units (2 lanes per cycle and
+// SM; ncu: 84 % busy): 128^3 on all SMs 506 us against 867, 32^3 13.1 against 32.1 (there the
+// flat node groups halve it as well), 256^3 3.98 ms against 6.85. The FP32 pass stays at the
+// copy bandwidth (256^3: 366 us); 16-bit storage, 256^3 BF16 on 112 SMs 223 us against 229.
+// The rounding of u enters at second order only, where a form with rho u rounds it into the
+// linear term: u of the 256^3 FP32 run is 1.2e-7 off 64 bits after 40 steps, against 3.6e-7.
+template <bool FORCE, typename real>
+__device__ __forceinline__ void collide(real f[Q], real drho, const real j[3], real ir,
+                                        const CollideCoef<real> &k) {
+  real u[3], K[3], L[3];
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    u[a] = mul_(FORCE ? add_(j[a], k.Fh[a]) : j[a], ir);
+    K[a] = FORCE ? add_(j[a], k.Kc[a]) : j[a];
+    L[a] = FORCE ? add_(j[a], k.Lc[a]) : j[a];
   }
-  // u = j'/(rho_hi + rho_lo): a first quotient and one residual correction by fused
-  // multiply-adds, which keeps u within about an ulp of the exact quotient. The float
-  // rounding of u is what the FP32 path's drift from the FP64 solution grows from (the other
-  // roundings of the collision, the storage and the interface part matter two to three
-  // orders of magnitude less), so it is worth the six extra multiply-adds.
-  ux = quotient(ux, rho_hi, rho_lo, r1);
-  uy = quotient(uy, rho_hi, rho_lo, r1);
-  uz = quotient(uz, rho_hi, rho_lo, r1);
-  const real uu15 = real(1.5) * (ux * ux + uy * uy + uz * uz);
-  const real om = P.omega;
-  real uF3 = 0;
-  if (FORCE) uF3 = real(3) * (ux * F[0] + uy * F[1] + uz * F[2]);
-  {  // rest population
-    const real w = (real)wgt(0);
-    const real feq = w * (drho - P.rho0 * uu15 - drho * uu15);
-    real out = f[0] + om * (feq - f[0]);
-    if (FORCE) out -= w * P.guo * uF3;
-    f[0] = out;
+  const real qxx = mul_(u[0], K[0]), qyy = mul_(u[1], K[1]), qzz = mul_(u[2], K[2]);
+  const real s = fma_(real(-1.5), add_(add_(qxx, qyy), qzz), drho);
+  f[0] = relaxed(f[0], mul_(k.b0, s), k);
+  const real pa = mul_(k.ba, s), pd = mul_(k.bd, s);
+  const real qk[3] = {qxx, qyy, qzz};
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const real P = fma_(k.qa, qk[a], pa);
+    f[2 * a + 1] = relaxed(f[2 * a + 1], P, k.la, L[a], k);
+    f[2 * a + 2] = relaxed(f[2 * a + 2], P, -k.la, L[a], k);
   }
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const real w = (real)wgt(i);
-    const real cu = cx(i) * ux + cy(i) * uy + cz(i) * uz;
-    const real xs = real(4.5) * cu * cu - uu15;
-    const real xa = real(3) * cu;
-    const real sym = w * (drho + P.rho0 * xs + drho * xs);
-    const real asym = w * (P.rho0 * xa + drho * xa);
-    real a = f[i] + om * (sym + asym - f[i]);
-    real b = f[i + 1] + om * (sym - asym - f[i + 1]);
-    if (FORCE) {
-      const real cF = cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2];
-      const real ssym = w * P.guo * (real(9) * cF * cu - uF3);
-      const real sasym = w * P.guo * real(3) * cF;
-      a += ssym + sasym;
-      b += ssym - sasym;
-    }
-    f[i] = a;
-    f[i + 1] = b;
+  for (int p = 0; p < 3; p++) {  // planes xy, xz, yz: directions 7 + 4 p .. 10 + 4 p
+    const int a = p == 2 ? 1 : 0, b = p == 0 ? 1 : 2, i = 7 + 4 * p;
+    const real P = fma_(k.qd, add_(qk[a], qk[b]), pd);
+    // the mixed term u_a K_b + u_b K_a (twice u_a K_b without a force)
+    const real m = FORCE ? fma_(u[a], K[b], mul_(u[b], K[a])) : mul_(u[a], K[b]);
+    const real qm = FORCE ? k.qd : k.qa;
+    const real Pp = fma_(qm, m, P), Pm = fma_(-qm, m, P);
+    const real lp = add_(L[a], L[b]), lm = add_(L[a], -L[b]);
+    f[i] = relaxed(f[i], Pp, k.ld, lp, k);
+    f[i + 1] = relaxed(f[i + 1], Pp, -k.ld, lp, k);
+    f[i + 2] = relaxed(f[i + 2], Pm, k.ld, lm, k);
+    f[i + 3] = relaxed(f[i + 3], Pm, -k.ld, lm, k);
+  }
+}
+
+// The collision of the two nodes a and b of a pair.
+template <bool FORCE, typename real>
+__device__ __forceinline__ void collide_pair(real a[Q], real b[Q], const LatParams<real> &P) {
+  real da, db, ja[3], jb[3], ia, ib;
+  if constexpr (sizeof(real) == 4) {  // one after the other: fewer registers
+    node_moments(a, da, ja);
+    collide<FORCE>(a, da, ja, real(1) / add_(P.rho0, da), P.cc);
+    node_moments(b, db, jb);
+    collide<FORCE>(b, db, jb, real(1) / add_(P.rho0, db), P.cc);
+  } else {
+    node_moments(a, da, ja);
+    node_moments(b, db, jb);
+    reciprocals(add_(P.rho0, da), add_(P.rho0, db), ia, ib);
+    collide<FORCE>(a, da, ja, ia, P.cc);
+    collide<FORCE>(b, db, jb, ib, P.cc);
   }
 }
 
@@ -396,21 +548,33 @@ __device__ __forceinline__ void store_pair(S *__restrict__ fout, const LatParams
 // their interface force, so this pass does not wait for the interface chain of the step.
 // Each thread owns the two nodes (x0, x0 + 1), x0 even: populations that do not move along x
 // and every store are one aligned 2-wide access, and the address arithmetic is shared.
-// With ROWS each block covers blockDim.y lattice rows (small lattices); without, one row
-// (kept as its own instance: the row arithmetic costs the single-row kernel registers).
-template <typename real, typename S, bool FIRST, bool FORCE, bool ROWS>
-__global__ void __launch_bounds__(128) stream_collide_kernel(const S *__restrict__ fin,
-                                                             S *__restrict__ fout,
-                                                             const LatParams<real> P, int z0) {
-  const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = ROWS ? blockIdx.y * blockDim.y + threadIdx.y : blockIdx.y;
-  const int z = blockIdx.z + z0;
-  if (x0 >= P.nx) return;
+// Each block covers (part of) one lattice row, or with FLAT the next blockDim.x pairs in memory
+// order: rows that are no whole number of warps would leave lanes idle (nx = 132: 66 pairs in 96
+// lanes, 45 us per pass of 132 x 100 x 77; nx = 32: 16 pairs in 32).
+template <typename real>
+struct K1MinBlocks {  // FP32: 72 registers, 28 warps per SM (64 registers spill and are no faster)
+  static constexpr int value = sizeof(real) == 4 ? 7 : 1;
+};
+
+template <typename real, typename S, bool FIRST, bool FORCE, bool FLAT>
+__global__ void __launch_bounds__(128, K1MinBlocks<real>::value) stream_collide_kernel(
+    const S *__restrict__ fin, S *__restrict__ fout, const LatParams<real> P, int z0,
+    const FlatGroups G) {
+  int x0, y, z;
+  if (FLAT) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= G.n) return;
+    G.at(g, x0, y, z);
+    x0 *= 2;
+    z += z0;
+  } else {
+    x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    y = blockIdx.y;
+    z = blockIdx.z + z0;
+  }
   real a[Q], b[Q];  // populations of nodes x0 and x0 + 1
   load_pair<real, S, FIRST>(fin, P, x0, y, z, a, b);
-  const real F[3] = {P.g[0], P.g[1], P.g[2]};
-  collide<real, FORCE>(a, F, P);
-  collide<real, FORCE>(b, F, P);
+  collide_pair<FORCE>(a, b, P);
   store_pair(fout, P, (size_t)z * P.nx * P.ny + (size_t)y * P.nx + x0, a, b);
 }
 
@@ -422,74 +586,59 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup(-1.0f), a); }
 
-// BGK collision with Guo forcing (Eqs. 9-10) of a node pair held in the scaled storage units
-// of a 16-bit type, g_i = (f_i - w_i rho0) K / w_i. The moments weigh g_i by w_i / K, and the
-// update is the one of `collide` multiplied through by k_i = K / w_i, where the weights cancel:
-//   g*_i = g_i + omega (K [drho + rho (4.5 (c.u)^2 - 1.5 u^2) +- 3 rho (c.u)] - g_i)
-//          + K (1 - 1/2tau) [9 (c.F)(c.u) - 3 u.F +- 3 (c.F)]
-// (F uniform over the pair). rho is rounded once here: the storage rounding of the 16-bit
-// types is four orders of magnitude above it.
+// The collision of `collide` for a node pair held in the scaled storage units of a 16-bit type,
+// g_i = (f_i - w_i rho0) K / w_i: the moments weigh g_i by w_i / K, and in the update the weights
+// cancel, so every direction has the coefficients
+//   g*_i = (1 - omega) g_i + omega K (drho - 1.5 u.K) + 4.5 omega K (c.u)(c.K) +- 3 omega K c.L.
 template <bool FORCE>
-__device__ __forceinline__ void collide_pair_scaled(float2 g[Q], const float F[3],
-                                                    const LatParams<float> &P, float K) {
-  const float iK = 1.0f / K;
-  float2 drho = mul2(g[0], dup(float(wgt(0)) * iK));
-  float2 jx = dup(0.0f), jy = dup(0.0f), jz = dup(0.0f);
+__device__ __forceinline__ void collide_pair_scaled(float2 g[Q], const LatParams<float> &P) {
+  const CollideCoef<float> &k = P.cc;
+  float2 s[9], d[9];
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const float2 w = dup(float(wgt(i)) * iK);
-    drho = fma2(add2(g[i], g[i + 1]), w, drho);
-    const float2 d = mul2(sub2(g[i], g[i + 1]), w);
-    if (cx(i)) jx = cx(i) > 0 ? add2(jx, d) : sub2(jx, d);
-    if (cy(i)) jy = cy(i) > 0 ? add2(jy, d) : sub2(jy, d);
-    if (cz(i)) jz = cz(i) > 0 ? add2(jz, d) : sub2(jz, d);
+  for (int p = 0; p < 9; p++) {
+    s[p] = add2(g[2 * p + 1], g[2 * p + 2]);
+    d[p] = sub2(g[2 * p + 1], g[2 * p + 2]);
   }
+  const float2 ma = dup(k.ma), md = dup(k.md);
+  const float2 sa = add2(add2(s[0], s[1]), s[2]);
+  const float2 sd = add2(add2(add2(s[3], s[4]), add2(s[5], s[6])), add2(s[7], s[8]));
+  const float2 drho = fma2(md, sd, fma2(ma, sa, mul2(dup(k.m0), g[0])));
+  float2 j[3];
+  j[0] = fma2(ma, d[0], mul2(md, add2(add2(d[3], d[4]), add2(d[5], d[6]))));
+  j[1] = fma2(ma, d[1], mul2(md, add2(sub2(d[3], d[4]), add2(d[7], d[8]))));
+  j[2] = fma2(ma, d[2], mul2(md, add2(sub2(d[5], d[6]), sub2(d[7], d[8]))));
   const float2 rho = add2(dup(P.rho0), drho);
-  const float2 inv_rho = make_float2(__frcp_rn(rho.x), __frcp_rn(rho.y));
-  float2 ux = jx, uy = jy, uz = jz;
-  if (FORCE) {
-    ux = fma2(dup(0.5f), dup(F[0]), ux);
-    uy = fma2(dup(0.5f), dup(F[1]), uy);
-    uz = fma2(dup(0.5f), dup(F[2]), uz);
-  }
-  ux = mul2(ux, inv_rho);
-  uy = mul2(uy, inv_rho);
-  uz = mul2(uz, inv_rho);
-  const float2 uu15 = mul2(dup(1.5f), fma2(ux, ux, fma2(uy, uy, mul2(uz, uz))));
-  const float2 om = dup(P.omega), omc = dup(1.0f - P.omega);
-  const float2 Kdrho = mul2(dup(K), drho), Krho = mul2(dup(K), rho);
-  const float2 Krho3 = mul2(dup(3.0f), Krho);
-  float2 KuF3 = dup(0.0f);
-  const float Kguo = K * P.guo;
-  if (FORCE)
-    KuF3 = mul2(dup(3.0f * Kguo),
-                fma2(ux, dup(F[0]), fma2(uy, dup(F[1]), mul2(uz, dup(F[2])))));
-  {  // rest population: g*_0 = (1 - omega) g_0 + omega K (drho - rho 1.5 u^2) - K guo 3 u.F
-    const float2 feq = sub2(Kdrho, mul2(Krho, uu15));
-    float2 out = fma2(omc, g[0], mul2(om, feq));
-    if (FORCE) out = sub2(out, KuF3);
-    g[0] = out;
-  }
+  const float2 ir = make_float2(__frcp_rn(rho.x), __frcp_rn(rho.y));
+  float2 u[3], K[3], L[3];
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    float2 cu = dup(0.0f);
-    if (cx(i)) cu = cx(i) > 0 ? add2(cu, ux) : sub2(cu, ux);
-    if (cy(i)) cu = cy(i) > 0 ? add2(cu, uy) : sub2(cu, uy);
-    if (cz(i)) cu = cz(i) > 0 ? add2(cu, uz) : sub2(cu, uz);
-    const float2 xs = fma2(mul2(dup(4.5f), cu), cu, mul2(dup(-1.0f), uu15));
-    const float2 sym = fma2(Krho, xs, Kdrho);
-    const float2 asym = mul2(Krho3, cu);
-    float2 a = fma2(omc, g[i], mul2(om, add2(sym, asym)));
-    float2 b = fma2(omc, g[i + 1], mul2(om, sub2(sym, asym)));
-    if (FORCE) {
-      const float cF = cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2];
-      const float2 ssym = sub2(mul2(dup(9.0f * Kguo * cF), cu), KuF3);
-      const float2 sasym = dup(3.0f * Kguo * cF);
-      a = add2(a, add2(ssym, sasym));
-      b = add2(b, sub2(ssym, sasym));
-    }
-    g[i] = a;
-    g[i + 1] = b;
+  for (int a = 0; a < 3; a++) {
+    u[a] = mul2(FORCE ? add2(j[a], dup(k.Fh[a])) : j[a], ir);
+    K[a] = FORCE ? add2(j[a], dup(k.Kc[a])) : j[a];
+    L[a] = FORCE ? add2(j[a], dup(k.Lc[a])) : j[a];
+  }
+  const float2 q[3] = {mul2(u[0], K[0]), mul2(u[1], K[1]), mul2(u[2], K[2])};
+  const float2 tr = fma2(dup(-1.5f), add2(add2(q[0], q[1]), q[2]), drho);
+  const float2 base = mul2(dup(k.bd), tr);
+  const float2 omc = dup(k.omc), qd = dup(k.qd), l = dup(k.ld), nl = dup(-k.ld);
+  g[0] = fma2(omc, g[0], base);
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float2 Pq = fma2(qd, q[a], base);
+    g[2 * a + 1] = fma2(l, L[a], fma2(omc, g[2 * a + 1], Pq));
+    g[2 * a + 2] = fma2(nl, L[a], fma2(omc, g[2 * a + 2], Pq));
+  }
+  const float2 qm = dup(FORCE ? k.qd : 2.0f * k.qd), nqm = dup(FORCE ? -k.qd : -2.0f * k.qd);
+#pragma unroll
+  for (int p = 0; p < 3; p++) {
+    const int a = p == 2 ? 1 : 0, b = p == 0 ? 1 : 2, i = 7 + 4 * p;
+    const float2 Pq = fma2(qd, add2(q[a], q[b]), base);
+    const float2 m = FORCE ? fma2(u[a], K[b], mul2(u[b], K[a])) : mul2(u[a], K[b]);
+    const float2 Pp = fma2(qm, m, Pq), Pm = fma2(nqm, m, Pq);
+    const float2 lp = add2(L[a], L[b]), lm = sub2(L[a], L[b]);
+    g[i] = fma2(l, lp, fma2(omc, g[i], Pp));
+    g[i + 1] = fma2(nl, lp, fma2(omc, g[i + 1], Pp));
+    g[i + 2] = fma2(l, lm, fma2(omc, g[i + 2], Pm));
+    g[i + 3] = fma2(nl, lm, fma2(omc, g[i + 3], Pm));
   }
 }
 
@@ -581,7 +730,6 @@ __device__ __forceinline__ void quad_nodes(const S *__restrict__ fin, S *__restr
       }
     }
   }
-  const float F[3] = {P.g[0], P.g[1], P.g[2]};
 #pragma unroll
   for (int h = 0; h < 2; h++) {  // node pairs (x0, x0 + 1), (x0 + 2, x0 + 3)
     unsigned int *pk = h ? hi : lo;
@@ -594,7 +742,7 @@ __device__ __forceinline__ void quad_nodes(const S *__restrict__ fin, S *__restr
         g[i] = add2(g[i], dup(wall));
       }
     }
-    collide_pair_scaled<FORCE>(g, F, P, float(Storage<S>::K));
+    collide_pair_scaled<FORCE>(g, P);
 #pragma unroll
     for (int i = 0; i < Q; i++) pk[i] = as_bits(narrow_pair<V2>(g[i]));
   }
@@ -603,16 +751,17 @@ __device__ __forceinline__ void quad_nodes(const S *__restrict__ fin, S *__restr
     *reinterpret_cast<uint2 *>(fout + (size_t)i * P.ncell + n) = make_uint2(lo[i], hi[i]);
 }
 
+// (its threads always take the quads in memory order)
 template <typename S, bool FIRST, bool FORCE>
 __global__ void __launch_bounds__(128) stream_collide_quad_kernel(const S *__restrict__ fin,
                                                                   S *__restrict__ fout,
                                                                   const LatParams<float> P,
-                                                                  int z0) {
-  const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;  // blockDim.y rows per block
-  const int z = blockIdx.z + z0;
-  if (x0 >= P.nx) return;
-  quad_nodes<S, FIRST, FORCE>(fin, fout, P, x0, y, z);
+                                                                  int z0, const FlatGroups G) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= G.n) return;
+  int gx, y, z;
+  G.at(g, gx, y, z);
+  quad_nodes<S, FIRST, FORCE>(fin, fout, P, 4 * gx, y, z + z0);
 }
 
 // --- K1s: stream-collide with the pulled rows staged in shared memory by bulk copies ----------
@@ -821,9 +970,7 @@ __device__ __forceinline__ void staged_pair(const float *rows, int stride, int x
       b[i] = row[xp];
     }
   }
-  const float F[3] = {P.g[0], P.g[1], P.g[2]};
-  collide<float, FORCE>(a, F, P);
-  collide<float, FORCE>(b, F, P);
+  collide_pair<FORCE>(a, b, P);
   store_pair(fout, P, n, a, b);
 }
 
@@ -855,7 +1002,6 @@ __device__ __forceinline__ void staged_quad(const S *rows, int stride, int x0, c
       hi[i] = __byte_perm(v.y, e, 0x5432);
     }
   }
-  const float F[3] = {P.g[0], P.g[1], P.g[2]};
 #pragma unroll
   for (int h = 0; h < 2; h++) {  // node pairs (x0, x0 + 1), (x0 + 2, x0 + 3)
     unsigned int *pk = h ? hi : lo;
@@ -868,7 +1014,7 @@ __device__ __forceinline__ void staged_quad(const S *rows, int stride, int x0, c
         g[i] = add2(g[i], dup(wall));
       }
     }
-    collide_pair_scaled<FORCE>(g, F, P, float(Storage<S>::K));
+    collide_pair_scaled<FORCE>(g, P);
 #pragma unroll
     for (int i = 0; i < Q; i++) pk[i] = as_bits(narrow_pair<V2>(g[i]));
   }
@@ -909,8 +1055,7 @@ __device__ __forceinline__ void staged_pair16(const S *rows, int stride, int x0,
       g[i] = add2(g[i], dup(wall));
     }
   }
-  const float F[3] = {P.g[0], P.g[1], P.g[2]};
-  collide_pair_scaled<FORCE>(g, F, P, float(Storage<S>::K));
+  collide_pair_scaled<FORCE>(g, P);
 #pragma unroll
   for (int i = 0; i < Q; i++)
     *reinterpret_cast<unsigned int *>(fout + (size_t)i * P.ncell + n) = as_bits(narrow_pair<V2>(g[i]));
@@ -1021,10 +1166,9 @@ struct StreamArgs {
   const S *fin;
   S *fout;
   LatParams<real> P;
-  int z0;       // first fluid layer
-  int per_row;  // node groups per lattice row
-  int ngroups;  // node groups of the context
-  int force;    // the body force is non-zero
+  FlatGroups G;  // node groups of the context
+  int z0;        // first fluid layer
+  int force;     // the body force is non-zero
 };
 
 // Blocks per SM the batched pass is compiled for: 6 (80 registers) for FP32, where it keeps
@@ -1051,30 +1195,24 @@ __global__ void __launch_bounds__(128, MultiMinBlocks<real, S>::value) stream_co
   __syncthreads();
   const int total = s_start[n];
   for (int vb = blockIdx.x; vb < total; vb += gridDim.x) {
-  const MultiBlock m = multi_block_of(s_start, n, vb);
-  const StreamArgs<real, S> &A = all[m.inst];
-  const int g = m.block * blockDim.x + threadIdx.x;
-  if (g >= A.ngroups) continue;
-  const int row = g / A.per_row;
-  const int y = row % A.P.ny, z = A.z0 + row / A.P.ny;
-  if constexpr (sizeof(S) == 2) {
-    const int x0 = 4 * (g - row * A.per_row);
-    if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, x0, y, z);
-    else quad_nodes<S, false, false>(A.fin, A.fout, A.P, x0, y, z);
-  } else {
-    const int x0 = 2 * (g - row * A.per_row);
-    real a[Q], b[Q];
-    load_pair<real, S, false>(A.fin, A.P, x0, y, z, a, b);
-    const real F[3] = {A.P.g[0], A.P.g[1], A.P.g[2]};
-    if (A.force) {
-      collide<real, true>(a, F, A.P);
-      collide<real, true>(b, F, A.P);
+    const MultiBlock m = multi_block_of(s_start, n, vb);
+    const StreamArgs<real, S> &A = all[m.inst];
+    const int g = m.block * blockDim.x + threadIdx.x;
+    if (g >= A.G.n) continue;
+    int gx, y, z;
+    A.G.at(g, gx, y, z);
+    z += A.z0;
+    if constexpr (sizeof(S) == 2) {
+      if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z);
+      else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z);
     } else {
-      collide<real, false>(a, F, A.P);
-      collide<real, false>(b, F, A.P);
+      const int x0 = 2 * gx;
+      real a[Q], b[Q];
+      load_pair<real, S, false>(A.fin, A.P, x0, y, z, a, b);
+      if (A.force) collide_pair<true>(a, b, A.P);
+      else collide_pair<false>(a, b, A.P);
+      store_pair(A.fout, A.P, (size_t)z * A.P.nx * A.P.ny + (size_t)y * A.P.nx + x0, a, b);
     }
-    store_pair(A.fout, A.P, (size_t)z * A.P.nx * A.P.ny + (size_t)y * A.P.nx + x0, a, b);
-  }
   }
 }
 
@@ -1380,24 +1518,37 @@ __global__ void init_equilibrium_kernel(S *__restrict__ fstate, const LatParams<
   }
 }
 
+// Node groups of K1's direct kernels: pairs along x, four nodes with 16-bit storage.
+template <typename S>
+FlatGroups k1_groups(const Ctx &c) {
+  return flat_groups(c.nx / (sizeof(S) == 2 ? 4 : 2), c.ny, c.has_walls ? c.nz - 2 : c.nz);
+}
+
+// Threads per block of K1's flat kernels: what the tuner chose, as the threads of that many
+// lattice rows (whole warps, at most 128), else 128, or 64 with FP64 arithmetic, whose small
+// lattices spread more evenly over the SMs (the pass is bound by each SM's FP64 units).
+template <typename S>
+int k1_flat_threads(const Ctx &c, int per_row) {
+  if (c.k1_rows <= 0) return sizeof(S) == 8 ? 64 : 128;
+  const int t = (per_row * k1_block_rows(c) + 31) / 32 * 32;
+  return t < 128 ? t : 128;
+}
+
 template <typename S>
 cudaError_t stream_collide_quad_t(Ctx &c, int first, cudaStream_t st) {
   const LatParams<float> P = lat_params<float>(c);
   const int z0 = c.has_walls ? 1 : 0;
-  const int nzf = c.has_walls ? c.nz - 2 : c.nz;
-  const int quads = c.nx / 4;  // four nodes per thread along x
-  const int bx = quads < 128 ? quads : 128;
-  const int rows = k1_block_rows(c);
-  const dim3 grid((quads + bx - 1) / bx, c.ny / rows, nzf), block(bx, rows);
+  const FlatGroups G = k1_groups<S>(c);
+  const int block = k1_flat_threads<S>(c, G.per_row.d), grid = (G.n + block - 1) / block;
   const S *fin = (const S *)c.f[c.cur];
   S *fout = (S *)c.f[c.cur ^ 1];
   const bool force = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
   if (first) {
-    if (force) stream_collide_quad_kernel<S, true, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-    else stream_collide_quad_kernel<S, true, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
+    if (force) stream_collide_quad_kernel<S, true, true><<<grid, block, 0, st>>>(fin, fout, P, z0, G);
+    else stream_collide_quad_kernel<S, true, false><<<grid, block, 0, st>>>(fin, fout, P, z0, G);
   } else {
-    if (force) stream_collide_quad_kernel<S, false, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-    else stream_collide_quad_kernel<S, false, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
+    if (force) stream_collide_quad_kernel<S, false, true><<<grid, block, 0, st>>>(fin, fout, P, z0, G);
+    else stream_collide_quad_kernel<S, false, false><<<grid, block, 0, st>>>(fin, fout, P, z0, G);
   }
   return cudaGetLastError();
 }
@@ -1503,35 +1654,38 @@ cudaError_t stream_collide_t(Ctx &c, int first, cudaStream_t st) {
     const cudaError_t e = stream_collide_staged_t<real, S>(c, st, &used);
     if (used) return e;
   }
-  if constexpr (sizeof(S) == 2) return stream_collide_quad_t<S>(c, first, st);
-  const LatParams<real> P = lat_params<real>(c);
-  const int z0 = c.has_walls ? 1 : 0;
-  const int nzf = c.has_walls ? c.nz - 2 : c.nz;
-  const int half = c.nx / 2;  // two nodes per thread along x
-  const int bx = half < 128 ? half : 128;
-  const int rows = k1_block_rows(c);
-  const dim3 grid((half + bx - 1) / bx, c.ny / rows, nzf), block(bx, rows);
-  const S *fin = (const S *)c.f[c.cur];
-  S *fout = (S *)c.f[c.cur ^ 1];
-  const bool force = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
-  if (rows > 1) {
-    if (first) {
-      if (force) stream_collide_kernel<real, S, true, true, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-      else stream_collide_kernel<real, S, true, false, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-    } else {
-      if (force) stream_collide_kernel<real, S, false, true, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-      else stream_collide_kernel<real, S, false, false, true><<<grid, block, 0, st>>>(fin, fout, P, z0);
-    }
+  if constexpr (sizeof(S) == 2) {
+    return stream_collide_quad_t<S>(c, first, st);
   } else {
+    const LatParams<real> P = lat_params<real>(c);
+    const int z0 = c.has_walls ? 1 : 0;
+    const FlatGroups G = k1_groups<S>(c);
+    const int per_row = G.per_row.d;
+    // a block per row where a row is a whole number of warps, at least two of them, and of
+    // 128-thread blocks (it saves the flat form's index arithmetic), else the flat form
+    const bool rows = c.k1_rows <= 1 && (per_row <= 128 ? per_row >= 64 && per_row % 32 == 0
+                                                        : per_row % 128 == 0);
+    const int block = rows ? (per_row < 128 ? per_row : 128) : k1_flat_threads<S>(c, per_row);
+    const dim3 grid = rows ? dim3(per_row / block, c.ny, c.has_walls ? c.nz - 2 : c.nz)
+                           : dim3((G.n + block - 1) / block);
+    const S *fin = (const S *)c.f[c.cur];
+    S *fout = (S *)c.f[c.cur ^ 1];
+    const bool force = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
+    auto launch = [&](auto first_c, auto force_c, auto flat_c) {
+      stream_collide_kernel<real, S, decltype(first_c)::value, decltype(force_c)::value,
+                            decltype(flat_c)::value><<<grid, block, 0, st>>>(fin, fout, P, z0, G);
+    };
+    using T = std::true_type;
+    using F = std::false_type;
     if (first) {
-      if (force) stream_collide_kernel<real, S, true, true, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
-      else stream_collide_kernel<real, S, true, false, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
+      if (force) rows ? launch(T(), T(), F()) : launch(T(), T(), T());
+      else rows ? launch(T(), F(), F()) : launch(T(), F(), T());
     } else {
-      if (force) stream_collide_kernel<real, S, false, true, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
-      else stream_collide_kernel<real, S, false, false, false><<<grid, block, 0, st>>>(fin, fout, P, z0);
+      if (force) rows ? launch(F(), T(), F()) : launch(F(), T(), T());
+      else rows ? launch(F(), F(), F()) : launch(F(), F(), T());
     }
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 // Argument records of K1t and K1b for the step that starts from c's current state (K1t pulls
@@ -1585,8 +1739,7 @@ StreamArgs<real, S> stream_args(const Ctx &c) {
   a.fout = (S *)c.f[c.cur ^ 1];
   a.P = lat_params<real>(c);
   a.z0 = c.has_walls ? 1 : 0;
-  a.per_row = sizeof(S) == 2 ? c.nx / 4 : c.nx / 2;
-  a.ngroups = a.per_row * c.ny * (c.has_walls ? c.nz - 2 : c.nz);
+  a.G = k1_groups<S>(c);
   a.force = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
   return a;
 }
@@ -1619,7 +1772,7 @@ int lattice_multi_record_t(const Ctx &c, MultiKernel k, std::vector<unsigned cha
     case MK_STREAM_COLLIDE: {
       const StreamArgs<real, S> a = stream_args<real, S>(c);
       append_record(bytes, a);
-      const int b = (a.ngroups + 127) / 128;
+      const int b = (a.G.n + 127) / 128;
       return b < 1 ? 1 : b;
     }
     case MK_TILES: append_record(bytes, tiles_args<real, S>(c)); return tiles_blocks(c, true);
