@@ -64,8 +64,8 @@ typedef struct {
                               the GPU (green context); the stream-collide passes get the rest.
                               0: when the stream-collide pass moves at least 1 GiB
                               (2 x 19 x nx ny nz x storage bytes) 24, 40 with 16-bit
-                              storage and none with FP64; below that 64 (rounded to the device's
-                              partition granularity), < 0: no
+                              storage; below that 64 (rounded to the device's partition
+                              granularity); none with FP64 from 192 MiB up. < 0: no
                               partition (both share all SMs, interface stream at top priority).
                               If the device or driver cannot partition, no partition is used. */
   double tau;              /* BGK relaxation time, > 1/2 (viscosity (tau - 1/2)/3) */
