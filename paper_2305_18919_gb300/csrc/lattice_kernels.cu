@@ -288,6 +288,13 @@ __device__ __forceinline__ real dev_scattered(const S *__restrict__ p, int i, si
   return real(widen(ld_scattered(p + idx))) * real(kinv<S>(i));
 }
 
+// Single roundings that the compiler does not fuse, so that every kernel that collides a node
+// gives the same bits.
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+
 // Pull the 19 post-streaming populations of fluid node (x, y, z) from post-collision array
 // `fp`. A link whose source is a wall node is bounced back: the opposite post-collision
 // population of the same node plus the moving-wall term.
@@ -316,58 +323,52 @@ __device__ __forceinline__ void pull(const S *__restrict__ fp, const LatParams<r
     const size_t idx = bounce ? (size_t)opp(i) * P.ncell + n
                               : (size_t)i * P.ncell + zo[1 - cz(i)] + yo[1 - cy(i)] + xo[1 - cx(i)];
     f[i] = SCATTERED ? dev_scattered<real>(fp, i, idx) : dev<real>(fp, i, idx);
-    if (bounce) f[i] += cz(i) > 0 ? P.wb[i] : P.wt[i];
+    if (bounce) f[i] = add_(f[i], cz(i) > 0 ? P.wb[i] : P.wt[i]);
   }
 }
 
-// Interface force density of node (x, y, z) from the active-tile table (0 if inactive).
+// Force density (body force and interface) of the node pair (x0, x0 + 1) from the active-tile
+// table; the two nodes lie in one tile.
 template <typename real>
-__device__ __forceinline__ void tile_force(const int *__restrict__ tile_slot,
-                                           const Vec4<real> *__restrict__ Fslot,
-                                           const LatParams<real> &P, int x, int y, int z,
-                                           real F[3]) {
-  F[0] = P.g[0];
-  F[1] = P.g[1];
-  F[2] = P.g[2];
+__device__ __forceinline__ void tile_force_pair(const int *__restrict__ tile_slot,
+                                                const Vec4<real> *__restrict__ Fslot,
+                                                const LatParams<real> &P, int x0, int y, int z,
+                                                real Fa[3], real Fb[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; k++) Fa[k] = Fb[k] = P.g[k];
   if (tile_slot == nullptr) return;
-  const int t = ((z >> 2) * P.nty + (y >> 2)) * P.ntx + (x >> 2);
-  const int s = tile_slot[t];
-  if (s >= 0) {
-    const int cell = (x & 3) + 4 * (y & 3) + 16 * (z & 3);
-    const Vec4<real> Fs = Fslot[(size_t)s * TILE_CELLS + cell];
-    F[0] += Fs.x;
-    F[1] += Fs.y;
-    F[2] += Fs.z;
-  }
+  const int s = tile_slot[((z >> 2) * P.nty + (y >> 2)) * P.ntx + (x0 >> 2)];
+  if (s < 0) return;
+  const Vec4<real> *F = Fslot + (size_t)s * TILE_CELLS + (x0 & 3) + 4 * (y & 3) + 16 * (z & 3);
+  const Vec4<real> fa = F[0], fb = F[1];
+  Fa[0] += fa.x;
+  Fa[1] += fa.y;
+  Fa[2] += fa.z;
+  Fb[0] += fb.x;
+  Fb[1] += fb.y;
+  Fb[2] += fb.z;
 }
 
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 
-// Single roundings that the compiler does not fuse, so that every kernel that collides a node
-// gives the same bits.
-__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
-
 // 1/a and 1/b of two nodes' densities. FP64 divides cost an order of magnitude more than an
 // FP64 multiply-add, so the two share one reciprocal, 1/(ab), by Newton's iteration
 // r <- r + r (1 - x r) from a float seed (relative error 2^-23, then 2^-46, then rounding);
-// outside the seed's range it is a plain division. u enters the collision only at second order.
+// outside the seed's range they are plain divisions. u enters the collision only at second order.
 __device__ __forceinline__ void reciprocals(double a, double b, double &ra, double &rb) {
   const double x = mul_(a, b);
   const float s = (float)x;
-  double r;
   if (s > 1e-30f && s < 1e30f) {
-    r = (double)(1.0f / s);
+    double r = (double)(1.0f / s);
     r = fma(r, fma(-x, r, 1.0), r);
     r = fma(r, fma(-x, r, 1.0), r);
-  } else {
-    r = 1.0 / x;
+    ra = mul_(r, b);
+    rb = mul_(r, a);
+  } else {  // also a node whose density is zero or not finite: the other keeps its own
+    ra = 1.0 / a;
+    rb = 1.0 / b;
   }
-  ra = mul_(r, b);
-  rb = mul_(r, a);
 }
 
 // Density and momentum of a node's shifted populations: rho = rho0 + sum f, j = sum c f (the
@@ -514,8 +515,8 @@ __device__ __forceinline__ void load_pair(const S *__restrict__ fin, const LatPa
     if ((cz(i) > 0 && wall_below) || (cz(i) < 0 && wall_above)) {
       widen2(*reinterpret_cast<const V2 *>(fin + (size_t)opp(i) * P.ncell + n), a[i], b[i]);
       const real wall = cz(i) > 0 ? P.wb[i] : P.wt[i];
-      a[i] = a[i] * real(kinv<S>(opp(i))) + wall;
-      b[i] = b[i] * real(kinv<S>(opp(i))) + wall;
+      a[i] = add_(a[i] * real(kinv<S>(opp(i))), wall);
+      b[i] = add_(b[i] * real(kinv<S>(opp(i))), wall);
       continue;
     }
     const S *row = fin + (size_t)i * P.ncell + zo[1 - cz(i)] + yo[1 - cy(i)];
@@ -1444,40 +1445,172 @@ __global__ void __launch_bounds__(128) shell_velocity_kernel_multi(
   shell_body<real, S>(all[m.inst], m.block, m.nblocks);
 }
 
-// rho and u of every node of the current post-streaming state (read-back, not on the step).
-template <typename real, typename S>
-__global__ void fields_kernel(const S *__restrict__ fstate, int fresh,
-                              const int *__restrict__ tile_slot,
-                              const Vec4<real> *__restrict__ Fslot,
-                              const LatParams<real> P, double3 ub, double3 ut, double rho0,
-                              double *__restrict__ rho_out, double *__restrict__ u_out) {
-  const size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (n >= P.ncell) return;
-  const int x = (int)(n % P.nx), y = (int)((n / P.nx) % P.ny), z = (int)(n / ((size_t)P.nx * P.ny));
+// rho - rho0 and u of one node for the read-back, in double.
+//
+// FP64 contexts compute in double, with one residual correction of each quotient by the
+// reciprocal. Float contexts carry every value as an unevaluated pair of floats hi + lo: sums by
+// TwoSum (Knuth: the exact error of each addition, six float operations), quotients by one
+// residual step (Dekker), about 2^-45 of the value, and widen the pair once at the end. One FP64
+// operation takes the issue slots of 64 float operations on this GPU; in double, the sums and
+// quotients of a node took 18 times as long as its bytes.
+
+// (double)f by moving its bits: zeros and normal floats, the conversion instruction otherwise.
+__device__ __forceinline__ double widened(float f) {
+  const unsigned u = __float_as_uint(f), sign = u & 0x80000000u, mag = u ^ sign;
+  if (mag == 0u) return __hiloint2double((int)sign, 0);
+  if (mag - 0x00800000u >= 0x7f000000u) return (double)f;  // subnormal, infinite or NaN
+  return __hiloint2double((int)(sign | ((mag >> 3) + 0x38000000u)), (int)(mag << 29));
+}
+
+template <typename real>
+struct Pair;  // a value of the read-back's arithmetic
+template <>
+struct Pair<double> {
+  double v;
+  __device__ __forceinline__ explicit Pair(double f) : v(f) {}
+  __device__ __forceinline__ void add(double f) { v = add_(v, f); }
+  __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct Pair<float> {
+  float hi, lo;
+  __device__ __forceinline__ explicit Pair(float f, float e = 0.0f) : hi(f), lo(e) {}
+  __device__ __forceinline__ void add(float f) {
+    const float s = __fadd_rn(hi, f), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(f, b)));
+    hi = s;
+  }
+  __device__ __forceinline__ double value() const {  // (the error of inf is no number)
+    return isfinite(hi) ? widened(hi) + widened(lo) : (double)hi;
+  }
+};
+
+// u = j / (rho0 + drho) of the two nodes of a pair.
+__device__ __forceinline__ void field_quotients(const Pair<double> &ma, const Pair<double> &mb,
+                                                const Pair<double> ja[3], const Pair<double> jb[3],
+                                                double rho0, double ua[3], double ub[3]) {
+  const double ra = rho0 + ma.v, rb = rho0 + mb.v;
+  double ia, ib;
+  reciprocals(ra, rb, ia, ib);
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    ua[k] = mul_(ja[k].v, ia);
+    ub[k] = mul_(jb[k].v, ib);
+    // (no residual of an infinity; the exponent's bits cost no FP64 issue slot)
+    if ((__double2hiint(ua[k]) & 0x7ff00000) != 0x7ff00000)
+      ua[k] = fma(fma(-ua[k], ra, ja[k].v), ia, ua[k]);
+    if ((__double2hiint(ub[k]) & 0x7ff00000) != 0x7ff00000)
+      ub[k] = fma(fma(-ub[k], rb, jb[k].v), ib, ub[k]);
+  }
+}
+__device__ __forceinline__ void field_quotient(const Pair<float> &m, const Pair<float> j[3],
+                                               double rho0, double u[3]) {
+  const float r0 = (float)rho0, r0e = (float)(rho0 - (double)r0);
+  Pair<float> r(r0, __fadd_rn(r0e, m.lo));
+  r.add(m.hi);
+  const float rh = __fadd_rn(r.hi, r.lo), rl = __fsub_rn(r.lo, __fsub_rn(rh, r.hi));
+  const float inv = 1.0f / rh;
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const float jh = __fadd_rn(j[k].hi, j[k].lo);
+    const float jl = __fsub_rn(j[k].lo, __fsub_rn(jh, j[k].hi));
+    const float q = __fmul_rn(jh, inv);
+    // jh - q rh is a float (q is jh / rh to within two roundings), the fused form gives it
+    const float res = __fadd_rn(__fmaf_rn(-q, rh, jh), __fmaf_rn(-q, rl, jl));
+    u[k] = Pair<float>(q, __fmul_rn(res, inv)).value();
+  }
+}
+__device__ __forceinline__ void field_quotients(const Pair<float> &ma, const Pair<float> &mb,
+                                                const Pair<float> ja[3], const Pair<float> jb[3],
+                                                double rho0, double ua[3], double ub[3]) {
+  field_quotient(ma, ja, rho0, ua);
+  field_quotient(mb, jb, rho0, ub);
+}
+
+// drho and the momentum j (with half the force F) of one node; m and j hold f[0] and f[1], f[3],
+// f[5] on entry.
+__device__ __forceinline__ void field_sums(const double f[Q], const double F[3], Pair<double> &m,
+                                           Pair<double> j[3]) {
+  double jd[3];
+  node_moments(f, m.v, jd);
+#pragma unroll
+  for (int k = 0; k < 3; k++) j[k].v = F[k] != 0.0 ? fma(0.5, F[k], jd[k]) : jd[k];
+}
+__device__ __forceinline__ void field_sums(const float f[Q], const float F[3], Pair<float> &m,
+                                           Pair<float> j[3]) {
+#pragma unroll
+  for (int i = 1; i < Q; i++) {
+    m.add(f[i]);
+    if (cx(i) && i != 1) j[0].add(cx(i) > 0 ? f[i] : -f[i]);
+    if (cy(i) && i != 3) j[1].add(cy(i) > 0 ? f[i] : -f[i]);
+    if (cz(i) && i != 5) j[2].add(cz(i) > 0 ? f[i] : -f[i]);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+    if (F[k] != 0.0f) j[k].add(0.5f * F[k]);
+}
+
+// rho and u of every node of the current post-streaming state (read-back, not on the step). A
+// thread per node pair: the pair's populations as the stream-collide pass loads them, 16-byte
+// stores. 256^3 FP32: 0.370 ms (0.72 of the copy bandwidth) against 4.81 ms with a thread per
+// node in double; FP16 0.388 against 4.82; 128^3 FP64, bound by the FP64 units, 0.30 against 0.56.
+struct FieldsArgs {
+  double3 ub, ut;
+  double rho0;
+  double *rho, *u;
+};
+
+template <typename real, typename S, bool FRESH>
+__global__ void __launch_bounds__(128) fields_kernel(const S *__restrict__ fstate,
+                                                     const int *__restrict__ tile_slot,
+                                                     const Vec4<real> *__restrict__ Fslot,
+                                                     const LatParams<real> P, const FieldsArgs A,
+                                                     const FlatGroups G) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= G.n) return;
+  int x0, y, z;
+  G.at(g, x0, y, z);
+  x0 *= 2;
+  const size_t n = ((size_t)z * P.ny + y) * P.nx + x0;
+  double2 rho, u[3];
   if (P.has_walls && (z == 0 || z == P.nz - 1)) {
-    const double3 w = z == 0 ? ub : ut;
-    rho_out[n] = rho0;
-    u_out[3 * n] = w.x; u_out[3 * n + 1] = w.y; u_out[3 * n + 2] = w.z;
-    return;
-  }
-  real f[Q];
-  if (fresh) {
-    for (int i = 0; i < Q; i++) f[i] = dev<real>(fstate, i, (size_t)i * P.ncell + n);
+    const double3 w = z == 0 ? A.ub : A.ut;
+    rho = make_double2(A.rho0, A.rho0);
+    u[0] = make_double2(w.x, w.y);
+    u[1] = make_double2(w.z, w.x);
+    u[2] = make_double2(w.y, w.z);
   } else {
-    pull(fstate, P, x, y, z, f);
+    real a[Q], b[Q];
+    load_pair<real, S, FRESH>(fstate, P, x0, y, z, a, b);
+    real Fa[3], Fb[3];
+    tile_force_pair(tile_slot, Fslot, P, x0, y, z, Fa, Fb);
+    Pair<real> ma(a[0]), mb(b[0]);
+    Pair<real> ja[3] = {Pair<real>(a[1]), Pair<real>(a[3]), Pair<real>(a[5])};
+    Pair<real> jb[3] = {Pair<real>(b[1]), Pair<real>(b[3]), Pair<real>(b[5])};
+    field_sums(a, Fa, ma, ja);
+    field_sums(b, Fb, mb, jb);
+    double ua[3], ub[3];
+    field_quotients(ma, mb, ja, jb, A.rho0, ua, ub);
+    rho = make_double2(A.rho0 + ma.value(), A.rho0 + mb.value());
+    u[0] = make_double2(ua[0], ua[1]);
+    u[1] = make_double2(ua[2], ub[0]);
+    u[2] = make_double2(ub[1], ub[2]);
   }
-  double drho = 0, j[3] = {0, 0, 0};
-  for (int i = 0; i < Q; i++) {
-    drho += (double)f[i];
-    j[0] += cx(i) * (double)f[i];
-    j[1] += cy(i) * (double)f[i];
-    j[2] += cz(i) * (double)f[i];
+  // the caller's buffers are doubles: 16-byte stores where they are aligned to them
+  double *ro = A.rho + n, *uo = A.u + 3 * n;
+  if ((((size_t)A.rho | (size_t)A.u) & 15) == 0) {
+    *reinterpret_cast<double2 *>(ro) = rho;
+#pragma unroll
+    for (int k = 0; k < 3; k++) reinterpret_cast<double2 *>(uo)[k] = u[k];
+  } else {
+    ro[0] = rho.x;
+    ro[1] = rho.y;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      uo[2 * k] = u[k].x;
+      uo[2 * k + 1] = u[k].y;
+    }
   }
-  real F[3];
-  tile_force(tile_slot, Fslot, P, x, y, z, F);
-  const double rho = rho0 + drho;
-  rho_out[n] = rho;
-  for (int k = 0; k < 3; k++) u_out[3 * n + k] = (j[k] + 0.5 * (double)F[k]) / rho;
 }
 
 template <typename real, typename S>
@@ -1822,14 +1955,21 @@ size_t lattice_record_align_t(MultiKernel k) {
 
 template <typename real, typename S>
 cudaError_t fields_t(Ctx &c, double *rho_dev, double *u_dev) {
-  const int blocks = (int)((c.ncell + 255) / 256);
-  const double3 ub = make_double3(c.ub[0], c.ub[1], c.ub[2]);
-  const double3 ut = make_double3(c.ut[0], c.ut[1], c.ut[2]);
+  const FlatGroups G = flat_groups(c.nx / 2, c.ny, c.nz);
+  const int block = 128, grid = (G.n + block - 1) / block;
+  FieldsArgs A;
+  A.ub = make_double3(c.ub[0], c.ub[1], c.ub[2]);
+  A.ut = make_double3(c.ut[0], c.ut[1], c.ut[2]);
+  A.rho0 = c.rho0;
+  A.rho = rho_dev;
+  A.u = u_dev;
   // the force of the last spreading step lives in the map that step used
   const int *ts = (c.nv && c.have_force) ? c.tile_slot[c.map ^ 1] : nullptr;
-  fields_kernel<real, S><<<blocks, 256, 0, c.stream>>>(
-      (const S *)c.f[c.cur], c.fresh, ts, (const Vec4<real> *)c.Fslot[c.map ^ 1],
-      lat_params<real>(c), ub, ut, c.rho0, rho_dev, u_dev);
+  const S *f = (const S *)c.f[c.cur];
+  const Vec4<real> *F = (const Vec4<real> *)c.Fslot[c.map ^ 1];
+  const LatParams<real> P = lat_params<real>(c);
+  if (c.fresh) fields_kernel<real, S, true><<<grid, block, 0, c.stream>>>(f, ts, F, P, A, G);
+  else fields_kernel<real, S, false><<<grid, block, 0, c.stream>>>(f, ts, F, P, A, G);
   return cudaGetLastError();
 }
 
