@@ -362,7 +362,7 @@ void iblb_destroy(iblb_ctx *h) {
     dfree(c.out_src[b]);
     dfree(c.Fslot[b]);
   }
-  dfree(c.counters); dfree(c.slot_count); dfree(c.src_index); dfree(c.Rslot); dfree(c.bucket); dfree(c.spill_bits); dfree(c.Uslot); dfree(c.pair_list);
+  dfree(c.counters); dfree(c.slot_count); dfree(c.src_slot); dfree(c.Rslot); dfree(c.bucket); dfree(c.spill_bits); dfree(c.Uslot); dfree(c.pair_list);
   dfree(c.q); dfree(c.qdot); dfree(c.faces); dfree(c.fref); dfree(c.xref); dfree(c.fgeo); dfree(c.vcoef); dfree(c.disp); dfree(c.vf_start); dfree(c.vf_list);
   dfree(c.fcontrib); dfree(c.fnorm); dfree(c.vol_partial); dfree(c.phi); dfree(c.gvol); dfree(c.stencil);
   dfree(c.dscratch);
@@ -426,7 +426,8 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   c.nf = nf;
   c.V0 = V0;
   for (int k = 0; k < 3; k++) c.centre[k] = centre[k];
-  c.vol_blocks = (nf + 255) / 256;  // one partial volume change per face block
+  const int ft = iblb::face_block_threads(c.precision);
+  c.vol_blocks = (nf + ft - 1) / ft;  // one partial volume change per face block
   const size_t rs = c.real_size;
   long ms = 8L * nv;
   if ((size_t)ms > c.ntiles) ms = (long)c.ntiles;
@@ -446,10 +447,11 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   CUDA_TRY(c, dalloc_bytes(&c.fgeo, (size_t)16 * nf * rs));
   CUDA_TRY(c, dalloc_bytes(&c.vcoef, sizeof(double)));
   CUDA_TRY(c, dalloc_bytes(&c.disp, (size_t)4 * nv * rs));
+  CUDA_TRY(c, cudaMemsetAsync(c.disp, 0, (size_t)4 * nv * rs, c.stream));
   CUDA_TRY(c, dalloc(&c.vf_start, (size_t)nv + 1));
   CUDA_TRY(c, dalloc(&c.vf_list, (size_t)3 * nf));
-  CUDA_TRY(c, dalloc_bytes(&c.fcontrib, (size_t)9 * nf * rs));
-  CUDA_TRY(c, dalloc_bytes(&c.fnorm, (size_t)3 * nf * rs));
+  CUDA_TRY(c, dalloc_bytes(&c.fcontrib, (size_t)12 * nf * rs));
+  CUDA_TRY(c, dalloc_bytes(&c.fnorm, (size_t)4 * nf * rs));
   CUDA_TRY(c, dalloc(&c.vol_partial, (size_t)c.vol_blocks));
   CUDA_TRY(c, dalloc_bytes(&c.phi, (size_t)4 * nv * rs));
   CUDA_TRY(c, dalloc_bytes(&c.gvol, (size_t)4 * nv * rs));
@@ -463,8 +465,8 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   }
   CUDA_TRY(c, dalloc(&c.slot_count, (size_t)c.max_slots));
   CUDA_TRY(c, dalloc(&c.pair_list, (size_t)32 * c.max_slots));
-  CUDA_TRY(c, dalloc(&c.src_index, (size_t)c.max_slots));
   c.max_sources = nv < c.max_slots ? nv : c.max_slots;  // a source tile holds >= 1 vertex base
+  CUDA_TRY(c, dalloc(&c.src_slot, (size_t)c.max_sources));
   CUDA_TRY(c, dalloc_bytes(&c.Rslot, (size_t)c.max_sources * 343 * 4 * rs));
   CUDA_TRY(c, dalloc(&c.bucket, (size_t)c.max_slots * iblb::BUCKET_CAP));
   c.spill_words = (nv + 31) / 32;

@@ -31,12 +31,28 @@ Dims dims_of(const Ctx &c) {
   return d;
 }
 
-__device__ __forceinline__ int floor_div4(int a) { return a >> 2; }  // arithmetic shift floors
+// i reduced to [0, n).
+__device__ __forceinline__ int wrap_index(int i, int n) {
+  if ((unsigned)i >= (unsigned)n) {
+    i += i < 0 ? n : -n;
+    if ((unsigned)i >= (unsigned)n) {  // positions are stored unwrapped
+      i %= n;
+      i += i < 0 ? n : 0;
+    }
+  }
+  return i;
+}
 
-// p reduced to [0, n) for a periodic axis (positions are stored unwrapped); inv_n = 1/n, so
-// no double division is issued (slow on this part). Rounding may leave p at -tiny or n.
-__device__ __forceinline__ double wrap_pos(double p, int n, double inv_n) {
-  return p - n * floor(p * inv_n);
+// Base node floor(p) - 1 of the delta stencil of coordinate p on an axis of n nodes, and
+// r = p - floor(p). Periodic axes: the base in [0, n); a walled axis: not wrapped. Integer work
+// but for one conversion each way and one subtraction (FP64 issues at 1/64 of the FP32 rate);
+// the stencil and the tile marking take the same base.
+__device__ __forceinline__ int stencil_base(double p, int n, double inv_n, bool periodic, double &r) {
+  if ((__double2hiint(p) & 0x7fffffff) >= 0x41d00000)  // |p| >= 2^30 or no number
+    p = periodic ? p - n * floor(p * inv_n) : fmin(fmax(p, -8.0), n + 8.0);
+  const int i = __double2int_rd(p);
+  r = p - (double)i;
+  return periodic ? wrap_index(i - 1, n) : i - 1;
 }
 
 __device__ __forceinline__ float log_(float v) { return logf(v); }
@@ -87,7 +103,7 @@ struct FaceArgs {
   const int *faces;
   const Vec4<real> *disp;
   const real *fgeo;
-  real *fcontrib, *fnorm;
+  Vec4<real> *fcontrib, *fnorm;
   double *vol_partial;
   FaceParams<real> fp;
   Dims D;
@@ -99,6 +115,16 @@ struct FaceArgs {
   int spill_words;
 };
 
+// Threads per block of K3a and K3b: few, so that a mesh of some thousand faces and vertices
+// spreads over all SMs of the chain (each SM's FP64 unit and each warp's chain of loads, not
+// memory, set their time). K3b with its loads a vector each, 10242 vertices on 64 SMs: 9.3 us
+// against 10.8 with 256-thread blocks; 40962 on 24 SMs: 30 against 40; K3a there 19 against 27.
+template <typename real>
+struct FaceThreads {
+  static constexpr int value = sizeof(real) == 4 ? 128 : 64;
+};
+constexpr int kVertexThreads = 64;
+
 // K3a for block `bid` of `nb` (the single-context kernel and the batched one share it).
 template <typename real>
 __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int nb) {
@@ -106,12 +132,12 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int 
   const int *__restrict__ faces = A.faces;
   const Vec4<real> *__restrict__ disp = A.disp;
   const real *__restrict__ fgeo = A.fgeo;
-  real *__restrict__ fcontrib = A.fcontrib;
-  real *__restrict__ fnorm = A.fnorm;
+  Vec4<real> *__restrict__ fcontrib = A.fcontrib;
+  Vec4<real> *__restrict__ fnorm = A.fnorm;
   double *__restrict__ vol_partial = A.vol_partial;
   const FaceParams<real> fp = A.fp;
   const Dims D = A.D;
-  __shared__ double warp_sum[8];
+  __shared__ double warp_sum[FaceThreads<real>::value / 32];
   const int j = bid * blockDim.x + threadIdx.x;
   real dvj = 0;
   if (j < nf) {
@@ -144,16 +170,17 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int 
     const real G22 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
     const real detG = G11 * G22 - G12 * G12;
     const real L = log_(detG / (real(4) * A0 * A0));  // log(I2 + 1), det G0 = 4 A0^2
-    const real dE_dI1 = real(0.5) * fp.a3 * A0;
-    const real dE_dL = A0 * (fp.cL0 + fp.cL1 * L);
-    const real inv_detG = real(1) / detG;
+    // dE/da = paa a + pab b and dE/db = pab a + pbb b, with I1 = H11 G11 + 2 H12 G12 + H22 G22 - 2
+    // and L = log det G + const
+    const real eI = fp.a3 * A0;                                          // 2 dE/dI1
+    const real eL = real(2) * A0 * (fp.cL0 + fp.cL1 * L) / detG;          // 2 dE/dL / det G
+    const real paa = eI * H11 + eL * G22;
+    const real pab = eI * H12 - eL * G12;
+    const real pbb = eI * H22 + eL * G11;
     real f0[3], f1[3], f2[3];
     for (int k = 0; k < 3; k++) {
-      // dE/da and dE/db with I1 = H11 G11 + 2 H12 G12 + H22 G22 - 2, L = log det G + const
-      const real ga = dE_dI1 * real(2) * (H11 * a[k] + H12 * b[k]) +
-                      dE_dL * real(2) * (a[k] * G22 - G12 * b[k]) * inv_detG;
-      const real gb = dE_dI1 * real(2) * (H12 * a[k] + H22 * b[k]) +
-                      dE_dL * real(2) * (b[k] * G11 - G12 * a[k]) * inv_detG;
+      const real ga = paa * a[k] + pab * b[k];
+      const real gb = pab * a[k] + pbb * b[k];
       f1[k] = -ga;
       f2[k] = -gb;
       f0[k] = ga + gb;
@@ -169,12 +196,10 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int 
       f1[2] += third;
       f2[2] += third;
     }
-    real *fc = fcontrib + 9 * (size_t)j;
-    for (int k = 0; k < 3; k++) {
-      fc[k] = f0[k];
-      fc[3 + k] = f1[k];
-      fc[6 + k] = f2[k];
-    }
+    Vec4<real> *fc = fcontrib + 3 * (size_t)j;
+    fc[0] = Vec4<real>{f0[0], f0[1], f0[2], real(0)};
+    fc[1] = Vec4<real>{f1[0], f1[1], f1[2], real(0)};
+    fc[2] = Vec4<real>{f2[0], f2[1], f2[2], real(0)};
     // For a closed surface the gradient of V at vertex i does not depend on the point about
     // which the tetrahedra are taken; with that point at x_i every face around i contributes
     // (a x b)/6, the same edge cross product for all three corners.
@@ -184,10 +209,7 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int 
                        da[2] * b[0] - da[0] * b[2] + A[2] * db[0] - A[0] * db[2],
                        da[0] * b[1] - da[1] * b[0] + A[0] * db[1] - A[1] * db[0]};
     const real sixth = real(1.0 / 6.0);
-    real *fn = fnorm + 3 * (size_t)j;
-    fn[0] = n[0] * sixth;
-    fn[1] = n[1] * sixth;
-    fn[2] = n[2] * sixth;
+    fnorm[j] = Vec4<real>{n[0] * sixth, n[1] * sixth, n[2] * sixth, real(0)};
     dvj = (u[0][0] * n[0] + u[0][1] * n[1] + u[0][2] * n[2] + X0c[0] * m[0] + X0c[1] * m[1] +
            X0c[2] * m[2]) * sixth;
   }
@@ -216,13 +238,13 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int bid, int 
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) face_kernel(const FaceArgs<real> A) {
+__global__ void __launch_bounds__(FaceThreads<real>::value) face_kernel(const FaceArgs<real> A) {
   face_body(A, blockIdx.x, gridDim.x);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) face_kernel_multi(const FaceArgs<real> *__restrict__ all,
-                                                         const int *__restrict__ start, int n) {
+__global__ void __launch_bounds__(FaceThreads<real>::value) face_kernel_multi(
+    const FaceArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   face_body(all[m.inst], m.block, m.nblocks);
 }
@@ -231,8 +253,14 @@ __global__ void __launch_bounds__(256) face_kernel_multi(const FaceArgs<real> *_
 // also returns V.
 __device__ __forceinline__ double volume_coef(const double *__restrict__ part, int n, double V0,
                                               double kV, int volume_on, double *V_out) {
-  double dv = 0.0;
-  for (int k = threadIdx.x & 31; k < n; k += 32) dv += part[k];
+  double s[4] = {0.0, 0.0, 0.0, 0.0};  // four chains of additions per lane
+  for (int k0 = 0; k0 < n; k0 += 128)
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const int k = k0 + 32 * c + (threadIdx.x & 31);
+      if (k < n) s[c] += part[k];
+    }
+  double dv = (s[0] + s[1]) + (s[2] + s[3]);
   for (int o = 16; o > 0; o >>= 1) dv += __shfl_down_sync(0xffffffffu, dv, o);
   dv = __shfl_sync(0xffffffffu, dv, 0);
   if (V_out) *V_out = V0 + dv;
@@ -243,10 +271,7 @@ __device__ __forceinline__ double volume_coef(const double *__restrict__ part, i
 // With r = p - floor(p) and s = sqrt(1 + 4r - 4r^2) the four branches reduce to
 // (3-2r-s)/8, (3-2r+s)/8, (1+2r+s)/8, (1+2r-s)/8, which sum to one.
 template <typename real>
-__device__ __forceinline__ void peskin_weights(double p, int &base, real w[4]) {
-  const double fl = floor(p);
-  base = (int)fl - 1;
-  const real r = (real)(p - fl);
+__device__ __forceinline__ void peskin_weights(real r, real w[4]) {
   const real s = sqrt_(real(1) + real(4) * r - real(4) * r * r);
   w[0] = (real(3) - real(2) * r - s) * real(0.125);
   w[1] = (real(3) - real(2) * r + s) * real(0.125);
@@ -271,13 +296,13 @@ template <typename real>
 struct VertexArgs {
   int nv;
   const int *vf_start, *vf_list;
-  const real *fcontrib, *fnorm;
+  const Vec4<real> *fcontrib, *fnorm;
   const double *q;
   Vec4<real> *phi, *gvol;
   StencilRec<real> *stencil;
   int bin;
   const int *tile_slot;
-  int *slot_count, *bucket, *ovf_count, *src_index, *nsources, *health, *zero_counter;
+  int *slot_count, *bucket, *ovf_count, *src_slot, *nsources, *health, *zero_counter;
   unsigned *spill_bits;  // bit i: vertex i did not fit in its tile's bucket
   const double *vol_partial;  // per-block V_j - V0_j partials of the face kernel
   VolumeParams vp;
@@ -290,14 +315,14 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
   const int nv = A.nv;
   const int *__restrict__ vf_start = A.vf_start;
   const int *__restrict__ vf_list = A.vf_list;
-  const real *__restrict__ fcontrib = A.fcontrib;
-  const real *__restrict__ fnorm = A.fnorm;
+  const Vec4<real> *__restrict__ fcontrib = A.fcontrib;
+  const Vec4<real> *__restrict__ fnorm = A.fnorm;
   const double *__restrict__ q = A.q;
   const int bin = A.bin;
   const Dims D = A.D;
-  const int i = bid * blockDim.x + threadIdx.x;
-  if (bid == 0 && threadIdx.x == 0 && A.zero_counter) *A.zero_counter = 0;
-  if (bid == 0 && threadIdx.x < 32) {
+  if (bid == 0) {  // the first block has no vertices
+    if (threadIdx.x == 32 && A.zero_counter) *A.zero_counter = 0;
+    if (threadIdx.x >= 32) return;
     // the volume-force coefficient of the step, once (the spreading pass reads it), and the
     // volume health check
     double V;
@@ -307,9 +332,14 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
       *A.vcoef = coef;
       if (!(fabs(V / A.vp.V0 - 1.0) <= 0.05)) atomicOr(A.health, H_VOLUME);
     }
+    return;
   }
+  const int i = (bid - 1) * blockDim.x + threadIdx.x;
   if (i >= nv) return;
   const int e0 = vf_start[i], e1 = vf_start[i + 1];
+  double p[3] = {0, 0, 0};
+  if (bin)
+    for (int k = 0; k < 3; k++) p[k] = q[3 * (size_t)i + k];
   real F[3] = {0, 0, 0}, g[3] = {0, 0, 0};
   for (int eb = e0; eb < e1; eb += GATHER_UNROLL) {
     int fcs[GATHER_UNROLL];
@@ -318,12 +348,14 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
 #pragma unroll
     for (int u = 0; u < GATHER_UNROLL; u++) {
       if (fcs[u] < 0) continue;
-      const int fc = fcs[u];  // face * 3 + corner
-      const int f = fc / 3;
-      for (int k = 0; k < 3; k++) {
-        F[k] += fcontrib[3 * (size_t)fc + k];
-        g[k] += fnorm[3 * (size_t)f + k];
-      }
+      const Vec4<real> fc = fcontrib[fcs[u]];   // face * 3 + corner
+      const Vec4<real> fn = fnorm[fcs[u] / 3];
+      F[0] += fc.x;
+      F[1] += fc.y;
+      F[2] += fc.z;
+      g[0] += fn.x;
+      g[1] += fn.y;
+      g[2] += fn.z;
     }
   }
   Vec4<real> pv, gv;
@@ -333,14 +365,11 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
   A.gvol[i] = gv;
   if (!bin) return;
   StencilRec<real> rec;
-  peskin_weights<real>(wrap_pos(q[3 * (size_t)i], D.nx, D.inx), rec.base[0], rec.w[0]);
-  peskin_weights<real>(wrap_pos(q[3 * (size_t)i + 1], D.ny, D.iny), rec.base[1], rec.w[1]);
-  const double pz = q[3 * (size_t)i + 2];
-  peskin_weights<real>(D.has_walls ? pz : wrap_pos(pz, D.nz, D.inz), rec.base[2], rec.w[2]);
-  // base in [-2, n - 1] on the periodic axes (rounding of the wrap): bring it into [0, n)
-  if (rec.base[0] < 0) rec.base[0] += D.nx;
-  if (rec.base[1] < 0) rec.base[1] += D.ny;
-  if (!D.has_walls && rec.base[2] < 0) rec.base[2] += D.nz;
+  double r[3];
+  rec.base[0] = stencil_base(p[0], D.nx, D.inx, true, r[0]);
+  rec.base[1] = stencil_base(p[1], D.ny, D.iny, true, r[1]);
+  rec.base[2] = stencil_base(p[2], D.nz, D.inz, !D.has_walls, r[2]);
+  for (int k = 0; k < 3; k++) peskin_weights<real>((real)r[k], rec.w[k]);
   rec.pad = 0;
   A.stencil[i] = rec;
   const int bz = min(max(rec.base[2], 0), D.nz - 1);
@@ -351,7 +380,7 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
     return;
   }
   const int rank = atomicAdd(&A.slot_count[s], 1);
-  if (rank == 0) A.src_index[s] = atomicAdd(A.nsources, 1);  // first vertex: the tile gets a region
+  if (rank == 0) A.src_slot[atomicAdd(A.nsources, 1)] = s;  // first vertex: the tile gets a region
   if (rank < BUCKET_CAP) {
     A.bucket[(size_t)s * BUCKET_CAP + rank] = i;
   } else {
@@ -363,12 +392,12 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int bid) 
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) vertex_kernel(const VertexArgs<real> A) {
+__global__ void __launch_bounds__(kVertexThreads) vertex_kernel(const VertexArgs<real> A) {
   vertex_body(A, blockIdx.x);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) vertex_kernel_multi(
+__global__ void __launch_bounds__(kVertexThreads) vertex_kernel_multi(
     const VertexArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   vertex_body(all[m.inst], m.block);
@@ -378,11 +407,9 @@ __global__ void __launch_bounds__(256) vertex_kernel_multi(
 // node in S) cover the 7x7x7 nodes S_lo .. S_lo + 6.
 constexpr int REGION = 7;
 constexpr int REGION_NODES = REGION * REGION * REGION;
-// Source tiles per block of K4a (shared memory per warp: the region and the staged records).
-template <typename real>
-struct SrcWarps {
-  static constexpr int value = sizeof(real) == 4 ? 4 : 2;
-};
+// Threads per block of K4a: one block per source tile, one bucket entry per thread.
+constexpr int kSourceThreads = BUCKET_CAP;
+static_assert(kSourceThreads == 128, "four warps: one per z plane of a stencil");
 
 // w[d] for a run-time d in 0..3 without indexing a local array.
 template <typename real>
@@ -390,21 +417,26 @@ __device__ __forceinline__ real pick4(const real w[4], int d) {
   return d == 0 ? w[0] : d == 1 ? w[1] : d == 2 ? w[2] : w[3];
 }
 
-// K4a: spreading, first pass (Eq. 13). One warp per source tile S: its bucket is sorted by
-// vertex index (rank by comparison, at most 64 entries), the vertices' stencil records and
-// forces (completed with the volume term -kV (V - V0)/V0 dV/dq) are staged in shared memory,
-// and the vertices are then added one after another into the 7x7x7 region of S, each lane
-// adding two of the 64 stencil nodes of a vertex (distinct nodes, so no atomics). The region
-// is written out and its index pushed to the (up to 8) tiles T = S + {0,1}^3 it overlaps.
-// A tile with more than 64 vertices (its bucket holds 64 of them, chosen by the order of the
+// K4a: spreading, first pass (Eq. 13). One block of four warps per source tile S: its bucket is
+// sorted by vertex index (rank by comparison, at most 128 entries) and the vertices' stencil
+// records and forces (completed with the volume term -kV (V - V0)/V0 dV/dq) are staged in shared
+// memory in that order. Of the 7x7x7 region of S warp w owns the z planes w and w + 4, of which
+// every vertex's stencil covers exactly one; a half warp adds the 16 nodes of that plane, the
+// lower half for the even vertices, the upper half for the odd ones into a copy of its own (no
+// atomics, no waiting between warps). The two copies are added and written out, and the region's
+// index is pushed to the (up to 8) tiles T = S + {0,1}^3 it overlaps. The time is the chain of
+// additions into shared memory, a quarter as long as with one warp per tile, whose lanes added two
+// nodes of every vertex one vertex after the other (10242 vertices on 64 SMs: 9.3 us against 12.5;
+// 96 wetting boxes 134 us against 180; 40962 vertices on 24 SMs, where the SMs are full: 89 both).
+// A tile with more than 128 vertices (its bucket holds 128 of them, chosen by the order of the
 // binning atomics) marks its bucket's vertices in the spill bitmap, which already holds its
 // spilled ones, and adds all of its vertices in increasing vertex index instead, found by a
 // scan of the bitmap. Either way the order of summation depends only on the vertex set.
 template <typename real>
 struct SourceArgs {
-  const int *tile_slot, *slot_tile, *nslots_ptr, *slot_count, *src_index, *bucket;
+  const int *tile_slot, *slot_tile, *nsources_ptr, *slot_count, *src_slot, *bucket;
   unsigned *spill_bits;
-  int spill_words;
+  int spill_words, max_sources;
   const StencilRec<real> *stencil;
   const Vec4<real> *phi, *gvol;
   const real *vcoef;  // kV (V - V0)/V0, written by the vertex kernel of the step
@@ -413,12 +445,30 @@ struct SourceArgs {
   Dims D;
 };
 
+// One vertex's plane of nodes added by a half warp: base (bx, by, bz) in the region, weights w
+// (x, y, z), force f. Lane l of the half owns the node (l & 3, l >> 2) of the plane.
+template <typename real>
+__device__ __forceinline__ void add_plane(Vec4<real> *region, int plane, int l, int bx, int by,
+                                          int bz, const real *wx, const real *wy, const real *wz,
+                                          real fx, real fy, real fz) {
+  const int dz = (plane - bz) & 3, rz = bz + dz;  // the stencil's plane that this warp owns
+  if (rz < 0 || rz >= REGION) return;             // beyond the lattice in z
+  const int dx = l & 3, dy = l >> 2;
+  const real w = wx[dx] * wy[dy] * wz[dz];
+  Vec4<real> &o = region[(rz * REGION + by + dy) * REGION + bx + dx];
+  Vec4<real> v = o;
+  v.x += w * fx;
+  v.y += w * fy;
+  v.z += w * fz;
+  v.w = real(1);  // a stencil node of some vertex (the interpolation reads it)
+  o = v;
+}
+
 template <typename real>
 __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, int bid, int nb) {
   const int *__restrict__ tile_slot = A.tile_slot;
   const int *__restrict__ slot_tile = A.slot_tile;
   const int *__restrict__ slot_count = A.slot_count;
-  const int *__restrict__ src_index = A.src_index;
   const int *__restrict__ bucket = A.bucket;
   unsigned *spill_bits = A.spill_bits;
   const StencilRec<real> *__restrict__ stencil = A.stencil;
@@ -426,28 +476,29 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, in
   const Vec4<real> *__restrict__ gvol = A.gvol;
   int *__restrict__ out_src = A.out_src;
   const Dims D = A.D;
-  constexpr int W = SrcWarps<real>::value;
-  __shared__ Vec4<real> s_region[W][REGION_NODES];
-  __shared__ real s_w[W][BUCKET_CAP][12];
-  __shared__ Vec4<real> s_f[W][BUCKET_CAP];
-  __shared__ int s_b[W][BUCKET_CAP][3];
-  const int nslots = min(*A.nslots_ptr, D.max_slots);
-  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  __shared__ Vec4<real> s_region[2][REGION_NODES];
+  __shared__ real s_w[BUCKET_CAP][12];
+  __shared__ Vec4<real> s_f[BUCKET_CAP];
+  __shared__ int s_b[BUCKET_CAP];
+  __shared__ int s_v[BUCKET_CAP];
+  const int nsources = min(*A.nsources_ptr, A.max_sources);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int half = lane >> 4, l16 = lane & 15;
   const real coef = *A.vcoef;
-  Vec4<real> *region = s_region[wq];
-  // the two stencil nodes of this lane
-  const int dxa = lane & 3, dya = (lane >> 2) & 3, dza = lane >> 4;  // node lane; node lane + 32
-  for (int s = bid * W + wq; s < nslots; s += nb * W) {
+  for (int reg = bid; reg < nsources; reg += nb) {
+    const int s = A.src_slot[reg];
     const int cnt = slot_count[s];
-    if (cnt == 0) continue;  // no vertex has its base node here: no region
-    const int n = min(cnt, BUCKET_CAP);
     const int t = slot_tile[s];
+    const int *bk = bucket + (size_t)s * BUCKET_CAP;
+    const int v = tid < cnt ? bk[tid] : 0x7fffffff;
+    for (int k = tid; k < 2 * REGION_NODES; k += kSourceThreads)
+      s_region[0][k] = Vec4<real>{0, 0, 0, 0};
     const int tsx = t % D.ntx, tsy = (t / D.ntx) % D.nty, tsz = t / (D.ntx * D.nty);
     const int Sx = tsx * TILE, Sy = tsy * TILE, Sz = tsz * TILE;
-    const int reg = src_index[s];
     // push the region to the tiles it overlaps: T = S + e, seen from T as source e
-    if (lane < 8) {
-      int ux = tsx + (lane & 1), uy = tsy + ((lane >> 1) & 1), uz = tsz + (lane >> 2);
+    if (tid >= kSourceThreads - 8) {
+      const int e = tid & 7;
+      int ux = tsx + (e & 1), uy = tsy + ((e >> 1) & 1), uz = tsz + (e >> 2);
       ux = ux >= D.ntx ? ux - D.ntx : ux;
       uy = uy >= D.nty ? uy - D.nty : uy;
       bool ok = true;
@@ -457,63 +508,52 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, in
       }
       if (ok) {
         const int slot_t = tile_slot[(uz * D.nty + uy) * D.ntx + ux];
-        if (slot_t >= 0) out_src[8 * (size_t)slot_t + lane] = reg;
+        if (slot_t >= 0) out_src[8 * (size_t)slot_t + e] = reg;
       }
     }
-    const int *bk = bucket + (size_t)s * BUCKET_CAP;
     if (cnt <= BUCKET_CAP) {
       // sort the bucket by vertex index and stage the records in that order
-      const int v0 = lane < n ? bk[lane] : 0x7fffffff;
-      const int v1 = lane + 32 < n ? bk[lane + 32] : 0x7fffffff;
-      int r0 = 0, r1 = 0;
-      for (int m = 0; m < n; m++) {
-        const int vm = __shfl_sync(0xffffffffu, m < 32 ? v0 : v1, m & 31);
-        r0 += vm < v0;
-        r1 += vm < v1;
+      StencilRec<real> rec;
+      Vec4<real> pv, gv;
+      s_v[tid] = v;
+      if (tid < cnt) {
+        rec = stencil[v];
+        pv = phi[v];
+        gv = gvol[v];
       }
-      for (int h = 0; h < 2; h++) {
-        const int v = h ? v1 : v0;
-        const int r = h ? r1 : r0;
-        if ((h ? lane + 32 : lane) >= n) continue;
-        const StencilRec<real> rec = stencil[v];
-        const Vec4<real> pv = phi[v], gv = gvol[v];
+      __syncthreads();
+      if (tid < cnt) {
+        int r = 0;
+        for (int m = 0; m < cnt; m++) r += s_v[m] < v;
         for (int k = 0; k < 4; k++) {
-          s_w[wq][r][k] = rec.w[0][k];
-          s_w[wq][r][4 + k] = rec.w[1][k];
-          s_w[wq][r][8 + k] = rec.w[2][k];
+          s_w[r][k] = rec.w[0][k];
+          s_w[r][4 + k] = rec.w[1][k];
+          s_w[r][8 + k] = rec.w[2][k];
         }
-        s_f[wq][r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
-        // base relative to S_lo (x, y wrapped into [0, n) by the vertex kernel)
-        s_b[wq][r][0] = rec.base[0] - Sx;
-        s_b[wq][r][1] = rec.base[1] - Sy;
-        s_b[wq][r][2] = rec.base[2] - Sz;
+        s_f[r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
+        // base relative to S_lo (x, y wrapped into [0, n) by the vertex kernel): x, y in 0..3,
+        // z in -4..3 (below 0 only at a wall), in a byte each
+        const int bz = max(rec.base[2] - Sz, -4);
+        s_b[r] = (rec.base[0] - Sx) | (rec.base[1] - Sy) << 8 | (bz + 4) << 16;
       }
-      for (int k = lane; k < REGION_NODES; k += 32) region[k] = Vec4<real>{0, 0, 0, 0};
-      __syncwarp();
-      for (int c = 0; c < n; c++) {
-        const int bx = s_b[wq][c][0], by = s_b[wq][c][1], bz = s_b[wq][c][2];
-        const Vec4<real> f = s_f[wq][c];
-        const real wxy = s_w[wq][c][dxa] * s_w[wq][c][4 + dya];
-        for (int h = 0; h < 2; h++) {
-          const int dz = dza + 2 * h;  // node lane + 32 h has the same dx, dy and dz + 2
-          const int rz = bz + dz;
-          if (rz < 0 || rz >= REGION) continue;  // beyond the lattice in z
-          const real w = wxy * s_w[wq][c][8 + dz];
-          Vec4<real> &o = region[(rz * REGION + by + dya) * REGION + bx + dxa];
-          o.x += w * f.x;
-          o.y += w * f.y;
-          o.z += w * f.z;
-          o.w = real(1);  // a stencil node of some vertex (the interpolation reads it)
+      __syncthreads();
+      for (int c0 = 0; c0 < cnt; c0 += 2) {
+        const int c = c0 + half;
+        if (c < cnt) {
+          const int b = s_b[c];
+          const Vec4<real> f = s_f[c];
+          add_plane(s_region[half], warp, l16, b & 255, (b >> 8) & 255, (b >> 16) - 4, s_w[c],
+                    s_w[c] + 4, s_w[c] + 8, f.x, f.y, f.z);
         }
         __syncwarp();
       }
     } else {
       // the tile spilled: mark its bucket's vertices too, then add every vertex of the tile in
-      // increasing index (bitmap words read through L2, where the atomics are performed)
-      atomicOr(&spill_bits[bk[lane] >> 5], 1u << (bk[lane] & 31));
-      atomicOr(&spill_bits[bk[lane + 32] >> 5], 1u << (bk[lane + 32] & 31));
-      for (int k = lane; k < REGION_NODES; k += 32) region[k] = Vec4<real>{0, 0, 0, 0};
-      __syncwarp();
+      // increasing index (bitmap words read through L2, where the atomics are performed); every
+      // warp scans for itself and adds the planes it owns
+      atomicOr(&spill_bits[v >> 5], 1u << (v & 31));
+      __syncthreads();
+      int rank = 0;
       for (int wb = 0; wb < A.spill_words; wb += 32) {
         const unsigned word_l = wb + lane < A.spill_words ? __ldcg(&spill_bits[wb + lane]) : 0u;
         unsigned nonzero = __ballot_sync(0xffffffffu, word_l != 0u);
@@ -524,7 +564,7 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, in
           const int vl = (wb + l) * 32 + lane;  // this lane's vertex of the word
           bool mine = false;
           if ((word >> lane) & 1u) {
-            const StencilRec<real> rl = stencil[vl];
+            const StencilRec<real> &rl = stencil[vl];
             const int bzc = min(max(rl.base[2], 0), D.nz - 1);
             mine = (rl.base[0] >> 2) == tsx && (rl.base[1] >> 2) == tsy && (bzc >> 2) == tsz;
           }
@@ -532,42 +572,36 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, in
           while (members) {  // the tile's vertices of this word, in index order
             const int b = __ffs(members) - 1;
             members &= members - 1;
-            const int v = (wb + l) * 32 + b;
-            const StencilRec<real> rec = stencil[v];
-            const int bx = rec.base[0] - Sx, by = rec.base[1] - Sy, bz = rec.base[2] - Sz;
-            const Vec4<real> pv = phi[v], gv = gvol[v];
-            const real fx = pv.x - coef * gv.x, fy = pv.y - coef * gv.y, fz = pv.z - coef * gv.z;
-            const real wxy = pick4(rec.w[0], dxa) * pick4(rec.w[1], dya);
-            for (int h = 0; h < 2; h++) {
-              const int dz = dza + 2 * h;
-              const int rz = bz + dz;
-              if (rz < 0 || rz >= REGION) continue;
-              const real w = wxy * pick4(rec.w[2], dz);
-              Vec4<real> &o = region[(rz * REGION + by + dya) * REGION + bx + dxa];
-              o.x += w * fx;
-              o.y += w * fy;
-              o.z += w * fz;
-              o.w = real(1);
+            if ((rank++ & 1) == half) {
+              const int vm = (wb + l) * 32 + b;
+              const StencilRec<real> &rec = stencil[vm];
+              const Vec4<real> pv = phi[vm], gv = gvol[vm];
+              add_plane(s_region[half], warp, l16, rec.base[0] - Sx, rec.base[1] - Sy,
+                        max(rec.base[2] - Sz, -4), rec.w[0], rec.w[1], rec.w[2],
+                        pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z);
             }
             __syncwarp();
           }
         }
       }
     }
+    __syncthreads();
     Vec4<real> *out = A.Rslot + (size_t)reg * REGION_NODES;
-    for (int k = lane; k < REGION_NODES; k += 32) out[k] = region[k];
-    __syncwarp();
+    for (int k = tid; k < REGION_NODES; k += kSourceThreads) {
+      const Vec4<real> a = s_region[0][k], b = s_region[1][k];
+      out[k] = Vec4<real>{a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
+    }
+    __syncthreads();  // the region is cleared for the next tile
   }
 }
 
 template <typename real>
-__global__ void __launch_bounds__(32 * SrcWarps<real>::value) spread_source_kernel(
-    const SourceArgs<real> A) {
+__global__ void __launch_bounds__(kSourceThreads) spread_source_kernel(const SourceArgs<real> A) {
   spread_source_body(A, blockIdx.x, gridDim.x);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(32 * SrcWarps<real>::value) spread_source_kernel_multi(
+__global__ void __launch_bounds__(kSourceThreads) spread_source_kernel_multi(
     const SourceArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   spread_source_body(all[m.inst], m.block, m.nblocks);
@@ -648,18 +682,20 @@ __global__ void __launch_bounds__(64) spread_gather_kernel_multi(
   spread_gather_body(all[m.inst], m.block, m.nblocks);
 }
 
-// Claim tile t in map (tile_slot, slot_tile, nslots): the first claimant takes a new slot.
-// A plain read first keeps the many vertices of an already-claimed tile off the atomic.
-__device__ __forceinline__ void claim_tile(int t, int *tile_slot, int *slot_tile, int *nslots,
-                                           int *slot_count, int *out_src, int *health,
+// Claim tile t in map (tile_slot, slot_tile, nslots), whose entry read `seen` a moment ago: the
+// first claimant takes a new slot. (The plain read keeps the many vertices of an already-claimed
+// tile off the atomic.)
+__device__ __forceinline__ void claim_tile(int t, int seen, int *tile_slot, int *slot_tile,
+                                           int *nslots, int *slot_count, int *out_src, int *health,
                                            int max_slots) {
-  if (*(volatile int *)&tile_slot[t] != -1) return;
+  if (seen != -1) return;
   if (atomicCAS(&tile_slot[t], -1, -2) == -1) {
     const int s = atomicAdd(nslots, 1);
     if (s < max_slots) {
       slot_tile[s] = t;
       slot_count[s] = 0;
-      for (int e = 0; e < 8; e++) out_src[8 * (size_t)s + e] = -1;
+      int4 *o = reinterpret_cast<int4 *>(out_src + 8 * (size_t)s);
+      o[0] = o[1] = make_int4(-1, -1, -1, -1);
       atomicExch(&tile_slot[t], s);
     } else {
       atomicOr(health, H_CAPACITY);
@@ -676,45 +712,42 @@ struct AxisTiles {
   bool ok0, ok1;
 };
 
-__device__ __forceinline__ AxisTiles axis_tiles(double p, int nt, double inv_n, bool periodic) {
+// of an axis of n nodes (nt tiles)
+__device__ __forceinline__ AxisTiles axis_tiles(double p, int n, int nt, double inv_n, bool periodic) {
   AxisTiles a;
-  if (periodic) p = wrap_pos(p, 4 * nt, inv_n);
-  const int b = (int)floor(p) - 1;
-  int t0 = floor_div4(b), t1 = floor_div4(b + 3);
-  a.ok1 = t1 != t0;
-  if (periodic) {  // b in [-2, 4 nt - 1]: t0 in [-1, nt - 1], t1 in [0, nt]
-    t0 = t0 < 0 ? t0 + nt : t0;
-    t1 = t1 >= nt ? t1 - nt : t1;
+  double r;
+  const int b = stencil_base(p, n, inv_n, periodic, r);
+  a.t0 = b >> 2;  // (arithmetic shift: floors)
+  a.t1 = (b + 3) >> 2;
+  if (periodic) {
+    a.t1 = a.t1 >= nt ? a.t1 - nt : a.t1;
     a.ok0 = true;
-    a.ok1 = a.ok1 && t1 != t0;  // a short periodic axis may wrap onto the same tile
+    a.ok1 = a.t1 != a.t0;  // a short periodic axis may wrap onto the same tile
   } else {
-    a.ok0 = t0 >= 0 && t0 < nt;
-    a.ok1 = a.ok1 && t1 >= 0 && t1 < nt;
+    a.ok0 = a.t0 >= 0 && a.t0 < nt;
+    a.ok1 = a.t1 != a.t0 && a.t1 >= 0 && a.t1 < nt;
   }
-  a.t0 = t0;
-  a.t1 = t1;
   return a;
 }
 
-// Claim, in map (tile_slot, slot_tile, nslots), tile e (bit k picks the upper tile along
-// axis k) of the stencil described by ax.
-__device__ __forceinline__ void mark_tile(const AxisTiles ax[3], int e, const Dims &D,
-                                          int *tile_slot, int *slot_tile, int *nslots,
-                                          int *slot_count, int *out_src, int *health) {
+// Tile e (bit k picks the upper tile along axis k) of the stencil described by ax, or -1.
+__device__ __forceinline__ int stencil_tile(const AxisTiles ax[3], int e, const Dims &D) {
   int t[3];
   for (int k = 0; k < 3; k++) {
     const bool up = (e >> k) & 1;
-    if (up ? !ax[k].ok1 : !ax[k].ok0) return;
+    if (up ? !ax[k].ok1 : !ax[k].ok0) return -1;
     t[k] = up ? ax[k].t1 : ax[k].t0;
   }
-  claim_tile((t[2] * D.nty + t[1]) * D.ntx + t[0], tile_slot, slot_tile, nslots, slot_count,
-             out_src, health, D.max_slots);
+  return (t[2] * D.nty + t[1]) * D.ntx + t[0];
 }
 
 // K2: interpolation (Eq. 11) and the Euler update (Eq. 12); 4 lanes per vertex, lane dz
-// sums the 16 nodes of its z-plane of the stencil, the 4 planes are summed by shuffles and
-// the update is added to the double position by lane 0, which also finds the tiles of the new
-// stencil; each lane then marks two of those (up to 8) tiles in the other map.
+// sums the 16 nodes of its z-plane of the stencil, the 4 planes are summed by shuffles; lane k
+// then adds the update to coordinate k of the double position and finds the tiles of the new
+// stencil along that axis; each lane marks two of the (up to 8) tiles in the other map. One
+// lane per axis issues a third of the FP64 instructions of one lane per vertex (an FP64
+// instruction holds the SM's FP64 unit for 16 cycles however few lanes take part): 10242 vertices
+// on 64 SMs 12.8 us against 17.2, 40962 on 24 SMs 88 against 127, 96 wetting boxes 108 against 262.
 // The delta-weight accumulation of a vertex is carried at double precision in every
 // precision (VertexSum): each stencil row's four products w_x u (one x row of a tile, in the
 // arithmetic type) is added to the vertex's sum with its weight w_y w_z, and the four planes'
@@ -731,7 +764,8 @@ struct VertexSum<double> {
   __device__ __forceinline__ void add_lanes(int o) {
     for (int k = 0; k < 3; k++) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
   }
-  __device__ __forceinline__ double value(int k) const { return s[k]; }
+  // component k of a run-time k
+  __device__ __forceinline__ double value(int k) const { return k == 0 ? s[0] : k == 1 ? s[1] : s[2]; }
 };
 
 // Float contexts: the sum is a pair of floats hi + lo (double-float arithmetic), kept exact
@@ -768,7 +802,11 @@ struct VertexSum<float> {
       add(k, h, 0.f);
     }
   }
-  __device__ __forceinline__ double value(int k) const { return (double)hi[k] + (double)lo[k]; }
+  __device__ __forceinline__ double value(int k) const {
+    const float h = k == 0 ? hi[0] : k == 1 ? hi[1] : hi[2];
+    const float l = k == 0 ? lo[0] : k == 1 ? lo[1] : lo[2];
+    return (double)h + (double)l;
+  }
 };
 
 template <typename real>
@@ -803,6 +841,10 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int bid) 
   const int v = gid >> 2;
   const int dz = gid & 3;
   const bool valid = v < nv;
+  // lane k < 3 of the vertex updates coordinate k: its position is read ahead
+  const bool axis = valid && dz < 3;
+  const double qk = axis ? q[3 * (size_t)v + dz] : 0.0;
+  const double xk = axis ? xref[3 * (size_t)v + dz] : 0.0;
   VertexSum<real> acc;
   if (valid) {
     const StencilRec<real> rec = stencil[v];
@@ -859,65 +901,58 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int bid) 
   }
   // sum of the 4 planes (fixed butterfly order)
   for (int o = 2; o > 0; o >>= 1) acc.add_lanes(o);
-  // lane dz == 0 updates the vertex in double and finds the tiles of its new stencil; the
-  // other three lanes take the tiles from it (FP64 issues at 1/64 of the FP32 rate on this
-  // GPU, so that work is done once per vertex)
-  int tq[6] = {0, 0, 0, 0, 0, 0};  // t0, t1 of each axis
-  int flags = 0;                   // bit 2k / 2k + 1: ok0 / ok1 of axis k; bit 6: mark
-  if (valid && dz == 0) {
-    double pn[3], qd[3];
+  int t0 = 0, t1 = 0, flags = 0;  // bit 0 / 1: ok0 / ok1 of the axis; bit 2: a number
+  if (axis) {
+    const double qd = acc.value(dz);
+    const double pn = qk + qd;
+    qdot[3 * (size_t)v + dz] = qd;
+    q[3 * (size_t)v + dz] = pn;
     int h = 0;
-    for (int k = 0; k < 3; k++) {
-      qd[k] = acc.value(k);
-      pn[k] = q[3 * (size_t)v + k] + qd[k];
-      qdot[3 * (size_t)v + k] = qd[k];
-      q[3 * (size_t)v + k] = pn[k];
-      if (!(fabs(qd[k]) < 0.1)) h |= (qd[k] == qd[k]) ? H_FAST : H_NAN;
-    }
-    if (D.has_walls && (pn[2] - D.zb < 0.05 || D.zt - pn[2] < 0.05)) h |= H_WALL;
+    if (!(fabs(qd) < 0.1)) h |= (qd == qd) ? H_FAST : H_NAN;
+    if (dz == 2 && D.has_walls && (pn - D.zb < 0.05 || D.zt - pn < 0.05)) h |= H_WALL;
     if (h) atomicOr(health, h);
-    Vec4<real> d;
-    d.x = (real)(pn[0] - xref[3 * (size_t)v]);
-    d.y = (real)(pn[1] - xref[3 * (size_t)v + 1]);
-    d.z = (real)(pn[2] - xref[3 * (size_t)v + 2]);
-    d.w = real(0);
-    disp[v] = d;
-    if (next_tile_slot != nullptr && pn[0] == pn[0] && pn[1] == pn[1] && pn[2] == pn[2]) {
-      const AxisTiles ax[3] = {axis_tiles(pn[0], D.ntx, D.inx, true),
-                               axis_tiles(pn[1], D.nty, D.iny, true),
-                               axis_tiles(pn[2], D.ntz, D.inz, !D.has_walls)};
-      for (int k = 0; k < 3; k++) {
-        tq[2 * k] = ax[k].t0;
-        tq[2 * k + 1] = ax[k].t1;
-        flags |= (ax[k].ok0 ? 1 : 0) << (2 * k) | (ax[k].ok1 ? 1 : 0) << (2 * k + 1);
-      }
-      flags |= 64;
+    reinterpret_cast<real *>(disp + v)[dz] = (real)(pn - xk);
+    if (next_tile_slot != nullptr && pn == pn) {
+      const int n = dz == 0 ? D.nx : dz == 1 ? D.ny : D.nz;
+      const int nt = dz == 0 ? D.ntx : dz == 1 ? D.nty : D.ntz;
+      const double inv = dz == 0 ? D.inx : dz == 1 ? D.iny : D.inz;
+      const AxisTiles ax = axis_tiles(pn, n, nt, inv, dz < 2 || !D.has_walls);
+      t0 = ax.t0;
+      t1 = ax.t1;
+      flags = (ax.ok0 ? 1 : 0) | (ax.ok1 ? 2 : 0) | 4;
     }
   }
-  for (int k = 0; k < 6; k++) tq[k] = __shfl_sync(0xffffffffu, tq[k], 0, 4);
-  flags = __shfl_sync(0xffffffffu, flags, 0, 4);
-  if (valid && (flags & 64)) {  // each lane claims two of the (up to 8) tiles
-    AxisTiles ax[3];
-    for (int k = 0; k < 3; k++) {
-      ax[k].t0 = tq[2 * k];
-      ax[k].t1 = tq[2 * k + 1];
-      ax[k].ok0 = (flags >> (2 * k)) & 1;
-      ax[k].ok1 = (flags >> (2 * k + 1)) & 1;
-    }
-    mark_tile(ax, dz, D, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count,
-              A.out_src, health);
-    mark_tile(ax, dz + 4, D, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count,
-              A.out_src, health);
+  AxisTiles ax[3];
+  int all = 4;
+  for (int k = 0; k < 3; k++) {
+    ax[k].t0 = __shfl_sync(0xffffffffu, t0, k, 4);
+    ax[k].t1 = __shfl_sync(0xffffffffu, t1, k, 4);
+    const int fl = __shfl_sync(0xffffffffu, flags, k, 4);
+    ax[k].ok0 = fl & 1;
+    ax[k].ok1 = fl & 2;
+    all &= fl;
+  }
+  if (valid && all) {  // each lane claims two of the (up to 8) tiles
+    const int ta = stencil_tile(ax, dz, D), tb = stencil_tile(ax, dz + 4, D);
+    const int sa = ta >= 0 ? *(volatile int *)&next_tile_slot[ta] : 0;
+    const int sb = tb >= 0 ? *(volatile int *)&next_tile_slot[tb] : 0;
+    claim_tile(ta, sa, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count, A.out_src,
+               health, D.max_slots);
+    claim_tile(tb, sb, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count, A.out_src,
+               health, D.max_slots);
   }
 }
 
+// Threads per block of K2.
+constexpr int kInterpThreads = 128;
+
 template <typename real>
-__global__ void __launch_bounds__(256) interp_kernel(const InterpArgs<real> A) {
+__global__ void __launch_bounds__(kInterpThreads) interp_kernel(const InterpArgs<real> A) {
   interp_body(A, blockIdx.x);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) interp_kernel_multi(
+__global__ void __launch_bounds__(kInterpThreads) interp_kernel_multi(
     const InterpArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   interp_body(all[m.inst], m.block);
@@ -944,10 +979,12 @@ __global__ void mark_kernel(int nv, const double *__restrict__ q, const double *
   }
   if (p[0] == p[0] && p[1] == p[1] && p[2] == p[2]) {
     AxisTiles ax[3];
-    ax[0] = axis_tiles(p[0], D.ntx, D.inx, true);
-    ax[1] = axis_tiles(p[1], D.nty, D.iny, true);
-    ax[2] = axis_tiles(p[2], D.ntz, D.inz, !D.has_walls);
-    mark_tile(ax, e, D, tile_slot, slot_tile, nslots, slot_count, out_src, health);
+    ax[0] = axis_tiles(p[0], D.nx, D.ntx, D.inx, true);
+    ax[1] = axis_tiles(p[1], D.ny, D.nty, D.iny, true);
+    ax[2] = axis_tiles(p[2], D.nz, D.ntz, D.inz, !D.has_walls);
+    const int t = stencil_tile(ax, e, D);
+    claim_tile(t, t >= 0 ? *(volatile int *)&tile_slot[t] : 0, tile_slot, slot_tile, nslots,
+               slot_count, out_src, health, D.max_slots);
   }
 }
 
@@ -1036,8 +1073,8 @@ FaceArgs<real> face_args(const Ctx &c, int reset) {
   a.faces = c.faces;
   a.disp = (const Vec4<real> *)c.disp;
   a.fgeo = (const real *)c.fgeo;
-  a.fcontrib = (real *)c.fcontrib;
-  a.fnorm = (real *)c.fnorm;
+  a.fcontrib = (Vec4<real> *)c.fcontrib;
+  a.fnorm = (Vec4<real> *)c.fnorm;
   a.vol_partial = c.vol_partial;
   a.D = dims_of(c);
   a.other_tile_slot = c.tile_slot[other];
@@ -1057,8 +1094,8 @@ VertexArgs<real> vertex_args(const Ctx &c, int bin) {
   a.nv = c.nv;
   a.vf_start = c.vf_start;
   a.vf_list = c.vf_list;
-  a.fcontrib = (const real *)c.fcontrib;
-  a.fnorm = (const real *)c.fnorm;
+  a.fcontrib = (const Vec4<real> *)c.fcontrib;
+  a.fnorm = (const Vec4<real> *)c.fnorm;
   a.q = c.q;
   a.phi = (Vec4<real> *)c.phi;
   a.gvol = (Vec4<real> *)c.gvol;
@@ -1069,7 +1106,7 @@ VertexArgs<real> vertex_args(const Ctx &c, int bin) {
   a.bucket = c.bucket;
   a.ovf_count = c.counters + 2;
   a.spill_bits = c.spill_bits;
-  a.src_index = c.src_index;
+  a.src_slot = c.src_slot;
   a.nsources = c.counters + 4;
   a.health = c.counters + 3;
   a.zero_counter = bin == 2 ? c.counters + (c.map ^ 1) : nullptr;
@@ -1079,16 +1116,18 @@ VertexArgs<real> vertex_args(const Ctx &c, int bin) {
   a.D = dims_of(c);
   return a;
 }
-int vertex_blocks(const Ctx &c) { return (c.nv + 255) / 256; }
+// the first block takes the volume coefficient
+int vertex_blocks(const Ctx &c) { return (c.nv + kVertexThreads - 1) / kVertexThreads + 1; }
 
 template <typename real>
 SourceArgs<real> source_args(const Ctx &c) {
   SourceArgs<real> a;
   a.tile_slot = c.tile_slot[c.map];
   a.slot_tile = c.slot_tile[c.map];
-  a.nslots_ptr = c.counters + c.map;
+  a.nsources_ptr = c.counters + 4;
+  a.max_sources = c.max_sources;
   a.slot_count = c.slot_count;
-  a.src_index = c.src_index;
+  a.src_slot = c.src_slot;
   a.bucket = c.bucket;
   a.spill_bits = c.spill_bits;
   a.spill_words = c.spill_words;
@@ -1102,14 +1141,13 @@ SourceArgs<real> source_args(const Ctx &c) {
   return a;
 }
 // persistent grids sized to the SMs the interface chain runs on; in a batch (no partition,
-// many contexts side by side) to the context's expected active tiles instead: one warp per
-// two (source) tiles
+// many contexts side by side) to the context's expected active tiles instead, about half of
+// them source tiles: a block per source tile
 template <typename real>
 int source_blocks(const Ctx &c, bool batched) {
-  constexpr int W = SrcWarps<real>::value;
   const int sms = c.ib_sms > 0 ? c.ib_sms : c.sm_count;
-  int g = batched ? (c.tile_estimate + 2 * W - 1) / (2 * W) : sms * 8;
-  if (g * W > c.max_slots) g = (c.max_slots + W - 1) / W;
+  int g = batched ? (c.tile_estimate + 3) / 4 : sms * (sizeof(real) == 4 ? 10 : 5);
+  if (g > c.max_sources) g = c.max_sources;
   return g < 1 ? 1 : g;
 }
 
@@ -1156,24 +1194,24 @@ InterpArgs<real> interp_args(const Ctx &c) {
   a.health = c.counters + 3;
   return a;
 }
-int interp_blocks(const Ctx &c) { return (int)((4L * c.nv + 255) / 256); }
+int interp_blocks(const Ctx &c) { return (int)((4L * c.nv + kInterpThreads - 1) / kInterpThreads); }
 
 template <typename real>
 cudaError_t face_forces_t(Ctx &c, int reset, cudaStream_t st) {
-  face_kernel<real><<<face_blocks(c), 256, 0, st>>>(face_args<real>(c, reset));
+  face_kernel<real><<<face_blocks(c), FaceThreads<real>::value, 0, st>>>(face_args<real>(c, reset));
   return cudaGetLastError();
 }
 
 template <typename real>
 cudaError_t vertex_forces_t(Ctx &c, int bin, cudaStream_t st) {
-  vertex_kernel<real><<<vertex_blocks(c), 256, 0, st>>>(vertex_args<real>(c, bin));
+  vertex_kernel<real><<<vertex_blocks(c), kVertexThreads, 0, st>>>(vertex_args<real>(c, bin));
   return cudaGetLastError();
 }
 
 template <typename real>
 cudaError_t spread_t(Ctx &c, cudaStream_t st) {
-  constexpr int W = SrcWarps<real>::value;
-  spread_source_kernel<real><<<source_blocks<real>(c, false), 32 * W, 0, st>>>(source_args<real>(c));
+  spread_source_kernel<real><<<source_blocks<real>(c, false), kSourceThreads, 0, st>>>(
+      source_args<real>(c));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   spread_gather_kernel<real><<<gather_blocks(c, false), TILE_CELLS, 0, st>>>(gather_args<real>(c));
@@ -1182,7 +1220,7 @@ cudaError_t spread_t(Ctx &c, cudaStream_t st) {
 
 template <typename real>
 cudaError_t interp_t(Ctx &c, cudaStream_t st) {
-  interp_kernel<real><<<interp_blocks(c), 256, 0, st>>>(interp_args<real>(c));
+  interp_kernel<real><<<interp_blocks(c), kInterpThreads, 0, st>>>(interp_args<real>(c));
   return cudaGetLastError();
 }
 
@@ -1207,17 +1245,17 @@ int ib_multi_record_t(const Ctx &c, MultiKernel k, std::vector<unsigned char> &b
 
 template <typename real>
 cudaError_t ib_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStream_t s) {
-  constexpr int W = SrcWarps<real>::value;
   switch (k) {
     case MK_FACE:
-      face_kernel_multi<real><<<m.blocks, 256, 0, s>>>((const FaceArgs<real> *)m.args, m.start, m.n);
+      face_kernel_multi<real><<<m.blocks, FaceThreads<real>::value, 0, s>>>(
+          (const FaceArgs<real> *)m.args, m.start, m.n);
       break;
     case MK_VERTEX:
-      vertex_kernel_multi<real><<<m.blocks, 256, 0, s>>>((const VertexArgs<real> *)m.args, m.start,
-                                                          m.n);
+      vertex_kernel_multi<real><<<m.blocks, kVertexThreads, 0, s>>>(
+          (const VertexArgs<real> *)m.args, m.start, m.n);
       break;
     case MK_SOURCE:
-      spread_source_kernel_multi<real><<<m.blocks, 32 * W, 0, s>>>(
+      spread_source_kernel_multi<real><<<m.blocks, kSourceThreads, 0, s>>>(
           (const SourceArgs<real> *)m.args, m.start, m.n);
       break;
     case MK_GATHER:
@@ -1225,8 +1263,8 @@ cudaError_t ib_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStream_t 
           (const GatherArgs<real> *)m.args, m.start, m.n);
       break;
     case MK_INTERP:
-      interp_kernel_multi<real><<<m.blocks, 256, 0, s>>>((const InterpArgs<real> *)m.args, m.start,
-                                                          m.n);
+      interp_kernel_multi<real><<<m.blocks, kInterpThreads, 0, s>>>(
+          (const InterpArgs<real> *)m.args, m.start, m.n);
       break;
     default:
       return cudaErrorInvalidValue;
@@ -1260,6 +1298,10 @@ cudaError_t ib_launch_multi(int precision, MultiKernel k, const MultiLaunch &m, 
 
 size_t ib_multi_record_align(int precision, MultiKernel k) {
   return precision == IBLB_FP64 ? ib_record_align<double>(k) : ib_record_align<float>(k);
+}
+
+int face_block_threads(int precision) {
+  return precision == IBLB_FP64 ? FaceThreads<double>::value : FaceThreads<float>::value;
 }
 
 size_t stencil_record_bytes(const Ctx &c) {

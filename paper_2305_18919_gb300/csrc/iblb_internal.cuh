@@ -39,7 +39,7 @@ __host__ __device__ constexpr double wgt(int i) {
 constexpr int TILE = 4;
 constexpr int TILE_CELLS = TILE * TILE * TILE;
 // vertices per source-tile bucket; the rest of a fuller tile is marked in a spill bitmap
-constexpr int BUCKET_CAP = 64;
+constexpr int BUCKET_CAP = 128;
 
 // Health word bits (read back by iblb_step).
 constexpr int H_NAN = 1, H_FAST = 2, H_WALL = 4, H_VOLUME = 8, H_CAPACITY = 16;
@@ -107,7 +107,7 @@ struct alignas(4 * sizeof(real)) Vec4 {
 // Per-vertex stencil record written by the vertex kernel and read by spreading and
 // interpolation: base node (floor(q) - 1, x/y wrapped), the 3x4 one-dimensional weights.
 template <typename real>
-struct StencilRec {
+struct alignas(16) StencilRec {
   int base[3];
   int pad;
   real w[3][4];
@@ -142,7 +142,7 @@ struct Ctx {
   int *slot_tile[2] = {nullptr, nullptr};  // [max_slots] tile id of each active slot
   int *counters = nullptr;  // [0..1] nslots per map, [2] spilled vertices, [3] health, [4] sources,
                             // [5] listed force pairs
-  int *src_index = nullptr;                // [max_slots] region of a source tile (slot)
+  int *src_slot = nullptr;                 // [max_sources] slot of each source tile
   void *Rslot = nullptr;                   // [max_sources][343] Vec4 spreading regions
   int *out_src[2] = {nullptr, nullptr};    // per map: [max_slots][8] region of source T - e
   int max_sources = 0;
@@ -169,8 +169,8 @@ struct Ctx {
   void *vcoef = nullptr;     // kV (V - V0)/V0 of the step, in the population type (K3b writes it)
   int *vf_start = nullptr;   // [nv+1] CSR vertex -> (face*3 + corner)
   int *vf_list = nullptr;    // [3 nf]
-  void *fcontrib = nullptr;  // [nf][3 corners][3]: strain + wall force per corner
-  void *fnorm = nullptr;     // [nf][3]: (a x b)/6, the face's volume gradient at each corner
+  void *fcontrib = nullptr;  // [nf][3 corners] Vec4: strain + wall force per corner
+  void *fnorm = nullptr;     // [nf] Vec4: (a x b)/6, the face's volume gradient at each corner
   double *vol_partial = nullptr;  // [vol_blocks] partial sums of V - V0 (one per face block)
   int vol_blocks = 0;
   void *phi = nullptr;       // [nv] Vec4: strain + wall part of the nodal force (Eq. 16 without
@@ -245,6 +245,8 @@ cudaError_t launch_populations(Ctx &c, double *f_dev);
 cudaError_t launch_init_equilibrium(Ctx &c, const double *rho_dev, const double *u_dev);
 
 cudaError_t launch_face_forces(Ctx &c, int reset_other_map, cudaStream_t s);
+// Threads per block of the face kernel (one partial volume sum per block).
+int face_block_threads(int precision);
 // Device bytes of one stencil record in the context's precision.
 size_t stencil_record_bytes(const Ctx &c);
 cudaError_t launch_vertex_forces(Ctx &c, int bin, cudaStream_t s);

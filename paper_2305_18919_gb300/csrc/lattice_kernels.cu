@@ -35,6 +35,16 @@ struct CollideCoef {
   real Lc[3];         // g/omega:        L = j + g/omega
 };
 
+// Coefficients of the active-tile correction (in the arithmetic's units, see Correction).
+template <typename real>
+struct CorrectionCoef {
+  real ba, bd, b0, qa, qd;  // as in CollideCoef
+  real la, ld;              // 3 w
+  real kappa;               // 2 tau - 1/2
+  real Gh[3];               // g/2:              u0 = (J - g/2)/rho
+  real Kt[3];               // (2 tau - 3/2) g:  K0 = J + (2 tau - 3/2) g
+};
+
 template <typename real>
 struct LatParams {
   int nx, ny, nz, has_walls;
@@ -47,6 +57,7 @@ struct LatParams {
   real wb[19];       // 6 w_i rho0 (c_i . u_bottom): moving-wall term, bottom wall
   real wt[19];       // same for the top wall
   CollideCoef<real> cc;
+  CorrectionCoef<real> ct;
 };
 
 // The collision's coefficients. Rounding them one by one would make the collision gain or lose
@@ -93,6 +104,25 @@ CollideCoef<real> collide_coef(const Ctx &c, double scale) {
 }
 
 template <typename real>
+CorrectionCoef<real> correction_coef(const Ctx &c) {
+  CorrectionCoef<real> k;
+  const double om = 1.0 / c.tau;
+  k.bd = (real)(om / 36.0);
+  k.ba = (real)(om / 18.0);
+  k.b0 = (real)(om / 3.0);
+  k.qd = (real)(om / 8.0);
+  k.qa = (real)(om / 4.0);
+  k.ld = (real)(1.0 / 12.0);
+  k.la = (real)(1.0 / 6.0);
+  k.kappa = (real)(2.0 * c.tau - 0.5);
+  for (int a = 0; a < 3; a++) {
+    k.Gh[a] = (real)(0.5 * c.g[a]);
+    k.Kt[a] = (real)((2.0 * c.tau - 1.5) * c.g[a]);
+  }
+  return k;
+}
+
+template <typename real>
 LatParams<real> lat_params(const Ctx &c) {
   LatParams<real> p;
   p.nx = c.nx; p.ny = c.ny; p.nz = c.nz; p.has_walls = c.has_walls;
@@ -109,6 +139,7 @@ LatParams<real> lat_params(const Ctx &c) {
     p.wt[i] = (real)(6.0 * wgt(i) * c.rho0 * ct);
   }
   p.cc = collide_coef<real>(c, c.precision == IBLB_FP16 ? 1024.0 : c.precision == IBLB_BF16 ? 1.0 : 0.0);
+  p.ct = correction_coef<real>(c);
   return p;
 }
 
@@ -356,6 +387,10 @@ __device__ __forceinline__ double fma_(double a, double b, double c) { return fm
 // FP64 multiply-add, so the two share one reciprocal, 1/(ab), by Newton's iteration
 // r <- r + r (1 - x r) from a float seed (relative error 2^-23, then 2^-46, then rounding);
 // outside the seed's range they are plain divisions. u enters the collision only at second order.
+__device__ __forceinline__ void reciprocals(float a, float b, float &ra, float &rb) {
+  ra = 1.0f / a;
+  rb = 1.0f / b;
+}
 __device__ __forceinline__ void reciprocals(double a, double b, double &ra, double &rb) {
   const double x = mul_(a, b);
   const float s = (float)x;
@@ -1221,11 +1256,8 @@ __global__ void __launch_bounds__(128, MultiMinBlocks<real, S>::value) stream_co
 // same step and corrects K1's result there in place. The collision (BGK with Guo forcing,
 // Eqs. 9-10) keeps rho and turns the momentum j into j + Ft (Ft the total force), so K1's
 // output f0 at a node (the collision with the body force g alone) gives rho = rho0 + sum f0
-// and u0 = (sum c f0 - g/2)/rho without the pre-collision populations; with the interface
-// force F the post-collision populations are f0 + D,
-//   D_i = omega (f^eq_i(rho, uF) - f^eq_i(rho, u0)) + S_i(uF, g + F) - S_i(u0, g),
-//   uF = u0 + F/(2 rho).
-// K1t therefore reads and writes only each node's own populations, no pulled neighbours.
+// and j = J - g, J = sum c f0, without the pre-collision populations. K1t therefore reads and
+// writes only each node's own populations, no pulled neighbours.
 // Its work list is the node pairs (x0, x0 + 1), x0 even, that hold a node of some vertex's
 // stencil, appended by the spreading's gather pass (K4b) as slot * 32 + pair; one thread per
 // listed pair. Pairs without force keep K1's result, which is already final.
@@ -1238,79 +1270,45 @@ struct TilesArgs {
   int max_pairs;
 };
 
-// f (deviations, after the collision with the body force g alone) becomes the collision
-// with g + F; see K1t above. D is a quadratic form in the lattice vector: for a direction i
-// and its opposite,
-//   D_i = w_i (c_i^T M c_i + q0 + c_i . v),   D_opp(i) = w_i (c_i^T M c_i + q0 - c_i . v),
-//   M = 9/4 omega rho (dl s^T + s dl^T) + 9/2 gamma (Ft uF^T + uF Ft^T - g u0^T - u0 g^T),
-//   v = 3 (omega rho dl + gamma F),  dl = uF - u0,  s = uF + u0,  Ft = g + F,
-// so a node needs ten numbers (M's diagonal, twice its off-diagonal, q0, v) once its
-// moments are known, and each direction a few adds.
+// f (deviations, after the collision with the body force g alone) becomes the collision with
+// g + F. In the collision's form (see collide) the interface force F shifts u by h = F/(2 rho),
+// K by e = (2 tau - 1/2) F and L by F/omega, so the second-order products u_a K_b change by
+//   D_ab = u0_a e_b + h_a K1_b,   K1 = K0 + e,
+// and the populations by w omega (-1.5 tr D) + 4.5 w omega c.D c +- 3 w c.F.
 template <typename real>
-struct Correction {
-  real dx, dy, dz;     // M_aa
-  real oxy, oxz, oyz;  // 2 M_ab
-  real q0;             // -1.5 omega rho (uF^2 - u0^2) - 3 gamma (uF.Ft - u0.g)
-  real vx, vy, vz;
-};
-
-// Moments of K1's output at one node: drho = sum f, J = sum c f (deviations).
-template <typename real>
-struct Moments {
-  real drho = 0, Jx = 0, Jy = 0, Jz = 0;
-  __device__ __forceinline__ void add(int i, real f) {
-    drho += f;
-    if (cx(i)) Jx += cx(i) > 0 ? f : -f;
-    if (cy(i)) Jy += cy(i) > 0 ? f : -f;
-    if (cz(i)) Jz += cz(i) > 0 ? f : -f;
+__device__ __forceinline__ void apply_force(real f[Q], real drho, const real J[3], real ir,
+                                            const real F[3], const CorrectionCoef<real> &k) {
+  real u0[3], h[3], e[3], K1[3], D[3];
+  const real hr = mul_(real(0.5), ir);
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    u0[a] = mul_(add_(J[a], -k.Gh[a]), ir);
+    h[a] = mul_(F[a], hr);
+    e[a] = mul_(F[a], k.kappa);
+    K1[a] = add_(add_(J[a], k.Kt[a]), e[a]);
+    D[a] = fma_(u0[a], e[a], mul_(h[a], K1[a]));
   }
-};
-
-template <typename real>
-__device__ __forceinline__ Correction<real> correction_of(const Moments<real> &m, const real F[3],
-                                                         const LatParams<real> &P) {
-  const real drho = m.drho, Jx = m.Jx, Jy = m.Jy, Jz = m.Jz;
-  const real rho = P.rho0 + drho;
-  const real ir = real(1) / rho;
-  const real u0[3] = {(Jx - real(0.5) * P.g[0]) * ir, (Jy - real(0.5) * P.g[1]) * ir,
-                      (Jz - real(0.5) * P.g[2]) * ir};
-  const real dl[3] = {real(0.5) * F[0] * ir, real(0.5) * F[1] * ir, real(0.5) * F[2] * ir};
-  const real uF[3] = {u0[0] + dl[0], u0[1] + dl[1], u0[2] + dl[2]};
-  const real sm[3] = {uF[0] + u0[0], uF[1] + u0[1], uF[2] + u0[2]};
-  const real Ft[3] = {P.g[0] + F[0], P.g[1] + F[1], P.g[2] + F[2]};
-  const real a = real(4.5) * P.omega * rho, b = real(9) * P.guo;
-  Correction<real> k;
-  k.q0 = real(-1.5) * P.omega * rho * (dl[0] * sm[0] + dl[1] * sm[1] + dl[2] * sm[2]) -
-         real(3) * P.guo *
-             ((uF[0] * Ft[0] + uF[1] * Ft[1] + uF[2] * Ft[2]) -
-              (u0[0] * P.g[0] + u0[1] * P.g[1] + u0[2] * P.g[2]));
-  k.dx = a * dl[0] * sm[0] + b * (Ft[0] * uF[0] - P.g[0] * u0[0]);
-  k.dy = a * dl[1] * sm[1] + b * (Ft[1] * uF[1] - P.g[1] * u0[1]);
-  k.dz = a * dl[2] * sm[2] + b * (Ft[2] * uF[2] - P.g[2] * u0[2]);
-  k.oxy = a * (dl[0] * sm[1] + dl[1] * sm[0]) +
-          b * (Ft[0] * uF[1] + Ft[1] * uF[0] - P.g[0] * u0[1] - P.g[1] * u0[0]);
-  k.oxz = a * (dl[0] * sm[2] + dl[2] * sm[0]) +
-          b * (Ft[0] * uF[2] + Ft[2] * uF[0] - P.g[0] * u0[2] - P.g[2] * u0[0]);
-  k.oyz = a * (dl[1] * sm[2] + dl[2] * sm[1]) +
-          b * (Ft[1] * uF[2] + Ft[2] * uF[1] - P.g[1] * u0[2] - P.g[2] * u0[1]);
-  const real oa = P.omega * rho;
-  k.vx = real(3) * (oa * dl[0] + P.guo * F[0]);
-  k.vy = real(3) * (oa * dl[1] + P.guo * F[1]);
-  k.vz = real(3) * (oa * dl[2] + P.guo * F[2]);
-  return k;
-}
-
-// D_i of one node (i and its opposite share M and v; c_opp = -c_i flips only c_i . v).
-template <typename real>
-__device__ __forceinline__ real correction_delta(int i, const Correction<real> &k) {
-  real quad = k.q0, lin = 0;
-  if (cx(i)) { quad += k.dx; lin += cx(i) > 0 ? k.vx : -k.vx; }
-  if (cy(i)) { quad += k.dy; lin += cy(i) > 0 ? k.vy : -k.vy; }
-  if (cz(i)) { quad += k.dz; lin += cz(i) > 0 ? k.vz : -k.vz; }
-  if (cx(i) && cy(i)) quad += cx(i) * cy(i) > 0 ? k.oxy : -k.oxy;
-  if (cx(i) && cz(i)) quad += cx(i) * cz(i) > 0 ? k.oxz : -k.oxz;
-  if (cy(i) && cz(i)) quad += cy(i) * cz(i) > 0 ? k.oyz : -k.oyz;
-  return real(wgt(i)) * (quad + lin);
+  const real s = mul_(real(-1.5), add_(add_(D[0], D[1]), D[2]));
+  f[0] = fma_(k.b0, s, f[0]);
+  const real pa = mul_(k.ba, s), pd = mul_(k.bd, s);
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const real P = fma_(k.qa, D[a], pa);
+    f[2 * a + 1] = add_(f[2 * a + 1], fma_(k.la, F[a], P));
+    f[2 * a + 2] = add_(f[2 * a + 2], fma_(-k.la, F[a], P));
+  }
+#pragma unroll
+  for (int p = 0; p < 3; p++) {  // planes xy, xz, yz
+    const int a = p == 2 ? 1 : 0, b = p == 0 ? 1 : 2, i = 7 + 4 * p;
+    const real m = add_(fma_(u0[a], e[b], mul_(h[a], K1[b])), fma_(u0[b], e[a], mul_(h[b], K1[a])));
+    const real P = fma_(k.qd, add_(D[a], D[b]), pd);
+    const real Pp = fma_(k.qd, m, P), Pm = fma_(-k.qd, m, P);
+    const real lp = add_(F[a], F[b]), lm = add_(F[a], -F[b]);
+    f[i] = add_(f[i], fma_(k.ld, lp, Pp));
+    f[i + 1] = add_(f[i + 1], fma_(-k.ld, lp, Pp));
+    f[i + 2] = add_(f[i + 2], fma_(k.ld, lm, Pm));
+    f[i + 3] = add_(f[i + 3], fma_(-k.ld, lm, Pm));
+  }
 }
 
 template <typename real, typename S>
@@ -1337,40 +1335,39 @@ __device__ __forceinline__ void tiles_body(const TilesArgs<real, S> &A, int bid,
     if (z >= P.nz || (P.has_walls && (z == 0 || z == P.nz - 1))) continue;
     const size_t n = (size_t)z * P.nx * P.ny + (size_t)y * P.nx + x0;
     real a[Q], b[Q];
-    Moments<real> ma, mb;
 #pragma unroll
     for (int i = 0; i < Q; i++) {
       widen2(*reinterpret_cast<const V2 *>(fout + (size_t)i * P.ncell + n), a[i], b[i]);
       a[i] *= real(kinv<S>(i));
       b[i] *= real(kinv<S>(i));
-      ma.add(i, a[i]);
-      mb.add(i, b[i]);
     }
     const real FA[3] = {Fa.x, Fa.y, Fa.z};
     const real FB[3] = {Fb.x, Fb.y, Fb.z};
-    const Correction<real> ka = correction_of<real>(ma, FA, P);
-    const Correction<real> kb = correction_of<real>(mb, FB, P);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      a[i] += correction_delta<real>(i, ka);
-      b[i] += correction_delta<real>(i, kb);
-    }
+    real da, db, Ja[3], Jb[3], ia, ib;
+    node_moments(a, da, Ja);
+    node_moments(b, db, Jb);
+    reciprocals(add_(P.rho0, da), add_(P.rho0, db), ia, ib);
+    apply_force(a, da, Ja, ia, FA, P.ct);
+    apply_force(b, db, Jb, ib, FB, P.ct);
     store_pair(fout, P, n, a, b);
   }
 }
 
+// Threads per block of K1t: few, so that a short list spreads over all SMs (the kernel's time
+// there is one pair's chain of loads and arithmetic).
+constexpr int kTilesThreads = 64;
+
 template <typename real, typename S>
-__global__ void __launch_bounds__(128) stream_collide_tiles_kernel(const TilesArgs<real, S> A) {
+__global__ void __launch_bounds__(kTilesThreads) stream_collide_tiles_kernel(const TilesArgs<real, S> A) {
   tiles_body<real, S>(A, blockIdx.x, gridDim.x);
 }
 
-// the batched form reads its argument record as well: held to 128 registers (4 blocks per SM,
-// as the single-context kernel) for float arithmetic
+// the batched form reads its argument record as well: held to 128 registers for float arithmetic
 template <typename real>
-struct TilesMultiMinBlocks { static constexpr int value = sizeof(real) == 4 ? 4 : 1; };
+struct TilesMultiMinBlocks { static constexpr int value = sizeof(real) == 4 ? 8 : 1; };
 
 template <typename real, typename S>
-__global__ void __launch_bounds__(128, TilesMultiMinBlocks<real>::value) stream_collide_tiles_kernel_multi(
+__global__ void __launch_bounds__(kTilesThreads, TilesMultiMinBlocks<real>::value) stream_collide_tiles_kernel_multi(
     const TilesArgs<real, S> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   tiles_body<real, S>(all[m.inst], m.block, m.nblocks);
@@ -1835,10 +1832,10 @@ TilesArgs<real, S> tiles_args(const Ctx &c) {
   a.max_pairs = 32 * c.max_slots;
   return a;
 }
-// a thread per listed pair; single context: four 128-thread blocks per SM (about 78k pairs
-// in one pass); in a batch a block per eight of the context's expected active tiles
+// a thread per listed pair; single context: eight 64-thread blocks per SM (about 78k pairs
+// in one pass); in a batch a block per four of the context's expected active tiles
 int tiles_blocks(const Ctx &c, bool batched) {
-  int grid = batched ? (c.tile_estimate + 7) / 8 : c.sm_count * 4;
+  int grid = batched ? (c.tile_estimate + 3) / 4 : c.sm_count * 8;
   if (grid > c.max_slots) grid = c.max_slots;
   return grid < 1 ? 1 : grid;
 }
@@ -1881,7 +1878,7 @@ template <typename real, typename S>
 cudaError_t stream_collide_tiles_t(Ctx &c, int first, cudaStream_t st) {
   const int grid = tiles_blocks(c, false);
   (void)first;  // K1t corrects K1's output in place, whatever K1 read
-  stream_collide_tiles_kernel<real, S><<<grid, 128, 0, st>>>(tiles_args<real, S>(c));
+  stream_collide_tiles_kernel<real, S><<<grid, kTilesThreads, 0, st>>>(tiles_args<real, S>(c));
   return cudaGetLastError();
 }
 
@@ -1930,7 +1927,7 @@ cudaError_t lattice_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStre
       break;
     }
     case MK_TILES:
-      stream_collide_tiles_kernel_multi<real, S><<<m.blocks, 128, 0, s>>>(
+      stream_collide_tiles_kernel_multi<real, S><<<m.blocks, kTilesThreads, 0, s>>>(
           (const TilesArgs<real, S> *)m.args, m.start, m.n);
       break;
     case MK_SHELL:
