@@ -140,6 +140,9 @@ bool green_api(GreenApi &g) {
   return true;
 }
 
+// Largest stream-collide pass (bytes read and written) of a lattice whose steps run as one kernel.
+constexpr size_t kFusedPassBytes = (size_t)1 << 30;
+
 // Split the device's SMs into an interface partition of about `want` SMs and a lattice
 // partition with the rest, each with its own stream. Returns false (and leaves nothing
 // behind) when the device or driver cannot partition.
@@ -339,6 +342,9 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ev_sync, cudaEventDisableTiming);
   if (e == cudaSuccess) e = dalloc(&c.counters, 8);
   if (e == cudaSuccess) e = cudaMallocHost((void **)&c.health_host, sizeof(int));
+  if (e == cudaSuccess) e = dalloc_bytes(&c.fused_ctl, iblb::kFusedControlBytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c.fused_ctl, 0, iblb::kFusedControlBytes, c.stream);
+  c.fused = e == cudaSuccess && d->ib_sms == 0 && pass_bytes < kFusedPassBytes && iblb::fused_steps_fit(c);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.counters, 0, 8 * sizeof(int), c.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
   if (e != cudaSuccess) {
@@ -366,6 +372,7 @@ void iblb_destroy(iblb_ctx *h) {
   dfree(c.q); dfree(c.qdot); dfree(c.faces); dfree(c.fref); dfree(c.xref); dfree(c.fgeo); dfree(c.vcoef); dfree(c.disp); dfree(c.vf_start); dfree(c.vf_list);
   dfree(c.fcontrib); dfree(c.fnorm); dfree(c.vol_partial); dfree(c.phi); dfree(c.gvol); dfree(c.stencil);
   dfree(c.dscratch);
+  dfree(c.fused_ctl);
   if (c.health_host) cudaFreeHost(c.health_host);
   iblb::adjoint_free(c);
   for (cudaEvent_t ev : c.ev_pool) cudaEventDestroy(ev);
@@ -426,8 +433,7 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   c.nf = nf;
   c.V0 = V0;
   for (int k = 0; k < 3; k++) c.centre[k] = centre[k];
-  const int ft = iblb::face_block_threads(c.precision);
-  c.vol_blocks = (nf + ft - 1) / ft;  // one partial volume change per face block
+  c.vol_blocks = (nf + 31) / 32;  // one partial volume change per warp of faces
   const size_t rs = c.real_size;
   long ms = 8L * nv;
   if ((size_t)ms > c.ntiles) ms = (long)c.ntiles;
@@ -587,7 +593,44 @@ namespace iblb {
 bool split_sms(Ctx &c, int want, int prio_hi) { return make_partitions(c, want, prio_hi); }
 void release_sms(Ctx &c) { free_partitions(c); }
 
+namespace {
+
+// Whether the context's steps after the first run as one kernel: a lattice chosen for it at its
+// creation, and nothing asked for that only the separate kernels have (their timing, a choice of
+// the stream-collide kernel or of its waits).
+bool takes_fused(const Ctx &c) {
+  return c.fused && c.nv && !c.profiling && c.k1_kind == IBLB_STREAM_COLLIDE_AUTO && !c.stage_wait_set;
+}
+
+// Steps of one fused launch: the GPU is the launch's own while it runs, so work of other streams
+// waits this long at most (some milliseconds).
+constexpr int kFusedSteps = 64;
+
+int enqueue_fused(Ctx &c, int nsteps) {
+  for (int done = 0; done < nsteps;) {
+    const int n = nsteps - done < kFusedSteps ? nsteps - done : kFusedSteps;
+    CUDA_TRY(c, launch_fused_steps(c, n, c.stream));
+    c.k1_launches += n;
+    c.kernel_launches += 1;
+    c.cur ^= n & 1;
+    c.map ^= n & 1;
+    c.have_force = 1;
+    c.steps_done += n;
+    done += n;
+  }
+  return 0;
+}
+
+}  // namespace
+
 int enqueue_steps(Ctx &c, int nsteps) {
+  if (takes_fused(c) && nsteps > (c.fresh ? 1 : 0)) {
+    if (c.fresh) {  // the in-place first step by the separate kernels
+      if (int rc = enqueue_steps(c, 1)) return rc;
+      nsteps--;
+    }
+    return enqueue_fused(c, nsteps);
+  }
   // the library streams start after everything queued so far on the context's stream
   CUDA_TRY(c, cudaEventRecord(c.ev_sync, c.stream));
   CUDA_TRY(c, cudaStreamWaitEvent(c.ib, c.ev_sync, 0));
@@ -956,6 +999,7 @@ int iblb_set_stage_wait_limit(iblb_ctx *h, int64_t ns) {
   if (!h) return IBLB_EINVAL;
   if (ns < 0 || ns > 60000000000ll) return fail(h->c, IBLB_EINVAL, "wait limit must be 0 .. 60 s");
   h->c.stage_wait_ns = (unsigned long long)ns;
+  h->c.stage_wait_set = 1;
   h->c.config_gen++;
   return IBLB_OK;
 }

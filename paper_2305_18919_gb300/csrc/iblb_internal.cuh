@@ -171,7 +171,7 @@ struct Ctx {
   int *vf_list = nullptr;    // [3 nf]
   void *fcontrib = nullptr;  // [nf][3 corners] Vec4: strain + wall force per corner
   void *fnorm = nullptr;     // [nf] Vec4: (a x b)/6, the face's volume gradient at each corner
-  double *vol_partial = nullptr;  // [vol_blocks] partial sums of V - V0 (one per face block)
+  double *vol_partial = nullptr;  // [vol_blocks] partial sums of V - V0 (one per 32 faces)
   int vol_blocks = 0;
   void *phi = nullptr;       // [nv] Vec4: strain + wall part of the nodal force (Eq. 16 without
                              //   the volume term, which is applied where the force is used)
@@ -198,10 +198,13 @@ struct Ctx {
   int k1_unit_rows = 0;     // lattice rows per unit of the staged pass (0: by copy size)
   int k1_nodes = 0;         // nodes per compute lane of the staged pass, 16-bit (0: default)
   unsigned long long stage_wait_ns = 1000000000ull;  // limit of a staged pass's waits (ns)
+  int stage_wait_set = 0;   // that limit was set by the caller
   int smem_optin = 0;       // shared memory a block may opt in to (bytes)
   int health_every = 1000;  // iblb_step reads the health word every this many steps (0: at its end)
   int health_pending = 0;   // steps queued by iblb_step_async whose health word is unread
   int *health_host = nullptr;  // pinned: the health word read with a call's own transfers
+  int fused = 0;               // small lattice: iblb_step's steps run as one kernel (fused.cu)
+  void *fused_ctl = nullptr;   // control words of the fused kernel (kFusedControlBytes, zeroed)
   uint64_t config_gen = 0;  // bumped by every call that changes what a queued step launches
   std::string err;
 };
@@ -234,6 +237,13 @@ int k1_block_rows(const Ctx &c);
 // Whether the stream-collide steps after the first take the staged kernel.
 bool stream_collide_staged(const Ctx &c);
 
+// Device bytes of the fused step kernel's control words.
+constexpr size_t kFusedControlBytes = 64;
+// nsteps coupled steps (not the first, in-place one; a mesh) as one cooperative launch (fused.cu).
+cudaError_t launch_fused_steps(Ctx &c, int nsteps, cudaStream_t s);
+// Whether that kernel's grid is resident at once on the context's device.
+bool fused_steps_fit(const Ctx &c);
+
 // Launchers (each returns cudaGetLastError() of its launch) on stream `s`.
 // Stream-collide of every fluid node with the body force only (no interface force).
 cudaError_t launch_stream_collide(Ctx &c, int first, cudaStream_t s);
@@ -245,8 +255,6 @@ cudaError_t launch_populations(Ctx &c, double *f_dev);
 cudaError_t launch_init_equilibrium(Ctx &c, const double *rho_dev, const double *u_dev);
 
 cudaError_t launch_face_forces(Ctx &c, int reset_other_map, cudaStream_t s);
-// Threads per block of the face kernel (one partial volume sum per block).
-int face_block_threads(int precision);
 // Device bytes of one stencil record in the context's precision.
 size_t stencil_record_bytes(const Ctx &c);
 cudaError_t launch_vertex_forces(Ctx &c, int bin, cudaStream_t s);
