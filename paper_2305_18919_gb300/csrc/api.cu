@@ -62,15 +62,15 @@ int check_mesh_id(Ctx &c, int mesh_id) {
   return 0;
 }
 
-// Clear a tile map and mark it for the current vertex positions.
-int remark(Ctx &c, int which) {
-  CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[which], 0xff, c.ntiles * sizeof(int), c.stream));
-  CUDA_TRY(c, cudaMemsetAsync(c.counters + which, 0, sizeof(int), c.stream));
-  const int saved = c.map;
-  c.map = which;
-  cudaError_t e = iblb::launch_mark(c);
-  c.map = saved;
-  CUDA_TRY(c, e);
+// The vertex positions were replaced: refresh the displacements, and empty the tile map if it was
+// marked for the old ones (a step's face pass marks it).
+int positions_changed(Ctx &c) {
+  if (c.marked) {
+    CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[c.map], 0xff, c.ntiles * sizeof(int), c.stream));
+    CUDA_TRY(c, cudaMemsetAsync(c.counters + c.map, 0, sizeof(int), c.stream));
+    c.marked = 0;
+  }
+  CUDA_TRY(c, iblb::launch_displacement(c));
   return 0;
 }
 
@@ -491,7 +491,8 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   c.map = 0;
   c.config_gen++;
   c.have_force = 0;
-  int rc = remark(c, 0);
+  c.marked = 0;
+  int rc = positions_changed(c);
   if (rc) return rc;
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
   if (mesh_id) *mesh_id = 0;
@@ -517,7 +518,7 @@ int iblb_set_vertices(iblb_ctx *h, int32_t mesh_id, const double *q) {
   if (int rc = check_mesh_id(c, mesh_id)) return rc;
   CUDA_TRY(c, cudaMemcpyAsync(c.q, q, (size_t)3 * c.nv * sizeof(double), cudaMemcpyHostToDevice, c.stream));
   // the map of the last spreading step (map ^ 1) stays: read_fields still uses its force
-  return remark(c, c.map);
+  return positions_changed(c);
 }
 
 int iblb_init_equilibrium(iblb_ctx *h, const double *rho, const double *u) {
@@ -614,6 +615,7 @@ int enqueue_fused(Ctx &c, int nsteps) {
     c.kernel_launches += 1;
     c.cur ^= n & 1;
     c.map ^= n & 1;
+    c.marked = 0;
     c.have_force = 1;
     c.steps_done += n;
     done += n;
@@ -675,6 +677,7 @@ int enqueue_steps(Ctx &c, int nsteps) {
       CUDA_TRY(c, iblb::launch_interpolate_advect(c, tail));
       c.kernel_launches += 2;
       c.map ^= 1;
+      c.marked = 0;
       c.have_force = 1;
     }
     c.steps_done++;
@@ -718,7 +721,7 @@ int restore_state(Ctx &c, const void *P, const double *q, int fresh) {
   CUDA_TRY(c, cudaMemcpyAsync(c.q, q, (size_t)3 * c.nv * sizeof(double), cudaMemcpyDeviceToDevice,
                               c.stream));
   c.fresh = fresh;
-  return remark(c, c.map);
+  return positions_changed(c);
 }
 
 }  // namespace iblb
@@ -804,6 +807,8 @@ int iblb_read_force_field(iblb_ctx *h, double *F) {
   CUDA_TRY(c, cudaMemsetAsync(c.dscratch, 0, 3 * c.ncell * sizeof(double), c.stream));
   if (c.nv) {
     CUDA_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
+    if (!c.marked) CUDA_TRY(c, iblb::launch_mark(c));
+    c.marked = 1;
     CUDA_TRY(c, iblb::launch_face_forces(c, 0, c.stream));
     CUDA_TRY(c, iblb::launch_vertex_forces(c, 1, c.stream));
     CUDA_TRY(c, iblb::launch_spread(c, c.stream));
@@ -937,7 +942,7 @@ int iblb_load_state(iblb_ctx *h, const char *path) {
     CUDA_TRY(c, cudaMemcpyAsync(c.q, qbuf.data(), qbuf.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
     CUDA_TRY(c, cudaMemcpyAsync(c.qdot, qdbuf.data(), qdbuf.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
     c.have_force = 0;
-    if (int rc = remark(c, c.map)) return rc;
+    if (int rc = positions_changed(c)) return rc;
     c.config_gen++;
   }
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));

@@ -23,10 +23,22 @@ using iblb::Ctx;
 
 namespace {
 
-// Instances of one precision, stepped by the same batched launches (at most kMultiMax).
+// Instances of one precision, stepped by the same batched launches (at most kMultiMax), on the
+// streams of one lane.
 struct Group {
   int precision = 0;
+  int lane = 0;
   std::vector<int> members;
+};
+
+// A pair of streams on which a part of the instances steps, independent of the other lanes: the
+// interface passes of one lane's instances run beside the lattice pass of another's. Three lanes
+// from kLaneNodes nodes up (96 wetting boxes, 33 M nodes: 1.162 ms per step against 1.253 on one
+// lane and 1.19 on two; 24 boxes, 8 M nodes: 0.304 against 0.336); below, one, whose third of the
+// launches the host issues in time.
+struct Lane {
+  cudaStream_t ib = nullptr, ls = nullptr;
+  cudaEvent_t ev_force = nullptr, ev_coll = nullptr;
 };
 
 // Host image of one batched launch: the records of its instances and its block table.
@@ -39,12 +51,14 @@ struct Table {
 using iblb::MultiKernel;
 constexpr MultiKernel kKernels[] = {iblb::MK_FACE,   iblb::MK_VERTEX,          iblb::MK_SOURCE,
                                     iblb::MK_GATHER, iblb::MK_STREAM_COLLIDE, iblb::MK_TILES,
-                                    iblb::MK_SHELL,  iblb::MK_INTERP};
+                                    iblb::MK_SHELL,  iblb::MK_INTERP,          iblb::MK_FORCED};
 constexpr int kNumKernels = sizeof(kKernels) / sizeof(kKernels[0]);
+constexpr size_t kLaneNodes = (size_t)4 << 20;
 constexpr int kPairSteps = 2;  // records are built for both parities of a pair of steps
 
 bool lattice_kernel(MultiKernel k) {
-  return k == iblb::MK_STREAM_COLLIDE || k == iblb::MK_TILES || k == iblb::MK_SHELL;
+  return k == iblb::MK_STREAM_COLLIDE || k == iblb::MK_TILES || k == iblb::MK_SHELL ||
+         k == iblb::MK_FORCED;
 }
 
 }  // namespace
@@ -55,7 +69,8 @@ struct iblb_batch {
   std::vector<cudaEvent_t> joins;     // one per instance
   cudaStream_t stream = nullptr;      // caller's stream
   iblb::Ctx part;                     // the batch's SM partitions and their streams (ib, ls)
-  cudaEvent_t ev_force = nullptr, ev_coll = nullptr, ev_join = nullptr;
+  std::vector<Lane> lanes;            // lane 0 on part's streams
+  cudaEvent_t ev_join = nullptr;
   std::vector<Group> groups;
   std::vector<Table> tabs;     // [parity][group][kernel]
   void *arena = nullptr;       // device: every table's records and block offsets
@@ -106,14 +121,27 @@ std::vector<Group> make_groups(const iblb_batch *b) {
   for (size_t i = 0; i < b->inst.size(); i++)
     by_precision[b->inst[i]->c.precision].push_back((int)i);
   std::vector<Group> groups;
-  for (const auto &kv : by_precision)
-    for (size_t o = 0; o < kv.second.size(); o += iblb::kMultiMax) {
+  const size_t L = b->lanes.size();
+  for (auto &kv : by_precision) {
+    // dealt to the lanes by size, so that each gets a like share of the nodes
+    std::vector<int> &m = kv.second;
+    std::stable_sort(m.begin(), m.end(),
+                     [&](int x, int y) { return b->inst[x]->c.ncell > b->inst[y]->c.ncell; });
+    for (size_t l = 0; l < L; l++) {
       Group g;
       g.precision = kv.first;
-      const size_t e = std::min(kv.second.size(), o + (size_t)iblb::kMultiMax);
-      g.members.assign(kv.second.begin() + o, kv.second.begin() + e);
-      groups.push_back(g);
+      g.lane = (int)l;
+      for (size_t o = 0; o < m.size(); o++) {
+        if ((o / L % 2 ? L - 1 - o % L : o % L) != l) continue;
+        g.members.push_back(m[o]);
+        if (g.members.size() == (size_t)iblb::kMultiMax) {
+          groups.push_back(g);
+          g.members.clear();
+        }
+      }
+      if (!g.members.empty()) groups.push_back(g);
     }
+  }
   return groups;
 }
 
@@ -147,7 +175,8 @@ int build_tables(iblb_batch *b) {
         const MultiKernel k = kKernels[ki];
         for (int i : b->groups[g].members) {
           const Ctx &c = b->inst[i]->c;
-          if (k != iblb::MK_STREAM_COLLIDE && c.nv == 0) continue;  // no mesh: lattice only
+          const bool lattice_pass = k == iblb::MK_STREAM_COLLIDE || k == iblb::MK_FORCED;
+          if (!lattice_pass && c.nv == 0) continue;  // no mesh: lattice only
           const int blocks = lattice_kernel(k) ? iblb::lattice_multi_record(c, k, t.bytes)
                                                : iblb::ib_multi_record(c, k, t.bytes);
           if (blocks < 1) {
@@ -189,10 +218,11 @@ int build_tables(iblb_batch *b) {
   return 0;
 }
 
-// Queue kernel ki of every group (records of step parity p) on stream s.
-int launch_kernel(iblb_batch *b, int p, int ki, cudaStream_t s) {
+// Queue kernel ki of the lane's groups (records of step parity p) on stream s.
+int launch_kernel(iblb_batch *b, int lane, int p, int ki, cudaStream_t s) {
   const size_t G = b->groups.size();
   for (size_t g = 0; g < G; g++) {
+    if (b->groups[g].lane != lane) continue;
     const Table &t = b->tabs[(p * G + g) * kNumKernels + ki];
     iblb::MultiLaunch m;
     m.n = (int)t.start.size() - 1;
@@ -209,21 +239,27 @@ int launch_kernel(iblb_batch *b, int p, int ki, cudaStream_t s) {
   return 0;
 }
 
-// Queue one coupled step of every instance (records of parity p): the interface chain on the
-// interface stream, the stream-collide passes on the lattice stream, joined by events as in
-// iblb_step.
+// Queue one coupled step of every instance (records of parity p): per lane the interface chain on
+// its interface stream, the stream-collide passes on its lattice stream, joined by events.
 int enqueue_batched_step(iblb_batch *b, int p) {
-  cudaStream_t ifc = b->part.ib, lat = b->part.ls;
-  for (int ki = 0; ki < 4; ki++)  // K3a, K3b, K4a, K4b
-    if (int rc = launch_kernel(b, p, ki, ifc)) return rc;
-  BATCH_TRY(b, cudaEventRecord(b->ev_force, ifc));
-  if (int rc = launch_kernel(b, p, 4, lat)) return rc;  // K1
-  BATCH_TRY(b, cudaStreamWaitEvent(lat, b->ev_force, 0));
-  if (int rc = launch_kernel(b, p, 5, lat)) return rc;  // K1t
-  BATCH_TRY(b, cudaEventRecord(b->ev_coll, lat));
-  BATCH_TRY(b, cudaStreamWaitEvent(ifc, b->ev_coll, 0));
-  for (int ki = 6; ki < 8; ki++)  // K1b, K2
-    if (int rc = launch_kernel(b, p, ki, ifc)) return rc;
+  for (size_t l = 0; l < b->lanes.size(); l++) {
+    Lane &n = b->lanes[l];
+    for (int ki = 0; ki < 4; ki++)  // K3a, K3b, K4a, K4b
+      if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
+    BATCH_TRY(b, cudaEventRecord(n.ev_force, n.ib));
+    // Without a partition the lattice pass waits for the step's force and takes it in (K1 and K1t
+    // in one: K1t's scattered rows are a sixth of the step's traffic; 96 boxes 1.253 ms per step
+    // against 1.310). On a partition the pass runs beside the chain instead, then K1t.
+    const bool beside = b->part.green[0] != nullptr;
+    if (beside)
+      if (int rc = launch_kernel(b, (int)l, p, 4, n.ls)) return rc;  // K1
+    BATCH_TRY(b, cudaStreamWaitEvent(n.ls, n.ev_force, 0));
+    if (int rc = launch_kernel(b, (int)l, p, beside ? 5 : 8, n.ls)) return rc;  // K1t, or both
+    BATCH_TRY(b, cudaEventRecord(n.ev_coll, n.ls));
+    BATCH_TRY(b, cudaStreamWaitEvent(n.ib, n.ev_coll, 0));
+    for (int ki = 6; ki < 8; ki++)  // K1b, K2
+      if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
+  }
   return 0;
 }
 
@@ -250,8 +286,23 @@ int iblb_batch_create(const iblb_lattice_desc *descs, int32_t n, void *cuda_stre
     e = cudaStreamCreateWithFlags(&b->part.ib, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->part.ls, cudaStreamNonBlocking);
   }
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_force, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_coll, cudaEventDisableTiming);
+  size_t nodes = 0;
+  for (int i = 0; i < n; i++)
+    if (descs[i].nx > 0 && descs[i].ny > 0 && descs[i].nz > 0)
+      nodes += (size_t)descs[i].nx * descs[i].ny * descs[i].nz;
+  const int nlanes = b->part.green[0] || nodes < kLaneNodes ? 1 : 3;
+  for (int l = 0; l < nlanes && e == cudaSuccess; l++) {
+    b->lanes.emplace_back();
+    Lane &n = b->lanes.back();
+    n.ib = b->part.ib;
+    n.ls = b->part.ls;
+    if (l > 0) {
+      e = cudaStreamCreateWithFlags(&n.ib, cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&n.ls, cudaStreamNonBlocking);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n.ev_force, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n.ev_coll, cudaEventDisableTiming);
+  }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocHost((void **)&b->health, sizeof(int) * n);
   for (int i = 0; i < n && e == cudaSuccess && rc == 0; i++) {
@@ -286,14 +337,22 @@ void iblb_batch_destroy(iblb_batch *b) {
   if (!b) return;
   for (cudaStream_t s : b->streams) cudaStreamSynchronize(s);
   cudaStreamSynchronize(b->stream);
-  if (b->part.ib) cudaStreamSynchronize(b->part.ib);
-  if (b->part.ls) cudaStreamSynchronize(b->part.ls);
+  for (const Lane &n : b->lanes) {
+    if (n.ib) cudaStreamSynchronize(n.ib);
+    if (n.ls) cudaStreamSynchronize(n.ls);
+  }
   if (b->arena) cudaFree(b->arena);
   for (iblb_ctx *h : b->inst) iblb_destroy(h);
   for (cudaEvent_t ev : b->joins) cudaEventDestroy(ev);
   for (cudaStream_t s : b->streams) cudaStreamDestroy(s);
-  for (cudaEvent_t ev : {b->ev_force, b->ev_coll, b->ev_join})
-    if (ev) cudaEventDestroy(ev);
+  if (b->ev_join) cudaEventDestroy(b->ev_join);
+  for (size_t l = 0; l < b->lanes.size(); l++) {
+    const Lane &n = b->lanes[l];
+    if (n.ev_force) cudaEventDestroy(n.ev_force);
+    if (n.ev_coll) cudaEventDestroy(n.ev_coll);
+    if (l > 0 && n.ib) cudaStreamDestroy(n.ib);  // (lane 0's are the partition's)
+    if (l > 0 && n.ls) cudaStreamDestroy(n.ls);
+  }
   if (b->part.green[0]) {
     iblb::release_sms(b->part);
   } else {
@@ -393,8 +452,10 @@ int iblb_batch_step(iblb_batch *b, int32_t nsteps) {
       if (int rc = build_tables(b)) return rc;
     // the partition streams start after everything queued on the instances' streams
     for (size_t i = 0; i < n; i++) BATCH_TRY(b, follow(b->stream, b->inst[i]->c.stream, b->joins[i]));
-    BATCH_TRY(b, follow(b->part.ib, b->stream, b->ev_join));
-    BATCH_TRY(b, follow(b->part.ls, b->stream, b->ev_join));
+    for (Lane &n : b->lanes) {
+      BATCH_TRY(b, follow(n.ib, b->stream, b->ev_join));
+      BATCH_TRY(b, follow(n.ls, b->stream, b->ev_join));
+    }
     for (; nsteps - done >= kPairSteps; done += kPairSteps) {
       for (int p = 0; p < kPairSteps; p++)
         if (int rc = enqueue_batched_step(b, p)) return rc;
@@ -402,11 +463,14 @@ int iblb_batch_step(iblb_batch *b, int32_t nsteps) {
         Ctx &c = b->inst[i]->c;
         c.steps_done += kPairSteps;
         if (c.nv) c.have_force = 1;
+        c.marked = 0;
         c.fresh = 0;
       }
     }
-    BATCH_TRY(b, follow(b->stream, b->part.ib, b->ev_join));
-    BATCH_TRY(b, follow(b->stream, b->part.ls, b->ev_join));
+    for (Lane &n : b->lanes) {
+      BATCH_TRY(b, follow(b->stream, n.ib, b->ev_join));
+      BATCH_TRY(b, follow(b->stream, n.ls, b->ev_join));
+    }
     for (size_t i = 0; i < n; i++) BATCH_TRY(b, follow(b->inst[i]->c.stream, b->stream, b->joins[i]));
   }
   if (nsteps > done)

@@ -132,8 +132,8 @@ __device__ __forceinline__ void lattice_chunks(const StreamArgs<real, S> &A, int
       A.G.at(g, gx, y, z);
       z += A.z0;
       if constexpr (sizeof(S) == 2) {
-        if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z);
-        else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z);
+        if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
+        else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
       } else {
         const int x0 = 2 * gx;
         real a[Q], b[Q];
@@ -181,7 +181,7 @@ __device__ __forceinline__ void fused_steps(const FusedArgs<real, S> &P, SourceS
     lattice_chunks(A.stream, &ctl->next[s & 1]);
     ALL_BARRIER();
     if (blockIdx.x == 0 && tid == 0) ctl->next[s & 1] = 0;  // used again two steps on
-    tiles_body<real, S>(A.tiles, all_first, all_stride);
+    tiles_body<false>(A.tiles, all_first, all_stride);
     ALL_BARRIER();
     if (chain) {
       shell_body<real, S>(A.shell, chain_first, chain_stride);

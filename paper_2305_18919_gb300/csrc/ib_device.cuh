@@ -79,6 +79,105 @@ __device__ __forceinline__ real lj_fz(real dz, real eps48, real xi) {
   return eps48 * (s6 * s6 - real(0.5) * s6) * dz * inv_d2;
 }
 
+// Tiles covered along one axis by the stencil of coordinate p: t0 (lower) and t1 (upper,
+// equal to t0 when the four nodes fall in one tile); `ok1` tells whether t1 is a distinct
+// tile that exists. Periodic axes wrap; along a walled z axis tiles beyond the lattice are
+// skipped (valid flags).
+struct AxisTiles {
+  int t0, t1;
+  bool ok0, ok1;
+};
+
+// of an axis of n nodes (nt tiles)
+__device__ __forceinline__ AxisTiles axis_tiles(double p, int n, int nt, double inv_n, bool periodic) {
+  AxisTiles a;
+  double r;
+  const int b = stencil_base(p, n, inv_n, periodic, r);
+  a.t0 = b >> 2;  // (arithmetic shift: floors)
+  a.t1 = (b + 3) >> 2;
+  if (periodic) {
+    a.t1 = a.t1 >= nt ? a.t1 - nt : a.t1;
+    a.ok0 = true;
+    a.ok1 = a.t1 != a.t0;  // a short periodic axis may wrap onto the same tile
+  } else {
+    a.ok0 = a.t0 >= 0 && a.t0 < nt;
+    a.ok1 = a.t1 != a.t0 && a.t1 >= 0 && a.t1 < nt;
+  }
+  return a;
+}
+
+// Tile e (bit k picks the upper tile along axis k) of the stencil described by ax, or -1.
+__device__ __forceinline__ int stencil_tile(const AxisTiles ax[3], int e, const Dims &D) {
+  int t[3];
+  for (int k = 0; k < 3; k++) {
+    const bool up = (e >> k) & 1;
+    if (up ? !ax[k].ok1 : !ax[k].ok0) return -1;
+    t[k] = up ? ax[k].t1 : ax[k].t0;
+  }
+  return (t[2] * D.nty + t[1]) * D.ntx + t[0];
+}
+
+// A tile map: the active tiles of one step's positions. Marked by the face pass of that step.
+struct TileMap {
+  int *tile_slot, *slot_tile, *nslots, *slot_count, *out_src, *health;
+};
+
+// Mark the tiles of the stencils of eight vertices by one warp (called together): lane l takes
+// vertex v0 + l / 4 and, l % 4 = k < 3, its axis k; each lane then claims two of the vertex's (up
+// to 8) tiles. The first claimant of a tile takes a new slot; a plain read first keeps the many
+// vertices of an already-claimed tile off the atomics, and a lane's two claims are in flight
+// together.
+__device__ __forceinline__ void mark_vertices(const double *IBLB_RO q, int nv, int v0, const Dims &D,
+                                              const TileMap &M) {
+  const int lane = threadIdx.x & 31, k = lane & 3, v = v0 + (lane >> 2);
+  int t0 = 0, t1 = 0, flags = 0;  // bit 0 / 1: ok0 / ok1 of the axis; bit 2: a number
+  if (v < nv && k < 3) {
+    const double p = q[3 * (size_t)v + k];
+    if (p == p) {
+      const int n = k == 0 ? D.nx : k == 1 ? D.ny : D.nz;
+      const int nt = k == 0 ? D.ntx : k == 1 ? D.nty : D.ntz;
+      const double inv = k == 0 ? D.inx : k == 1 ? D.iny : D.inz;
+      const AxisTiles ax = axis_tiles(p, n, nt, inv, k < 2 || !D.has_walls);
+      t0 = ax.t0;
+      t1 = ax.t1;
+      flags = (ax.ok0 ? 1 : 0) | (ax.ok1 ? 2 : 0) | 4;
+    }
+  }
+  AxisTiles ax[3];
+  int all = 4;
+  for (int a = 0; a < 3; a++) {
+    ax[a].t0 = __shfl_sync(0xffffffffu, t0, a, 4);
+    ax[a].t1 = __shfl_sync(0xffffffffu, t1, a, 4);
+    const int fl = __shfl_sync(0xffffffffu, flags, a, 4);
+    ax[a].ok0 = fl & 1;
+    ax[a].ok1 = fl & 2;
+    all &= fl;
+  }
+  if (!all) return;  // (also beyond the last vertex)
+  int t[2], won[2];
+  for (int h = 0; h < 2; h++) {
+    t[h] = stencil_tile(ax, k + 4 * h, D);
+    won[h] = t[h] >= 0 && *(volatile int *)&M.tile_slot[t[h]] == -1;
+  }
+  for (int h = 0; h < 2; h++)
+    if (won[h]) won[h] = atomicCAS(&M.tile_slot[t[h]], -1, -2) == -1;
+  if (!(won[0] | won[1])) return;
+  int s = atomicAdd(M.nslots, won[0] + won[1]);
+  for (int h = 0; h < 2; h++) {
+    if (!won[h]) continue;
+    if (s < D.max_slots) {
+      M.slot_tile[s] = t[h];
+      M.slot_count[s] = 0;
+      int4 *o = reinterpret_cast<int4 *>(M.out_src + 8 * (size_t)s);
+      o[0] = o[1] = make_int4(-1, -1, -1, -1);
+      atomicExch(&M.tile_slot[t[h]], s);
+    } else {
+      atomicOr(M.health, H_CAPACITY);
+    }
+    s++;
+  }
+}
+
 // Per-face reference data in the population type, stored by component ([FGEO][nf]): A, B
 // (edges), X0 - c, the reference centroid height above the bottom and the top wall plane, a
 // pad, and the reference metric inverse H11, H12, H22 with the reference area A0 (rounded
@@ -98,7 +197,9 @@ struct FaceParams {
 // K3a: one thread per face, in the population type. Writes the strain + wall force of each
 // corner, the face's contribution (a x b)/6 to the volume gradient of each of its corners,
 // and one partial sum per warp of V_j - V0_j, the change of the face's share of the volume.
-// With reset != 0 it also clears the tile map that the previous step used.
+// With reset != 0 (a step) it also marks the tile map of the current positions and clears the one
+// that the previous step used. The marking runs beside the faces, by warps of its own: at the end
+// of the interpolation its two rounds of atomics were the longest chain of the step.
 //
 // V_j = (x0 - c) . (a x b) / 6 for a fixed point c. Written with the displacements
 // u_k = x_k - X_k from the reference shape (da = u1 - u0, db = u2 - u0, reference edges A, B)
@@ -119,6 +220,9 @@ struct FaceArgs {
   int *other_tile_slot;
   const int *other_slot_tile, *other_nslots;
   int reset;
+  TileMap map;           // with reset: the map of the current positions, marked by this pass
+  const double *q;
+  int nv;
   int *ovf_count;
   unsigned *spill_bits;  // [spill_words] cleared here, before the vertex kernel bins
   int spill_words;
@@ -134,8 +238,12 @@ struct FaceThreads {
 };
 constexpr int kVertexThreads = 64;
 
-// K3a for the faces first, first + stride, ... (`first`: of this thread; a warp's 32 threads hold
-// 32 consecutive ones and call it together).
+// Warps of K3a: one per eight vertices to mark, then one per 32 faces.
+template <typename real>
+__device__ __forceinline__ int mark_warps(const FaceArgs<real> &A) { return A.reset ? (A.nv + 7) / 8 : 0; }
+
+// K3a for the warps first / 32, first / 32 + stride / 32, ... (`first`: of this thread; a warp's 32
+// threads hold 32 consecutive ones and call it together).
 template <typename real>
 __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int first, int stride) {
   const int nf = A.nf;
@@ -148,7 +256,13 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int first, in
   const FaceParams<real> fp = A.fp;
   const Dims D = A.D;
   const int lane = threadIdx.x & 31;
-  for (int j = first; j - lane < nf; j += stride) {
+  const int marks = mark_warps(A), warps = marks + (nf + 31) / 32;
+  for (int w = first >> 5; w < warps; w += stride >> 5) {
+  if (w < marks) {
+    mark_vertices(A.q, A.nv, 8 * w, D, A.map);
+    continue;
+  }
+  const int j = 32 * (w - marks) + lane;
   real dvj = 0;
   if (j < nf) {
     const int iv[3] = {faces[3 * j], faces[3 * j + 1], faces[3 * j + 2]};
@@ -347,16 +461,16 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int i) {
 #pragma unroll
     for (int u = 0; u < GATHER_UNROLL; u++) fcs[u] = eb + u < e1 ? vf_list[eb + u] : -1;
 #pragma unroll
-    for (int u = 0; u < GATHER_UNROLL; u++) {
-      if (fcs[u] < 0) continue;
-      const Vec4<real> fc = fcontrib[fcs[u]];   // face * 3 + corner
-      const Vec4<real> fn = fnorm[fcs[u] / 3];
-      F[0] += fc.x;
-      F[1] += fc.y;
-      F[2] += fc.z;
-      g[0] += fn.x;
-      g[1] += fn.y;
-      g[2] += fn.z;
+    for (int u = 0; u < GATHER_UNROLL; u++) {  // (no branch between the loads: all in flight)
+      const int fc = max(fcs[u], 0);              // face * 3 + corner
+      Vec4<real> f = fcontrib[fc], n = fnorm[fc / 3];
+      if (fcs[u] < 0) f = n = Vec4<real>{0, 0, 0, 0};
+      F[0] += f.x;
+      F[1] += f.y;
+      F[2] += f.z;
+      g[0] += n.x;
+      g[1] += n.y;
+      g[2] += n.z;
     }
   }
   Vec4<real> pv, gv;
@@ -660,18 +774,25 @@ __device__ __forceinline__ void spread_gather_body(const GatherArgs<real> &A, in
   const int nslots = min(*A.nslots_ptr, D.max_slots);
   const int lx = tid & 3, ly = (tid >> 2) & 3, lz = tid >> 4;
   for (int b = bid; b < nslots; b += nb) {
-    const int *src = out_src + 8 * (size_t)b;
+    const int4 *src4 = reinterpret_cast<const int4 *>(out_src + 8 * (size_t)b);
+    const int4 lo = src4[0], hi = src4[1];
+    const int src[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
     real f[3] = {0, 0, 0};
     bool stencil_node = false;
+    Vec4<real> r[8];
+#pragma unroll
     for (int e = 0; e < 8; e++) {
-      const int reg = src[e];
       const int rx = lx + 4 * (e & 1), ry = ly + 4 * ((e >> 1) & 1), rz = lz + 4 * (e >> 2);
-      if (reg < 0 || rx >= REGION || ry >= REGION || rz >= REGION) continue;
-      const Vec4<real> r = Rslot[(size_t)reg * REGION_NODES + (rz * REGION + ry) * REGION + rx];
-      f[0] += r.x;
-      f[1] += r.y;
-      f[2] += r.z;
-      stencil_node |= r.w != real(0);
+      const bool in = src[e] >= 0 && rx < REGION && ry < REGION && rz < REGION;
+      r[e] = Vec4<real>{0, 0, 0, 0};
+      if (in) r[e] = Rslot[(size_t)src[e] * REGION_NODES + (rz * REGION + ry) * REGION + rx];
+    }
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      f[0] += r[e].x;
+      f[1] += r[e].y;
+      f[2] += r[e].z;
+      stencil_node |= r[e].w != real(0);
     }
     const int Z = (slot_tile[b] / (D.ntx * D.nty)) * TILE + lz;
     const bool drop = D.has_walls && (Z == 0 || Z >= D.nz - 1);
@@ -708,70 +829,9 @@ __global__ void __launch_bounds__(64) spread_gather_kernel_multi(
   spread_gather_body(all[m.inst], m.block, m.nblocks, threadIdx.x);
 }
 
-// Claim tile t in map (tile_slot, slot_tile, nslots), whose entry read `seen` a moment ago: the
-// first claimant takes a new slot. (The plain read keeps the many vertices of an already-claimed
-// tile off the atomic.)
-__device__ __forceinline__ void claim_tile(int t, int seen, int *tile_slot, int *slot_tile,
-                                           int *nslots, int *slot_count, int *out_src, int *health,
-                                           int max_slots) {
-  if (seen != -1) return;
-  if (atomicCAS(&tile_slot[t], -1, -2) == -1) {
-    const int s = atomicAdd(nslots, 1);
-    if (s < max_slots) {
-      slot_tile[s] = t;
-      slot_count[s] = 0;
-      int4 *o = reinterpret_cast<int4 *>(out_src + 8 * (size_t)s);
-      o[0] = o[1] = make_int4(-1, -1, -1, -1);
-      atomicExch(&tile_slot[t], s);
-    } else {
-      atomicOr(health, H_CAPACITY);
-    }
-  }
-}
-
-// Tiles covered along one axis by the stencil of coordinate p: t0 (lower) and t1 (upper,
-// equal to t0 when the four nodes fall in one tile); `ok1` tells whether t1 is a distinct
-// tile that exists. Periodic axes wrap; along a walled z axis tiles beyond the lattice are
-// skipped (valid flags).
-struct AxisTiles {
-  int t0, t1;
-  bool ok0, ok1;
-};
-
-// of an axis of n nodes (nt tiles)
-__device__ __forceinline__ AxisTiles axis_tiles(double p, int n, int nt, double inv_n, bool periodic) {
-  AxisTiles a;
-  double r;
-  const int b = stencil_base(p, n, inv_n, periodic, r);
-  a.t0 = b >> 2;  // (arithmetic shift: floors)
-  a.t1 = (b + 3) >> 2;
-  if (periodic) {
-    a.t1 = a.t1 >= nt ? a.t1 - nt : a.t1;
-    a.ok0 = true;
-    a.ok1 = a.t1 != a.t0;  // a short periodic axis may wrap onto the same tile
-  } else {
-    a.ok0 = a.t0 >= 0 && a.t0 < nt;
-    a.ok1 = a.t1 != a.t0 && a.t1 >= 0 && a.t1 < nt;
-  }
-  return a;
-}
-
-// Tile e (bit k picks the upper tile along axis k) of the stencil described by ax, or -1.
-__device__ __forceinline__ int stencil_tile(const AxisTiles ax[3], int e, const Dims &D) {
-  int t[3];
-  for (int k = 0; k < 3; k++) {
-    const bool up = (e >> k) & 1;
-    if (up ? !ax[k].ok1 : !ax[k].ok0) return -1;
-    t[k] = up ? ax[k].t1 : ax[k].t0;
-  }
-  return (t[2] * D.nty + t[1]) * D.ntx + t[0];
-}
-
 // K2: interpolation (Eq. 11) and the Euler update (Eq. 12); 4 lanes per vertex, lane dz
 // sums the 16 nodes of its z-plane of the stencil, the 4 planes are summed by shuffles; lane k
-// then adds the update to coordinate k of the double position and finds the tiles of the new
-// stencil along that axis; each lane marks two of the (up to 8) tiles in the other map. One
-// lane per axis issues a third of the FP64 instructions of one lane per vertex (an FP64
+// then adds the update to coordinate k of the double position. One lane per axis issues a third of the FP64 instructions of one lane per vertex (an FP64
 // instruction holds the SM's FP64 unit for 16 cycles however few lanes take part): 10242 vertices
 // on 64 SMs 12.8 us against 17.2, 40962 on 24 SMs 88 against 127, 96 wetting boxes 108 against 262.
 // The delta-weight accumulation of a vertex is carried at double precision in every
@@ -846,7 +906,7 @@ struct InterpArgs {
   Vec4<real> *disp;
   double3 ub, ut;
   Dims D;
-  int *next_tile_slot, *next_slot_tile, *next_nslots, *slot_count, *out_src, *health;
+  int *health;
 };
 
 // K2 for lane `gid` (vertex gid / 4, plane gid % 4); a warp's 32 lanes are consecutive and call it
@@ -863,7 +923,6 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) 
   Vec4<real> *IBLB_RO disp = A.disp;
   const double3 ub = A.ub, ut = A.ut;
   const Dims D = A.D;
-  int *next_tile_slot = A.next_tile_slot;
   int *IBLB_RO health = A.health;
   const int v = gid >> 2;
   const int dz = gid & 3;
@@ -902,21 +961,28 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) 
         for (int iy = 0; iy < 2; iy++)
           for (int ix = 0; ix < 2; ix++)
             sl[iy][ix] = tile_slot[(tzrow + (Y[3 * iy] >> 2)) * D.ntx + (X[3 * ix] >> 2)];
+        // an unmarked tile (only after a capacity failure) counts as at rest; checked ahead of the
+        // loads, so that no branch stands between them and they are all in flight at once
+        if (min(min(sl[0][0], sl[0][1]), min(sl[1][0], sl[1][1])) < 0) atomicOr(health, H_CAPACITY);
+#pragma unroll
         for (int dy = 0; dy < 4; dy++) {
-          const int iy = (Y[dy] >> 2) != (Y[0] >> 2);
+          const bool uy = (Y[dy] >> 2) != (Y[0] >> 2);
           const int crow = 4 * (Y[dy] & 3) + 16 * (Z & 3);
-          real r3[3] = {0, 0, 0};
+          const int s0 = uy ? sl[1][0] : sl[0][0], s1 = uy ? sl[1][1] : sl[0][1];
+          Vec4<real> u[4];
+#pragma unroll
           for (int dx = 0; dx < 4; dx++) {
-            const int sidx = sl[iy][(X[dx] >> 2) != (X[0] >> 2)];
-            if (sidx < 0) {  // unmarked tile: only after a capacity failure, flagged there
-              atomicOr(health, H_CAPACITY);
-              continue;
-            }
-            const Vec4<real> u = Uslot[(size_t)sidx * TILE_CELLS + (X[dx] & 3) + crow];
+            const int sidx = (X[dx] >> 2) != (X[0] >> 2) ? s1 : s0;
+            u[dx] = Uslot[(size_t)max(sidx, 0) * TILE_CELLS + (X[dx] & 3) + crow];
+            if (sidx < 0) u[dx] = Vec4<real>{0, 0, 0, 0};
+          }
+          real r3[3] = {0, 0, 0};
+#pragma unroll
+          for (int dx = 0; dx < 4; dx++) {
             const real w = rec.w[0][dx];
-            r3[0] += w * u.x;
-            r3[1] += w * u.y;
-            r3[2] += w * u.z;
+            r3[0] += w * u[dx].x;
+            r3[1] += w * u[dx].y;
+            r3[2] += w * u[dx].z;
           }
           const real wyz = rec.w[1][dy] * wz;
           acc.add_prod(0, wyz, r3[0]);
@@ -928,7 +994,6 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) 
   }
   // sum of the 4 planes (fixed butterfly order)
   for (int o = 2; o > 0; o >>= 1) acc.add_lanes(o);
-  int t0 = 0, t1 = 0, flags = 0;  // bit 0 / 1: ok0 / ok1 of the axis; bit 2: a number
   if (axis) {
     const double qd = acc.value(dz);
     const double pn = qk + qd;
@@ -939,34 +1004,6 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) 
     if (dz == 2 && D.has_walls && (pn - D.zb < 0.05 || D.zt - pn < 0.05)) h |= H_WALL;
     if (h) atomicOr(health, h);
     reinterpret_cast<real *>(disp + v)[dz] = (real)(pn - xk);
-    if (next_tile_slot != nullptr && pn == pn) {
-      const int n = dz == 0 ? D.nx : dz == 1 ? D.ny : D.nz;
-      const int nt = dz == 0 ? D.ntx : dz == 1 ? D.nty : D.ntz;
-      const double inv = dz == 0 ? D.inx : dz == 1 ? D.iny : D.inz;
-      const AxisTiles ax = axis_tiles(pn, n, nt, inv, dz < 2 || !D.has_walls);
-      t0 = ax.t0;
-      t1 = ax.t1;
-      flags = (ax.ok0 ? 1 : 0) | (ax.ok1 ? 2 : 0) | 4;
-    }
-  }
-  AxisTiles ax[3];
-  int all = 4;
-  for (int k = 0; k < 3; k++) {
-    ax[k].t0 = __shfl_sync(0xffffffffu, t0, k, 4);
-    ax[k].t1 = __shfl_sync(0xffffffffu, t1, k, 4);
-    const int fl = __shfl_sync(0xffffffffu, flags, k, 4);
-    ax[k].ok0 = fl & 1;
-    ax[k].ok1 = fl & 2;
-    all &= fl;
-  }
-  if (valid && all) {  // each lane claims two of the (up to 8) tiles
-    const int ta = stencil_tile(ax, dz, D), tb = stencil_tile(ax, dz + 4, D);
-    const int sa = ta >= 0 ? *(volatile int *)&next_tile_slot[ta] : 0;
-    const int sb = tb >= 0 ? *(volatile int *)&next_tile_slot[tb] : 0;
-    claim_tile(ta, sa, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count, A.out_src,
-               health, D.max_slots);
-    claim_tile(tb, sb, next_tile_slot, A.next_slot_tile, A.next_nslots, A.slot_count, A.out_src,
-               health, D.max_slots);
   }
 }
 
@@ -985,34 +1022,12 @@ __global__ void __launch_bounds__(kInterpThreads) interp_kernel_multi(
   interp_body(all[m.inst], m.block * blockDim.x + threadIdx.x);
 }
 
-// Standalone marking of the current positions (after setting vertices); also refreshes the
-// float displacement from the reference shape.
+// Displacement from the reference shape, after setting vertices; one thread per coordinate.
 template <typename real>
-__global__ void mark_kernel(int nv, const double *__restrict__ q, const double *__restrict__ xref,
-                            Vec4<real> *__restrict__ disp, Dims D, int *tile_slot,
-                            int *slot_tile, int *nslots, int *slot_count, int *out_src,
-                            int *health) {
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int v = gid >> 3, e = gid & 7;
-  if (v >= nv) return;
-  const double p[3] = {q[3 * (size_t)v], q[3 * (size_t)v + 1], q[3 * (size_t)v + 2]};
-  if (e == 0) {
-    Vec4<real> d;
-    d.x = (real)(p[0] - xref[3 * (size_t)v]);
-    d.y = (real)(p[1] - xref[3 * (size_t)v + 1]);
-    d.z = (real)(p[2] - xref[3 * (size_t)v + 2]);
-    d.w = real(0);
-    disp[v] = d;
-  }
-  if (p[0] == p[0] && p[1] == p[1] && p[2] == p[2]) {
-    AxisTiles ax[3];
-    ax[0] = axis_tiles(p[0], D.nx, D.ntx, D.inx, true);
-    ax[1] = axis_tiles(p[1], D.ny, D.nty, D.iny, true);
-    ax[2] = axis_tiles(p[2], D.nz, D.ntz, D.inz, !D.has_walls);
-    const int t = stencil_tile(ax, e, D);
-    claim_tile(t, t >= 0 ? *(volatile int *)&tile_slot[t] : 0, tile_slot, slot_tile, nslots,
-               slot_count, out_src, health, D.max_slots);
-  }
+__global__ void displacement_kernel(int nv, const double *__restrict__ q,
+                                    const double *__restrict__ xref, Vec4<real> *__restrict__ disp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 3 * nv) reinterpret_cast<real *>(disp + i / 3)[i % 3] = (real)(q[i] - xref[i]);
 }
 
 template <typename real>
@@ -1064,6 +1079,12 @@ VolumeParams volume_params(const Ctx &c) {
   return vp;
 }
 
+// The tile map of the context's current positions.
+TileMap tile_map(const Ctx &c) {
+  return TileMap{c.tile_slot[c.map], c.slot_tile[c.map], c.counters + c.map, c.slot_count,
+                 c.out_src[c.map], c.counters + 3};
+}
+
 // Argument records of the step kernels for context c as it is now (its cur and map), shared by
 // the single-context launches and the batched ones.
 template <typename real>
@@ -1089,14 +1110,18 @@ FaceArgs<real> face_args(const Ctx &c, int reset) {
   a.other_slot_tile = c.slot_tile[other];
   a.other_nslots = c.counters + other;
   a.reset = reset;
+  a.map = tile_map(c);
+  a.q = c.q;
+  a.nv = c.nv;
   a.ovf_count = c.counters + 2;
   a.spill_bits = c.spill_bits;
   a.spill_words = c.spill_words;
   return a;
 }
 template <typename real>
-int face_blocks(const Ctx &c) {
-  return (c.nf + FaceThreads<real>::value - 1) / FaceThreads<real>::value;
+int face_blocks(const Ctx &c, int reset) {
+  const int warps = (c.nf + 31) / 32 + (reset ? (c.nv + 7) / 8 : 0);
+  return (32 * warps + FaceThreads<real>::value - 1) / FaceThreads<real>::value;
 }
 
 template <typename real>
@@ -1184,7 +1209,6 @@ int gather_blocks(const Ctx &c, bool batched) {
 
 template <typename real>
 InterpArgs<real> interp_args(const Ctx &c) {
-  const int other = c.map ^ 1;
   InterpArgs<real> a;
   a.nv = c.nv;
   a.stencil = (const StencilRec<real> *)c.stencil;
@@ -1197,11 +1221,6 @@ InterpArgs<real> interp_args(const Ctx &c) {
   a.ub = make_double3(c.ub[0], c.ub[1], c.ub[2]);
   a.ut = make_double3(c.ut[0], c.ut[1], c.ut[2]);
   a.D = dims_of(c);
-  a.next_tile_slot = c.tile_slot[other];
-  a.next_slot_tile = c.slot_tile[other];
-  a.next_nslots = c.counters + other;
-  a.slot_count = c.slot_count;
-  a.out_src = c.out_src[other];
   a.health = c.counters + 3;
   return a;
 }

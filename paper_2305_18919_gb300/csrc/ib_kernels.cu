@@ -5,6 +5,11 @@
 namespace iblb {
 namespace {
 
+// Standalone marking of the current positions (a read of the spread field between steps).
+__global__ void mark_kernel(int nv, const double *IBLB_RO q, Dims D, TileMap M) {
+  mark_vertices(q, nv, 8 * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5), D, M);
+}
+
 __global__ void clear_counts_kernel(const int *__restrict__ nslots, int *__restrict__ slot_count,
                                     int *__restrict__ ovf_count, int max_slots) {
   const int n = min(*nslots, max_slots);
@@ -26,7 +31,7 @@ __global__ void volume_sum_kernel(const double *__restrict__ part, int n, double
 
 template <typename real>
 cudaError_t face_forces_t(Ctx &c, int reset, cudaStream_t st) {
-  face_kernel<real><<<face_blocks<real>(c), FaceThreads<real>::value, 0, st>>>(face_args<real>(c, reset));
+  face_kernel<real><<<face_blocks<real>(c, reset), FaceThreads<real>::value, 0, st>>>(face_args<real>(c, reset));
   return cudaGetLastError();
 }
 
@@ -62,7 +67,7 @@ void append_record(std::vector<unsigned char> &bytes, const T &rec) {
 template <typename real>
 int ib_multi_record_t(const Ctx &c, MultiKernel k, std::vector<unsigned char> &bytes) {
   switch (k) {
-    case MK_FACE: append_record(bytes, face_args<real>(c, 1)); return face_blocks<real>(c);
+    case MK_FACE: append_record(bytes, face_args<real>(c, 1)); return face_blocks<real>(c, 1);
     case MK_VERTEX: append_record(bytes, vertex_args<real>(c, 2)); return vertex_blocks(c);
     case MK_SOURCE: append_record(bytes, source_args<real>(c)); return source_blocks<real>(c, true);
     case MK_GATHER: append_record(bytes, gather_args<real>(c)); return gather_blocks(c, true);
@@ -153,16 +158,17 @@ cudaError_t launch_interpolate_advect(Ctx &c, cudaStream_t s) {
 }
 
 cudaError_t launch_mark(Ctx &c) {
-  const long threads = 8L * c.nv;
-  const unsigned blocks = (unsigned)((threads + 255) / 256);
+  const int warps = (c.nv + 7) / 8;
+  mark_kernel<<<(32 * warps + 127) / 128, 128, 0, c.stream>>>(c.nv, c.q, dims_of(c), tile_map(c));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_displacement(Ctx &c) {
+  const int blocks = (3 * c.nv + 127) / 128;
   if (c.precision == IBLB_FP64)
-    mark_kernel<double><<<blocks, 256, 0, c.stream>>>(
-        c.nv, c.q, c.xref, (Vec4<double> *)c.disp, dims_of(c), c.tile_slot[c.map],
-        c.slot_tile[c.map], c.counters + c.map, c.slot_count, c.out_src[c.map], c.counters + 3);
+    displacement_kernel<double><<<blocks, 128, 0, c.stream>>>(c.nv, c.q, c.xref, (Vec4<double> *)c.disp);
   else
-    mark_kernel<float><<<blocks, 256, 0, c.stream>>>(
-        c.nv, c.q, c.xref, (Vec4<float> *)c.disp, dims_of(c), c.tile_slot[c.map],
-        c.slot_tile[c.map], c.counters + c.map, c.slot_count, c.out_src[c.map], c.counters + 3);
+    displacement_kernel<float><<<blocks, 128, 0, c.stream>>>(c.nv, c.q, c.xref, (Vec4<float> *)c.disp);
   return cudaGetLastError();
 }
 

@@ -156,6 +156,8 @@ struct Ctx {
   int *pair_list = nullptr;                // [32 max_slots] slot * 32 + pair: the node pairs with
                                            //   a non-zero force (K4b appends, K1t reads)
   int map = 0;                             // tile map of the current vertex positions
+  int marked = 0;                          // that map holds their tiles (else it is empty and
+                                           //   the next step's face pass marks it)
   // mesh
   int nv = 0, nf = 0;
   double *q = nullptr;       // [nv][3] positions (double in every precision)
@@ -221,7 +223,7 @@ int enqueue_steps(Ctx &c, int nsteps);
 // IBLB_OK for a clear health word, else the matching error code (message in c.err).
 int health_status(Ctx &c, int health_word);
 // Replace the state by populations P (the storage layout of f[cur]) and positions q (device
-// arrays), with the given fresh flag, and mark the tiles of q: the next step continues from
+// arrays), with the given fresh flag: the next step continues from
 // there exactly as from the state that P and q were copied from.
 int restore_state(Ctx &c, const void *P, const double *q, int fresh);
 // A failure of steps queued by iblb_step_async: read with a synchronisation (settle_health), or
@@ -260,7 +262,9 @@ size_t stencil_record_bytes(const Ctx &c);
 cudaError_t launch_vertex_forces(Ctx &c, int bin, cudaStream_t s);
 cudaError_t launch_spread(Ctx &c, cudaStream_t s);
 cudaError_t launch_interpolate_advect(Ctx &c, cudaStream_t s);
+// Mark the (empty) tile map of the current positions; refresh the displacements from them.
 cudaError_t launch_mark(Ctx &c);
+cudaError_t launch_displacement(Ctx &c);
 cudaError_t launch_clear_counts(Ctx &c);
 cudaError_t launch_expand_force(Ctx &c, double *F_dev);
 cudaError_t launch_phi_to_double(Ctx &c, double *phi_dev);
@@ -275,6 +279,7 @@ enum MultiKernel {
   MK_SOURCE,          // K4a
   MK_GATHER,          // K4b
   MK_STREAM_COLLIDE,  // K1 (not the first, in-place step)
+  MK_FORCED,          // K1 and K1t in one
   MK_TILES,           // K1t
   MK_SHELL,           // K1b
   MK_INTERP,          // K2

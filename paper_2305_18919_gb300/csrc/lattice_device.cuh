@@ -396,9 +396,13 @@ __device__ __forceinline__ double fma_(double a, double b, double c) { return fm
 // FP64 multiply-add, so the two share one reciprocal, 1/(ab), by Newton's iteration
 // r <- r + r (1 - x r) from a float seed (relative error 2^-23, then 2^-46, then rounding);
 // outside the seed's range they are plain divisions. u enters the collision only at second order.
-__device__ __forceinline__ void reciprocals(float a, float b, float &ra, float &rb) {
-  ra = 1.0f / a;
-  rb = 1.0f / b;
+__device__ __forceinline__ float reciprocal(float a) { return 1.0f / a; }
+__device__ __forceinline__ double reciprocal(double a) {
+  const float s = (float)a;
+  if (!(s > 1e-30f && s < 1e30f)) return 1.0 / a;
+  double r = (double)(1.0f / s);
+  r = fma(r, fma(-a, r, 1.0), r);
+  return fma(r, fma(-a, r, 1.0), r);
 }
 __device__ __forceinline__ void reciprocals(double a, double b, double &ra, double &rb) {
   const double x = mul_(a, b);
@@ -686,9 +690,11 @@ __device__ __forceinline__ unsigned int as_bits(V2 v) {
 // 2-byte type needs to keep HBM busy. The loaded rows stay packed in registers (`lo` holds
 // nodes x0, x0 + 1, `hi` nodes x0 + 2, x0 + 3) and are widened one node pair at a time for
 // the collision; the results are packed back in place.
-template <typename S, bool FIRST, bool FORCE>
+// `After`: applied to the packed results lo, hi before they are stored.
+template <typename S, bool FIRST, bool FORCE, typename After>
 __device__ __forceinline__ void quad_nodes(const S *IBLB_RO fin, S *IBLB_RO fout,
-                                           const LatParams<float> &P, int x0, int y, int z) {
+                                           const LatParams<float> &P, int x0, int y, int z,
+                                           After after) {
   using V2 = typename Storage<S>::V2;
   const size_t plane = (size_t)P.nx * P.ny;
   const size_t n = (size_t)z * plane + (size_t)y * P.nx + x0;
@@ -756,10 +762,16 @@ __device__ __forceinline__ void quad_nodes(const S *IBLB_RO fin, S *IBLB_RO fout
 #pragma unroll
     for (int i = 0; i < Q; i++) pk[i] = as_bits(narrow_pair<V2>(g[i]));
   }
+  after(lo, hi);
 #pragma unroll
   for (int i = 0; i < Q; i++)
     *reinterpret_cast<uint2 *>(fout + (size_t)i * P.ncell + n) = make_uint2(lo[i], hi[i]);
 }
+
+// no step after the collision
+struct Nothing {
+  __device__ __forceinline__ void operator()(unsigned int *, unsigned int *) const {}
+};
 
 template <typename real, typename S>
 struct StreamArgs {
@@ -769,6 +781,8 @@ struct StreamArgs {
   FlatGroups G;  // node groups of the context
   int z0;        // first fluid layer
   int force;     // the body force is non-zero
+  const int *tile_slot;        // the interface force of the step, by active tile (null: no mesh)
+  const Vec4<real> *Fslot;
 };
 
 // K1t: the fluid nodes of the active tiles with body + interface force. Runs after K1 of the
@@ -778,8 +792,11 @@ struct StreamArgs {
 // and j = J - g, J = sum c f0, without the pre-collision populations. K1t therefore reads and
 // writes only each node's own populations, no pulled neighbours.
 // Its work list is the node pairs (x0, x0 + 1), x0 even, that hold a node of some vertex's
-// stencil, appended by the spreading's gather pass (K4b) as slot * 32 + pair; one thread per
-// listed pair. Pairs without force keep K1's result, which is already final.
+// stencil, appended by the spreading's gather pass (K4b) as slot * 32 + pair. Nodes without force
+// keep K1's result, which is already final. A thread takes a listed pair, or one node of it: long
+// lists are bound by the scattered rows' accesses, which the pair halves (96 wetting boxes: 1.29
+// ms per step against 1.36), short ones by one thread's chain, which the node halves (32^3 FP64 in
+// the fused kernel: 6.8 us against 11.5). Both give the same bits.
 template <typename real, typename S>
 struct TilesArgs {
   S *fout;
@@ -830,45 +847,115 @@ __device__ __forceinline__ void apply_force(real f[Q], real drho, const real J[3
   }
 }
 
-template <typename real, typename S>
+// apply_force at one node (deviations f after K1's collision) with its interface force.
+template <typename real>
+__device__ __forceinline__ void correct_node(real f[Q], const Vec4<real> &F, const LatParams<real> &P) {
+  const real Fk[3] = {F.x, F.y, F.z};
+  real drho, J[3];
+  node_moments(f, drho, J);
+  apply_force(f, drho, J, reciprocal(add_(P.rho0, drho)), Fk, P.ct);
+}
+template <typename real>
+__device__ __forceinline__ bool any_force(const Vec4<real> &F) {
+  return F.x != real(0) || F.y != real(0) || F.z != real(0);
+}
+
+template <bool PAIR, typename real, typename S>
 __device__ __forceinline__ void tiles_body(const TilesArgs<real, S> &A, int first, int stride) {
-  using V2 = typename Storage<S>::V2;
   S *IBLB_RO fout = A.fout;
   const int *IBLB_RO slot_tile = A.slot_tile;
   const int *IBLB_RO pair_list = A.pair_list;
   const Vec4<real> *IBLB_RO Fslot = A.Fslot;
   const LatParams<real> P = A.P;  // held in registers: the loop below is latency-bound
-  const int npairs = min(*A.npairs_ptr, A.max_pairs);
-  for (int k = first; k < npairs; k += stride) {
-    const int e = pair_list[k];
-    const int s = e >> 5, cell = 2 * (e & 31);  // slot, and the pair's first node in the tile
-    const Vec4<real> Fa = Fslot[(size_t)s * TILE_CELLS + cell];
-    const Vec4<real> Fb = Fslot[(size_t)s * TILE_CELLS + cell + 1];
-    if (Fa.x == real(0) && Fa.y == real(0) && Fa.z == real(0) && Fb.x == real(0) &&
-        Fb.y == real(0) && Fb.z == real(0))
-      continue;
+  constexpr int N = PAIR ? 2 : 1;  // nodes of a thread
+  const int items = (PAIR ? 1 : 2) * min(*A.npairs_ptr, A.max_pairs);
+  for (int k = first; k < items; k += stride) {
+    const int e = pair_list[PAIR ? k : k >> 1];
+    const int s = e >> 5;                                    // slot, and the first node in the tile
+    const int cell = 2 * (e & 31) + (PAIR ? 0 : k & 1);
+    Vec4<real> Fv[N];
+    bool any = false;
+#pragma unroll
+    for (int m = 0; m < N; m++) {
+      Fv[m] = Fslot[(size_t)s * TILE_CELLS + cell + m];
+      any |= any_force(Fv[m]);
+    }
     const int t = slot_tile[s];
     const int tx = t % P.ntx, ty = (t / P.ntx) % P.nty, tz = t / (P.ntx * P.nty);
     const int x0 = tx * TILE + (cell & 3), y = ty * TILE + ((cell >> 2) & 3);
     const int z = tz * TILE + (cell >> 4);
     if (z >= P.nz || (P.has_walls && (z == 0 || z == P.nz - 1))) continue;
     const size_t n = (size_t)z * P.nx * P.ny + (size_t)y * P.nx + x0;
-    real a[Q], b[Q];
+    real f[N][Q];
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-      widen2(*reinterpret_cast<const V2 *>(fout + (size_t)i * P.ncell + n), a[i], b[i]);
-      a[i] *= real(kinv<S>(i));
-      b[i] *= real(kinv<S>(i));
+      const S *row = fout + (size_t)i * P.ncell + n;
+      if constexpr (PAIR) {
+        widen2(*reinterpret_cast<const typename Storage<S>::V2 *>(row), f[0][i], f[1][i]);
+        f[0][i] *= real(kinv<S>(i));
+        f[1][i] *= real(kinv<S>(i));
+      } else {
+        f[0][i] = real(widen(*row)) * real(kinv<S>(i));
+      }
     }
-    const real FA[3] = {Fa.x, Fa.y, Fa.z};
-    const real FB[3] = {Fb.x, Fb.y, Fb.z};
-    real da, db, Ja[3], Jb[3], ia, ib;
-    node_moments(a, da, Ja);
-    node_moments(b, db, Jb);
-    reciprocals(add_(P.rho0, da), add_(P.rho0, db), ia, ib);
-    apply_force(a, da, Ja, ia, FA, P.ct);
-    apply_force(b, db, Jb, ib, FB, P.ct);
-    store_pair(fout, P, n, a, b);
+    if (!any) continue;
+#pragma unroll
+    for (int m = 0; m < N; m++) correct_node(f[m], Fv[m], P);
+    if constexpr (PAIR) {
+      store_pair(fout, P, n, f[0], f[1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < Q; i++)
+        fout[(size_t)i * P.ncell + n] = Narrow<S>::one(f[0][i] * real(kscale<S>(i)));
+    }
+  }
+}
+
+// K1 and K1t in one: node group (gx, y, z) of the lattice pass, its active-tile nodes corrected
+// before they are stored, rounded to the storage type in between as in the two passes, so that
+// the results are theirs bit for bit. For passes that start after the step's force is complete.
+template <typename real, typename S, bool FORCE>
+__device__ __forceinline__ void forced_group(const StreamArgs<real, S> &A, int gx, int y, int z) {
+  constexpr int N = sizeof(S) == 2 ? 4 : 2;  // nodes of the group, all in one tile row
+  const LatParams<real> &P = A.P;
+  const int x0 = N * gx;
+  int slot = -1;
+  if (A.tile_slot) slot = A.tile_slot[((z >> 2) * P.nty + (y >> 2)) * P.ntx + (x0 >> 2)];
+  const Vec4<real> *F = A.Fslot + ((x0 & 3) + 4 * (y & 3) + 16 * (z & 3));
+  if constexpr (sizeof(S) == 2) {
+    using V2 = typename Storage<S>::V2;
+    quad_nodes<S, false, FORCE>(A.fin, A.fout, P, x0, y, z, [&](unsigned int *lo, unsigned int *hi) {
+      if (slot < 0) return;
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        const Vec4<real> Fa = F[(size_t)slot * TILE_CELLS + 2 * h];
+        const Vec4<real> Fb = F[(size_t)slot * TILE_CELLS + 2 * h + 1];
+        if (!any_force(Fa) && !any_force(Fb)) continue;
+        unsigned int *pk = h ? hi : lo;
+        real a[Q], b[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+          widen2(as_pair<V2>(pk[i]), a[i], b[i]);
+          a[i] *= real(kinv<S>(i));
+          b[i] *= real(kinv<S>(i));
+        }
+        correct_node(a, Fa, P);
+        correct_node(b, Fb, P);
+#pragma unroll
+        for (int i = 0; i < Q; i++)
+          pk[i] = as_bits(Narrow<S>::two(a[i] * real(kscale<S>(i)), b[i] * real(kscale<S>(i))));
+      }
+    });
+  } else {
+    real a[Q], b[Q];
+    load_pair<real, S, false>(A.fin, P, x0, y, z, a, b);
+    collide_pair<FORCE>(a, b, P);
+    if (slot >= 0) {
+      const Vec4<real> Fa = F[(size_t)slot * TILE_CELLS], Fb = F[(size_t)slot * TILE_CELLS + 1];
+      if (any_force(Fa)) correct_node(a, Fa, P);
+      if (any_force(Fb)) correct_node(b, Fb, P);
+    }
+    store_pair(A.fout, P, (size_t)z * P.nx * P.ny + (size_t)y * P.nx + x0, a, b);
   }
 }
 
@@ -906,14 +993,8 @@ __device__ __forceinline__ void shell_body(const ShellArgs<real, S> &A, int firs
     if (z >= P.nz || (P.has_walls && (z == 0 || z == P.nz - 1))) continue;
     real f[Q];
     pull<real, S, true>(fpost, P, x, y, z, f);
-    real drho = 0, j[3] = {0, 0, 0};
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      drho += f[i];
-      j[0] += cx(i) * f[i];
-      j[1] += cy(i) * f[i];
-      j[2] += cz(i) * f[i];
-    }
+    real drho, j[3];
+    node_moments(f, drho, j);
     const Vec4<real> Fs = Fslot[(size_t)s * TILE_CELLS + cell];
     const real Fk[3] = {Fs.x, Fs.y, Fs.z};
     const real rho_hi = P.rho0 + drho;
@@ -971,6 +1052,8 @@ StreamArgs<real, S> stream_args(const Ctx &c) {
   a.z0 = c.has_walls ? 1 : 0;
   a.G = k1_groups<S>(c);
   a.force = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
+  a.tile_slot = c.nv ? c.tile_slot[c.map] : nullptr;
+  a.Fslot = (const Vec4<real> *)c.Fslot[c.map];
   return a;
 }
 

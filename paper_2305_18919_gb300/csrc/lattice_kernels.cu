@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(128) stream_collide_quad_kernel(const S *__res
   if (g >= G.n) return;
   int gx, y, z;
   G.at(g, gx, y, z);
-  quad_nodes<S, FIRST, FORCE>(fin, fout, P, 4 * gx, y, z + z0);
+  quad_nodes<S, FIRST, FORCE>(fin, fout, P, 4 * gx, y, z + z0, Nothing());
 }
 
 // --- K1s: stream-collide with the pulled rows staged in shared memory by bulk copies ----------
@@ -451,23 +451,21 @@ __global__ void __launch_bounds__(staged_threads(NPT), 1) stream_collide_staged_
 // each thread takes one node group in memory order, a pair (x0, x0 + 1) or, with 16-bit
 // storage, four nodes x0 .. x0 + 3, and runs the very code of the single-context kernels on it,
 // so each context's populations come out bit for bit as from those.
-// Blocks per SM the batched pass is compiled for: 6 (80 registers) for FP32, where it keeps
-// the occupancy it has without the velocity correction (93 registers otherwise); no bound for
-// the others, which would spill under it.
-// Blocks per SM of the batched pass, run as a persistent grid over its blocks (0: one launch
-// block per 128 node groups). A pass that does not fill the SMs leaves room for the interface
-// kernels of the other stream, which then run beside it instead of after it (96 wetting
-// boxes: 1.317 ms per step with 4, 1.322 with 3, 1.402 with 6, 1.425 with 2, against 1.342
-// ms with a block per 128 node groups).
-constexpr int kK1MultiPerSM = 4;
+// Blocks per SM of the batched pass, run as a persistent grid over its blocks. A pass that does not
+// fill the SMs leaves room for the interface kernels of the other streams, which then run beside
+// it instead of after it (96 wetting boxes, ms per step: with the interface force taken in, on
+// three lanes, 1.162 with 6, 1.178 with 4 or 3; without it, beside a partitioned chain, 1.317 with
+// 4, 1.402 with 6).
+constexpr int k1_multi_per_sm(bool forced) { return forced ? 6 : 4; }
 
+// Blocks per SM that the registers are bounded for with FP32 storage; the others would spill.
 template <typename real, typename S>
 struct MultiMinBlocks {
-  static constexpr int value =
-      sizeof(real) == 4 && sizeof(S) == 4 ? (kK1MultiPerSM > 0 ? kK1MultiPerSM : 6) : 1;
+  static constexpr int value = sizeof(real) == 4 && sizeof(S) == 4 ? 4 : 1;
 };
 
-template <typename real, typename S>
+// FORCED: with the interface force of the step (forced_group), else the body force only.
+template <typename real, typename S, bool FORCED>
 __global__ void __launch_bounds__(128, MultiMinBlocks<real, S>::value) stream_collide_kernel_multi(
     const StreamArgs<real, S> *__restrict__ all, const int *__restrict__ start, int n) {
   __shared__ int s_start[kMultiMax + 1];
@@ -482,9 +480,12 @@ __global__ void __launch_bounds__(128, MultiMinBlocks<real, S>::value) stream_co
     int gx, y, z;
     A.G.at(g, gx, y, z);
     z += A.z0;
-    if constexpr (sizeof(S) == 2) {
-      if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z);
-      else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z);
+    if constexpr (FORCED) {
+      if (A.force) forced_group<real, S, true>(A, gx, y, z);
+      else forced_group<real, S, false>(A, gx, y, z);
+    } else if constexpr (sizeof(S) == 2) {
+      if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
+      else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
     } else {
       const int x0 = 2 * gx;
       real a[Q], b[Q];
@@ -502,18 +503,14 @@ constexpr int kTilesThreads = 64;
 
 template <typename real, typename S>
 __global__ void __launch_bounds__(kTilesThreads) stream_collide_tiles_kernel(const TilesArgs<real, S> A) {
-  tiles_body<real, S>(A, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  tiles_body<true>(A, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// the batched form reads its argument record as well: held to 128 registers for float arithmetic
-template <typename real>
-struct TilesMultiMinBlocks { static constexpr int value = sizeof(real) == 4 ? 8 : 1; };
-
 template <typename real, typename S>
-__global__ void __launch_bounds__(kTilesThreads, TilesMultiMinBlocks<real>::value) stream_collide_tiles_kernel_multi(
+__global__ void __launch_bounds__(kTilesThreads, sizeof(real) == 4 ? 8 : 1) stream_collide_tiles_kernel_multi(
     const TilesArgs<real, S> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
-  tiles_body<real, S>(all[m.inst], m.block * blockDim.x + threadIdx.x, m.nblocks * blockDim.x);
+  tiles_body<true>(all[m.inst], m.block * blockDim.x + threadIdx.x, m.nblocks * blockDim.x);
 }
 
 template <typename real, typename S>
@@ -940,6 +937,7 @@ void append_record(std::vector<unsigned char> &bytes, const T &rec) {
 template <typename real, typename S>
 int lattice_multi_record_t(const Ctx &c, MultiKernel k, std::vector<unsigned char> &bytes) {
   switch (k) {
+    case MK_FORCED:
     case MK_STREAM_COLLIDE: {
       const StreamArgs<real, S> a = stream_args<real, S>(c);
       append_record(bytes, a);
@@ -957,14 +955,16 @@ int lattice_multi_record_t(const Ctx &c, MultiKernel k, std::vector<unsigned cha
 template <typename real, typename S>
 cudaError_t lattice_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStream_t s) {
   switch (k) {
+    case MK_FORCED:
     case MK_STREAM_COLLIDE: {
       static int sms = 0;
       if (!sms && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess)
         sms = 0;
-      const int cap = kK1MultiPerSM * sms;
+      const int cap = k1_multi_per_sm(k == MK_FORCED) * sms;
       const int grid = cap > 0 && m.blocks > cap ? cap : m.blocks;
-      stream_collide_kernel_multi<real, S><<<grid, 128, 0, s>>>(
-          (const StreamArgs<real, S> *)m.args, m.start, m.n);
+      const auto *args = (const StreamArgs<real, S> *)m.args;
+      if (k == MK_FORCED) stream_collide_kernel_multi<real, S, true><<<grid, 128, 0, s>>>(args, m.start, m.n);
+      else stream_collide_kernel_multi<real, S, false><<<grid, 128, 0, s>>>(args, m.start, m.n);
       break;
     }
     case MK_TILES:
@@ -984,6 +984,7 @@ cudaError_t lattice_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStre
 template <typename real, typename S>
 size_t lattice_record_align_t(MultiKernel k) {
   switch (k) {
+    case MK_FORCED:
     case MK_STREAM_COLLIDE: return alignof(StreamArgs<real, S>);
     case MK_TILES: return alignof(TilesArgs<real, S>);
     case MK_SHELL: return alignof(ShellArgs<real, S>);
