@@ -27,88 +27,16 @@
 #include <string>
 #include <vector>
 
-#include "iblb_internal.cuh"
+#include "lattice_device.cuh"
 
 namespace iblb {
 namespace {
 
 // --- device helpers --------------------------------------------------------------------
-
-struct Dual {
-  double v, d;
-};
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return {a.v + b.v, a.d + b.d}; }
-__device__ __forceinline__ Dual operator-(Dual a, Dual b) { return {a.v - b.v, a.d - b.d}; }
-__device__ __forceinline__ Dual operator-(Dual a) { return {-a.v, -a.d}; }
-__device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-__device__ __forceinline__ Dual operator*(double s, Dual a) { return {s * a.v, s * a.d}; }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-  const double r = 1.0 / b.v;
-  return {a.v * r, (a.d - a.v * r * b.d) * r};
-}
-__device__ __forceinline__ Dual operator/(Dual a, double s) { return {a.v / s, a.d / s}; }
-__device__ __forceinline__ Dual operator/(double s, Dual b) {
-  const double r = 1.0 / b.v;
-  return {s * r, -s * r * r * b.d};
-}
-__device__ __forceinline__ Dual operator+(double s, Dual a) { return {a.v + s, a.d}; }
-__device__ __forceinline__ Dual operator-(Dual a, double s) { return {a.v - s, a.d}; }
-__device__ __forceinline__ Dual dlog(Dual a) { return {log(a.v), a.d / a.v}; }
-__device__ __forceinline__ double dlog(double a) { return log(a); }
-__device__ __forceinline__ Dual dabs(Dual a) { return a.v < 0 ? -a : a; }
-__device__ __forceinline__ double dabs(double a) { return fabs(a); }
-template <typename T>
-__device__ __forceinline__ T make(double v, double d);
-template <>
-__device__ __forceinline__ double make<double>(double v, double) { return v; }
-template <>
-__device__ __forceinline__ Dual make<Dual>(double v, double d) { return {v, d}; }
-
-// Forces of one face on its three corners (out[3 c + k]): the strain part, the negative
-// gradient of A0 w_S of Eq. 2 with the Skalak invariants of the face (readings R4, R5),
-// and the Lennard-Jones wall part of Eq. 19 (thirds of the centroid force, readings R6-R8).
-template <typename T>
-__device__ void face_forces(const T x[3][3], double H11, double H12, double H22, double A0,
-                            double a1, double a2, double a3, double eps, double xi, bool lj,
-                            double zb, double zt, T out[9]) {
-  T a[3], b[3];
-  for (int k = 0; k < 3; k++) {
-    a[k] = x[1][k] - x[0][k];
-    b[k] = x[2][k] - x[0][k];
-  }
-  const T g11 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2];
-  const T g12 = a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-  const T g22 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-  const T detG = g11 * g22 - g12 * g12;
-  const double detG0 = 4.0 * A0 * A0;
-  const T L = dlog(detG / detG0);  // ln(I2 + 1)
-  const double dE_dI1 = A0 * 0.5 * a3;
-  const T dE_dL = A0 * (0.5 * (a1 - a3) + 0.25 * (a1 + a2) * L);
-  for (int k = 0; k < 3; k++) {
-    const T dI1_da = 2.0 * (H11 * a[k] + H12 * b[k]);
-    const T dI1_db = 2.0 * (H12 * a[k] + H22 * b[k]);
-    const T dL_da = (2.0 * (a[k] * g22) - 2.0 * (g12 * b[k])) / detG;
-    const T dL_db = (2.0 * (b[k] * g11) - 2.0 * (g12 * a[k])) / detG;
-    const T dE_da = dE_dI1 * dI1_da + dE_dL * dL_da;
-    const T dE_db = dE_dI1 * dI1_db + dE_dL * dL_db;
-    out[3 + k] = -dE_da;
-    out[6 + k] = -dE_db;
-    out[k] = dE_da + dE_db;
-  }
-  if (lj) {
-    const T gz = (x[0][2] + x[1][2] + x[2][2]) / 3.0;
-    T fz = make<T>(0.0, 0.0);
-    for (int w = 0; w < 2; w++) {
-      const T dz = gz - (w == 0 ? zb : zt);
-      const T d = dabs(dz);
-      const T r = xi / d;
-      const T r2 = r * r;
-      const T s6 = r2 * r2 * r2;
-      fz = fz + (48.0 * eps) * ((s6 * s6 - 0.5 * s6) * dz / (d * d));
-    }
-    for (int c = 0; c < 3; c++) out[3 * c + 2] = out[3 * c + 2] + fz / 3.0;
-  }
-}
+//
+// FP64 issues at 1/64 of the FP32 rate on this GPU, two lanes per cycle and SM whatever the number
+// of active lanes: the kernels count double operations, and give each pass enough warps to use
+// every SM's unit.
 
 struct FaceArgs {
   int nf;
@@ -120,114 +48,176 @@ struct FaceArgs {
   double zb, zt;
 };
 
+__device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
+  return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2]));
+}
+__device__ __forceinline__ void cross3(const double a[3], const double b[3], double o[3]) {
+  o[0] = fma(a[1], b[2], -a[2] * b[1]);
+  o[1] = fma(a[2], b[0], -a[0] * b[2]);
+  o[2] = fma(a[0], b[1], -a[1] * b[0]);
+}
+__device__ __forceinline__ double warp_sum(double x) {
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// Sum of the n values at p by one warp (every lane gets it), in a fixed order.
+__device__ __forceinline__ double warp_total(const double *__restrict__ p, int n) {
+  double s[4] = {0, 0, 0, 0};
+  for (int k0 = 0; k0 < n; k0 += 128)
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const int k = k0 + 32 * c + (threadIdx.x & 31);
+      if (k < n) s[c] += p[k];
+    }
+  return warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+}
+
+// Metric of a face and the Skalak energy's coefficients (Eq. 2, readings R4, R5): the strain
+// forces are -dE/da = -(paa a + pab b) on corner 1, -dE/db = -(pab a + pbb b) on corner 2 and
+// their opposite on corner 0, with eI = 2 dE/dI1 and eL = 2 dE/dL / det G.
+struct Strain {
+  double G11, G12, G22, id, L;  // metric, 1/det G, ln(det G / det G0)
+  double eI, eL, paa, pab, pbb;
+};
+__device__ __forceinline__ Strain strain_of(const FaceArgs &A, const double a[3], const double b[3],
+                                            const double H[4]) {
+  Strain s;
+  s.G11 = dot3(a, a);
+  s.G12 = dot3(a, b);
+  s.G22 = dot3(b, b);
+  const double det = fma(s.G11, s.G22, -s.G12 * s.G12);
+  s.id = 1.0 / det;
+  s.L = log(det / (4.0 * H[3] * H[3]));
+  s.eI = A.alpha[2] * H[3];
+  s.eL = H[3] * fma(0.5 * (A.alpha[0] + A.alpha[1]), s.L, A.alpha[0] - A.alpha[2]) * s.id;
+  s.paa = fma(s.eI, H[0], s.eL * s.G22);
+  s.pab = fma(s.eI, H[1], -s.eL * s.G12);
+  s.pbb = fma(s.eI, H[2], s.eL * s.G11);
+  return s;
+}
+// Lennard-Jones force along z of both wall planes on a centroid at height gz (Eq. 19, readings
+// R6-R8) per 48 eps, and its derivative in gz: with s = (xi/dz)^6, (s^2 - s/2)/dz and
+// (-13 s^2 + 3.5 s)/dz^2.
+__device__ __forceinline__ void lj_pair(const FaceArgs &A, double gz, double &f, double &df) {
+  f = df = 0.0;
+  for (int w = 0; w < 2; w++) {
+    const double r = 1.0 / (gz - (w == 0 ? A.zb : A.zt));
+    const double x = A.xi * r, x2 = x * x, s6 = x2 * x2 * x2;
+    f = fma(fma(s6, s6, -0.5 * s6), r, f);
+    df = fma(s6 * fma(-13.0, s6, 3.5), r * r, df);
+  }
+}
+
 // Forward pass over faces at positions q: corner forces fc [nf][9], volume gradient share
-// (a x b)/6 per corner fn [nf][3] and the face's share of V, fV [nf].
+// (a x b)/6 per corner fn [nf][3] and per warp of 32 faces their share of V, vpart.
 __global__ void adj_face_value_kernel(FaceArgs A, const double *__restrict__ q,
                                       double *__restrict__ fc, double *__restrict__ fn,
-                                      double *__restrict__ fV) {
+                                      double *__restrict__ vpart) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= A.nf) return;
-  double x[3][3];
-  for (int c = 0; c < 3; c++)
-    for (int k = 0; k < 3; k++) x[c][k] = q[3 * A.faces[3 * j + c] + k];
-  const double *H = A.fref + 4 * j;
-  double out[9];
-  face_forces<double>(x, H[0], H[1], H[2], H[3], A.alpha[0], A.alpha[1], A.alpha[2], A.eps,
-                      A.xi, A.lj, A.zb, A.zt, out);
-  for (int k = 0; k < 9; k++) fc[9 * j + k] = out[k];
-  double a[3], b[3], r[3][3];
-  for (int k = 0; k < 3; k++) {
-    a[k] = x[1][k] - x[0][k];
-    b[k] = x[2][k] - x[0][k];
-    for (int c = 0; c < 3; c++) r[c][k] = x[c][k] - A.centre[k];
+  double V = 0.0;
+  if (j < A.nf) {
+    double x[3][3];
+    for (int c = 0; c < 3; c++)
+      for (int k = 0; k < 3; k++) x[c][k] = q[3 * A.faces[3 * j + c] + k];
+    double a[3], b[3], r0[3], n[3];
+    for (int k = 0; k < 3; k++) {
+      a[k] = x[1][k] - x[0][k];
+      b[k] = x[2][k] - x[0][k];
+      r0[k] = x[0][k] - A.centre[k];
+    }
+    const Strain s = strain_of(A, a, b, A.fref + 4 * j);
+    double fz = 0.0;
+    if (A.lj) {
+      double f, df;
+      lj_pair(A, (x[0][2] + x[1][2] + x[2][2]) * (1.0 / 3.0), f, df);
+      fz = 16.0 * A.eps * f;  // a third to each corner
+    }
+    double *o = fc + 9 * (size_t)j;
+    for (int k = 0; k < 3; k++) {
+      const double ga = fma(s.paa, a[k], s.pab * b[k]), gb = fma(s.pab, a[k], s.pbb * b[k]);
+      const double w = k == 2 ? fz : 0.0;
+      o[k] = ga + gb + w;
+      o[3 + k] = w - ga;
+      o[6 + k] = w - gb;
+    }
+    cross3(a, b, n);
+    for (int k = 0; k < 3; k++) fn[3 * (size_t)j + k] = n[k] * (1.0 / 6.0);
+    V = dot3(r0, n) * (1.0 / 6.0);  // r0 . (r1 x r2) = r0 . (a x b)
   }
-  fn[3 * j] = (a[1] * b[2] - a[2] * b[1]) / 6.0;
-  fn[3 * j + 1] = (a[2] * b[0] - a[0] * b[2]) / 6.0;
-  fn[3 * j + 2] = (a[0] * b[1] - a[1] * b[0]) / 6.0;
-  fV[j] = (r[0][0] * (r[1][1] * r[2][2] - r[1][2] * r[2][1]) +
-           r[0][1] * (r[1][2] * r[2][0] - r[1][0] * r[2][2]) +
-           r[0][2] * (r[1][0] * r[2][1] - r[1][1] * r[2][0])) / 6.0;
+  V = warp_sum(V);
+  if ((threadIdx.x & 31) == 0 && j < A.nf) vpart[j >> 5] = V;
 }
 
 // Derivative pass over faces along the tangent t (the adjoint force lambda_phi):
-// d(corner forces) fj [nf][9], d((a x b)/6) dn [nf][3], ((a x b)/6) . (t0 + t1 + t2) fdot [nf]
-// (a share of grad V . t), and t . dphi/dtheta_k per face, fpar [nf][4].
+// d(corner forces) fj [nf][9], d((a x b)/6) dn [nf][3], and per warp of 32 faces the sums of
+// ((a x b)/6) . (t0 + t1 + t2), a share of grad V . t, and of t . dphi/dtheta_k: part [5][warps].
+// The strain forces' derivative follows from the metric's, dG = (2 a.ta, a.tb + b.ta, 2 b.tb) and
+// d det = dG11 G22 + G11 dG22 - 2 G12 dG12; the forces are linear in each parameter and their
+// component along t is -(eI (H : dG)/2 + eL d det / 2), so the four parameter derivatives need no
+// further pass.
 __global__ void adj_face_tangent_kernel(FaceArgs A, const double *__restrict__ q,
                                         const double *__restrict__ t, double *__restrict__ fj,
-                                        double *__restrict__ dn, double *__restrict__ fdot,
-                                        double *__restrict__ fpar) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= A.nf) return;
-  Dual x[3][3];
-  double xv[3][3], tv[3][3];
-  for (int c = 0; c < 3; c++)
-    for (int k = 0; k < 3; k++) {
-      const int v = A.faces[3 * j + c];
-      xv[c][k] = q[3 * v + k];
-      tv[c][k] = t[3 * v + k];
-      x[c][k] = {xv[c][k], tv[c][k]};
-    }
-  const double *H = A.fref + 4 * j;
-  Dual out[9];
-  face_forces<Dual>(x, H[0], H[1], H[2], H[3], A.alpha[0], A.alpha[1], A.alpha[2], A.eps, A.xi,
-                    A.lj, A.zb, A.zt, out);
-  for (int k = 0; k < 9; k++) fj[9 * j + k] = out[k].d;
-  Dual a[3], b[3];
-  for (int k = 0; k < 3; k++) {
-    a[k] = x[1][k] - x[0][k];
-    b[k] = x[2][k] - x[0][k];
-  }
-  const Dual n0 = (a[1] * b[2] - a[2] * b[1]) / 6.0;
-  const Dual n1 = (a[2] * b[0] - a[0] * b[2]) / 6.0;
-  const Dual n2 = (a[0] * b[1] - a[1] * b[0]) / 6.0;
-  dn[3 * j] = n0.d;
-  dn[3 * j + 1] = n1.d;
-  dn[3 * j + 2] = n2.d;
-  double ts[3];
-  for (int k = 0; k < 3; k++) ts[k] = tv[0][k] + tv[1][k] + tv[2][k];
-  fdot[j] = n0.v * ts[0] + n1.v * ts[1] + n2.v * ts[2];
-  // the forces are linear in each parameter: dphi/dtheta_k is the force with theta = e_k
-  for (int p = 0; p < 4; p++) {
-    double o[9];
-    const double e1 = p == 0, e2 = p == 1, e3 = p == 2, ee = p == 3;
-    face_forces<double>(xv, H[0], H[1], H[2], H[3], e1, e2, e3, ee, A.xi, p == 3 && A.lj, A.zb,
-                        A.zt, o);
-    double s = 0.0;
+                                        double *__restrict__ dn, double *__restrict__ part) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, warps = (A.nf + 31) / 32;
+  double sum[5] = {0, 0, 0, 0, 0};
+  if (j < A.nf) {
+    double x[3][3], u[3][3];
     for (int c = 0; c < 3; c++)
-      for (int k = 0; k < 3; k++) s += o[3 * c + k] * tv[c][k];
-    fpar[4 * j + p] = s;
-  }
-}
-
-// Fixed-order sums over faces (one block of 1024 threads): out[0] = sum a, out[1..m] = sums of
-// b's columns; with grad, the b sums (the parameter derivatives of the step) are also added to
-// grad[0..m-1]. Strided per-thread sums, then warp shuffles, then one warp over the warps.
-constexpr int kSumThreads = 1024;
-__global__ void __launch_bounds__(kSumThreads) adj_face_sums_kernel(
-    int nf, const double *__restrict__ a, const double *__restrict__ b, int m,
-    double *__restrict__ out, double *__restrict__ grad) {
-  __shared__ double sh[kSumThreads / 32][5];
-  const int t = threadIdx.x, lane = t & 31, wq = t >> 5;
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int j = t; j < nf; j += kSumThreads) {
-    acc[0] += a[j];
-    for (int k = 0; k < m; k++) acc[1 + k] += b[(size_t)m * j + k];
-  }
-  for (int k = 0; k <= m; k++) {
-    double v = acc[k];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[wq][k] = v;
-  }
-  __syncthreads();
-  if (wq == 0) {
-    for (int k = 0; k <= m; k++) {
-      double v = sh[lane][k];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) {
-        out[k] = v;
-        if (grad && k > 0) grad[k - 1] += v;
+      for (int k = 0; k < 3; k++) {
+        const int v = A.faces[3 * j + c];
+        x[c][k] = q[3 * v + k];
+        u[c][k] = t[3 * v + k];
       }
+    double a[3], b[3], ta[3], tb[3];
+    for (int k = 0; k < 3; k++) {
+      a[k] = x[1][k] - x[0][k];
+      b[k] = x[2][k] - x[0][k];
+      ta[k] = u[1][k] - u[0][k];
+      tb[k] = u[2][k] - u[0][k];
     }
+    const double *H = A.fref + 4 * j;
+    const double A0 = H[3];
+    const Strain s = strain_of(A, a, b, H);
+    const double hG11 = dot3(a, ta), dG12 = dot3(a, tb) + dot3(b, ta), hG22 = dot3(b, tb);
+    const double hdet = fma(hG11, s.G22, fma(s.G11, hG22, -s.G12 * dG12));  // d det / 2
+    const double dL = 2.0 * hdet * s.id;
+    const double deL = s.id * dL * A0 * 0.5 * (A.alpha[0] + A.alpha[1]) - s.eL * dL;
+    const double dpaa = fma(deL, s.G22, 2.0 * s.eL * hG22);
+    const double dpab = -fma(deL, s.G12, s.eL * dG12);
+    const double dpbb = fma(deL, s.G11, 2.0 * s.eL * hG11);
+    double f = 0.0, df = 0.0, tz = 0.0, dfz = 0.0;
+    if (A.lj) {
+      tz = (u[0][2] + u[1][2] + u[2][2]) * (1.0 / 3.0);
+      lj_pair(A, (x[0][2] + x[1][2] + x[2][2]) * (1.0 / 3.0), f, df);
+      dfz = 16.0 * A.eps * df * tz;
+    }
+    double *o = fj + 9 * (size_t)j;
+    for (int k = 0; k < 3; k++) {
+      const double ga = fma(dpaa, a[k], fma(s.paa, ta[k], fma(dpab, b[k], s.pab * tb[k])));
+      const double gb = fma(dpab, a[k], fma(s.pab, ta[k], fma(dpbb, b[k], s.pbb * tb[k])));
+      const double w = k == 2 ? dfz : 0.0;
+      o[k] = ga + gb + w;
+      o[3 + k] = w - ga;
+      o[6 + k] = w - gb;
+    }
+    double n[3], c1[3], c2[3], ts[3];
+    cross3(a, b, n);
+    cross3(ta, b, c1);
+    cross3(a, tb, c2);
+    for (int k = 0; k < 3; k++) {
+      dn[3 * (size_t)j + k] = (c1[k] + c2[k]) * (1.0 / 6.0);
+      ts[k] = u[0][k] + u[1][k] + u[2][k];
+    }
+    sum[0] = dot3(n, ts) * (1.0 / 6.0);
+    const double SI = fma(H[0], hG11, fma(H[1], dG12, H[2] * hG22));
+    sum[1] = -A0 * fma(0.25, s.L, 0.5) * dL;   // alpha1
+    sum[2] = -A0 * 0.25 * s.L * dL;            // alpha2
+    sum[3] = A0 * fma(0.5, dL, -SI);           // alpha3
+    sum[4] = 48.0 * f * tz;                    // eps
+  }
+  for (int k = 0; k < 5; k++) {
+    const double v = warp_sum(sum[k]);
+    if ((threadIdx.x & 31) == 0 && j < A.nf) part[(size_t)k * warps + (j >> 5)] = v;
   }
 }
 
@@ -236,35 +226,108 @@ struct VolArgs {
   double kV, V0;
 };
 
-// phi_v = sum over the faces at v of the corner forces - kV (V - V0)/V0 dV/dq_v (forward), or
-// lam_q_v += the tangent of that along lambda_phi (derivative pass, `tangent`):
-//   d(corner forces) - kV/V0 [(V - V0) d(dV/dq_v) + (grad V . t) dV/dq_v].
-__global__ void adj_vertex_kernel(int nv, const int *__restrict__ vf_start,
-                                  const int *__restrict__ vf_list, const double *__restrict__ corner,
-                                  const double *__restrict__ fn, const double *__restrict__ dn,
-                                  const double *__restrict__ sums,
-                                  const double *__restrict__ sums_t, VolArgs va, int tangent,
-                                  double *__restrict__ out) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= nv) return;
-  double f[3] = {0, 0, 0}, g[3] = {0, 0, 0}, dg[3] = {0, 0, 0};
-  for (int e = vf_start[v]; e < vf_start[v + 1]; e++) {
-    const int j = vf_list[e] / 3, c = vf_list[e] % 3;
-    for (int k = 0; k < 3; k++) {
-      f[k] += corner[9 * j + 3 * c + k];
-      g[k] += fn[3 * j + k];
-      if (tangent) dg[k] += dn[3 * j + k];
+// Peskin's 4-point function (Eq. 15, reading R2) on the four nodes floor(p) - 1 .. floor(p) + 2 and
+// its derivative with respect to p: with r = p - floor(p) and s = sqrt(1 + 4r - 4r^2) the weights
+// are (3-2r-s)/8, (3-2r+s)/8, (1+2r+s)/8, (1+2r-s)/8, and s' = (2 - 4r)/s.
+struct Stencil {
+  int base[3];
+  int pad;
+  double w[3][4], dw[3][4];
+};
+__device__ __forceinline__ void stencil_axis(double p, int &base, double w[4], double dw[4]) {
+  const double fl = floor(p);
+  base = (int)fl - 1;
+  const double r = p - fl;
+  const double s = sqrt(fma(4.0 * r, 1.0 - r, 1.0));
+  const double ds = (2.0 - 4.0 * r) / s;
+  const double lo = fma(-2.0, r, 3.0), hi = fma(2.0, r, 1.0);
+  w[0] = 0.125 * (lo - s);
+  w[1] = 0.125 * (lo + s);
+  w[2] = 0.125 * (hi + s);
+  w[3] = 0.125 * (hi - s);
+  dw[0] = 0.125 * (-2.0 - ds);
+  dw[1] = 0.125 * (-2.0 + ds);
+  dw[2] = 0.125 * (2.0 + ds);
+  dw[3] = 0.125 * (2.0 - ds);
+}
+
+constexpr int kFaceThreads = 32, kVertexThreads = 64;
+
+// Forward pass over vertices: phi_v, the sum over the faces at v of the corner forces
+// - kV (V - V0)/V0 dV/dq_v, and the stencil of v. Each block sums the volume's partials itself.
+// A thread per (vertex, coordinate).
+__global__ void __launch_bounds__(kVertexThreads) adj_vertex_value_kernel(
+    int nv, int nwarps, const int *__restrict__ vf_start, const int *__restrict__ vf_list,
+    const double *__restrict__ corner, const double *__restrict__ fn,
+    const double *__restrict__ vpart, VolArgs va, const double *__restrict__ q,
+    double *__restrict__ phi, Stencil *__restrict__ st) {
+  __shared__ double s_coef;
+  if (threadIdx.x < 32) {
+    const double V = warp_total(vpart, nwarps);
+    if (threadIdx.x == 0) s_coef = va.on ? va.kV * (V - va.V0) / va.V0 : 0.0;
+  }
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double f = 0, g = 0;
+  if (i < 3 * nv) {
+    const int v = i / 3, k = i - 3 * v;
+    for (int e = vf_start[v]; e < vf_start[v + 1]; e++) {
+      const int fcr = vf_list[e];  // face * 3 + corner
+      f += corner[3 * (size_t)fcr + k];
+      g += fn[3 * (size_t)(fcr / 3) + k];
+    }
+    double w[4], dw[4];
+    int base;
+    stencil_axis(q[i], base, w, dw);
+    Stencil &s = st[v];
+    s.base[k] = base;
+    for (int d = 0; d < 4; d++) {
+      s.w[k][d] = w[d];
+      s.dw[k][d] = dw[d];
     }
   }
-  if (!tangent) {
-    const double coef = va.on ? va.kV * (sums[0] - va.V0) / va.V0 : 0.0;
-    for (int k = 0; k < 3; k++) out[3 * v + k] = f[k] - coef * g[k];
+  __syncthreads();
+  if (i < 3 * nv) phi[i] = fma(-s_coef, g, f);
+}
+
+// Derivative pass over vertices: lam_q_v += the tangent of phi_v along lambda_phi,
+//   d(corner forces) - kV/V0 [(V - V0) d(dV/dq_v) + (grad V . t) dV/dq_v];
+// block 0 also adds the step's parameter derivatives to grad. A thread per (vertex, coordinate).
+__global__ void __launch_bounds__(kVertexThreads) adj_vertex_tangent_kernel(
+    int nv, int nwarps, const int *__restrict__ vf_start, const int *__restrict__ vf_list,
+    const double *__restrict__ corner, const double *__restrict__ fn, const double *__restrict__ dn,
+    const double *__restrict__ vpart, const double *__restrict__ part, VolArgs va,
+    double *__restrict__ lam_q, double *__restrict__ grad) {
+  __shared__ double s_coef, s_coef2;
+  if (threadIdx.x < 32) {
+    const double V = warp_total(vpart, nwarps);
+    if (threadIdx.x == 0) s_coef = va.on ? va.kV * (V - va.V0) / va.V0 : 0.0;
+    if (blockIdx.x == 0)
+      for (int k = 0; k < 2; k++) {
+        const double p = warp_total(part + (size_t)(1 + k) * nwarps, nwarps);
+        if (threadIdx.x == 0) grad[k] += p;
+      }
   } else {
-    // sums[0] = V (value pass), sums_t[0] = grad V . t (derivative pass)
-    const double coef = va.on ? va.kV * (sums[0] - va.V0) / va.V0 : 0.0;
-    const double coef2 = va.on ? va.kV / va.V0 * sums_t[0] : 0.0;
-    for (int k = 0; k < 3; k++) out[3 * v + k] += f[k] - coef * dg[k] - coef2 * g[k];
+    const double d = warp_total(part, nwarps);
+    if (threadIdx.x == 32) s_coef2 = va.on ? va.kV / va.V0 * d : 0.0;
+    if (blockIdx.x == 0)
+      for (int k = 2; k < 4; k++) {
+        const double p = warp_total(part + (size_t)(1 + k) * nwarps, nwarps);
+        if (threadIdx.x == 32) grad[k] += p;
+      }
   }
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double f = 0, g = 0, dg = 0;
+  if (i < 3 * nv) {
+    const int v = i / 3, k = i - 3 * v;
+    for (int e = vf_start[v]; e < vf_start[v + 1]; e++) {
+      const int fcr = vf_list[e];
+      f += corner[3 * (size_t)fcr + k];
+      g += fn[3 * (size_t)(fcr / 3) + k];
+      dg += dn[3 * (size_t)(fcr / 3) + k];
+    }
+  }
+  __syncthreads();
+  if (i < 3 * nv) lam_q[i] += fma(-s_coef2, g, fma(-s_coef, dg, f));
 }
 
 // --- immersed-boundary transposes ------------------------------------------------------
@@ -272,56 +335,13 @@ __global__ void adj_vertex_kernel(int nv, const int *__restrict__ vf_start,
 struct LatArgs {
   int nx, ny, nz, walls;
   size_t ncell;
+  FastDiv dx, dy;             // by nx, by ny
   double rho0, omega, gamma;  // 1/tau, 1 - 1/(2 tau)
   double g[3];
+  int has_g;                  // the body force is not zero
   double ub[3], ut[3];        // wall velocities
   double wb[19], wt[19];      // moving-wall terms of the bounce-back (deviation units)
 };
-
-// Peskin's 4-point function (Eq. 15, reading R2) and its derivative, sharing the root.
-__device__ __forceinline__ void peskin_wdw(double r, double &w, double &dwdr) {
-  const double a = fabs(r), sg = r < 0 ? -1.0 : 1.0;
-  if (a <= 1.0) {
-    const double s = sqrt(1.0 + 4.0 * a - 4.0 * a * a);
-    w = 0.125 * (3.0 - 2.0 * a + s);
-    dwdr = sg * 0.125 * (-2.0 + (2.0 - 4.0 * a) / s);
-  } else if (a <= 2.0) {
-    const double s = sqrt(-7.0 + 12.0 * a - 4.0 * a * a);
-    w = 0.125 * (5.0 - 2.0 * a - s);
-    dwdr = sg * 0.125 * (-2.0 - (6.0 - 4.0 * a) / s);
-  } else {
-    w = 0.0;
-    dwdr = 0.0;
-  }
-}
-
-// Stencil of a vertex position: base node floor(p) - 1 per axis, the 1D weights w and their
-// derivatives dw with respect to p (= -d peskin(x - p)/dx). Computed once per vertex and
-// reverse step, then read by the three per-vertex passes (double square roots and divisions
-// are costly here: FP64 runs at 1/64 of the FP32 rate).
-struct Stencil {
-  int base[3];
-  int pad;
-  double w[3][4], dw[3][4];
-};
-
-// one thread per (vertex, axis)
-__global__ void adj_stencil_kernel(int nv, const double *__restrict__ q, Stencil *__restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 3 * nv) return;
-  const int v = t / 3, k = t - 3 * v;
-  const double p = q[t];
-  const int base = (int)floor(p) - 1;
-  Stencil &s = out[v];
-  s.base[k] = base;
-  if (k == 0) s.pad = 0;
-  for (int d = 0; d < 4; d++) {
-    double w, dwdr;
-    peskin_wdw((double)(base + d) - p, w, dwdr);
-    s.w[k][d] = w;
-    s.dw[k][d] = -dwdr;
-  }
-}
 
 // z kind of a node: 0 fluid, 1 bottom wall, 2 top wall, -1 beyond the array (reading R9).
 __device__ __forceinline__ int zkind(int z, const LatArgs &L) {
@@ -332,55 +352,72 @@ __device__ __forceinline__ int zkind(int z, const LatArgs &L) {
   return 0;
 }
 __device__ __forceinline__ int wrapi(int a, int n) {
+  if ((unsigned)a < (unsigned)n) return a;
   const int r = a % n;
   return r < 0 ? r + n : r;
 }
-__device__ __forceinline__ size_t node_of(int x, int y, int z, const LatArgs &L) {
-  return ((size_t)wrapi(z, L.nz) * L.ny + wrapi(y, L.ny)) * L.nx + wrapi(x, L.nx);
+
+// A node and its neighbours' offsets along each axis, at 1 - c for a source x - c.
+struct Node {
+  size_t n, zo[3], yo[3];
+  int xo[3], z;
+  bool below, above;  // a link up starts at the bottom wall, one down at the top wall
+};
+__device__ __forceinline__ Node node_at(size_t n, const LatArgs &L) {
+  Node d;
+  d.n = n;
+  // (node numbers beyond 2^31 take the plain division)
+  const size_t row = n < ((size_t)1 << 31) ? (size_t)L.dx.div((int)n) : n / L.nx;
+  const int x = (int)(n - row * L.nx);
+  const int z = row < ((size_t)1 << 31) ? L.dy.div((int)row) : (int)(row / L.ny);
+  const int y = (int)(row - (size_t)z * L.ny);
+  d.z = z;
+  d.xo[0] = x == 0 ? L.nx - 1 : x - 1;
+  d.xo[1] = x;
+  d.xo[2] = x == L.nx - 1 ? 0 : x + 1;
+  d.yo[0] = (size_t)(y == 0 ? L.ny - 1 : y - 1) * L.nx;
+  d.yo[1] = (size_t)y * L.nx;
+  d.yo[2] = (size_t)(y == L.ny - 1 ? 0 : y + 1) * L.nx;
+  const size_t plane = (size_t)L.nx * L.ny;
+  d.zo[0] = (size_t)(z == 0 ? L.nz - 1 : z - 1) * plane;
+  d.zo[1] = (size_t)z * plane;
+  d.zo[2] = (size_t)(z == L.nz - 1 ? 0 : z + 1) * plane;
+  d.below = L.walls && z == 1;
+  d.above = L.walls && z == L.nz - 2;
+  return d;
+}
+// Source of the pulled population i at node d: element index into P (i-th array); a link from a
+// wall bounces back: population opp(i) at the same node, plus the wall term.
+__device__ __forceinline__ bool bounced(const Node &d, int i) {
+  return (cz(i) > 0 && d.below) || (cz(i) < 0 && d.above);
+}
+__device__ __forceinline__ size_t pull_source(const Node &d, int i, const LatArgs &L) {
+  if (bounced(d, i)) return (size_t)opp(i) * L.ncell + d.n;
+  return (size_t)i * L.ncell + d.zo[1 - cz(i)] + d.yo[1 - cy(i)] + d.xo[1 - cx(i)];
 }
 
-// Source of the pulled population i at fluid node (x, y, z): element index into P (i-th
-// array) and whether the link bounces back from a wall (then: population opp(i) at the same
-// node, plus the wall term).
-__device__ __forceinline__ size_t pull_source(int x, int y, int z, int i, const LatArgs &L,
-                                              bool &bounced) {
-  const int sz = z - cz(i);
-  bounced = L.walls && (sz == 0 || sz == L.nz - 1);
-  if (bounced) return (size_t)opp(i) * L.ncell + node_of(x, y, z, L);
-  return (size_t)i * L.ncell + node_of(x - cx(i), y - cy(i), sz, L);
-}
-
-// Post-streaming populations (deviations) at fluid node (x, y, z) from the post-collision
-// populations P as stored, in the arithmetic type A of the forward state: double for FP64
-// contexts; float for FP32 contexts, whose forward step ran in float (the reverse pass
-// linearises the double-precision step about that trajectory; its rho and u are formed in
-// float, like the forward step's, and the adjoint arithmetic itself stays double).
+// Post-streaming populations (deviations) at a fluid node from the post-collision populations P
+// as stored, in the arithmetic type A of the forward state: double for FP64 contexts; float for
+// FP32 contexts, whose forward step ran in float (the reverse pass linearises the double-precision
+// step about that trajectory; its rho and u are formed in float, like the forward step's, and the
+// adjoint arithmetic itself stays double).
 template <typename A, typename T>
-__device__ __forceinline__ void pull_dev(const T *__restrict__ P, int x, int y, int z,
-                                         const LatArgs &L, A f[Q]) {
+__device__ __forceinline__ void pull_dev(const T *__restrict__ P, const Node &d, const LatArgs &L,
+                                         A f[Q]) {
 #pragma unroll
   for (int i = 0; i < Q; i++) {
-    bool bb;
-    const size_t s = pull_source(x, y, z, i, L, bb);
-    f[i] = (A)P[s] + (bb ? (A)(cz(i) > 0 ? L.wb[i] : L.wt[i]) : A(0));
+    f[i] = (A)P[pull_source(d, i, L)];
+    if (bounced(d, i)) f[i] += (A)(cz(i) > 0 ? L.wb[i] : L.wt[i]);
   }
 }
 
-// Velocity (Guo shift with the total force g + F) of deviations f; returns rho. Opposite
-// directions are summed in pairs.
+// Velocity (Guo shift with the total force Ft) of deviations f; returns rho.
 template <typename A>
 __device__ __forceinline__ A velocity(const A f[Q], const A Ft[3], A rho0, A u[3]) {
-  A drho = f[0], j[3] = {0, 0, 0};
-#pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    drho += f[i] + f[i + 1];
-    const A d = f[i] - f[i + 1];
-    if (cx(i)) j[0] += cx(i) > 0 ? d : -d;
-    if (cy(i)) j[1] += cy(i) > 0 ? d : -d;
-    if (cz(i)) j[2] += cz(i) > 0 ? d : -d;
-  }
+  A drho, j[3];
+  node_moments(f, drho, j);
   const A rho = rho0 + drho;
-  const A ir = A(1) / rho;
+  const A ir = reciprocal(rho);
   for (int k = 0; k < 3; k++) u[k] = (j[k] + A(0.5) * Ft[k]) * ir;
   return rho;
 }
@@ -390,46 +427,80 @@ struct alignas(32) NodeU {
   double x, y, z, rho;
 };
 
-__device__ __forceinline__ double warp_sum(double x) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+// The per-vertex passes run sixteen lanes per vertex: lane l holds the stencil row (dy, dz) =
+// (l & 3, l >> 2), its four nodes along x one after another. Two rows' factors are shared by all
+// four nodes, so a vertex costs a third of the FP64 instructions of a lane per node pair.
+struct Row {
+  int v, z, kind;
+  size_t base;   // of node (0, y, z)
+  double wy, wz, dwy, dwz;
+};
+__device__ __forceinline__ Row row_of(const Stencil &s, int v, const LatArgs &L) {
+  Row r;
+  const int l = threadIdx.x & 15, dy = l & 3, dz = l >> 2;
+  r.v = v;
+  r.z = s.base[2] + dz;
+  r.kind = zkind(r.z, L);
+  r.base = ((size_t)wrapi(r.z, L.nz) * L.ny + wrapi(s.base[1] + dy, L.ny)) * L.nx;
+  r.wy = s.w[1][dy];
+  r.wz = s.w[2][dz];
+  r.dwy = s.dw[1][dy];
+  r.dwz = s.dw[2][dz];
+  return r;
+}
+// Sum over the sixteen lanes of a vertex.
+__device__ __forceinline__ double half_sum(double x) {
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
 }
+// Sums over the sixteen lanes of a vertex of 2 N values: the first step exchanges halves of the
+// values between two halves of the lanes, so each lane goes on with N of them. Lanes with
+// (l & 8) == 0 return the sums of v[0 .. N-1], the others of v[N .. 2N-1].
+template <int N>
+__device__ __forceinline__ void half_sums(const double v[2 * N], double out[N]) {
+  const bool up = threadIdx.x & 8;
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    const double other = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[N + k], 8);
+    out[k] = (up ? v[N + k] : v[k]) + other;
+  }
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < N; k++) out[k] += __shfl_xor_sync(0xffffffffu, out[k], o);
+}
 
-// The per-vertex passes run one warp per vertex: lane l handles the stencil nodes
-// (dx, dy, dz) = (l & 3, (l >> 2) & 3, (l >> 4) + 2 h) for h = 0, 1.
-
-// Spreading at q_n onto the fluid nodes (Eq. 13): F += W phi. F is zero on entry at every
-// stencil node: the spreading transpose of the previous reverse step cleared it.
+// Spreading at q_n onto the fluid nodes (Eq. 13): F += W phi, and the nodes' marks are set. F and
+// the marks are zero on entry: the spreading transpose that last used them cleared them.
 __global__ void adj_spread_kernel(int nv, const Stencil *__restrict__ st,
-                                  const double *__restrict__ phi, LatArgs L,
-                                  double *__restrict__ F) {
-  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+                                  const double *__restrict__ phi, LatArgs L, double *__restrict__ F,
+                                  unsigned char *__restrict__ mark) {
+  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
   if (v >= nv) return;
   const Stencil &s = st[v];
-  const double ph[3] = {phi[3 * v], phi[3 * v + 1], phi[3 * v + 2]};
-  const int dx = lane & 3, dy = (lane >> 2) & 3;
-  for (int h = 0; h < 2; h++) {
-    const int dz = (lane >> 4) + 2 * h;
-    const int z = s.base[2] + dz;
-    if (zkind(z, L) != 0) continue;  // wall layer: force dropped; beyond: skipped
-    const double w = s.w[0][dx] * s.w[1][dy] * s.w[2][dz];
-    const size_t n = node_of(s.base[0] + dx, s.base[1] + dy, z, L);
+  const Row r = row_of(s, v, L);
+  if (r.kind != 0) return;  // wall layer: force dropped; beyond: skipped
+  const double wyz = r.wy * r.wz;
+  const double ph[3] = {wyz * phi[3 * v], wyz * phi[3 * v + 1], wyz * phi[3 * v + 2]};
+  for (int dx = 0; dx < 4; dx++) {
+    const size_t n = r.base + wrapi(s.base[0] + dx, L.nx);
+    const double w = s.w[0][dx];
+    mark[n] = 1;
     for (int k = 0; k < 3; k++) atomicAdd(&F[3 * n + k], w * ph[k]);
   }
 }
 
-// Velocity and density after streaming at every fluid node, U = (u, rho), from the
-// post-collision populations P_{n+1} and the step's total force g + F.
+// Velocity and density after streaming at the marked nodes, U = (u, rho), from the post-collision
+// populations P_{n+1} and the step's total force g + F.
 template <typename T>
 __global__ void adj_moments_kernel(const T *__restrict__ P, const double *__restrict__ F,
-                                   LatArgs L, NodeU *__restrict__ U) {
+                                   const unsigned char *__restrict__ mark, LatArgs L,
+                                   NodeU *__restrict__ U) {
   const size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (n >= L.ncell) return;
-  const int x = (int)(n % L.nx), y = (int)((n / L.nx) % L.ny), z = (int)(n / ((size_t)L.nx * L.ny));
-  if (zkind(z, L) != 0) return;
+  if (n >= L.ncell || !mark[n]) return;
+  const Node d = node_at(n, L);
   using A = T;  // the forward state's arithmetic type
   A f[Q], u[3];
-  pull_dev<A>(P, x, y, z, L, f);
+  pull_dev<A>(P, d, L, f);
   const A Ft[3] = {(A)(L.g[0] + F[3 * n]), (A)(L.g[1] + F[3 * n + 1]), (A)(L.g[2] + F[3 * n + 2])};
   const A rho = velocity<A>(f, Ft, (A)L.rho0, u);
   U[n] = NodeU{(double)u[0], (double)u[1], (double)u[2], (double)rho};
@@ -441,240 +512,268 @@ __global__ void adj_interp_t_kernel(int nv, const Stencil *__restrict__ st,
                                     const double *__restrict__ lam, const NodeU *__restrict__ U,
                                     LatArgs L, double *__restrict__ lam_qn,
                                     double *__restrict__ lam_u) {
-  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (v >= nv) return;
-  const Stencil &s = st[v];
-  const double l[3] = {lam[3 * v], lam[3 * v + 1], lam[3 * v + 2]};
-  const int dx = lane & 3, dy = (lane >> 2) & 3;
-  double acc[3] = {0, 0, 0};
-  for (int h = 0; h < 2; h++) {
-    const int dz = (lane >> 4) + 2 * h;
-    const int z = s.base[2] + dz;
-    const int kind = zkind(z, L);
-    if (kind < 0) continue;
-    const double wx = s.w[0][dx], wy = s.w[1][dy], wz = s.w[2][dz];
-    double u[3];
-    if (kind == 1) {
-      for (int k = 0; k < 3; k++) u[k] = L.ub[k];
-    } else if (kind == 2) {
-      for (int k = 0; k < 3; k++) u[k] = L.ut[k];
-    } else {
-      const size_t n = node_of(s.base[0] + dx, s.base[1] + dy, z, L);
-      const NodeU un = U[n];
-      u[0] = un.x;
-      u[1] = un.y;
-      u[2] = un.z;
-      const double w = wx * wy * wz;
-      for (int k = 0; k < 3; k++) atomicAdd(&lam_u[3 * n + k], w * l[k]);
+  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  double c[3] = {0, 0, 0}, l[3] = {0, 0, 0};
+  if (v < nv) {
+    const Stencil &s = st[v];
+    const Row r = row_of(s, v, L);
+    for (int k = 0; k < 3; k++) l[k] = lam[3 * v + k];
+    if (r.kind >= 0) {
+      const double wyz = r.wy * r.wz;
+      double p = 0.0, dp = 0.0;  // sum over x of (u . lam) wx, (u . lam) dwx
+      if (r.kind > 0) {
+        const double *uw = r.kind == 1 ? L.ub : L.ut;
+        const double ul = dot3(uw, l);
+        for (int dx = 0; dx < 4; dx++) {
+          p = fma(ul, s.w[0][dx], p);
+          dp = fma(ul, s.dw[0][dx], dp);
+        }
+      } else {
+        const double lw[3] = {wyz * l[0], wyz * l[1], wyz * l[2]};
+        for (int dx = 0; dx < 4; dx++) {
+          const size_t n = r.base + wrapi(s.base[0] + dx, L.nx);
+          const NodeU un = U[n];
+          const double u[3] = {un.x, un.y, un.z};
+          const double ul = dot3(u, l), w = s.w[0][dx];
+          p = fma(ul, w, p);
+          dp = fma(ul, s.dw[0][dx], dp);
+          for (int k = 0; k < 3; k++) atomicAdd(&lam_u[3 * n + k], w * lw[k]);
+        }
+      }
+      c[0] = dp * wyz;
+      c[1] = p * (r.dwy * r.wz);
+      c[2] = p * (r.wy * r.dwz);
     }
-    const double ul = u[0] * l[0] + u[1] * l[1] + u[2] * l[2];
-    acc[0] += ul * s.dw[0][dx] * wy * wz;
-    acc[1] += ul * wx * s.dw[1][dy] * wz;
-    acc[2] += ul * wx * wy * s.dw[2][dz];
   }
-  for (int k = 0; k < 3; k++) acc[k] = warp_sum(acc[k]);
-  if (lane == 0)
-    for (int k = 0; k < 3; k++) lam_qn[3 * v + k] = l[k] + acc[k];
+  for (int k = 0; k < 3; k++) c[k] = half_sum(c[k]);
+  const int k = threadIdx.x & 15;
+  if (v < nv && k < 3) lam_qn[3 * v + k] = k == 0 ? l[0] + c[0] : k == 1 ? l[1] + c[1] : l[2] + c[2];
 }
 
-// Velocity moments^T at the fluid nodes with lam_u != 0: the adjoint of each pulled
-// population, (c_i - u) . lam_u / rho, added to its source in lam_P (its force part,
-// lam_u / (2 rho), is added by the collision transpose, which also clears lam_u).
+// Velocity moments^T at the marked nodes with lam_u != 0: the adjoint of each pulled population,
+// (c_i - u) . lam_u / rho, added to its source in lam_P (its force part, lam_u / (2 rho), is added
+// by the collision transpose, which also clears lam_u).
 __global__ void adj_velocity_t_kernel(const double *__restrict__ lam_u,
+                                      const unsigned char *__restrict__ mark,
                                       const NodeU *__restrict__ U, LatArgs L,
                                       double *__restrict__ lam_P) {
   const size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (n >= L.ncell) return;
-  const int x = (int)(n % L.nx), y = (int)((n / L.nx) % L.ny), z = (int)(n / ((size_t)L.nx * L.ny));
-  if (zkind(z, L) != 0) return;
+  if (n >= L.ncell || !mark[n]) return;
   const double lu[3] = {lam_u[3 * n], lam_u[3 * n + 1], lam_u[3 * n + 2]};
   if (lu[0] == 0.0 && lu[1] == 0.0 && lu[2] == 0.0) return;
+  const Node d = node_at(n, L);
   const NodeU un = U[n];
-  const double ir = 1.0 / un.rho;
-  const double ulu = (un.x * lu[0] + un.y * lu[1] + un.z * lu[2]) * ir;
+  const double ir = reciprocal(un.rho);
   const double l[3] = {lu[0] * ir, lu[1] * ir, lu[2] * ir};
+  const double u[3] = {un.x, un.y, un.z};
+  const double m = -dot3(u, l);
 #pragma unroll
   for (int i = 0; i < Q; i++) {
-    double a = -ulu;
+    double a = m;
     if (cx(i)) a += cx(i) > 0 ? l[0] : -l[0];
     if (cy(i)) a += cy(i) > 0 ? l[1] : -l[1];
     if (cz(i)) a += cz(i) > 0 ? l[2] : -l[2];
-    bool bb;
-    lam_P[pull_source(x, y, z, i, L, bb)] += a;  // each (source, direction) has one puller
+    lam_P[pull_source(d, i, L)] += a;  // each (source, direction) has one puller
   }
 }
 
 // Collision^T and streaming^T at every fluid node. mu = lam_P1 at the node is the adjoint of
 // the post-collision populations out_i = f_i - omega (f_i - feq_i(rho, u)) + S_i(u, F) of the
 // pulled pre-collision f (BGK with Guo forcing). With the moments of mu,
-//   m0 = sum w_i mu_i, m1 = sum w_i mu_i c_i, M2 = sum w_i mu_i c_i c_i^T,
+//   m0 = sum w_i mu_i, m1 = sum w_i mu_i c_i, M2 = sum w_i mu_i c_i c_i^T, N = 9 M2 - 3 m0 I,
 // the vector-Jacobian product is
-//   lam_f_j = (1 - omega) mu_j + A + B . (c_j - u) / rho,
-//   A = omega (m0 + 3 u.m1 + 4.5 u.M2 u - 1.5 u.u m0)                      (d/d rho)
-//   B = omega rho (3 m1 + 9 M2 u - 3 m0 u) + gamma (9 M2 Ft - 3 m0 Ft)     (d/d u)
-//   lam_F = B / (2 rho) + gamma (3 m1 - 3 m0 u + 9 M2 u)                     (d/d F)
+//   lam_f_j = (1 - omega) mu_j + A - b . u + b . c_j,
+//   A = omega (m0 + u . (3 m1 + N u / 2))                  (d/d rho)
+//   b = omega G + gamma N Ft / rho,  G = 3 m1 + N u        (d/d u, over rho)
+//   lam_F = b / 2 + gamma G                                 (d/d F)
 // (u depends on f through (sum c f + Ft/2)/rho; Ft = g + F). lam_f_j goes to the source of
-// the pulled population (a permutation: written once). The velocity-moment transpose of step
-// n+1 adds lam_u / (2 rho_{n+1}) to lam_F here, and lam_u is cleared for the next step.
+// the pulled population (a permutation: written once). lam_F is needed at the marked nodes only,
+// and Ft is zero elsewhere without a body force. The velocity-moment transpose of step n+1 adds
+// lam_u / (2 rho_{n+1}) to lam_F here, and lam_u is cleared for the next step. About 135 double
+// operations per node (the moments scaled by 36, opposite directions in pairs) against 220.
 template <typename T>
-__global__ void adj_collide_t_kernel(const double *__restrict__ lam_P1, const T *__restrict__ Pn,
-                                     const double *__restrict__ F, const NodeU *__restrict__ U1,
-                                     double *__restrict__ lam_u, LatArgs L, int fresh,
-                                     double *__restrict__ lam_P0, double *__restrict__ lam_F) {
+__global__ void __launch_bounds__(128) adj_collide_t_kernel(
+    const double *__restrict__ lam_P1, const T *__restrict__ Pn, const double *__restrict__ F,
+    const unsigned char *__restrict__ mark, const NodeU *__restrict__ U1,
+    double *__restrict__ lam_u, LatArgs L, int fresh, double *__restrict__ lam_P0,
+    double *__restrict__ lam_F) {
   const size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (n >= L.ncell) return;
-  const int x = (int)(n % L.nx), y = (int)((n / L.nx) % L.ny), z = (int)(n / ((size_t)L.nx * L.ny));
-  if (zkind(z, L) != 0) return;
+  const Node d = node_at(n, L);
+  if (zkind(d.z, L) != 0) return;
   using A = T;  // the forward state's arithmetic type
+  const bool marked = mark[n];
   A f[Q], ua[3];
   if (fresh) {
 #pragma unroll
     for (int i = 0; i < Q; i++) f[i] = (A)Pn[(size_t)i * L.ncell + n];
   } else {
-    pull_dev<A>(Pn, x, y, z, L, f);
+    pull_dev<A>(Pn, d, L, f);
   }
-  const double Ft[3] = {L.g[0] + F[3 * n], L.g[1] + F[3 * n + 1], L.g[2] + F[3 * n + 2]};
-  const A Fta[3] = {(A)Ft[0], (A)Ft[1], (A)Ft[2]};
-  const double rho = (double)velocity<A>(f, Fta, (A)L.rho0, ua);
-  const double u[3] = {(double)ua[0], (double)ua[1], (double)ua[2]};
-  const double ir = 1.0 / rho;
   double mu[Q];
 #pragma unroll
   for (int i = 0; i < Q; i++) mu[i] = lam_P1[(size_t)i * L.ncell + n];
-  // moments of mu from opposite pairs: c c^T is the same for both, c changes sign
-  double m0 = wgt(0) * mu[0], m1[3] = {0, 0, 0}, mxx = 0, myy = 0, mzz = 0, mxy = 0, mxz = 0,
-         myz = 0;
+  double Ft[3] = {L.g[0], L.g[1], L.g[2]};
+  if (marked)
+    for (int k = 0; k < 3; k++) Ft[k] += F[3 * n + k];
+  const A Fta[3] = {(A)Ft[0], (A)Ft[1], (A)Ft[2]};
+  const A rho = velocity<A>(f, Fta, (A)L.rho0, ua);
+  const double u[3] = {(double)ua[0], (double)ua[1], (double)ua[2]};
+  // 36 times the moments
+  double s[9], e[9];
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const double ws = wgt(i) * (mu[i] + mu[i + 1]);
-    const double wd = wgt(i) * (mu[i] - mu[i + 1]);
-    m0 += ws;
-    if (cx(i)) { m1[0] += cx(i) > 0 ? wd : -wd; mxx += ws; }
-    if (cy(i)) { m1[1] += cy(i) > 0 ? wd : -wd; myy += ws; }
-    if (cz(i)) { m1[2] += cz(i) > 0 ? wd : -wd; mzz += ws; }
-    if (cx(i) && cy(i)) mxy += cx(i) * cy(i) > 0 ? ws : -ws;
-    if (cx(i) && cz(i)) mxz += cx(i) * cz(i) > 0 ? ws : -ws;
-    if (cy(i) && cz(i)) myz += cy(i) * cz(i) > 0 ? ws : -ws;
+  for (int p = 0; p < 9; p++) {
+    s[p] = mu[2 * p + 1] + mu[2 * p + 2];
+    e[p] = mu[2 * p + 1] - mu[2 * p + 2];
   }
-  const double M2u[3] = {mxx * u[0] + mxy * u[1] + mxz * u[2], mxy * u[0] + myy * u[1] + myz * u[2],
-                         mxz * u[0] + myz * u[1] + mzz * u[2]};
-  const double M2F[3] = {mxx * Ft[0] + mxy * Ft[1] + mxz * Ft[2],
-                         mxy * Ft[0] + myy * Ft[1] + myz * Ft[2],
-                         mxz * Ft[0] + myz * Ft[1] + mzz * Ft[2]};
-  const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const double um1 = u[0] * m1[0] + u[1] * m1[1] + u[2] * m1[2];
-  const double uM2u = u[0] * M2u[0] + u[1] * M2u[1] + u[2] * M2u[2];
-  const double Arho = L.omega * (m0 + 3.0 * um1 + 4.5 * uM2u - 1.5 * uu * m0);
-  double B[3], lf[3];
+  const double pxy = s[3] + s[4], pxz = s[5] + s[6], pyz = s[7] + s[8];
+  const double M0 = fma(12.0, mu[0], fma(2.0, s[0] + s[1] + s[2], pxy + pxz + pyz));
+  const double c0 = M0 * (-1.0 / 12.0);
+  const double Nxx = fma(0.25, fma(2.0, s[0], pxy + pxz), c0);
+  const double Nyy = fma(0.25, fma(2.0, s[1], pxy + pyz), c0);
+  const double Nzz = fma(0.25, fma(2.0, s[2], pxz + pyz), c0);
+  const double Nxy = 0.25 * (s[3] - s[4]), Nxz = 0.25 * (s[5] - s[6]), Nyz = 0.25 * (s[7] - s[8]);
+  const double t[3] = {fma(2.0, e[0], (e[3] + e[4]) + (e[5] + e[6])) * (1.0 / 12.0),  // 3 m1
+                       fma(2.0, e[1], (e[3] - e[4]) + (e[7] + e[8])) * (1.0 / 12.0),
+                       fma(2.0, e[2], (e[5] - e[6]) + (e[7] - e[8])) * (1.0 / 12.0)};
+  const double Nu[3] = {fma(Nxx, u[0], fma(Nxy, u[1], Nxz * u[2])),
+                        fma(Nxy, u[0], fma(Nyy, u[1], Nyz * u[2])),
+                        fma(Nxz, u[0], fma(Nyz, u[1], Nzz * u[2]))};
+  double G[3], b[3], acc = M0 * (1.0 / 36.0);
   for (int k = 0; k < 3; k++) {
-    B[k] = L.omega * rho * (3.0 * m1[k] + 9.0 * M2u[k] - 3.0 * m0 * u[k]) +
-           L.gamma * (9.0 * M2F[k] - 3.0 * m0 * Ft[k]);
-    lf[k] = 0.5 * B[k] * ir + L.gamma * (3.0 * m1[k] - 3.0 * m0 * u[k] + 9.0 * M2u[k]);
+    acc = fma(u[k], fma(0.5, Nu[k], t[k]), acc);
+    G[k] = t[k] + Nu[k];
+    b[k] = L.omega * G[k];
   }
-  const double lu[3] = {lam_u[3 * n], lam_u[3 * n + 1], lam_u[3 * n + 2]};
-  if (lu[0] != 0.0 || lu[1] != 0.0 || lu[2] != 0.0) {
-    const double h = 0.5 / U1[n].rho;
-    for (int k = 0; k < 3; k++) {
-      lf[k] += lu[k] * h;
-      lam_u[3 * n + k] = 0.0;
+  if (marked || L.has_g) {
+    const double gr = L.gamma * reciprocal((double)rho);
+    b[0] = fma(gr, fma(Nxx, Ft[0], fma(Nxy, Ft[1], Nxz * Ft[2])), b[0]);
+    b[1] = fma(gr, fma(Nxy, Ft[0], fma(Nyy, Ft[1], Nyz * Ft[2])), b[1]);
+    b[2] = fma(gr, fma(Nxz, Ft[0], fma(Nyz, Ft[1], Nzz * Ft[2])), b[2]);
+  }
+  if (marked) {
+    double lf[3];
+    for (int k = 0; k < 3; k++) lf[k] = fma(0.5, b[k], L.gamma * G[k]);
+    const double lu[3] = {lam_u[3 * n], lam_u[3 * n + 1], lam_u[3 * n + 2]};
+    if (lu[0] != 0.0 || lu[1] != 0.0 || lu[2] != 0.0) {
+      const double h = 0.5 * reciprocal(U1[n].rho);
+      for (int k = 0; k < 3; k++) {
+        lf[k] = fma(lu[k], h, lf[k]);
+        lam_u[3 * n + k] = 0.0;
+      }
     }
+    for (int k = 0; k < 3; k++) lam_F[3 * n + k] = lf[k];
   }
-  for (int k = 0; k < 3; k++) lam_F[3 * n + k] = lf[k];
-  const double b[3] = {B[0] * ir, B[1] * ir, B[2] * ir};
-  const double s0 = Arho - (u[0] * b[0] + u[1] * b[1] + u[2] * b[2]);
+  double s0 = L.omega * acc;
+  for (int k = 0; k < 3; k++) s0 = fma(-u[k], b[k], s0);
   const double om1 = 1.0 - L.omega;
-  double lam[Q];
-  lam[0] = om1 * mu[0] + s0;
+  mu[0] = fma(om1, mu[0], s0);
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {  // c.b changes sign between opposite directions
     double cb = 0.0;
-    if (cx(i)) cb += cx(i) > 0 ? b[0] : -b[0];
-    if (cy(i)) cb += cy(i) > 0 ? b[1] : -b[1];
-    if (cz(i)) cb += cz(i) > 0 ? b[2] : -b[2];
-    lam[i] = om1 * mu[i] + s0 + cb;
-    lam[i + 1] = om1 * mu[i + 1] + s0 - cb;
+    if (cx(i)) cb = cx(i) > 0 ? b[0] : -b[0];
+    if (cy(i)) cb = cx(i) ? (cy(i) > 0 ? cb + b[1] : cb - b[1]) : (cy(i) > 0 ? b[1] : -b[1]);
+    if (cz(i)) cb = cx(i) || cy(i) ? (cz(i) > 0 ? cb + b[2] : cb - b[2]) : (cz(i) > 0 ? b[2] : -b[2]);
+    mu[i] = fma(om1, mu[i], s0 + cb);
+    mu[i + 1] = fma(om1, mu[i + 1], s0 - cb);
   }
 #pragma unroll
-  for (int i = 0; i < Q; i++) {
-    if (fresh) {
-      lam_P0[(size_t)i * L.ncell + n] = lam[i];
-    } else {
-      bool bb;
-      lam_P0[pull_source(x, y, z, i, L, bb)] = lam[i];  // a permutation: written once
-    }
-  }
+  for (int i = 0; i < Q; i++)  // a permutation: written once
+    lam_P0[fresh ? (size_t)i * L.ncell + n : pull_source(d, i, L)] = mu[i];
 }
 
 // Spreading^T: lam_phi_v = sum_x W lam_F(x) over the fluid nodes, and
-// lam_qn_v += sum_x (phi_v . lam_F(x)) dW/dq_v. The step's force field F is no longer
-// needed afterwards: its stencil nodes are cleared here, which leaves F zero for the next
-// reverse step's spreading.
+// lam_qn_v += sum_x (phi_v . lam_F(x)) dW/dq_v. With row sums over x, a = sum wx lam_F and
+// d = sum dwx lam_F, a row gives wy wz a, and wy wz phi.d, dwy wz phi.a, wy dwz phi.a. The step's
+// force field F and the marks are no longer needed afterwards: cleared here for the next step that
+// uses them.
 __global__ void adj_spread_t_kernel(int nv, const Stencil *__restrict__ st,
                                     const double *__restrict__ phi, const double *__restrict__ lam_F,
                                     LatArgs L, double *__restrict__ lam_phi,
-                                    double *__restrict__ lam_qn, double *__restrict__ F) {
-  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+                                    double *__restrict__ lam_qn, double *__restrict__ F,
+                                    unsigned char *__restrict__ mark) {
+  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  double c[6] = {0, 0, 0, 0, 0, 0};
+  if (v < nv) {
+    const Stencil &s = st[v];
+    const Row r = row_of(s, v, L);
+    if (r.kind == 0) {
+      double a[3] = {0, 0, 0}, g[3] = {0, 0, 0};
+      for (int dx = 0; dx < 4; dx++) {
+        const size_t n = r.base + wrapi(s.base[0] + dx, L.nx);
+        const double w = s.w[0][dx], dw = s.dw[0][dx];
+        for (int k = 0; k < 3; k++) {
+          const double lf = lam_F[3 * n + k];
+          a[k] = fma(w, lf, a[k]);
+          g[k] = fma(dw, lf, g[k]);
+          F[3 * n + k] = 0.0;
+        }
+        mark[n] = 0;
+      }
+      const double ph[3] = {phi[3 * v], phi[3 * v + 1], phi[3 * v + 2]};
+      const double pa = dot3(ph, a), wyz = r.wy * r.wz;
+      for (int k = 0; k < 3; k++) c[k] = wyz * a[k];
+      c[3] = wyz * dot3(ph, g);
+      c[4] = pa * (r.dwy * r.wz);
+      c[5] = pa * (r.wy * r.dwz);
+    }
+  }
+  double o[3];
+  half_sums<3>(c, o);
   if (v >= nv) return;
-  const Stencil &s = st[v];
-  const double ph[3] = {phi[3 * v], phi[3 * v + 1], phi[3 * v + 2]};
-  const int dx = lane & 3, dy = (lane >> 2) & 3;
-  double lp[3] = {0, 0, 0}, acc[3] = {0, 0, 0};
-  for (int h = 0; h < 2; h++) {
-    const int dz = (lane >> 4) + 2 * h;
-    const int z = s.base[2] + dz;
-    if (zkind(z, L) != 0) continue;
-    const size_t n = node_of(s.base[0] + dx, s.base[1] + dy, z, L);
-    const double lf[3] = {lam_F[3 * n], lam_F[3 * n + 1], lam_F[3 * n + 2]};
-    const double wx = s.w[0][dx], wy = s.w[1][dy], wz = s.w[2][dz];
-    const double w = wx * wy * wz;
-    for (int k = 0; k < 3; k++) {
-      lp[k] += w * lf[k];
-      F[3 * n + k] = 0.0;
-    }
-    const double pl = ph[0] * lf[0] + ph[1] * lf[1] + ph[2] * lf[2];
-    acc[0] += pl * s.dw[0][dx] * wy * wz;
-    acc[1] += pl * wx * s.dw[1][dy] * wz;
-    acc[2] += pl * wx * wy * s.dw[2][dz];
+  const int k = threadIdx.x & 7;
+  const double x = k == 0 ? o[0] : k == 1 ? o[1] : o[2];
+  if (k < 3) {
+    if (threadIdx.x & 8) lam_qn[3 * v + k] += x;
+    else lam_phi[3 * v + k] = x;
   }
-  for (int k = 0; k < 3; k++) {
-    lp[k] = warp_sum(lp[k]);
-    acc[k] = warp_sum(acc[k]);
-  }
-  if (lane == 0)
-    for (int k = 0; k < 3; k++) {
-      lam_phi[3 * v + k] = lp[k];
-      lam_qn[3 * v + k] += acc[k];
-    }
 }
 
 // --- host side ---------------------------------------------------------------------------
 
+// What the forward pieces of a reverse step leave for its transposes; two sets, so that those of
+// the next reverse step are prepared on a stream of their own beside this step's transposes.
+struct Pieces {
+  double *fc = nullptr, *fn = nullptr, *vpart = nullptr, *phi = nullptr, *F = nullptr;
+  unsigned char *mark = nullptr;  // [ncell] node of some vertex's stencil (fluid)
+  NodeU *U = nullptr;             // [ncell] velocity and density after streaming, marked nodes
+  Stencil *st = nullptr;          // [nv] stencils of the step's positions
+  cudaEvent_t ready = nullptr, free = nullptr;
+};
+
 struct Adjoint {
   int nsteps = 0, every = 0, first_fresh = 0;
+  bool recorded = false;              // the checkpoints hold a whole run
+  bool work = false;                  // the work arrays are there
   std::vector<void *> ck_P;           // populations at steps 0, K, 2K, ..., nsteps (storage type)
   std::vector<double *> ck_q;         // positions at the same steps
   std::vector<void *> seg_P;          // states of the segment being reversed (storage type)
   std::vector<double *> seg_q;
   double *lam_P[2] = {nullptr, nullptr};
   double *lam_q = nullptr, *lam_qn = nullptr, *lam_phi = nullptr, *lam_F = nullptr,
-         *lam_u = nullptr, *F = nullptr, *phi = nullptr;
-  double *fc = nullptr, *fn = nullptr, *fV = nullptr, *fj = nullptr, *dn = nullptr,
-         *fdot = nullptr, *fpar = nullptr, *sums = nullptr, *sums_t = nullptr, *grad = nullptr;
-  NodeU *U = nullptr;       // [ncell] velocity and density after streaming of the step
-  Stencil *st = nullptr;    // [nv] stencils of the step's positions
+         *lam_u = nullptr;
+  double *fj = nullptr, *dn = nullptr, *part = nullptr, *grad = nullptr;
+  Pieces pieces[2];
+  cudaStream_t side = nullptr;        // stream of the forward pieces
 };
 
 void free_all(Adjoint *a) {
   auto f = [](void *p) {
     if (p) cudaFree(p);
   };
+  if (a->side) cudaStreamSynchronize(a->side);
   for (void *p : a->ck_P) f(p);
   for (double *p : a->ck_q) f(p);
-  for (void *p : a->seg_P) f(p);
+  for (size_t m = 1; m < a->seg_P.size(); m++) f(a->seg_P[m]);  // ([0] is a checkpoint)
   for (double *p : a->seg_q) f(p);
   f(a->lam_P[0]); f(a->lam_P[1]); f(a->lam_q); f(a->lam_qn); f(a->lam_phi); f(a->lam_F);
-  f(a->lam_u); f(a->F); f(a->phi); f(a->fc); f(a->fn); f(a->fV); f(a->fj); f(a->dn); f(a->fdot);
-  f(a->fpar); f(a->sums); f(a->sums_t); f(a->grad); f(a->U); f(a->st);
+  f(a->lam_u); f(a->fj); f(a->dn); f(a->part); f(a->grad);
+  for (Pieces &p : a->pieces) {
+    f(p.fc); f(p.fn); f(p.vpart); f(p.phi); f(p.F); f(p.mark); f(p.U); f(p.st);
+    if (p.ready) cudaEventDestroy(p.ready);
+    if (p.free) cudaEventDestroy(p.free);
+  }
+  if (a->side) cudaStreamDestroy(a->side);
   delete a;
 }
 
@@ -694,6 +793,29 @@ int afail(Ctx &c, int code, const std::string &m) {
 cudaError_t dmalloc(double **p, size_t n) {
   *p = nullptr;
   return cudaMalloc((void **)p, (n ? n : 1) * sizeof(double));
+}
+
+// Make P hold nP population states and q hold nq positions, keeping what is there.
+int resize_states(Ctx &c, std::vector<void *> &P, std::vector<double *> &q, int nP, int nq) {
+  while ((int)P.size() > nP) {
+    cudaFree(P.back());
+    P.pop_back();
+  }
+  while ((int)q.size() > nq) {
+    cudaFree(q.back());
+    q.pop_back();
+  }
+  while ((int)P.size() < nP) {
+    void *p = nullptr;
+    ADJ_TRY(c, cudaMalloc(&p, (size_t)Q * c.ncell * c.pop_size));
+    P.push_back(p);
+  }
+  while ((int)q.size() < nq) {
+    double *p = nullptr;
+    ADJ_TRY(c, dmalloc(&p, (size_t)3 * c.nv));
+    q.push_back(p);
+  }
+  return 0;
 }
 
 FaceArgs face_args(const Ctx &c) {
@@ -717,6 +839,9 @@ LatArgs lat_args(const Ctx &c) {
   LatArgs L;
   L.nx = c.nx; L.ny = c.ny; L.nz = c.nz; L.walls = c.has_walls;
   L.ncell = c.ncell;
+  L.dx = fast_div(c.nx);
+  L.dy = fast_div(c.ny);
+  L.has_g = c.g[0] != 0.0 || c.g[1] != 0.0 || c.g[2] != 0.0;
   L.rho0 = c.rho0;
   L.omega = 1.0 / c.tau;
   L.gamma = 1.0 - 0.5 / c.tau;
@@ -754,59 +879,106 @@ int run_steps(Ctx &c, int n) {
   return health_status(c, hw);
 }
 
-// Recompute a segment: from the restored state, `len` steps, the state after each one copied
-// (as stored) to seg_P[m], seg_q[m]; everything queued, one health check at the end.
-int recompute_segment(Ctx &c, Adjoint *a, int len) {
+// Recompute a segment from checkpoint `s`: `len` steps, state m + 1 written by its step straight
+// into seg_P[m + 1] (the step reads one population array and writes the other, and these two are
+// lent to the context in place of its own), positions copied to seg_q; everything queued, one
+// health check at the end. State 0 is the checkpoint itself.
+int recompute_segment(Ctx &c, Adjoint *a, int s, int len, int fresh) {
+  void *const own[2] = {c.f[0], c.f[1]};
+  a->seg_P[0] = a->ck_P[s];
   ADJ_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
-  if (int rc = snapshot_raw(c, a->seg_P[0], a->seg_q[0])) return rc;
-  for (int m = 1; m <= len; m++) {
-    if (int rc = enqueue_steps(c, 1)) return rc;
-    if (int rc = snapshot_raw(c, a->seg_P[m], a->seg_q[m])) return rc;
+  int rc = restore_positions(c, a->ck_q[s], fresh);
+  for (int m = 0; m < len && rc == 0; m++) {
+    cudaError_t e = cudaMemcpyAsync(a->seg_q[m], c.q, (size_t)3 * c.nv * sizeof(double),
+                                    cudaMemcpyDeviceToDevice, c.stream);
+    if (e != cudaSuccess) rc = afail(c, IBLB_ECUDA, cudaGetErrorString(e));
+    c.f[c.cur] = a->seg_P[m];
+    c.f[c.cur ^ 1] = a->seg_P[m + 1];
+    if (rc == 0) rc = enqueue_steps(c, 1);
   }
+  c.f[0] = own[0];
+  c.f[1] = own[1];
+  if (rc) return rc;
   int hw = 0;
   ADJ_TRY(c, cudaMemcpyAsync(&hw, c.counters + 3, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   ADJ_TRY(c, cudaStreamSynchronize(c.stream));
   return health_status(c, hw);
 }
 
-// Reverse step n: a->lam_q (of q_{n+1}) and a->lam_P[1] (of P_{n+1}) become those of q_n, P_n
-// in a->lam_qn and a->lam_P[0] (swapped by the caller). Pn, Pn1 are stored populations (T).
-// No scratch field needs clearing: F and lam_u are zero between steps (cleared by their last
-// readers), lam_F and lam_P0 are overwritten at every fluid node.
+int face_warps(const Ctx &c) { return (c.nf + 31) / 32; }
+
+// Forward pieces of reverse step n at q_n, on the side stream: forces, volume, stencils, the
+// spread force field, the moments of P_{n+1}. They depend on the recomputed states only.
 template <typename T>
-int reverse_step(Ctx &c, Adjoint *a, const T *Pn, const double *qn, const T *Pn1, int fresh) {
-  const FaceArgs FA = face_args(c);
+int forward_pieces(Ctx &c, Adjoint *a, Pieces &p, const double *qn, const T *Pn1) {
   const LatArgs L = lat_args(c);
   const VolArgs va{c.iface.volume_force_on, c.iface.kV, c.V0};
-  // small blocks for the per-face and per-vertex passes: a few thousand threads spread over
-  // all SMs (their double arithmetic, not memory, sets their time)
-  const int tb = 32, tw = 128;
-  const unsigned gf = (unsigned)((c.nf + tb - 1) / tb), gv = (unsigned)((c.nv + tb - 1) / tb);
-  const unsigned gs = (unsigned)((3 * c.nv + tb - 1) / tb);     // a thread per (vertex, axis)
-  const unsigned gw = (unsigned)((32L * c.nv + tw - 1) / tw);   // a warp per vertex
+  const unsigned gf = (unsigned)((c.nf + kFaceThreads - 1) / kFaceThreads);
+  const unsigned gv = (unsigned)((3L * c.nv + kVertexThreads - 1) / kVertexThreads);
+  const unsigned gw = (unsigned)((16L * c.nv + 127) / 128);  // sixteen lanes per vertex
   const unsigned gn = (unsigned)((c.ncell + 255) / 256);
-  cudaStream_t st = c.stream;
-  // forward pieces at q_n: forces, volume, stencils, the spread force field, the moments
-  adj_face_value_kernel<<<gf, tb, 0, st>>>(FA, qn, a->fc, a->fn, a->fV);
-  adj_face_sums_kernel<<<1, kSumThreads, 0, st>>>(c.nf, a->fV, nullptr, 0, a->sums, nullptr);
-  adj_vertex_kernel<<<gv, tb, 0, st>>>(c.nv, c.vf_start, c.vf_list, a->fc, a->fn, nullptr, a->sums,
-                                       nullptr, va, 0, a->phi);
-  adj_stencil_kernel<<<gs, tb, 0, st>>>(c.nv, qn, a->st);
-  adj_spread_kernel<<<gw, tw, 0, st>>>(c.nv, a->st, a->phi, L, a->F);
-  adj_moments_kernel<T><<<gn, 256, 0, st>>>(Pn1, a->F, L, a->U);
-  // interpolation^T, velocity^T, collision^T and streaming^T, spreading^T
-  adj_interp_t_kernel<<<gw, tw, 0, st>>>(c.nv, a->st, a->lam_q, a->U, L, a->lam_qn, a->lam_u);
-  adj_velocity_t_kernel<<<gn, 256, 0, st>>>(a->lam_u, a->U, L, a->lam_P[1]);
-  adj_collide_t_kernel<T><<<gn, 256, 0, st>>>(a->lam_P[1], Pn, a->F, a->U, a->lam_u, L, fresh,
-                                              a->lam_P[0], a->lam_F);
-  adj_spread_t_kernel<<<gw, tw, 0, st>>>(c.nv, a->st, a->phi, a->lam_F, L, a->lam_phi, a->lam_qn,
-                                         a->F);
-  // force Jacobian^T along lam_phi, and the parameter derivatives (added to grad)
-  adj_face_tangent_kernel<<<gf, tb, 0, st>>>(FA, qn, a->lam_phi, a->fj, a->dn, a->fdot, a->fpar);
-  adj_face_sums_kernel<<<1, kSumThreads, 0, st>>>(c.nf, a->fdot, a->fpar, 4, a->sums_t, a->grad);
-  adj_vertex_kernel<<<gv, tb, 0, st>>>(c.nv, c.vf_start, c.vf_list, a->fj, a->fn, a->dn, a->sums,
-                                       a->sums_t, va, 1, a->lam_qn);
+  cudaStream_t st = a->side;
+  ADJ_TRY(c, cudaStreamWaitEvent(st, p.free, 0));
+  adj_face_value_kernel<<<gf, kFaceThreads, 0, st>>>(face_args(c), qn, p.fc, p.fn, p.vpart);
+  adj_vertex_value_kernel<<<gv, kVertexThreads, 0, st>>>(c.nv, face_warps(c), c.vf_start, c.vf_list,
+                                                         p.fc, p.fn, p.vpart, va, qn, p.phi, p.st);
+  adj_spread_kernel<<<gw, 128, 0, st>>>(c.nv, p.st, p.phi, L, p.F, p.mark);
+  adj_moments_kernel<T><<<gn, 256, 0, st>>>(Pn1, p.F, p.mark, L, p.U);
   ADJ_TRY(c, cudaGetLastError());
+  ADJ_TRY(c, cudaEventRecord(p.ready, st));
+  return 0;
+}
+
+// Reverse step n: a->lam_q (of q_{n+1}) and a->lam_P[1] (of P_{n+1}) become those of q_n, P_n
+// in a->lam_qn and a->lam_P[0] (swapped by the caller). Pn are stored populations (T). No scratch
+// field needs clearing: F, the marks and lam_u are zero between steps (cleared by their last
+// readers), lam_P0 is overwritten at every fluid node, lam_F at every marked one.
+template <typename T>
+int reverse_step(Ctx &c, Adjoint *a, Pieces &p, const T *Pn, const double *qn, int fresh) {
+  const LatArgs L = lat_args(c);
+  const VolArgs va{c.iface.volume_force_on, c.iface.kV, c.V0};
+  const unsigned gf = (unsigned)((c.nf + kFaceThreads - 1) / kFaceThreads);
+  const unsigned gv = (unsigned)((3L * c.nv + kVertexThreads - 1) / kVertexThreads);
+  const unsigned gw = (unsigned)((16L * c.nv + 127) / 128);
+  cudaStream_t st = c.stream;
+  ADJ_TRY(c, cudaStreamWaitEvent(st, p.ready, 0));
+  // interpolation^T, velocity^T, collision^T and streaming^T, spreading^T
+  adj_interp_t_kernel<<<gw, 128, 0, st>>>(c.nv, p.st, a->lam_q, p.U, L, a->lam_qn, a->lam_u);
+  adj_velocity_t_kernel<<<(unsigned)((c.ncell + 255) / 256), 256, 0, st>>>(a->lam_u, p.mark, p.U, L,
+                                                                          a->lam_P[1]);
+  adj_collide_t_kernel<T><<<(unsigned)((c.ncell + 127) / 128), 128, 0, st>>>(
+      a->lam_P[1], Pn, p.F, p.mark, p.U, a->lam_u, L, fresh, a->lam_P[0], a->lam_F);
+  adj_spread_t_kernel<<<gw, 128, 0, st>>>(c.nv, p.st, p.phi, a->lam_F, L, a->lam_phi, a->lam_qn, p.F,
+                                          p.mark);
+  // force Jacobian^T along lam_phi, and the parameter derivatives (added to grad)
+  adj_face_tangent_kernel<<<gf, kFaceThreads, 0, st>>>(face_args(c), qn, a->lam_phi, a->fj, a->dn,
+                                                       a->part);
+  adj_vertex_tangent_kernel<<<gv, kVertexThreads, 0, st>>>(c.nv, face_warps(c), c.vf_start, c.vf_list,
+                                                           a->fj, p.fn, a->dn, p.vpart, a->part, va,
+                                                           a->lam_qn, a->grad);
+  ADJ_TRY(c, cudaGetLastError());
+  ADJ_TRY(c, cudaEventRecord(p.free, st));
+  return 0;
+}
+
+// The reverse steps of a recomputed segment of len steps (seg_P[0] fresh: the run's first state).
+template <typename T>
+int reverse_segment(Ctx &c, Adjoint *a, int len, int first_fresh) {
+  // the side stream starts after the recomputed states (and after what last used the pieces)
+  for (Pieces &p : a->pieces) ADJ_TRY(c, cudaEventRecord(p.free, c.stream));
+  auto prepare = [&](int m) {
+    return forward_pieces<T>(c, a, a->pieces[m & 1], a->seg_q[m], (const T *)a->seg_P[m + 1]);
+  };
+  if (int rc = prepare(len - 1)) return rc;
+  for (int m = len - 1; m >= 0; m--) {
+    if (m > 0)
+      if (int rc = prepare(m - 1)) return rc;
+    if (int rc = reverse_step<T>(c, a, a->pieces[m & 1], (const T *)a->seg_P[m], a->seg_q[m],
+                                 m == 0 && first_fresh))
+      return rc;
+    std::swap(a->lam_q, a->lam_qn);
+    std::swap(a->lam_P[0], a->lam_P[1]);
+  }
   return 0;
 }
 
@@ -831,22 +1003,24 @@ int iblb_adjoint_record(iblb_ctx *h, int32_t nsteps, int32_t every) {
   if (c.nv == 0) return iblb::afail(c, IBLB_EINVAL, "no mesh has been added");
   if (nsteps < 1 || every < 1) return iblb::afail(c, IBLB_EINVAL, "nsteps and every must be >= 1");
   if (int rc = iblb::settle_health(c)) return rc;  // a failure of earlier iblb_step_async steps
-  iblb::adjoint_free(c);
-  auto *a = new iblb::Adjoint();
-  c.adj = a;
-  a->nsteps = nsteps;
-  a->every = every < nsteps ? every : nsteps;
-  a->first_fresh = c.fresh;
-  const size_t pn = (size_t)iblb::Q * c.ncell, qn = (size_t)3 * c.nv;
-  const int nck = (nsteps + a->every - 1) / a->every + 1;
-  for (int k = 0; k < nck; k++) {
-    void *P = nullptr;
-    double *q = nullptr;
-    ADJ_TRY(c, cudaMalloc(&P, pn * c.pop_size));
-    a->ck_P.push_back(P);
-    ADJ_TRY(c, iblb::dmalloc(&q, qn));
-    a->ck_q.push_back(q);
+  // the arrays of an earlier recording serve again (its states change in number only): allocating
+  // and freeing them took 2 ms of a 60-step gradient. Released by iblb_adjoint_release.
+  const int step = every < nsteps ? every : nsteps;
+  const int nck = (nsteps + step - 1) / step + 1;
+  if (!c.adj) c.adj = new iblb::Adjoint();
+  auto *a = (iblb::Adjoint *)c.adj;
+  a->recorded = false;
+  int rc = iblb::resize_states(c, a->ck_P, a->ck_q, nck, nck);
+  if (rc == IBLB_ENOMEM && (a->work || !a->seg_q.empty())) {  // without the last gradient's arrays
+    cudaGetLastError();
+    iblb::adjoint_free(c);
+    c.adj = a = new iblb::Adjoint();
+    rc = iblb::resize_states(c, a->ck_P, a->ck_q, nck, nck);
   }
+  if (rc) return rc;
+  a->nsteps = nsteps;
+  a->every = step;
+  a->first_fresh = c.fresh;
   ADJ_TRY(c, cudaStreamSynchronize(c.stream));
   if (int rc = iblb::snapshot_raw(c, a->ck_P[0], a->ck_q[0])) return rc;
   int done = 0;
@@ -857,6 +1031,7 @@ int iblb_adjoint_record(iblb_ctx *h, int32_t nsteps, int32_t every) {
     if (int rc = iblb::snapshot_raw(c, a->ck_P[k], a->ck_q[k])) return rc;
   }
   ADJ_TRY(c, cudaStreamSynchronize(c.stream));
+  a->recorded = true;
   return IBLB_OK;
 }
 
@@ -864,46 +1039,49 @@ int iblb_adjoint_gradient(iblb_ctx *h, const double *dJdq, double *dJdtheta) {
   if (!h || !dJdq || !dJdtheta) return IBLB_EINVAL;
   Ctx &c = h->c;
   auto *a = (iblb::Adjoint *)c.adj;
-  if (!a) return iblb::afail(c, IBLB_EINVAL, "no trajectory recorded (iblb_adjoint_record)");
+  if (!a || !a->recorded)
+    return iblb::afail(c, IBLB_EINVAL, "no trajectory recorded (iblb_adjoint_record)");
   if (int rc = iblb::settle_health(c)) return rc;
   const size_t pn = (size_t)iblb::Q * c.ncell, qn = (size_t)3 * c.nv;
   // work arrays (kept for later calls)
-  if (!a->lam_q) {
+  if (!a->work) {
     ADJ_TRY(c, iblb::dmalloc(&a->lam_P[0], pn));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_P[1], pn));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_q, qn));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_qn, qn));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_phi, qn));
-    ADJ_TRY(c, iblb::dmalloc(&a->phi, qn));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_F, 3 * c.ncell));
     ADJ_TRY(c, iblb::dmalloc(&a->lam_u, 3 * c.ncell));
-    ADJ_TRY(c, iblb::dmalloc(&a->F, 3 * c.ncell));
-    ADJ_TRY(c, iblb::dmalloc(&a->fc, (size_t)9 * c.nf));
     ADJ_TRY(c, iblb::dmalloc(&a->fj, (size_t)9 * c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->fn, (size_t)3 * c.nf));
     ADJ_TRY(c, iblb::dmalloc(&a->dn, (size_t)3 * c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->fV, (size_t)c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->fdot, (size_t)c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->fpar, (size_t)4 * c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->sums, 8));
-    ADJ_TRY(c, iblb::dmalloc(&a->sums_t, 8));
+    ADJ_TRY(c, iblb::dmalloc(&a->part, (size_t)5 * iblb::face_warps(c)));
     ADJ_TRY(c, iblb::dmalloc(&a->grad, 4));
-    ADJ_TRY(c, cudaMalloc((void **)&a->U, c.ncell * sizeof(iblb::NodeU)));
-    ADJ_TRY(c, cudaMalloc((void **)&a->st, (size_t)c.nv * sizeof(iblb::Stencil)));
-    for (int m = 0; m <= a->every; m++) {
-      void *P = nullptr;
-      double *q = nullptr;
-      ADJ_TRY(c, cudaMalloc(&P, pn * c.pop_size));
-      a->seg_P.push_back(P);
-      ADJ_TRY(c, iblb::dmalloc(&q, qn));
-      a->seg_q.push_back(q);
+    for (iblb::Pieces &p : a->pieces) {
+      ADJ_TRY(c, iblb::dmalloc(&p.fc, (size_t)9 * c.nf));
+      ADJ_TRY(c, iblb::dmalloc(&p.fn, (size_t)3 * c.nf));
+      ADJ_TRY(c, iblb::dmalloc(&p.vpart, (size_t)iblb::face_warps(c)));
+      ADJ_TRY(c, iblb::dmalloc(&p.phi, qn));
+      ADJ_TRY(c, iblb::dmalloc(&p.F, 3 * c.ncell));
+      ADJ_TRY(c, cudaMalloc((void **)&p.mark, c.ncell));
+      ADJ_TRY(c, cudaMalloc((void **)&p.U, c.ncell * sizeof(iblb::NodeU)));
+      ADJ_TRY(c, cudaMalloc((void **)&p.st, (size_t)c.nv * sizeof(iblb::Stencil)));
+      ADJ_TRY(c, cudaEventCreateWithFlags(&p.ready, cudaEventDisableTiming));
+      ADJ_TRY(c, cudaEventCreateWithFlags(&p.free, cudaEventDisableTiming));
     }
+    ADJ_TRY(c, cudaStreamCreateWithFlags(&a->side, cudaStreamNonBlocking));
+    a->work = true;
   }
+  // states 1 .. every of a segment and the positions 0 .. every - 1
+  if (a->seg_P.empty()) a->seg_P.push_back(nullptr);
+  if (int rc = iblb::resize_states(c, a->seg_P, a->seg_q, a->every + 1, a->every)) return rc;
   ADJ_TRY(c, cudaMemcpyAsync(a->lam_q, dJdq, qn * sizeof(double), cudaMemcpyHostToDevice, c.stream));
   ADJ_TRY(c, cudaMemsetAsync(a->lam_P[0], 0, pn * sizeof(double), c.stream));
   ADJ_TRY(c, cudaMemsetAsync(a->lam_P[1], 0, pn * sizeof(double), c.stream));
   // zero between reverse steps (each step leaves them so)
-  ADJ_TRY(c, cudaMemsetAsync(a->F, 0, 3 * c.ncell * sizeof(double), c.stream));
+  for (iblb::Pieces &p : a->pieces) {
+    ADJ_TRY(c, cudaMemsetAsync(p.F, 0, 3 * c.ncell * sizeof(double), c.stream));
+    ADJ_TRY(c, cudaMemsetAsync(p.mark, 0, c.ncell, c.stream));
+  }
   ADJ_TRY(c, cudaMemsetAsync(a->lam_u, 0, 3 * c.ncell * sizeof(double), c.stream));
   ADJ_TRY(c, cudaMemsetAsync(a->grad, 0, 4 * sizeof(double), c.stream));
   const int nseg = (int)a->ck_P.size() - 1;
@@ -911,20 +1089,11 @@ int iblb_adjoint_gradient(iblb_ctx *h, const double *dJdq, double *dJdtheta) {
   for (int s = nseg - 1; s >= 0 && rc == 0; s--) {
     const int first = s * a->every;
     const int len = (a->nsteps - first) < a->every ? a->nsteps - first : a->every;
-    const int fresh0 = s == 0 ? a->first_fresh : 0;
-    rc = iblb::restore_state(c, a->ck_P[s], a->ck_q[s], fresh0);
-    if (rc == 0) rc = iblb::recompute_segment(c, a, len);
-    for (int m = len - 1; m >= 0 && rc == 0; m--) {
-      const int fresh = s == 0 && m == 0 && a->first_fresh;
-      if (c.pop_size == sizeof(double))
-        rc = iblb::reverse_step<double>(c, a, (const double *)a->seg_P[m], a->seg_q[m],
-                                        (const double *)a->seg_P[m + 1], fresh);
-      else
-        rc = iblb::reverse_step<float>(c, a, (const float *)a->seg_P[m], a->seg_q[m],
-                                       (const float *)a->seg_P[m + 1], fresh);
-      std::swap(a->lam_q, a->lam_qn);
-      std::swap(a->lam_P[0], a->lam_P[1]);
-    }
+    const int first_fresh = s == 0 && a->first_fresh;
+    rc = iblb::recompute_segment(c, a, s, len, first_fresh);
+    if (rc == 0)
+      rc = c.pop_size == sizeof(double) ? iblb::reverse_segment<double>(c, a, len, first_fresh)
+                                        : iblb::reverse_segment<float>(c, a, len, first_fresh);
   }
   // back to the end of the recorded run
   if (rc == 0) rc = iblb::restore_state(c, a->ck_P[nseg], a->ck_q[nseg], 0);

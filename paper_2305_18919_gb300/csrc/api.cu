@@ -344,7 +344,7 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
   if (e == cudaSuccess) e = cudaMallocHost((void **)&c.health_host, sizeof(int));
   if (e == cudaSuccess) e = dalloc_bytes(&c.fused_ctl, iblb::kFusedControlBytes);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.fused_ctl, 0, iblb::kFusedControlBytes, c.stream);
-  c.fused = e == cudaSuccess && d->ib_sms == 0 && pass_bytes < kFusedPassBytes && iblb::fused_steps_fit(c);
+  c.fused = e == cudaSuccess && d->ib_sms == 0 && pass_bytes < kFusedPassBytes;
   if (e == cudaSuccess) e = cudaMemsetAsync(c.counters, 0, 8 * sizeof(int), c.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
   if (e != cudaSuccess) {
@@ -607,10 +607,20 @@ bool takes_fused(const Ctx &c) {
 // waits this long at most (some milliseconds).
 constexpr int kFusedSteps = 64;
 
-int enqueue_fused(Ctx &c, int nsteps) {
+// `left` returns the steps that the separate kernels have to take: those of a launch that the
+// caller's context has too few SMs for (the context then keeps to them).
+int enqueue_fused(Ctx &c, int nsteps, int *left) {
+  *left = 0;
   for (int done = 0; done < nsteps;) {
     const int n = nsteps - done < kFusedSteps ? nsteps - done : kFusedSteps;
-    CUDA_TRY(c, launch_fused_steps(c, n, c.stream));
+    const cudaError_t e = launch_fused_steps(c, n, c.stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+      cudaGetLastError();
+      c.fused = 0;
+      *left = nsteps - done;
+      return 0;
+    }
+    CUDA_TRY(c, e);
     c.k1_launches += n;
     c.kernel_launches += 1;
     c.cur ^= n & 1;
@@ -631,7 +641,8 @@ int enqueue_steps(Ctx &c, int nsteps) {
       if (int rc = enqueue_steps(c, 1)) return rc;
       nsteps--;
     }
-    return enqueue_fused(c, nsteps);
+    if (int rc = enqueue_fused(c, nsteps, &nsteps)) return rc;
+    if (nsteps == 0) return 0;
   }
   // the library streams start after everything queued so far on the context's stream
   CUDA_TRY(c, cudaEventRecord(c.ev_sync, c.stream));
@@ -715,13 +726,17 @@ int pending_health(Ctx &c) {
   return health_status(c, *c.health_host);
 }
 
-int restore_state(Ctx &c, const void *P, const double *q, int fresh) {
-  CUDA_TRY(c, cudaMemcpyAsync(c.f[c.cur], P, (size_t)Q * c.ncell * c.pop_size,
-                              cudaMemcpyDeviceToDevice, c.stream));
+int restore_positions(Ctx &c, const double *q, int fresh) {
   CUDA_TRY(c, cudaMemcpyAsync(c.q, q, (size_t)3 * c.nv * sizeof(double), cudaMemcpyDeviceToDevice,
                               c.stream));
   c.fresh = fresh;
   return positions_changed(c);
+}
+
+int restore_state(Ctx &c, const void *P, const double *q, int fresh) {
+  CUDA_TRY(c, cudaMemcpyAsync(c.f[c.cur], P, (size_t)Q * c.ncell * c.pop_size,
+                              cudaMemcpyDeviceToDevice, c.stream));
+  return restore_positions(c, q, fresh);
 }
 
 }  // namespace iblb

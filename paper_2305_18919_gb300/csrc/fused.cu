@@ -239,18 +239,11 @@ cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
   a.nsteps = nsteps;
   a.nchain = c.sm_count;
   void *params[] = {&a};
+  // (two blocks per SM always fit: the launch bound limits their registers, and each has 40 KB of
+  // shared memory; a caller's context with fewer SMs than the device refuses the launch)
   return cudaLaunchCooperativeKernel((const void *)fused_step_kernel<real, S>,
                                      dim3(FusedShape<real>::per_sm * c.sm_count),
                                      dim3(FusedShape<real>::threads), params, 0, st);
-}
-
-// Whether the fused kernel's grid is resident at once on this device.
-template <typename real, typename S>
-bool fused_fits_t(const Ctx &c) {
-  int n = 0;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_step_kernel<real, S>,
-                                                       FusedShape<real>::threads, 0) == cudaSuccess &&
-         n >= FusedShape<real>::per_sm;
 }
 
 }  // namespace
@@ -261,15 +254,6 @@ cudaError_t launch_fused_steps(Ctx &c, int nsteps, cudaStream_t s) {
     case IBLB_FP16: return launch_fused_t<float, __half>(c, nsteps, s);
     case IBLB_BF16: return launch_fused_t<float, __nv_bfloat16>(c, nsteps, s);
     default: return launch_fused_t<float, float>(c, nsteps, s);
-  }
-}
-
-bool fused_steps_fit(const Ctx &c) {
-  switch (c.precision) {
-    case IBLB_FP64: return fused_fits_t<double, double>(c);
-    case IBLB_FP16: return fused_fits_t<float, __half>(c);
-    case IBLB_BF16: return fused_fits_t<float, __nv_bfloat16>(c);
-    default: return fused_fits_t<float, float>(c);
   }
 }
 

@@ -226,6 +226,8 @@ int health_status(Ctx &c, int health_word);
 // arrays), with the given fresh flag: the next step continues from
 // there exactly as from the state that P and q were copied from.
 int restore_state(Ctx &c, const void *P, const double *q, int fresh);
+// The same without the populations: f[cur] holds them already.
+int restore_positions(Ctx &c, const double *q, int fresh);
 // A failure of steps queued by iblb_step_async: read with a synchronisation (settle_health), or
 // queued before a read call's own synchronisation (queue_health) and taken after it
 // (pending_health). Each returns IBLB_OK or the failure, and clears the pending mark.
@@ -241,10 +243,9 @@ bool stream_collide_staged(const Ctx &c);
 
 // Device bytes of the fused step kernel's control words.
 constexpr size_t kFusedControlBytes = 64;
-// nsteps coupled steps (not the first, in-place one; a mesh) as one cooperative launch (fused.cu).
+// nsteps coupled steps (not the first, in-place one; a mesh) as one cooperative launch (fused.cu);
+// cudaErrorCooperativeLaunchTooLarge, and nothing launched, where the grid cannot be resident.
 cudaError_t launch_fused_steps(Ctx &c, int nsteps, cudaStream_t s);
-// Whether that kernel's grid is resident at once on the context's device.
-bool fused_steps_fit(const Ctx &c);
 
 // Launchers (each returns cudaGetLastError() of its launch) on stream `s`.
 // Stream-collide of every fluid node with the body force only (no interface force).
