@@ -140,12 +140,27 @@ bool green_api(GreenApi &g) {
   return true;
 }
 
-// Largest stream-collide pass (bytes read and written) of a lattice whose steps run as one kernel.
-constexpr size_t kFusedPassBytes = (size_t)1 << 30;
+// Whether the steps of a default context run as one kernel (fused.cu), by the bytes that its
+// stream-collide pass reads and writes. With a mesh: below 1 GiB (us per step, fused against the
+// separate kernels: 24^3 FP32 28 / 46, 64^3 35 / 52, 128x128x96 65 / 69, 128^3 FP32 77 / 78 and
+// FP16 60 / 72, 192^3 FP32 189 / 187). Without one, where only the gap between two launches of
+// the pass is saved and the pass alone runs at a higher occupancy: below 30 MB in FP32 and 80 MB in
+// 16 bits, never in FP64 (32^3 FP32 3.2 / 4.3, FP16 3.3 / 6.3; 64^3 FP32 9.3 / 8.4, FP16 5.3 / 8.4;
+// 128^3 FP16 30.6 / 30.1; 48^3 FP64 37.5 / 35.1).
+bool fused_by_size(const Ctx &c) {
+  const size_t pass = (size_t)2 * iblb::Q * c.ncell * c.pop_size;
+  if (c.nv) return pass < ((size_t)1 << 30);
+  return c.pop_size == 4 ? pass < 30000000 : c.pop_size == 2 && pass < 80000000;
+}
+
+// SMs of the interface partition that the lattice partition may use as well: the interface chain
+// is idle for a part of every step (256^3: FP16 244 us per step against 249 without any, 275 with
+// 16; FP32 409 against 413).
+constexpr int kSharedSms = 8;
 
 // Split the device's SMs into an interface partition of about `want` SMs and a lattice
-// partition with the rest, each with its own stream. Returns false (and leaves nothing
-// behind) when the device or driver cannot partition.
+// partition with the rest and kSharedSms of the first, each with its own stream. Returns false
+// (and leaves nothing behind) when the device or driver cannot partition.
 bool make_partitions(Ctx &c, int want, int prio_hi) {
   GreenApi g;
   if (!green_api(g)) return false;
@@ -158,6 +173,12 @@ bool make_partitions(Ctx &c, int want, int prio_hi) {
   if (g.split(&part, &groups, &all, &rest, 0, (unsigned)want) != CUDA_SUCCESS || groups != 1 ||
       rest.sm.smCount < part.sm.smCount)
     return false;
+  if (want > 2 * kSharedSms) {
+    CUdevResource less, more;
+    unsigned int one = 1;
+    if (g.split(&less, &one, &all, &more, 0, (unsigned)(want - kSharedSms)) == CUDA_SUCCESS && one == 1)
+      rest = more;
+  }
   CUdevResourceDesc d_ib, d_lat;
   if (g.make_desc(&d_ib, &part, 1) != CUDA_SUCCESS || g.make_desc(&d_lat, &rest, 1) != CUDA_SUCCESS)
     return false;
@@ -344,7 +365,7 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
   if (e == cudaSuccess) e = cudaMallocHost((void **)&c.health_host, sizeof(int));
   if (e == cudaSuccess) e = dalloc_bytes(&c.fused_ctl, iblb::kFusedControlBytes);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.fused_ctl, 0, iblb::kFusedControlBytes, c.stream);
-  c.fused = e == cudaSuccess && d->ib_sms == 0 && pass_bytes < kFusedPassBytes;
+  c.fused = e == cudaSuccess && d->ib_sms == 0;
   if (e == cudaSuccess) e = cudaMemsetAsync(c.counters, 0, 8 * sizeof(int), c.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
   if (e != cudaSuccess) {
@@ -596,11 +617,11 @@ void release_sms(Ctx &c) { free_partitions(c); }
 
 namespace {
 
-// Whether the context's steps after the first run as one kernel: a lattice chosen for it at its
-// creation, and nothing asked for that only the separate kernels have (their timing, a choice of
-// the stream-collide kernel or of its waits).
+// Whether the context's steps after the first run as one kernel: of a size for it, and nothing
+// asked for that only the separate kernels have (an SM partition, their timing, a choice of the
+// stream-collide kernel or of its waits).
 bool takes_fused(const Ctx &c) {
-  return c.fused && c.nv && !c.profiling && c.k1_kind == IBLB_STREAM_COLLIDE_AUTO && !c.stage_wait_set;
+  return c.fused && fused_by_size(c) && !c.profiling && c.k1_kind == IBLB_STREAM_COLLIDE_AUTO && !c.stage_wait_set;
 }
 
 // Steps of one fused launch: the GPU is the launch's own while it runs, so work of other streams
@@ -624,9 +645,11 @@ int enqueue_fused(Ctx &c, int nsteps, int *left) {
     c.k1_launches += n;
     c.kernel_launches += 1;
     c.cur ^= n & 1;
-    c.map ^= n & 1;
-    c.marked = 0;
-    c.have_force = 1;
+    if (c.nv) {
+      c.map ^= n & 1;
+      c.marked = 0;
+      c.have_force = 1;
+    }
     c.steps_done += n;
     done += n;
   }
@@ -647,7 +670,9 @@ int enqueue_steps(Ctx &c, int nsteps) {
   // the library streams start after everything queued so far on the context's stream
   CUDA_TRY(c, cudaEventRecord(c.ev_sync, c.stream));
   CUDA_TRY(c, cudaStreamWaitEvent(c.ib, c.ev_sync, 0));
-  if (c.ls != c.stream) CUDA_TRY(c, cudaStreamWaitEvent(c.ls, c.ev_sync, 0));
+  // without a mesh there is no chain to share the SMs with: the passes run on all of them
+  cudaStream_t ls = c.nv ? c.ls : c.stream;
+  if (ls != c.stream) CUDA_TRY(c, cudaStreamWaitEvent(ls, c.ev_sync, 0));
   for (int s = 0; s < nsteps; s++) {
     if (c.nv) {
       CUDA_TRY(c, iblb::launch_face_forces(c, 1, c.ib));
@@ -661,16 +686,16 @@ int enqueue_steps(Ctx &c, int nsteps) {
       e0 = pooled_event(c);
       e1 = pooled_event(c);
       if (!e0 || !e1) return fail(c, IBLB_ECUDA, "cudaEventCreate failed");
-      CUDA_TRY(c, cudaEventRecord(e0, c.ls));
+      CUDA_TRY(c, cudaEventRecord(e0, ls));
     }
-    CUDA_TRY(c, iblb::launch_stream_collide(c, c.fresh, c.ls));
-    if (c.profiling) CUDA_TRY(c, cudaEventRecord(e1, c.ls));
+    CUDA_TRY(c, iblb::launch_stream_collide(c, c.fresh, ls));
+    if (c.profiling) CUDA_TRY(c, cudaEventRecord(e1, ls));
     c.k1_launches += 1;
     c.kernel_launches += 1;
     if (c.nv) {
-      CUDA_TRY(c, cudaStreamWaitEvent(c.ls, c.ev_force, 0));
-      CUDA_TRY(c, iblb::launch_stream_collide_tiles(c, c.fresh, c.ls));
-      CUDA_TRY(c, cudaEventRecord(c.ev_coll, c.ls));
+      CUDA_TRY(c, cudaStreamWaitEvent(ls, c.ev_force, 0));
+      CUDA_TRY(c, iblb::launch_stream_collide_tiles(c, c.fresh, ls));
+      CUDA_TRY(c, cudaEventRecord(c.ev_coll, ls));
       c.kernel_launches += 1;
     }
     c.cur ^= 1;
@@ -696,8 +721,8 @@ int enqueue_steps(Ctx &c, int nsteps) {
   // the context's stream continues after the last step on both library streams
   CUDA_TRY(c, cudaEventRecord(c.ev_sync, c.ib));
   CUDA_TRY(c, cudaStreamWaitEvent(c.stream, c.ev_sync, 0));
-  if (c.ls != c.stream) {
-    CUDA_TRY(c, cudaEventRecord(c.ev_coll, c.ls));
+  if (ls != c.stream) {
+    CUDA_TRY(c, cudaEventRecord(c.ev_coll, ls));
     CUDA_TRY(c, cudaStreamWaitEvent(c.stream, c.ev_coll, 0));
   }
   return 0;

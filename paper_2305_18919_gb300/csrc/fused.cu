@@ -112,6 +112,40 @@ __device__ __forceinline__ bool grid_barrier(unsigned *ctr, unsigned target, Fus
   return s_go != 0;
 }
 
+// The last block to leave clears the control words for the next launch.
+__device__ __forceinline__ void leave_grid(FusedControl *ctl) {
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(&ctl->left, 1u) == gridDim.x - 1) {
+    ctl->chain = 0;
+    ctl->all = 0;
+    ctl->abort = 0;
+    ctl->next[0] = ctl->next[1] = 0;
+    __threadfence();
+    ctl->left = 0;
+  }
+}
+
+// Node group g of the lattice pass (K1, body force only).
+template <typename real, typename S>
+__device__ __forceinline__ void lattice_group(const StreamArgs<real, S> &A, int g) {
+  int gx, y, z;
+  A.G.at(g, gx, y, z);
+  z += A.z0;
+  if constexpr (sizeof(S) == 2) {
+    if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
+    else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
+  } else {
+    const int x0 = 2 * gx;
+    real a[Q], b[Q];
+    load_pair<real, S, false>(A.fin, A.P, x0, y, z, a, b);
+    if (A.force) collide_pair<true>(a, b, A.P);
+    else collide_pair<false>(a, b, A.P);
+    store_pair(A.fout, A.P, (size_t)z * A.P.nx * A.P.ny + (size_t)y * A.P.nx + x0, a, b);
+  }
+}
+
 // The lattice pass of a step (K1, body force only): blocks take chunks of one node group per
 // thread until none is left. The next chunk's number is fetched while the current one is worked on.
 template <typename real, typename S>
@@ -127,22 +161,7 @@ __device__ __forceinline__ void lattice_chunks(const StreamArgs<real, S> &A, int
     if (c >= chunks) break;
     if (threadIdx.x == 0) s_chunk[(k & 1) ^ 1] = atomicAdd(next, 1);
     const int g = c * nt + threadIdx.x;
-    if (g < A.G.n) {
-      int gx, y, z;
-      A.G.at(g, gx, y, z);
-      z += A.z0;
-      if constexpr (sizeof(S) == 2) {
-        if (A.force) quad_nodes<S, false, true>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
-        else quad_nodes<S, false, false>(A.fin, A.fout, A.P, 4 * gx, y, z, Nothing());
-      } else {
-        const int x0 = 2 * gx;
-        real a[Q], b[Q];
-        load_pair<real, S, false>(A.fin, A.P, x0, y, z, a, b);
-        if (A.force) collide_pair<true>(a, b, A.P);
-        else collide_pair<false>(a, b, A.P);
-        store_pair(A.fout, A.P, (size_t)z * A.P.nx * A.P.ny + (size_t)y * A.P.nx + x0, a, b);
-      }
-    }
+    if (g < A.G.n) lattice_group(A, g);
     __syncthreads();
   }
 }
@@ -186,8 +205,12 @@ __device__ __forceinline__ void fused_steps(const FusedArgs<real, S> &P, SourceS
     if (chain) {
       shell_body<real, S>(A.shell, chain_first, chain_stride);
       CHAIN_BARRIER();
-      for (int g0 = chain_first; g0 - lane < 4 * A.interp.nv; g0 += chain_stride)
-        interp_body(A.interp, g0);
+      if (4 * A.interp.nv <= chain_stride) {
+        interp_body<1>(A.interp, chain_first, 0);
+      } else {  // two vertices at a time per lane
+        for (int g0 = chain_first; g0 - lane < 4 * A.interp.nv; g0 += 2 * chain_stride)
+          interp_body<2>(A.interp, g0, chain_stride >> 2);
+      }
       if (s + 1 < P.nsteps) CHAIN_BARRIER();
     }
   }
@@ -200,23 +223,57 @@ __global__ void __launch_bounds__(FusedShape<real>::threads, FusedShape<real>::p
     fused_step_kernel(const __grid_constant__ FusedArgs<real, S> P) {
   __shared__ SourceShared<real> sh[FusedShape<real>::threads / kSourceThreads];
   fused_steps(P, sh);
-  // the last block to leave clears the control words for the next launch
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(&P.ctl->left, 1u) == gridDim.x - 1) {
-      P.ctl->chain = 0;
-      P.ctl->all = 0;
-      P.ctl->abort = 0;
-      P.ctl->next[0] = P.ctl->next[1] = 0;
-      __threadfence();
-      P.ctl->left = 0;
-    }
+  leave_grid(P.ctl);
+}
+
+// Steps of a lattice without a mesh: the lattice pass alone, a barrier between two steps. Groups
+// go to the threads of the grid in memory order, round after round.
+template <typename real, typename S>
+struct LatticeSteps {
+  StreamArgs<real, S> step[2];
+  FusedControl *ctl;
+  int *health;
+  int nsteps;
+};
+// Blocks of 128 threads per SM: what the pass's registers allow.
+template <typename real, typename S>
+struct LatticeShape {
+  static constexpr int per_sm = sizeof(S) == 2 ? 4 : sizeof(real) == 4 ? 7 : 3;
+};
+
+template <typename real, typename S>
+__global__ void __launch_bounds__(128, (LatticeShape<real, S>::per_sm))
+    lattice_steps_kernel(const __grid_constant__ LatticeSteps<real, S> P) {
+  unsigned n_all = 0;
+  for (int s = 0; s < P.nsteps; s++) {
+    const StreamArgs<real, S> &A = P.step[s & 1];
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < A.G.n; g += gridDim.x * blockDim.x)
+      lattice_group(A, g);
+    if (s + 1 < P.nsteps && !grid_barrier(&P.ctl->all, n_all += gridDim.x, P.ctl, P.health)) break;
   }
+  leave_grid(P.ctl);
+}
+
+template <typename real, typename S>
+cudaError_t launch_lattice_steps_t(Ctx &c, int nsteps, cudaStream_t st) {
+  LatticeSteps<real, S> a;
+  for (int p = 0; p < 2; p++) {
+    c.cur ^= p;
+    a.step[p] = stream_args<real, S>(c);
+    c.cur ^= p;
+  }
+  a.ctl = (FusedControl *)c.fused_ctl;
+  a.health = c.counters + 3;
+  a.nsteps = nsteps;
+  const int need = (a.step[0].G.n + 127) / 128, room = LatticeShape<real, S>::per_sm * c.sm_count;
+  void *params[] = {&a};
+  return cudaLaunchCooperativeKernel((const void *)lattice_steps_kernel<real, S>,
+                                     dim3(need < room ? need : room), dim3(128), params, 0, st);
 }
 
 template <typename real, typename S>
 cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
+  if (c.nv == 0) return launch_lattice_steps_t<real, S>(c, nsteps, st);
   FusedArgs<real, S> a;
   const int cur = c.cur, map = c.map;
   for (int p = 0; p < 2; p++) {

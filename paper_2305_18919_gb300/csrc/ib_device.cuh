@@ -122,6 +122,9 @@ struct TileMap {
   int *tile_slot, *slot_tile, *nslots, *slot_count, *out_src, *health;
 };
 
+// Vertices that one warp marks.
+constexpr int kMarkVertices = 8;
+
 // Mark the tiles of the stencils of eight vertices by one warp (called together): lane l takes
 // vertex v0 + l / 4 and, l % 4 = k < 3, its axis k; each lane then claims two of the vertex's (up
 // to 8) tiles. The first claimant of a tile takes a new slot; a plain read first keeps the many
@@ -238,9 +241,11 @@ struct FaceThreads {
 };
 constexpr int kVertexThreads = 64;
 
-// Warps of K3a: one per eight vertices to mark, then one per 32 faces.
+// Warps of K3a: one per kMarkVertices vertices to mark, then one per 32 faces.
 template <typename real>
-__device__ __forceinline__ int mark_warps(const FaceArgs<real> &A) { return A.reset ? (A.nv + 7) / 8 : 0; }
+__device__ __forceinline__ int mark_warps(const FaceArgs<real> &A) {
+  return A.reset ? (A.nv + kMarkVertices - 1) / kMarkVertices : 0;
+}
 
 // K3a for the warps first / 32, first / 32 + stride / 32, ... (`first`: of this thread; a warp's 32
 // threads hold 32 consecutive ones and call it together).
@@ -259,7 +264,7 @@ __device__ __forceinline__ void face_body(const FaceArgs<real> &A, int first, in
   const int marks = mark_warps(A), warps = marks + (nf + 31) / 32;
   for (int w = first >> 5; w < warps; w += stride >> 5) {
   if (w < marks) {
-    mark_vertices(A.q, A.nv, 8 * w, D, A.map);
+    mark_vertices(A.q, A.nv, kMarkVertices * w, D, A.map);
     continue;
   }
   const int j = 32 * (w - marks) + lane;
@@ -909,30 +914,17 @@ struct InterpArgs {
   int *health;
 };
 
-// K2 for lane `gid` (vertex gid / 4, plane gid % 4); a warp's 32 lanes are consecutive and call it
-// together.
+// K2's sum over plane dz of vertex v's stencil.
 template <typename real>
-__device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) {
-  const int nv = A.nv;
+__device__ __forceinline__ void interp_plane(const InterpArgs<real> &A, int v, int dz,
+                                             VertexSum<real> &acc) {
   const StencilRec<real> *IBLB_RO stencil = A.stencil;
   const int *IBLB_RO tile_slot = A.tile_slot;
   const Vec4<real> *IBLB_RO Uslot = A.Uslot;
-  double *IBLB_RO q = A.q;
-  double *IBLB_RO qdot = A.qdot;
-  const double *IBLB_RO xref = A.xref;
-  Vec4<real> *IBLB_RO disp = A.disp;
-  const double3 ub = A.ub, ut = A.ut;
-  const Dims D = A.D;
   int *IBLB_RO health = A.health;
-  const int v = gid >> 2;
-  const int dz = gid & 3;
-  const bool valid = v < nv;
-  // lane k < 3 of the vertex updates coordinate k: its position is read ahead
-  const bool axis = valid && dz < 3;
-  const double qk = axis ? q[3 * (size_t)v + dz] : 0.0;
-  const double xk = axis ? xref[3 * (size_t)v + dz] : 0.0;
-  VertexSum<real> acc;
-  if (valid) {
+  const double3 ub = A.ub, ut = A.ut;
+  const Dims &D = A.D;
+  {
     const StencilRec<real> rec = stencil[v];
     int Z = rec.base[2] + dz;
     if (!D.has_walls) Z = Z >= D.nz ? Z - D.nz : Z;
@@ -992,18 +984,47 @@ __device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid) 
       }
     }
   }
+}
+
+// K2 for N vertices per four lanes: lane `gid` takes plane gid % 4 of the vertices gid / 4,
+// gid / 4 + step, ... A warp's 32 lanes are consecutive and call it together. With N = 2 the two
+// vertices' loads are in flight together, for a grid that has fewer lanes than the mesh asks for.
+template <int N, typename real>
+__device__ __forceinline__ void interp_body(const InterpArgs<real> &A, int gid, int step) {
+  const Dims &D = A.D;
+  const int dz = gid & 3;
+  // lane k < 3 of a vertex updates coordinate k: its position is read ahead
+  double qk[N], xk[N];
+  VertexSum<real> acc[N];
+#pragma unroll
+  for (int m = 0; m < N; m++) {
+    const int v = (gid >> 2) + m * step;
+    const bool axis = v < A.nv && dz < 3;
+    qk[m] = axis ? A.q[3 * (size_t)v + dz] : 0.0;
+    xk[m] = axis ? A.xref[3 * (size_t)v + dz] : 0.0;
+  }
+#pragma unroll
+  for (int m = 0; m < N; m++) {
+    const int v = (gid >> 2) + m * step;
+    if (v < A.nv) interp_plane(A, v, dz, acc[m]);
+  }
   // sum of the 4 planes (fixed butterfly order)
-  for (int o = 2; o > 0; o >>= 1) acc.add_lanes(o);
-  if (axis) {
-    const double qd = acc.value(dz);
-    const double pn = qk + qd;
-    qdot[3 * (size_t)v + dz] = qd;
-    q[3 * (size_t)v + dz] = pn;
+  for (int o = 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int m = 0; m < N; m++) acc[m].add_lanes(o);
+#pragma unroll
+  for (int m = 0; m < N; m++) {
+    const int v = (gid >> 2) + m * step;
+    if (v >= A.nv || dz >= 3) continue;
+    const double qd = acc[m].value(dz);
+    const double pn = qk[m] + qd;
+    A.qdot[3 * (size_t)v + dz] = qd;
+    A.q[3 * (size_t)v + dz] = pn;
     int h = 0;
     if (!(fabs(qd) < 0.1)) h |= (qd == qd) ? H_FAST : H_NAN;
     if (dz == 2 && D.has_walls && (pn - D.zb < 0.05 || D.zt - pn < 0.05)) h |= H_WALL;
-    if (h) atomicOr(health, h);
-    reinterpret_cast<real *>(disp + v)[dz] = (real)(pn - xk);
+    if (h) atomicOr(A.health, h);
+    reinterpret_cast<real *>(A.disp + v)[dz] = (real)(pn - xk[m]);
   }
 }
 
@@ -1012,14 +1033,14 @@ constexpr int kInterpThreads = 128;
 
 template <typename real>
 __global__ void __launch_bounds__(kInterpThreads) interp_kernel(const InterpArgs<real> A) {
-  interp_body(A, blockIdx.x * blockDim.x + threadIdx.x);
+  interp_body<1>(A, blockIdx.x * blockDim.x + threadIdx.x, 0);
 }
 
 template <typename real>
 __global__ void __launch_bounds__(kInterpThreads) interp_kernel_multi(
     const InterpArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
-  interp_body(all[m.inst], m.block * blockDim.x + threadIdx.x);
+  interp_body<1>(all[m.inst], m.block * blockDim.x + threadIdx.x, 0);
 }
 
 // Displacement from the reference shape, after setting vertices; one thread per coordinate.
@@ -1120,7 +1141,7 @@ FaceArgs<real> face_args(const Ctx &c, int reset) {
 }
 template <typename real>
 int face_blocks(const Ctx &c, int reset) {
-  const int warps = (c.nf + 31) / 32 + (reset ? (c.nv + 7) / 8 : 0);
+  const int warps = (c.nf + 31) / 32 + (reset ? (c.nv + kMarkVertices - 1) / kMarkVertices : 0);
   return (32 * warps + FaceThreads<real>::value - 1) / FaceThreads<real>::value;
 }
 

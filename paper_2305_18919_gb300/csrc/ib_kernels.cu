@@ -7,7 +7,7 @@ namespace {
 
 // Standalone marking of the current positions (a read of the spread field between steps).
 __global__ void mark_kernel(int nv, const double *IBLB_RO q, Dims D, TileMap M) {
-  mark_vertices(q, nv, 8 * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5), D, M);
+  mark_vertices(q, nv, kMarkVertices * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5), D, M);
 }
 
 __global__ void clear_counts_kernel(const int *__restrict__ nslots, int *__restrict__ slot_count,
@@ -158,7 +158,7 @@ cudaError_t launch_interpolate_advect(Ctx &c, cudaStream_t s) {
 }
 
 cudaError_t launch_mark(Ctx &c) {
-  const int warps = (c.nv + 7) / 8;
+  const int warps = (c.nv + kMarkVertices - 1) / kMarkVertices;
   mark_kernel<<<(32 * warps + 127) / 128, 128, 0, c.stream>>>(c.nv, c.q, dims_of(c), tile_map(c));
   return cudaGetLastError();
 }

@@ -205,7 +205,7 @@ struct Ctx {
   int health_every = 1000;  // iblb_step reads the health word every this many steps (0: at its end)
   int health_pending = 0;   // steps queued by iblb_step_async whose health word is unread
   int *health_host = nullptr;  // pinned: the health word read with a call's own transfers
-  int fused = 0;               // small lattice: iblb_step's steps run as one kernel (fused.cu)
+  int fused = 0;               // iblb_step's steps may run as one kernel (fused.cu)
   void *fused_ctl = nullptr;   // control words of the fused kernel (kFusedControlBytes, zeroed)
   uint64_t config_gen = 0;  // bumped by every call that changes what a queued step launches
   std::string err;

@@ -805,8 +805,9 @@ cudaError_t launch_staged(Ctx &c, const StageGeom &G, size_t smem, int nc, cudaS
   if (32 * (nc + 1) > staged_threads(NPT)) nc = staged_threads(NPT) / 32 - 1;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // one block per SM of the lattice partition, each working through its share of the units
-  const int sms = c.green[0] ? c.lat_sms : c.sm_count;
+  // one block per SM of the lattice partition (of all SMs without a mesh), each working through
+  // its share of the units
+  const int sms = c.green[0] && c.nv ? c.lat_sms : c.sm_count;
   const int grid = G.nunits < sms ? G.nunits : sms;
   kern<<<grid, 32 * (nc + 1), smem, st>>>((const S *)c.f[c.cur], (S *)c.f[c.cur ^ 1],
                                           lat_params<float>(c), G, c.counters + 3);
