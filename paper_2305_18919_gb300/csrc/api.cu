@@ -143,14 +143,15 @@ bool green_api(GreenApi &g) {
 // Whether the steps of a default context run as one kernel (fused.cu), by the bytes that its
 // stream-collide pass reads and writes. With a mesh: below 1 GiB (us per step, fused against the
 // separate kernels: 24^3 FP32 28 / 46, 64^3 35 / 52, 128x128x96 65 / 69, 128^3 FP32 77 / 78 and
-// FP16 60 / 72, 192^3 FP32 189 / 187). Without one, where only the gap between two launches of
-// the pass is saved and the pass alone runs at a higher occupancy: below 30 MB in FP32 and 80 MB in
-// 16 bits, never in FP64 (32^3 FP32 3.2 / 4.3, FP16 3.3 / 6.3; 64^3 FP32 9.3 / 8.4, FP16 5.3 / 8.4;
-// 128^3 FP16 30.6 / 30.1; 48^3 FP64 37.5 / 35.1).
+// FP16 60 / 72, 192^3 FP32 189 / 187). Without one, where the separate passes are launched early
+// (except the staged one): below 20 MB in FP32 and 8 MB in 16 bits, 80 MB where the staged pass
+// would be taken, never in FP64 (32^3 FP32 3.2 / 3.4, 48^3 4.8 / 6.0, 64^3 9.3 / 6.5; FP16 staged
+// 64^3 5.3 / 8.4, 128^3 30.6 / 29.8, not staged 84x68x64 7.9 / 5.5; FP64 48^3 37.5 / 32.4).
 bool fused_by_size(const Ctx &c) {
   const size_t pass = (size_t)2 * iblb::Q * c.ncell * c.pop_size;
   if (c.nv) return pass < ((size_t)1 << 30);
-  return c.pop_size == 4 ? pass < 30000000 : c.pop_size == 2 && pass < 80000000;
+  if (c.pop_size == 2) return pass < (iblb::stream_collide_staged(c) ? 80000000u : 8000000u);
+  return c.pop_size == 4 && pass < 20000000;
 }
 
 // SMs of the interface partition that the lattice partition may use as well: the interface chain

@@ -228,6 +228,10 @@ int launch_kernel(iblb_batch *b, int lane, int p, int ki, cudaStream_t s) {
     m.n = (int)t.start.size() - 1;
     if (m.n == 0) continue;
     m.blocks = t.start.back();
+    // one lane's chain is a row of short kernels: each is launched early (12 boxes of 32 to 64 nodes
+    // an edge, FP16: 77 us per step against 86). Lanes lose by it (96 boxes 1.175 ms against 1.202:
+    // the waiting blocks take the other lanes' room), and FP64 (493 us against 504).
+    m.early = b->lanes.size() == 1 && !b->part.green[0] && b->groups[g].precision != IBLB_FP64;
     m.args = (const unsigned char *)b->arena + t.args_off;
     m.start = (const int *)((const unsigned char *)b->arena + t.start_off);
     const MultiKernel k = kKernels[ki];
@@ -246,17 +250,19 @@ int enqueue_batched_step(iblb_batch *b, int p) {
     Lane &n = b->lanes[l];
     for (int ki = 0; ki < 4; ki++)  // K3a, K3b, K4a, K4b
       if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
-    BATCH_TRY(b, cudaEventRecord(n.ev_force, n.ib));
     // Without a partition the lattice pass waits for the step's force and takes it in (K1 and K1t
     // in one: K1t's scattered rows are a sixth of the step's traffic; 96 boxes 1.253 ms per step
-    // against 1.310). On a partition the pass runs beside the chain instead, then K1t.
-    const bool beside = b->part.green[0] != nullptr;
-    if (beside)
+    // against 1.310), all on one stream. On a partition the pass runs beside the chain, then K1t.
+    if (b->part.green[0]) {
+      BATCH_TRY(b, cudaEventRecord(n.ev_force, n.ib));
       if (int rc = launch_kernel(b, (int)l, p, 4, n.ls)) return rc;  // K1
-    BATCH_TRY(b, cudaStreamWaitEvent(n.ls, n.ev_force, 0));
-    if (int rc = launch_kernel(b, (int)l, p, beside ? 5 : 8, n.ls)) return rc;  // K1t, or both
-    BATCH_TRY(b, cudaEventRecord(n.ev_coll, n.ls));
-    BATCH_TRY(b, cudaStreamWaitEvent(n.ib, n.ev_coll, 0));
+      BATCH_TRY(b, cudaStreamWaitEvent(n.ls, n.ev_force, 0));
+      if (int rc = launch_kernel(b, (int)l, p, 5, n.ls)) return rc;  // K1t
+      BATCH_TRY(b, cudaEventRecord(n.ev_coll, n.ls));
+      BATCH_TRY(b, cudaStreamWaitEvent(n.ib, n.ev_coll, 0));
+    } else if (int rc = launch_kernel(b, (int)l, p, 8, n.ib)) {  // both
+      return rc;
+    }
     for (int ki = 6; ki < 8; ki++)  // K1b, K2
       if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
   }

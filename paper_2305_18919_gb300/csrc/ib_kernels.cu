@@ -80,29 +80,23 @@ template <typename real>
 cudaError_t ib_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStream_t s) {
   switch (k) {
     case MK_FACE:
-      face_kernel_multi<real><<<m.blocks, FaceThreads<real>::value, 0, s>>>(
-          (const FaceArgs<real> *)m.args, m.start, m.n);
-      break;
+      return launch_after(m.early, face_kernel_multi<real>, m.blocks, FaceThreads<real>::value, s,
+                          (const FaceArgs<real> *)m.args, m.start, m.n);
     case MK_VERTEX:
-      vertex_kernel_multi<real><<<m.blocks, kVertexThreads, 0, s>>>(
-          (const VertexArgs<real> *)m.args, m.start, m.n);
-      break;
+      return launch_after(m.early, vertex_kernel_multi<real>, m.blocks, kVertexThreads, s,
+                          (const VertexArgs<real> *)m.args, m.start, m.n);
     case MK_SOURCE:
-      spread_source_kernel_multi<real><<<m.blocks, kSourceThreads, 0, s>>>(
-          (const SourceArgs<real> *)m.args, m.start, m.n);
-      break;
+      return launch_after(m.early, spread_source_kernel_multi<real>, m.blocks, kSourceThreads, s,
+                          (const SourceArgs<real> *)m.args, m.start, m.n);
     case MK_GATHER:
-      spread_gather_kernel_multi<real><<<m.blocks, TILE_CELLS, 0, s>>>(
-          (const GatherArgs<real> *)m.args, m.start, m.n);
-      break;
+      return launch_after(m.early, spread_gather_kernel_multi<real>, m.blocks, TILE_CELLS, s,
+                          (const GatherArgs<real> *)m.args, m.start, m.n);
     case MK_INTERP:
-      interp_kernel_multi<real><<<m.blocks, kInterpThreads, 0, s>>>(
-          (const InterpArgs<real> *)m.args, m.start, m.n);
-      break;
+      return launch_after(m.early, interp_kernel_multi<real>, m.blocks, kInterpThreads, s,
+                          (const InterpArgs<real> *)m.args, m.start, m.n);
     default:
       return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename real>

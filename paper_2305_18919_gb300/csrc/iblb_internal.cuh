@@ -53,6 +53,27 @@ constexpr int kStageNodes16 = 4;
 // Default size of one population's copy in the staged pass (bytes): rows per unit follow.
 constexpr size_t kStageCopyBytes = 4096;
 
+// Programmatic dependent launch, for chains of kernels on one stream: a kernel lets its successor's
+// blocks onto the SMs at once, and the successor reads and writes nothing that a predecessor uses
+// before its own wait, which returns when every kernel before it is complete. Launched without the
+// attribute (`early` false), both are no-ops.
+__device__ __forceinline__ void pdl_let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_after(bool early, void (*kernel)(P...), dim3 grid, int block, cudaStream_t s,
+                         A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Batched launches: one grid over the blocks of many contexts. Instance i of a launch owns the
 // grid's blocks start[i] .. start[i + 1] - 1 (start[0] = 0, start[n] = the grid size).
 constexpr int kMultiMax = 256;  // instances per batched launch
@@ -81,8 +102,10 @@ __device__ __forceinline__ MultiBlock multi_block_of(const int *s_start, int n, 
 
 __device__ __forceinline__ MultiBlock multi_block(const int *__restrict__ start, int n) {
   __shared__ int s_start[kMultiMax + 1];
+  pdl_let_next();
   for (int k = threadIdx.x; k <= n; k += blockDim.x) s_start[k] = start[k];
   __syncthreads();
+  pdl_wait();  // (the block table is no predecessor's output)
   const int b = blockIdx.x;
   int lo = 0, hi = n;  // the largest lo with start[lo] <= b
   while (hi - lo > 1) {
@@ -289,6 +312,7 @@ struct MultiLaunch {
   const void *args = nullptr;  // device: the n records, one per context
   const int *start = nullptr;  // device: n + 1 block offsets
   int n = 0, blocks = 0;
+  bool early = false;          // programmatic launch after the kernel before it on the stream
 };
 // Append context c's record for kernel k to `bytes` and return its number of blocks (at least
 // 1), or -1 where k does not belong to this file.
