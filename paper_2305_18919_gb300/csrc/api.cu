@@ -74,6 +74,16 @@ int positions_changed(Ctx &c) {
   return 0;
 }
 
+// Whether the stream is being captured into a graph, whose replays see none of the host's decisions.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {  // the legacy stream beside another's capture
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 int read_health(Ctx &c, int *h) {
   CUDA_TRY(c, cudaMemcpyAsync(h, c.counters + 3, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
@@ -83,7 +93,7 @@ int read_health(Ctx &c, int *h) {
 // An unstable run reports that first: its garbage positions can also leave tiles unmarked.
 int health_error(Ctx &c, int h) {
   if (h & iblb::H_TIMEOUT)
-    return fail(c, IBLB_ETIMEOUT, "stream-collide pipeline: a bounded wait for staged data gave up");
+    return fail(c, IBLB_ETIMEOUT, "a bounded wait inside a kernel gave up (staged copies or the step's grid barrier)");
   const int unstable = iblb::H_NAN | iblb::H_FAST | iblb::H_WALL | iblb::H_VOLUME;
   if (!(h & unstable))
     return fail(c, IBLB_ECAPACITY, "active-tile table capacity exceeded");
@@ -590,8 +600,10 @@ int iblb_step_async(iblb_ctx *h, int32_t nsteps) {
   Ctx &c = h->c;
   if (nsteps < 0) return fail(c, IBLB_EINVAL, "nsteps < 0");
   if (nsteps == 0) return IBLB_OK;
-  // a failure still unread stays in the health word; otherwise it starts clear
-  if (!c.health_pending) CUDA_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
+  // a failure still unread stays in the health word; otherwise it starts clear (as it is where the
+  // last steps' word was read and none has run since: a loop that exchanges data every step)
+  if (!c.health_pending && (!c.health_clear || capturing(c.stream)))
+    CUDA_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
   if (int rc = iblb::enqueue_steps(c, nsteps)) return rc;
   c.health_pending = 1;
   return IBLB_OK;
@@ -620,9 +632,10 @@ namespace {
 
 // Whether the context's steps after the first run as one kernel: of a size for it, and nothing
 // asked for that only the separate kernels have (an SM partition, their timing, a choice of the
-// stream-collide kernel or of its waits).
+// stream-collide kernel or of its waits), nor a capture, which keeps to plain launches.
 bool takes_fused(const Ctx &c) {
-  return c.fused && fused_by_size(c) && !c.profiling && c.k1_kind == IBLB_STREAM_COLLIDE_AUTO && !c.stage_wait_set;
+  return c.fused && fused_by_size(c) && !c.profiling && c.k1_kind == IBLB_STREAM_COLLIDE_AUTO &&
+         !c.stage_wait_set && !capturing(c.stream);
 }
 
 // Steps of one fused launch: the GPU is the launch's own while it runs, so work of other streams
@@ -660,6 +673,7 @@ int enqueue_fused(Ctx &c, int nsteps, int *left) {
 }  // namespace
 
 int enqueue_steps(Ctx &c, int nsteps) {
+  c.health_clear = 0;
   if (takes_fused(c) && nsteps > (c.fresh ? 1 : 0)) {
     if (c.fresh) {  // the in-place first step by the separate kernels
       if (int rc = enqueue_steps(c, 1)) return rc;
@@ -749,6 +763,7 @@ int queue_health(Ctx &c) {
 int pending_health(Ctx &c) {
   if (!c.health_pending) return IBLB_OK;
   c.health_pending = 0;
+  c.health_clear = *c.health_host == 0;
   return health_status(c, *c.health_host);
 }
 
@@ -837,7 +852,9 @@ int iblb_read_forces(iblb_ctx *h, int32_t mesh_id, double *phi) {
   CUDA_TRY(c, iblb::launch_phi_to_double(c, c.dscratch));
   CUDA_TRY(c, cudaMemcpyAsync(phi, c.dscratch, (size_t)3 * c.nv * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
-  return iblb::pending_health(c);
+  const int rc = iblb::pending_health(c);
+  c.health_clear = 0;  // the force pass above checks the volume, after that word was read
+  return rc;
 }
 
 int iblb_read_force_field(iblb_ctx *h, double *F) {

@@ -493,6 +493,7 @@ int iblb_batch_step(iblb_batch *b, int32_t nsteps) {
   int first = IBLB_OK;
   for (size_t i = 0; i < n; i++) {
     b->inst[i]->c.health_pending = 0;
+    b->inst[i]->c.health_clear = 0;
     b->status[i] = iblb::health_status(b->inst[i]->c, b->health[i]);
     if (b->status[i] != IBLB_OK && first == IBLB_OK) {
       first = b->status[i];

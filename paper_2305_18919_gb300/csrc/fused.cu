@@ -87,8 +87,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *ctr, unsigned target, Fus
   __shared__ int s_go;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1u);
+    // (release and acquire at the GPU's scope, cumulative over the block by its barriers: no full
+    // fences, each a microsecond's part of a barrier that a step passes seven times)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
     int go = 1;
     if ((int)(ld_acquire(ctr) - target) < 0) {
       const unsigned long long t0 = now_ns();
@@ -105,7 +106,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *ctr, unsigned target, Fus
         }
       }
     }
-    __threadfence();
     s_go = go;
   }
   __syncthreads();
@@ -188,7 +188,7 @@ __device__ __forceinline__ void fused_steps(const FusedArgs<real, S> &P, SourceS
       face_body(A.face, chain_first, chain_stride);
       CHAIN_BARRIER();
       if ((int)blockIdx.x == nchain - 1 && tid >= nt - 32) volume_task(A.vertex);
-      for (int i = chain_first; i < A.vertex.nv; i += chain_stride) vertex_body(A.vertex, i);
+      for (int g = chain_first; g - lane < 4 * A.vertex.nv; g += chain_stride) vertex_body(A.vertex, g);
       CHAIN_BARRIER();
       const int g = tid / kSourceThreads, ng = nt / kSourceThreads;
       spread_source_body(A.source, sh[g], blockIdx.x + g * nchain, ng * nchain, g,

@@ -233,13 +233,12 @@ struct FaceArgs {
 
 // Threads per block of K3a and K3b: few, so that a mesh of some thousand faces and vertices
 // spreads over all SMs of the chain (each SM's FP64 unit and each warp's chain of loads, not
-// memory, set their time). K3b with its loads a vector each, 10242 vertices on 64 SMs: 9.3 us
-// against 10.8 with 256-thread blocks; 40962 on 24 SMs: 30 against 40; K3a there 19 against 27.
+// memory, set their time): K3a of 81920 faces on 24 SMs 19 us against 27 with 256-thread blocks.
 template <typename real>
 struct FaceThreads {
   static constexpr int value = sizeof(real) == 4 ? 128 : 64;
 };
-constexpr int kVertexThreads = 64;
+constexpr int kVertexThreads = 128;
 
 // Warps of K3a: one per kMarkVertices vertices to mark, then one per 32 faces.
 template <typename real>
@@ -446,54 +445,60 @@ __device__ __forceinline__ void volume_task(const VertexArgs<real> &A) {
   }
 }
 
-// K3b for vertex i.
+// K3b for lane `gid`: vertex gid / 4; lane k = gid % 4 < 3 gathers component k of its forces and
+// finds the stencil along axis k, lane 0 then bins the vertex. A third of the serial FP64 work and
+// of the loads per lane of one lane per vertex, whose chain set the pass's time where the vertices
+// are few (fused step, with the lighter grid barrier, against one lane per vertex: 32^3 FP64, 642
+// vertices, 47.6 us against 53; 24^3 FP32 23 against 28; 64^3, 2562 vertices, 31 against 35); with
+// many the two are equal (128x128x96, 10242 vertices, 64.9 against 65). A warp's 32 lanes are
+// consecutive and call it together.
 template <typename real>
-__device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int i) {
+__device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int gid) {
   const int *IBLB_RO vf_start = A.vf_start;
   const int *IBLB_RO vf_list = A.vf_list;
-  const Vec4<real> *IBLB_RO fcontrib = A.fcontrib;
-  const Vec4<real> *IBLB_RO fnorm = A.fnorm;
+  const real *IBLB_RO fcontrib = reinterpret_cast<const real *>(A.fcontrib);  // [3 nf][4]
+  const real *IBLB_RO fnorm = reinterpret_cast<const real *>(A.fnorm);        // [nf][4]
   const double *IBLB_RO q = A.q;
-  const int bin = A.bin;
   const Dims D = A.D;
-  const int e0 = vf_start[i], e1 = vf_start[i + 1];
-  double p[3] = {0, 0, 0};
-  if (bin)
-    for (int k = 0; k < 3; k++) p[k] = q[3 * (size_t)i + k];
-  real F[3] = {0, 0, 0}, g[3] = {0, 0, 0};
-  for (int eb = e0; eb < e1; eb += GATHER_UNROLL) {
-    int fcs[GATHER_UNROLL];
+  const int i = gid >> 2, k = gid & 3;
+  const bool mine = i < A.nv && k < 3;
+  int base = 0;
+  if (mine) {
+    const int e0 = vf_start[i], e1 = vf_start[i + 1];
+    const double p = A.bin ? q[3 * (size_t)i + k] : 0.0;
+    real F = 0, g = 0;
+    for (int eb = e0; eb < e1; eb += GATHER_UNROLL) {
+      int fcs[GATHER_UNROLL];
 #pragma unroll
-    for (int u = 0; u < GATHER_UNROLL; u++) fcs[u] = eb + u < e1 ? vf_list[eb + u] : -1;
+      for (int u = 0; u < GATHER_UNROLL; u++) fcs[u] = eb + u < e1 ? vf_list[eb + u] : -1;
 #pragma unroll
-    for (int u = 0; u < GATHER_UNROLL; u++) {  // (no branch between the loads: all in flight)
-      const int fc = max(fcs[u], 0);              // face * 3 + corner
-      Vec4<real> f = fcontrib[fc], n = fnorm[fc / 3];
-      if (fcs[u] < 0) f = n = Vec4<real>{0, 0, 0, 0};
-      F[0] += f.x;
-      F[1] += f.y;
-      F[2] += f.z;
-      g[0] += n.x;
-      g[1] += n.y;
-      g[2] += n.z;
+      for (int u = 0; u < GATHER_UNROLL; u++) {  // (no branch between the loads: all in flight)
+        const int fc = max(fcs[u], 0);            // face * 3 + corner
+        const real f = fcontrib[4 * (size_t)fc + k], n = fnorm[4 * (size_t)(fc / 3) + k];
+        F += fcs[u] < 0 ? real(0) : f;
+        g += fcs[u] < 0 ? real(0) : n;
+      }
+    }
+    reinterpret_cast<real *>(A.phi + i)[k] = F;
+    reinterpret_cast<real *>(A.gvol + i)[k] = g;
+    if (A.bin) {
+      double r;
+      const int n = k == 0 ? D.nx : k == 1 ? D.ny : D.nz;
+      const double inv = k == 0 ? D.inx : k == 1 ? D.iny : D.inz;
+      base = stencil_base(p, n, inv, k < 2 || !D.has_walls, r);
+      real w[4];
+      peskin_weights<real>((real)r, w);
+      StencilRec<real> &rec = A.stencil[i];
+      rec.base[k] = base;
+#pragma unroll
+      for (int d = 0; d < 4; d++) rec.w[k][d] = w[d];
     }
   }
-  Vec4<real> pv, gv;
-  pv.x = F[0]; pv.y = F[1]; pv.z = F[2]; pv.w = real(0);
-  gv.x = g[0]; gv.y = g[1]; gv.z = g[2]; gv.w = real(0);
-  A.phi[i] = pv;
-  A.gvol[i] = gv;
-  if (!bin) return;
-  StencilRec<real> rec;
-  double r[3];
-  rec.base[0] = stencil_base(p[0], D.nx, D.inx, true, r[0]);
-  rec.base[1] = stencil_base(p[1], D.ny, D.iny, true, r[1]);
-  rec.base[2] = stencil_base(p[2], D.nz, D.inz, !D.has_walls, r[2]);
-  for (int k = 0; k < 3; k++) peskin_weights<real>((real)r[k], rec.w[k]);
-  rec.pad = 0;
-  A.stencil[i] = rec;
-  const int bz = min(max(rec.base[2], 0), D.nz - 1);
-  const int t = ((bz >> 2) * D.nty + (rec.base[1] >> 2)) * D.ntx + (rec.base[0] >> 2);
+  if (!A.bin) return;
+  const int by = __shfl_sync(0xffffffffu, base, 1, 4), bz_ = __shfl_sync(0xffffffffu, base, 2, 4);
+  if (!mine || k != 0) return;
+  const int bz = min(max(bz_, 0), D.nz - 1);
+  const int t = ((bz >> 2) * D.nty + (by >> 2)) * D.ntx + (base >> 2);
   const int s = A.tile_slot[t];
   if (s < 0) {
     atomicOr(A.health, H_CAPACITY);
@@ -511,15 +516,14 @@ __device__ __forceinline__ void vertex_body(const VertexArgs<real> &A, int i) {
   }
 }
 
-// Block `bid` of K3b: the first takes the scalars, the others a vertex per thread.
+// Block `bid` of K3b: the first takes the scalars, the others a vertex per four threads.
 template <typename real>
 __device__ __forceinline__ void vertex_block(const VertexArgs<real> &A, int bid) {
   if (bid == 0) {
     if (threadIdx.x < 32) volume_task(A);
     return;
   }
-  const int i = (bid - 1) * blockDim.x + threadIdx.x;
-  if (i < A.nv) vertex_body(A, i);
+  vertex_body(A, (bid - 1) * blockDim.x + threadIdx.x);
 }
 
 template <typename real>
@@ -836,9 +840,10 @@ __global__ void __launch_bounds__(64) spread_gather_kernel_multi(
 
 // K2: interpolation (Eq. 11) and the Euler update (Eq. 12); 4 lanes per vertex, lane dz
 // sums the 16 nodes of its z-plane of the stencil, the 4 planes are summed by shuffles; lane k
-// then adds the update to coordinate k of the double position. One lane per axis issues a third of the FP64 instructions of one lane per vertex (an FP64
-// instruction holds the SM's FP64 unit for 16 cycles however few lanes take part): 10242 vertices
-// on 64 SMs 12.8 us against 17.2, 40962 on 24 SMs 88 against 127, 96 wetting boxes 108 against 262.
+// then adds the update to coordinate k of the double position. One lane per axis issues a third of
+// the FP64 instructions of one lane per vertex (an FP64 instruction holds the SM's FP64 unit for 16
+// cycles however few lanes take part): 10242 vertices on 64 SMs 12.8 us against 17.2, 40962 on 24
+// SMs 88 against 127, 96 wetting boxes 108 against 262.
 // The delta-weight accumulation of a vertex is carried at double precision in every
 // precision (VertexSum): each stencil row's four products w_x u (one x row of a tile, in the
 // arithmetic type) is added to the vertex's sum with its weight w_y w_z, and the four planes'
@@ -1174,7 +1179,7 @@ VertexArgs<real> vertex_args(const Ctx &c, int bin) {
   return a;
 }
 // the first block takes the volume coefficient
-int vertex_blocks(const Ctx &c) { return (c.nv + kVertexThreads - 1) / kVertexThreads + 1; }
+int vertex_blocks(const Ctx &c) { return (int)((4L * c.nv + kVertexThreads - 1) / kVertexThreads) + 1; }
 
 template <typename real>
 SourceArgs<real> source_args(const Ctx &c) {

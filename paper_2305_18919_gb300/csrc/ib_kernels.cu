@@ -139,6 +139,7 @@ cudaError_t launch_face_forces(Ctx &c, int reset_other_map, cudaStream_t s) {
 // bin: 0 forces only; 1 forces + stencil + binning; 2 as 1 and also zero the other map's
 // tile counter (inside a step, after that map was cleared by the face kernel).
 cudaError_t launch_vertex_forces(Ctx &c, int bin, cudaStream_t s) {
+  c.health_clear = 0;  // (the volume check)
   return c.precision == IBLB_FP64 ? vertex_forces_t<double>(c, bin, s)
                                   : vertex_forces_t<float>(c, bin, s);
 }
@@ -152,6 +153,7 @@ cudaError_t launch_interpolate_advect(Ctx &c, cudaStream_t s) {
 }
 
 cudaError_t launch_mark(Ctx &c) {
+  c.health_clear = 0;
   const int warps = (c.nv + kMarkVertices - 1) / kMarkVertices;
   mark_kernel<<<(32 * warps + 127) / 128, 128, 0, c.stream>>>(c.nv, c.q, dims_of(c), tile_map(c));
   return cudaGetLastError();

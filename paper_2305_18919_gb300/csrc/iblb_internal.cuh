@@ -43,7 +43,8 @@ constexpr int BUCKET_CAP = 128;
 
 // Health word bits (read back by iblb_step).
 constexpr int H_NAN = 1, H_FAST = 2, H_WALL = 4, H_VOLUME = 8, H_CAPACITY = 16;
-// a bounded wait of the staged stream-collide pipeline gave up (the kernel returned early)
+// a bounded wait (staged stream-collide copies, the fused step's grid barrier) gave up: the kernel
+// returned early
 constexpr int H_TIMEOUT = 32;
 
 // Default shape of the staged stream-collide pass: stages per block, compute warps per block.
@@ -227,6 +228,7 @@ struct Ctx {
   int smem_optin = 0;       // shared memory a block may opt in to (bytes)
   int health_every = 1000;  // iblb_step reads the health word every this many steps (0: at its end)
   int health_pending = 0;   // steps queued by iblb_step_async whose health word is unread
+  int health_clear = 0;     // the health word is known to be 0 (read so, and nothing run since)
   int *health_host = nullptr;  // pinned: the health word read with a call's own transfers
   int fused = 0;               // iblb_step's steps may run as one kernel (fused.cu)
   void *fused_ctl = nullptr;   // control words of the fused kernel (kFusedControlBytes, zeroed)
