@@ -218,11 +218,22 @@ int build_tables(iblb_batch *b) {
   return 0;
 }
 
-// Queue kernel ki of the lane's groups (records of step parity p) on stream s.
-int launch_kernel(iblb_batch *b, int lane, int p, int ki, cudaStream_t s) {
+// Whether a group's lattice pass (K1, then K1t) runs on the lattice stream beside the interface
+// chain of the step: on a partition, and in FP64, where the FP64 units bound the pass and the chain
+// leaves them idle (12 boxes 391 us per step against 491). Otherwise the pass waits for the step's
+// force and takes it in (K1 and K1t in one: K1t's scattered rows are a sixth of the step's traffic;
+// 96 boxes 1.253 ms per step against 1.310), on the chain's own stream.
+bool beside(const iblb_batch *b, const Group &g) {
+  return b->part.green[0] != nullptr || g.precision == IBLB_FP64;
+}
+
+// Queue kernel ki of the lane's groups (records of step parity p) on stream s; which: 0 all of them,
+// 1 those whose lattice pass runs beside the chain, 2 the others.
+int launch_kernel(iblb_batch *b, int lane, int p, int ki, cudaStream_t s, int which = 0) {
   const size_t G = b->groups.size();
   for (size_t g = 0; g < G; g++) {
     if (b->groups[g].lane != lane) continue;
+    if (which && beside(b, b->groups[g]) != (which == 1)) continue;
     const Table &t = b->tabs[(p * G + g) * kNumKernels + ki];
     iblb::MultiLaunch m;
     m.n = (int)t.start.size() - 1;
@@ -250,19 +261,17 @@ int enqueue_batched_step(iblb_batch *b, int p) {
     Lane &n = b->lanes[l];
     for (int ki = 0; ki < 4; ki++)  // K3a, K3b, K4a, K4b
       if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
-    // Without a partition the lattice pass waits for the step's force and takes it in (K1 and K1t
-    // in one: K1t's scattered rows are a sixth of the step's traffic; 96 boxes 1.253 ms per step
-    // against 1.310), all on one stream. On a partition the pass runs beside the chain, then K1t.
-    if (b->part.green[0]) {
+    bool some = false;
+    for (const Group &g : b->groups) some = some || (g.lane == (int)l && beside(b, g));
+    if (some) {
       BATCH_TRY(b, cudaEventRecord(n.ev_force, n.ib));
-      if (int rc = launch_kernel(b, (int)l, p, 4, n.ls)) return rc;  // K1
+      if (int rc = launch_kernel(b, (int)l, p, 4, n.ls, 1)) return rc;  // K1
       BATCH_TRY(b, cudaStreamWaitEvent(n.ls, n.ev_force, 0));
-      if (int rc = launch_kernel(b, (int)l, p, 5, n.ls)) return rc;  // K1t
+      if (int rc = launch_kernel(b, (int)l, p, 5, n.ls, 1)) return rc;  // K1t
       BATCH_TRY(b, cudaEventRecord(n.ev_coll, n.ls));
-      BATCH_TRY(b, cudaStreamWaitEvent(n.ib, n.ev_coll, 0));
-    } else if (int rc = launch_kernel(b, (int)l, p, 8, n.ib)) {  // both
-      return rc;
     }
+    if (int rc = launch_kernel(b, (int)l, p, 8, n.ib, 2)) return rc;  // both
+    if (some) BATCH_TRY(b, cudaStreamWaitEvent(n.ib, n.ev_coll, 0));
     for (int ki = 6; ki < 8; ki++)  // K1b, K2
       if (int rc = launch_kernel(b, (int)l, p, ki, n.ib)) return rc;
   }
