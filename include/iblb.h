@@ -67,7 +67,9 @@ typedef struct {
                               storage; below that 64 (rounded to the device's partition
                               granularity); none with FP64 from 192 MiB up. < 0: no
                               partition (both share all SMs, interface stream at top priority).
-                              If the device or driver cannot partition, no partition is used. */
+                              If the device or driver cannot partition, no partition is used.
+                              With 0, a mesh and less than 1 GiB a step runs as one kernel on
+                              all SMs, and the partition serves the steps that cannot. */
   double tau;              /* BGK relaxation time, > 1/2 (viscosity (tau - 1/2)/3) */
   double rho0;             /* reference density (initial state and moving-wall term) */
   double wall_u_bottom[3]; /* wall velocity at z = 0.5 (tangential components only) */
@@ -118,7 +120,8 @@ int iblb_init_equilibrium(iblb_ctx *ctx, const double *rho, const double *u);
    synchronises to read the health word every `every` steps of iblb_set_health_interval (1000
    by default) and at its end, and returns IBLB_EUNSTABLE or IBLB_ECAPACITY if a check failed
    during the steps read so far (the steps done then stop at the end of that interval),
-   IBLB_ETIMEOUT if a bounded wait of the staged stream-collide pass gave up. */
+   IBLB_ETIMEOUT if a bounded wait inside a kernel gave up (the staged stream-collide pass; the
+   grid barriers of the kernel that runs all of a small lattice's step). */
 int iblb_step(iblb_ctx *ctx, int32_t nsteps);
 
 /* Steps between health-word reads in iblb_step: every >= 1, or 0 for one read at the end of
@@ -187,7 +190,8 @@ int64_t iblb_steps_done(const iblb_ctx *ctx);
 /* Profiling of the dominant kernel. When on, iblb_step() brackets every stream-collide launch
    with CUDA events on the context's stream. iblb_profile() synchronises and returns the summed
    stream-collide time in milliseconds, the number of stream-collide launches and the number of
-   kernel launches made by iblb_step() since profiling was switched on. */
+   kernel launches made by iblb_step() since profiling was switched on. A small lattice's steps,
+   which otherwise run as one kernel, then run as separate kernels (with the same results). */
 int iblb_set_profiling(iblb_ctx *ctx, int32_t on);
 int iblb_profile(iblb_ctx *ctx, double *k1_ms, int64_t *k1_launches, int64_t *kernel_launches);
 
@@ -231,7 +235,8 @@ int iblb_mesh_volume_noalloc(const double *q_dev, const int32_t *faces_dev, int3
 
    iblb_batch_step advances every instance by nsteps coupled steps (the iblb_step sequence).
    Each kernel of a step is one launch over all instances of a precision (up to 256 per
-   launch), whose blocks read their instance's arguments from tables the batch builds at its
+   launch; ensembles of 4 Mi nodes and more in three groups that run beside one another), whose
+   blocks read their instance's arguments from tables the batch builds at its
    first use and again after any instance was reconfigured (mesh, interface parameters,
    initial state, kernel choice) or stepped alone by an odd count; steps run in pairs, and a
    freshly initialised instance takes its first step, and an odd last step is taken, through
@@ -274,7 +279,8 @@ int iblb_batch_status(const iblb_batch *batch, int32_t *status);
    the transposed step is applied state by state. The context is returned to the end of the run;
    the recording stays valid for further calls with other dJdq.
 
-   iblb_adjoint_release frees the recording and the work arrays (iblb_destroy also does).
+   iblb_adjoint_release frees the recording and the work arrays (iblb_destroy also does); until
+   then a further recording uses the arrays of the last one that have its size.
    Errors: IBLB_EINVAL (16-bit storage, no mesh, nothing recorded, nsteps or every < 1), the health
    errors of iblb_step during the record or the recomputation, IBLB_ENOMEM, IBLB_ECUDA. */
 int iblb_adjoint_record(iblb_ctx *ctx, int32_t nsteps, int32_t every);
@@ -317,7 +323,8 @@ int iblb_set_stage_wait_limit(iblb_ctx *ctx, int64_t ns);
 
 /* 1 if the stream-collide steps after the first take the staged kernel (as configured by
    iblb_set_stream_collide for this lattice and storage type), 0 for the direct kernel, -1 for
-   a NULL context. */
+   a NULL context. (While a small lattice's whole step runs as one kernel, that kernel loads
+   directly; the populations are the same.) */
 int32_t iblb_stream_collide_staged(const iblb_ctx *ctx);
 
 /* SMs of the interface partition of iblb_step (0: no partition, -1: NULL context). */
