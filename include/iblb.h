@@ -62,10 +62,11 @@ typedef struct {
   int32_t z_periodic;      /* 0: bounce-back walls at both z ends; 1: periodic z (tests) */
   int32_t ib_sms;          /* SMs given to the interface chain of iblb_step as a partition of
                               the GPU (green context); the stream-collide passes get the rest.
-                              0: when the stream-collide pass moves at least 1 GiB
-                              (2 x 19 x nx ny nz x storage bytes) 24, 40 with 16-bit
-                              storage; below that 64 (rounded to the device's partition
-                              granularity); none with FP64 from 192 MiB up. < 0: no
+                              0: by the bytes that the stream-collide pass moves
+                              (2 x 19 x nx ny nz x storage bytes), 64 below 1 GiB, 40 below
+                              1.5 GiB, then 32 with 16-bit storage or below 2 GiB, else 24
+                              (rounded to the device's partition granularity); none with
+                              FP64 from 192 MiB up. < 0: no
                               partition (both share all SMs, interface stream at top priority).
                               If the device or driver cannot partition, no partition is used.
                               With 0, a mesh and less than 1 GiB a step runs as one kernel on

@@ -343,19 +343,22 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
     e = cudaDeviceGetAttribute(&c.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   for (int b = 0; b < 2 && e == cudaSuccess; b++) e = dalloc_bytes(&c.f[b], (size_t)iblb::Q * c.ncell * c.pop_size);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.f[0], 0, (size_t)iblb::Q * c.ncell * c.pop_size, c.stream);
-  // The interface chain runs on its own partition of SMs (default 32) so that the concurrent
+  // The interface chain runs on its own partition of SMs so that the concurrent
   // full-lattice pass keeps the rest undisturbed; without partitions both share the GPU and
   // the interface stream gets the highest priority, so that its small kernels are scheduled
   // between the blocks of the full-lattice pass instead of after it.
   int prio_lo = 0, prio_hi = 0;
   if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-  // Default split, from sweeps of the interface SMs. A full-lattice pass of at least 1 GiB
-  // hides the interface chain on 24 SMs (256^3 FP32, 2.5 GB: 40.3k MLUPS against 39.3k on 32,
-  // 31.5k on 16 and 34.8k unpartitioned); 16-bit storage halves the pass, so the chain takes
-  // 40 (256^3 FP16: 66.0k against 59.0k on 32). A shorter pass leaves the chain as the
-  // critical path, which then takes 64 SMs (128x128x96 FP32 wetting, 1.5 M nodes: 0.090 ms
-  // against 0.115 ms on 32 SMs; 32^3 FP64 shear: 0.136 ms against 0.138 ms on 32 and
-  // 0.149 ms unpartitioned). An FP64 pass is bound by the FP64 units (1/64 of the FP32 rate),
+  // Default split, from sweeps of the interface SMs: the longer the full-lattice pass, the fewer
+  // SMs hide the chain beside it. us per step on 24 / 32 / 40 SMs, with 40962 and, after the
+  // comma, 10242 vertices. FP32: 192^3 (1.08 GB per pass) 308 / 264 / 226, 193 / 183 / 187; 208^3
+  // (1.37 GB) 348 / 302 / 259, 239 / 223 / 225; 224^3 (1.71 GB) 380 / 323 / 297, 269 / 269 / 273;
+  // 240^3 (2.10 GB) 401 / 357 / 340; 256^3 (2.55 GB) 408 / 414 / 423, 390 / 397 / 406. 16 bits, whose
+  // pass has twice the arithmetic per byte: 256^3 (1.28 GB) 348 / 292 / 248; 288^3 (1.82 GB) 385 /
+  // 385 / 408, 371 / 378 / 403; 320^3 (2.49 GB) 498 / 471 / 500; 384^3 (4.30 GB) 780 / 726 / 720.
+  // A pass below 1 GiB leaves the chain as the critical path, which then takes 64 SMs where the
+  // separate kernels run (128x128x96 FP32 wetting, 1.5 M nodes: 0.090 ms against 0.115 ms on 32
+  // SMs). An FP64 pass is bound by the FP64 units (1/64 of the FP32 rate),
   // not by memory, and from 192 MiB (about 650k nodes) up the interface chain is short beside
   // it: no partition (96^3 FP64: 0.301 ms per step against 0.407 on 64 interface SMs and 0.309
   // on 24; 128^3: 0.583 against 0.899 and 0.632; below it, 64^3: 0.147 against 0.137 on 64).
@@ -363,7 +366,8 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
   const int want = d->ib_sms != 0 ? d->ib_sms
                    : c.pop_size == 8 && pass_bytes >= ((size_t)192 << 20) ? -1
                    : pass_bytes < ((size_t)1 << 30) ? 64
-                   : c.pop_size == 2 ? 40
+                   : pass_bytes < ((size_t)3 << 29) ? 40
+                   : pass_bytes < ((size_t)2 << 30) || c.pop_size == 2 ? 32
                    : 24;
   if (e == cudaSuccess && !(want > 0 && make_partitions(c, want, prio_hi))) {
     e = cudaStreamCreateWithPriority(&c.ib, cudaStreamNonBlocking, prio_hi);
