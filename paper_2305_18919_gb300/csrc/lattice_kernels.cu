@@ -14,6 +14,9 @@ namespace {
 // Each block covers (part of) one lattice row, or with FLAT the next blockDim.x pairs in memory
 // order: rows that are no whole number of warps would leave lanes idle (nx = 132: 66 pairs in 96
 // lanes, 45 us per pass of 132 x 100 x 77; nx = 32: 16 pairs in 32).
+// fin and fout carry no __restrict__: launched early, the kernel is there while the one before it
+// still writes fin, and `const __restrict__` would promise that nothing does. The loads, all after
+// the wait, are those of load_pair.
 template <typename real>
 struct K1MinBlocks {  // FP32: 72 registers, 28 warps per SM (64 registers spill and are no faster)
   static constexpr int value = sizeof(real) == 4 ? 7 : 1;
@@ -21,8 +24,7 @@ struct K1MinBlocks {  // FP32: 72 registers, 28 warps per SM (64 registers spill
 
 template <typename real, typename S, bool FIRST, bool FORCE, bool FLAT>
 __global__ void __launch_bounds__(128, K1MinBlocks<real>::value) stream_collide_kernel(
-    const S *__restrict__ fin, S *__restrict__ fout, const LatParams<real> P, int z0,
-    const FlatGroups G) {
+    const S *fin, S *fout, const LatParams<real> P, int z0, const FlatGroups G) {
   int x0, y, z;
   pdl_let_next();
   pdl_wait();
@@ -45,8 +47,7 @@ __global__ void __launch_bounds__(128, K1MinBlocks<real>::value) stream_collide_
 
 // (its threads always take the quads in memory order)
 template <typename S, bool FIRST, bool FORCE>
-__global__ void __launch_bounds__(128) stream_collide_quad_kernel(const S *__restrict__ fin,
-                                                                  S *__restrict__ fout,
+__global__ void __launch_bounds__(128) stream_collide_quad_kernel(const S *fin, S *fout,
                                                                   const LatParams<float> P,
                                                                   int z0, const FlatGroups G) {
   pdl_let_next();
