@@ -44,7 +44,9 @@ extern "C" {
                                wall plane, or |V/V0 - 1| > 0.05 */
 #define IBLB_ECAPACITY (-5) /* an internal bound was exceeded (active-tile table) */
 #define IBLB_ETIMEOUT (-6)  /* a bounded wait inside a kernel gave up (the staged stream-collide
-                               pass, iblb_set_stage_wait_limit); the context stays usable */
+                               pass, iblb_set_stage_wait_limit; the grid barriers of a small
+                               lattice's step, iblb_set_barrier_wait_limit); the context stays
+                               usable */
 
 #define IBLB_FP64 1 /* populations and interface arithmetic in double */
 #define IBLB_FP32 2 /* populations (stored as f_i - w_i rho0) and interface forces in float;
@@ -321,6 +323,15 @@ int iblb_set_stream_collide(iblb_ctx *ctx, int32_t kind, int32_t stages, int32_t
    step are incomplete; the context stays usable (iblb_init_equilibrium or iblb_load_state restore
    a state). IBLB_EINVAL outside the range. */
 int iblb_set_stage_wait_limit(iblb_ctx *ctx, int64_t ns);
+
+/* Limit in nanoseconds of each wait at a grid barrier of the kernel that runs all of a small
+   lattice's step (default 2e9, range 0 .. 6e10; 0: one test, so that the first block to arrive gives
+   up; this exercises the timeout path). A wait that runs out records the timeout in the health word
+   and every block stops; steps queued behind do nothing. iblb_step, or the call that reads the health
+   word, then returns IBLB_ETIMEOUT and the state is incomplete; the context stays usable
+   (iblb_init_equilibrium with iblb_set_vertices, or iblb_load_state, restore a state).
+   IBLB_EINVAL outside the range. */
+int iblb_set_barrier_wait_limit(iblb_ctx *ctx, int64_t ns);
 
 /* 1 if the stream-collide steps after the first take the staged kernel (as configured by
    iblb_set_stream_collide for this lattice and storage type), 0 for the direct kernel, -1 for

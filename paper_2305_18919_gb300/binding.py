@@ -91,6 +91,7 @@ SIGNATURES = {
     "iblb_set_stream_collide": (_i32, [_vp, _i32, _i32, _i32, _i32, _i32]),
     "iblb_stream_collide_staged": (_i32, [_vp]),
     "iblb_set_stage_wait_limit": (_i32, [_vp, _i64]),
+    "iblb_set_barrier_wait_limit": (_i32, [_vp, _i64]),
     "iblb_set_health_interval": (_i32, [_vp, _i32]),
     "iblb_mesh_volume_noalloc": (_i32, [_vp, _vp, _i32, _dp, _vp, _vp]),
     "iblb_batch_create": (_i32, [ctypes.POINTER(iblb_lattice_desc), _i32, _vp, ctypes.POINTER(_vp)]),
@@ -360,6 +361,11 @@ class Lattice:
     def set_stage_wait_limit(self, ns):
         """Limit (ns) of each wait of the staged stream-collide kernel (iblb_set_stage_wait_limit)."""
         self._check(self._L.iblb_set_stage_wait_limit(self.h, int(ns)))
+
+    def set_barrier_wait_limit(self, ns):
+        """Limit (ns) of each wait at a grid barrier of a small lattice's step kernel
+        (iblb_set_barrier_wait_limit)."""
+        self._check(self._L.iblb_set_barrier_wait_limit(self.h, int(ns)))
 
     def stream_collide_staged(self) -> bool:
         """Whether the steps after the first take the staged stream-collide kernel."""

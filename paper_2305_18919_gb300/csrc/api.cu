@@ -90,10 +90,27 @@ int read_health(Ctx &c, int *h) {
   return 0;
 }
 
+// Both tile maps and their counts as iblb_add_mesh left them: a step that gave up in the middle has
+// marked and binned into part of one, and the other may have lost its tiles but not their count.
+int empty_maps(Ctx &c) {
+  if (c.nv == 0) return 0;
+  for (int b = 0; b < 2; b++)
+    CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[b], 0xff, c.ntiles * sizeof(int), c.stream));
+  CUDA_TRY(c, cudaMemsetAsync(c.counters, 0, 3 * sizeof(int), c.stream));      // [3]: health
+  CUDA_TRY(c, cudaMemsetAsync(c.counters + 4, 0, 2 * sizeof(int), c.stream));
+  CUDA_TRY(c, cudaMemsetAsync(c.slot_count, 0, (size_t)c.max_slots * sizeof(int), c.stream));
+  CUDA_TRY(c, cudaMemsetAsync(c.spill_bits, 0, (size_t)c.spill_words * sizeof(unsigned), c.stream));
+  c.marked = 0;
+  c.have_force = 0;
+  return 0;
+}
+
 // An unstable run reports that first: its garbage positions can also leave tiles unmarked.
 int health_error(Ctx &c, int h) {
-  if (h & iblb::H_TIMEOUT)
+  if (h & iblb::H_TIMEOUT) {
+    if (int rc = empty_maps(c)) return rc;
     return fail(c, IBLB_ETIMEOUT, "a bounded wait inside a kernel gave up (staged copies or the step's grid barrier)");
+  }
   const int unstable = iblb::H_NAN | iblb::H_FAST | iblb::H_WALL | iblb::H_VOLUME;
   if (!(h & unstable))
     return fail(c, IBLB_ECAPACITY, "active-tile table capacity exceeded");
@@ -104,6 +121,16 @@ int health_error(Ctx &c, int h) {
   if (h & iblb::H_VOLUME) m += " |V/V0 - 1| > 0.05;";
   if (h & iblb::H_CAPACITY) m += " (active-tile table capacity also exceeded);";
   return fail(c, IBLB_EUNSTABLE, m);
+}
+
+// An unread failure of iblb_step_async steps goes with the state they left; what a step that gave up
+// did to the maps does not.
+int discard_health(Ctx &c) {
+  if (!c.health_pending) return 0;
+  c.health_pending = 0;
+  int h = 0;
+  if (int rc = read_health(c, &h)) return rc;
+  return h & iblb::H_TIMEOUT ? empty_maps(c) : 0;
 }
 
 cudaEvent_t pooled_event(Ctx &c) {
@@ -561,13 +588,13 @@ int iblb_init_equilibrium(iblb_ctx *h, const double *rho, const double *u) {
   if (!h || !rho || !u) return IBLB_EINVAL;
   Ctx &c = h->c;
   if (int rc = staging(c, 4 * c.ncell)) return rc;
+  if (int rc = discard_health(c)) return rc;
   CUDA_TRY(c, cudaMemcpyAsync(c.dscratch, rho, c.ncell * sizeof(double), cudaMemcpyHostToDevice, c.stream));
   CUDA_TRY(c, cudaMemcpyAsync(c.dscratch + c.ncell, u, 3 * c.ncell * sizeof(double), cudaMemcpyHostToDevice, c.stream));
   CUDA_TRY(c, iblb::launch_init_equilibrium(c, c.dscratch, c.dscratch + c.ncell));
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
   c.fresh = 1;
   c.have_force = 0;
-  c.health_pending = 0;  // the state those steps left is gone
   c.config_gen++;
   return IBLB_OK;
 }
@@ -985,11 +1012,11 @@ int iblb_load_state(iblb_ctx *h, const char *path) {
     CUDA_TRY(c, cudaMemcpy(mine.data(), c.faces, mine.size() * sizeof(int), cudaMemcpyDeviceToHost));
     if (mine != fcs) return fail(c, IBLB_EINVAL, "state file has a different face list");
   }
+  if (int rc = discard_health(c)) return rc;
   c.tau = hd.tau; c.rho0 = hd.rho0;
   for (int k = 0; k < 3; k++) { c.ub[k] = hd.ub[k]; c.ut[k] = hd.ut[k]; c.g[k] = hd.g[k]; }
   c.fresh = hd.fresh;
   c.steps_done = hd.steps_done;
-  c.health_pending = 0;  // the state of any unread iblb_step_async steps is replaced
   CUDA_TRY(c, cudaMemcpyAsync(c.f[c.cur], fbuf.data(), fbytes, cudaMemcpyHostToDevice, c.stream));
   if (c.nv) {
     std::vector<double> fref, fgeo;
@@ -1068,6 +1095,13 @@ int iblb_set_stage_wait_limit(iblb_ctx *h, int64_t ns) {
   h->c.stage_wait_ns = (unsigned long long)ns;
   h->c.stage_wait_set = 1;
   h->c.config_gen++;
+  return IBLB_OK;
+}
+
+int iblb_set_barrier_wait_limit(iblb_ctx *h, int64_t ns) {
+  if (!h) return IBLB_EINVAL;
+  if (ns < 0 || ns > 60000000000ll) return fail(h->c, IBLB_EINVAL, "wait limit must be 0 .. 60 s");
+  h->c.barrier_wait_ns = (unsigned long long)ns;
   return IBLB_OK;
 }
 

@@ -20,7 +20,9 @@
 //                     (| barrier of the interface blocks, || barrier of all blocks)
 //
 // The grid is launched cooperatively (all blocks resident). Every wait is bounded: a barrier that
-// does not complete within kBarrierWaitNs sets H_TIMEOUT and an abort flag that ends every block.
+// does not complete within the context's limit (iblb_set_barrier_wait_limit) sets H_TIMEOUT and an
+// abort flag that ends every block. A launch that finds H_TIMEOUT set, by one queued before it, does
+// nothing; the host empties the tile maps, which an abort leaves half marked, when it reads the word.
 #define IBLB_RO               // phases read what earlier phases of the same kernel wrote
 #define IBLB_SCATTER_ASM asm volatile
 #include "ib_device.cuh"
@@ -28,8 +30,6 @@
 
 namespace iblb {
 namespace {
-
-constexpr unsigned long long kBarrierWaitNs = 2000000000ull;
 
 // Control words of a launch, zero between launches (the last block to leave clears them).
 struct FusedControl {
@@ -58,6 +58,7 @@ struct FusedArgs {
   FusedStep<real, S> step[2];
   FusedControl *ctl;
   int *health;
+  unsigned long long wait_ns;
   int nsteps, nchain;
 };
 
@@ -80,10 +81,18 @@ __device__ __forceinline__ unsigned long long now_ns() {
   return t;
 }
 
+// Whether an earlier launch gave up (called by every thread of the block; one answer for all).
+__device__ __forceinline__ bool gave_up(const int *health) {
+  __shared__ int s_word;
+  if (threadIdx.x == 0) s_word = *(const volatile int *)health;
+  __syncthreads();
+  return s_word & H_TIMEOUT;
+}
+
 // Wait until `target` blocks have arrived on *ctr, this one included (called by every thread of the
-// block). False if the wait gave up or another block's did.
+// block). False if the wait gave up (after wait_ns; 0: after one test) or another block's did.
 __device__ __forceinline__ bool grid_barrier(unsigned *ctr, unsigned target, FusedControl *ctl,
-                                             int *health) {
+                                             int *health, unsigned long long wait_ns) {
   __shared__ int s_go;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -95,9 +104,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *ctr, unsigned target, Fus
       const unsigned long long t0 = now_ns();
       for (int k = 0;; k++) {
         if ((int)(ld_acquire(ctr) - target) >= 0) break;
-        if ((k & 63) == 63) {
+        if ((k & 63) == 63 || wait_ns == 0) {
           if (*(volatile int *)&ctl->abort) go = 0;
-          if (go && now_ns() - t0 > kBarrierWaitNs) {
+          if (go && now_ns() - t0 >= wait_ns) {
             atomicOr(health, H_TIMEOUT);
             atomicExch(&ctl->abort, 1);
             go = 0;
@@ -179,9 +188,9 @@ __device__ __forceinline__ void fused_steps(const FusedArgs<real, S> &P, SourceS
             all_stride = gridDim.x * nt;
   unsigned n_chain = 0, n_all = 0;  // arrivals expected at the next barrier
 #define CHAIN_BARRIER() \
-  if (!grid_barrier(&ctl->chain, n_chain += nchain, ctl, P.health)) return
+  if (!grid_barrier(&ctl->chain, n_chain += nchain, ctl, P.health, P.wait_ns)) return
 #define ALL_BARRIER() \
-  if (!grid_barrier(&ctl->all, n_all += gridDim.x, ctl, P.health)) return
+  if (!grid_barrier(&ctl->all, n_all += gridDim.x, ctl, P.health, P.wait_ns)) return
   for (int s = 0; s < P.nsteps; s++) {
     const FusedStep<real, S> &A = P.step[s & 1];
     if (chain) {
@@ -222,7 +231,7 @@ template <typename real, typename S>
 __global__ void __launch_bounds__(FusedShape<real>::threads, FusedShape<real>::per_sm)
     fused_step_kernel(const __grid_constant__ FusedArgs<real, S> P) {
   __shared__ SourceShared<real> sh[FusedShape<real>::threads / kSourceThreads];
-  fused_steps(P, sh);
+  if (!gave_up(P.health)) fused_steps(P, sh);
   leave_grid(P.ctl);
 }
 
@@ -233,6 +242,7 @@ struct LatticeSteps {
   StreamArgs<real, S> step[2];
   FusedControl *ctl;
   int *health;
+  unsigned long long wait_ns;
   int nsteps;
 };
 // Blocks of 128 threads per SM: what the pass's registers allow.
@@ -245,11 +255,14 @@ template <typename real, typename S>
 __global__ void __launch_bounds__(128, (LatticeShape<real, S>::per_sm))
     lattice_steps_kernel(const __grid_constant__ LatticeSteps<real, S> P) {
   unsigned n_all = 0;
-  for (int s = 0; s < P.nsteps; s++) {
+  const int nsteps = gave_up(P.health) ? 0 : P.nsteps;
+  for (int s = 0; s < nsteps; s++) {
     const StreamArgs<real, S> &A = P.step[s & 1];
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < A.G.n; g += gridDim.x * blockDim.x)
       lattice_group(A, g);
-    if (s + 1 < P.nsteps && !grid_barrier(&P.ctl->all, n_all += gridDim.x, P.ctl, P.health)) break;
+    if (s + 1 < nsteps &&
+        !grid_barrier(&P.ctl->all, n_all += gridDim.x, P.ctl, P.health, P.wait_ns))
+      break;
   }
   leave_grid(P.ctl);
 }
@@ -264,6 +277,7 @@ cudaError_t launch_lattice_steps_t(Ctx &c, int nsteps, cudaStream_t st) {
   }
   a.ctl = (FusedControl *)c.fused_ctl;
   a.health = c.counters + 3;
+  a.wait_ns = c.barrier_wait_ns;
   a.nsteps = nsteps;
   const int need = (a.step[0].G.n + 127) / 128, room = LatticeShape<real, S>::per_sm * c.sm_count;
   void *params[] = {&a};
@@ -293,6 +307,7 @@ cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
   c.map = map;
   a.ctl = (FusedControl *)c.fused_ctl;
   a.health = c.counters + 3;
+  a.wait_ns = c.barrier_wait_ns;
   a.nsteps = nsteps;
   a.nchain = c.sm_count;
   void *params[] = {&a};

@@ -225,6 +225,7 @@ struct Ctx {
   int k1_nodes = 0;         // nodes per compute lane of the staged pass, 16-bit (0: default)
   unsigned long long stage_wait_ns = 1000000000ull;  // limit of a staged pass's waits (ns)
   int stage_wait_set = 0;   // that limit was set by the caller
+  unsigned long long barrier_wait_ns = 2000000000ull;  // limit of a grid barrier's wait (ns)
   int smem_optin = 0;       // shared memory a block may opt in to (bytes)
   int health_every = 1000;  // iblb_step reads the health word every this many steps (0: at its end)
   int health_pending = 0;   // steps queued by iblb_step_async whose health word is unread
