@@ -757,23 +757,32 @@ struct Adjoint {
   cudaStream_t side = nullptr;        // stream of the forward pieces
 };
 
-void free_all(Adjoint *a) {
-  auto f = [](void *p) {
+// Free the work arrays of a gradient (also a part of them, after a failed allocation).
+void free_work(Adjoint *a) {
+  auto f = [](auto *&p) {
     if (p) cudaFree(p);
+    p = nullptr;
   };
   if (a->side) cudaStreamSynchronize(a->side);
-  for (void *p : a->ck_P) f(p);
-  for (double *p : a->ck_q) f(p);
-  for (size_t m = 1; m < a->seg_P.size(); m++) f(a->seg_P[m]);  // ([0] is a checkpoint)
-  for (double *p : a->seg_q) f(p);
   f(a->lam_P[0]); f(a->lam_P[1]); f(a->lam_q); f(a->lam_qn); f(a->lam_phi); f(a->lam_F);
   f(a->lam_u); f(a->fj); f(a->dn); f(a->part); f(a->grad);
   for (Pieces &p : a->pieces) {
     f(p.fc); f(p.fn); f(p.vpart); f(p.phi); f(p.F); f(p.mark); f(p.U); f(p.st);
     if (p.ready) cudaEventDestroy(p.ready);
     if (p.free) cudaEventDestroy(p.free);
+    p.ready = p.free = nullptr;
   }
   if (a->side) cudaStreamDestroy(a->side);
+  a->side = nullptr;
+  a->work = false;
+}
+
+void free_all(Adjoint *a) {
+  free_work(a);
+  for (void *p : a->ck_P) cudaFree(p);
+  for (double *p : a->ck_q) cudaFree(p);
+  for (size_t m = 1; m < a->seg_P.size(); m++) cudaFree(a->seg_P[m]);  // ([0] is a checkpoint)
+  for (double *p : a->seg_q) cudaFree(p);
   delete a;
 }
 
@@ -782,12 +791,15 @@ int afail(Ctx &c, int code, const std::string &m) {
   return code;
 }
 
+// (the error is taken: the next launch's check would find it)
 #define ADJ_TRY(c, expr)                                                                   \
   do {                                                                                     \
     cudaError_t e_ = (expr);                                                               \
-    if (e_ != cudaSuccess)                                                                 \
+    if (e_ != cudaSuccess) {                                                               \
+      cudaGetLastError();                                                                  \
       return iblb::afail((c), e_ == cudaErrorMemoryAllocation ? IBLB_ENOMEM : IBLB_ECUDA,   \
                    std::string(#expr) + ": " + cudaGetErrorString(e_));                    \
+    }                                                                                      \
   } while (0)
 
 cudaError_t dmalloc(double **p, size_t n) {
@@ -907,6 +919,37 @@ int recompute_segment(Ctx &c, Adjoint *a, int s, int len, int fresh) {
 
 int face_warps(const Ctx &c) { return (c.nf + 31) / 32; }
 
+// Allocate the work arrays of a gradient; what a failure leaves is for free_work.
+int allocate_work(Ctx &c, Adjoint *a) {
+  const size_t pn = (size_t)Q * c.ncell, qn = (size_t)3 * c.nv;
+  ADJ_TRY(c, dmalloc(&a->lam_P[0], pn));
+  ADJ_TRY(c, dmalloc(&a->lam_P[1], pn));
+  ADJ_TRY(c, dmalloc(&a->lam_q, qn));
+  ADJ_TRY(c, dmalloc(&a->lam_qn, qn));
+  ADJ_TRY(c, dmalloc(&a->lam_phi, qn));
+  ADJ_TRY(c, dmalloc(&a->lam_F, 3 * c.ncell));
+  ADJ_TRY(c, dmalloc(&a->lam_u, 3 * c.ncell));
+  ADJ_TRY(c, dmalloc(&a->fj, (size_t)9 * c.nf));
+  ADJ_TRY(c, dmalloc(&a->dn, (size_t)3 * c.nf));
+  ADJ_TRY(c, dmalloc(&a->part, (size_t)5 * face_warps(c)));
+  ADJ_TRY(c, dmalloc(&a->grad, 4));
+  for (Pieces &p : a->pieces) {
+    ADJ_TRY(c, dmalloc(&p.fc, (size_t)9 * c.nf));
+    ADJ_TRY(c, dmalloc(&p.fn, (size_t)3 * c.nf));
+    ADJ_TRY(c, dmalloc(&p.vpart, (size_t)face_warps(c)));
+    ADJ_TRY(c, dmalloc(&p.phi, qn));
+    ADJ_TRY(c, dmalloc(&p.F, 3 * c.ncell));
+    ADJ_TRY(c, cudaMalloc((void **)&p.mark, c.ncell));
+    ADJ_TRY(c, cudaMalloc((void **)&p.U, c.ncell * sizeof(NodeU)));
+    ADJ_TRY(c, cudaMalloc((void **)&p.st, (size_t)c.nv * sizeof(Stencil)));
+    ADJ_TRY(c, cudaEventCreateWithFlags(&p.ready, cudaEventDisableTiming));
+    ADJ_TRY(c, cudaEventCreateWithFlags(&p.free, cudaEventDisableTiming));
+  }
+  ADJ_TRY(c, cudaStreamCreateWithFlags(&a->side, cudaStreamNonBlocking));
+  a->work = true;
+  return 0;
+}
+
 // Forward pieces of reverse step n at q_n, on the side stream: forces, volume, stencils, the
 // spread force field, the moments of P_{n+1}. They depend on the recomputed states only.
 template <typename T>
@@ -1011,8 +1054,8 @@ int iblb_adjoint_record(iblb_ctx *h, int32_t nsteps, int32_t every) {
   auto *a = (iblb::Adjoint *)c.adj;
   a->recorded = false;
   int rc = iblb::resize_states(c, a->ck_P, a->ck_q, nck, nck);
-  if (rc == IBLB_ENOMEM && (a->work || !a->seg_q.empty())) {  // without the last gradient's arrays
-    cudaGetLastError();
+  if (rc == IBLB_ENOMEM && (a->work || a->seg_P.size() > 1 || !a->seg_q.empty())) {
+    // without the last gradient's arrays
     iblb::adjoint_free(c);
     c.adj = a = new iblb::Adjoint();
     rc = iblb::resize_states(c, a->ck_P, a->ck_q, nck, nck);
@@ -1044,33 +1087,11 @@ int iblb_adjoint_gradient(iblb_ctx *h, const double *dJdq, double *dJdtheta) {
   if (int rc = iblb::settle_health(c)) return rc;
   const size_t pn = (size_t)iblb::Q * c.ncell, qn = (size_t)3 * c.nv;
   // work arrays (kept for later calls)
-  if (!a->work) {
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_P[0], pn));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_P[1], pn));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_q, qn));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_qn, qn));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_phi, qn));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_F, 3 * c.ncell));
-    ADJ_TRY(c, iblb::dmalloc(&a->lam_u, 3 * c.ncell));
-    ADJ_TRY(c, iblb::dmalloc(&a->fj, (size_t)9 * c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->dn, (size_t)3 * c.nf));
-    ADJ_TRY(c, iblb::dmalloc(&a->part, (size_t)5 * iblb::face_warps(c)));
-    ADJ_TRY(c, iblb::dmalloc(&a->grad, 4));
-    for (iblb::Pieces &p : a->pieces) {
-      ADJ_TRY(c, iblb::dmalloc(&p.fc, (size_t)9 * c.nf));
-      ADJ_TRY(c, iblb::dmalloc(&p.fn, (size_t)3 * c.nf));
-      ADJ_TRY(c, iblb::dmalloc(&p.vpart, (size_t)iblb::face_warps(c)));
-      ADJ_TRY(c, iblb::dmalloc(&p.phi, qn));
-      ADJ_TRY(c, iblb::dmalloc(&p.F, 3 * c.ncell));
-      ADJ_TRY(c, cudaMalloc((void **)&p.mark, c.ncell));
-      ADJ_TRY(c, cudaMalloc((void **)&p.U, c.ncell * sizeof(iblb::NodeU)));
-      ADJ_TRY(c, cudaMalloc((void **)&p.st, (size_t)c.nv * sizeof(iblb::Stencil)));
-      ADJ_TRY(c, cudaEventCreateWithFlags(&p.ready, cudaEventDisableTiming));
-      ADJ_TRY(c, cudaEventCreateWithFlags(&p.free, cudaEventDisableTiming));
+  if (!a->work)
+    if (int rc = iblb::allocate_work(c, a)) {
+      iblb::free_work(a);
+      return rc;
     }
-    ADJ_TRY(c, cudaStreamCreateWithFlags(&a->side, cudaStreamNonBlocking));
-    a->work = true;
-  }
   // states 1 .. every of a segment and the positions 0 .. every - 1
   if (a->seg_P.empty()) a->seg_P.push_back(nullptr);
   if (int rc = iblb::resize_states(c, a->seg_P, a->seg_q, a->every + 1, a->every)) return rc;
