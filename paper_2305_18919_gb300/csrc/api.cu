@@ -1017,6 +1017,7 @@ int iblb_load_state(iblb_ctx *h, const char *path) {
   for (int k = 0; k < 3; k++) { c.ub[k] = hd.ub[k]; c.ut[k] = hd.ut[k]; c.g[k] = hd.g[k]; }
   c.fresh = hd.fresh;
   c.steps_done = hd.steps_done;
+  c.config_gen++;  // a batch's records hold the parameters replaced above
   CUDA_TRY(c, cudaMemcpyAsync(c.f[c.cur], fbuf.data(), fbytes, cudaMemcpyHostToDevice, c.stream));
   if (c.nv) {
     std::vector<double> fref, fgeo;
@@ -1032,7 +1033,6 @@ int iblb_load_state(iblb_ctx *h, const char *path) {
     CUDA_TRY(c, cudaMemcpyAsync(c.qdot, qdbuf.data(), qdbuf.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
     c.have_force = 0;
     if (int rc = positions_changed(c)) return rc;
-    c.config_gen++;
   }
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
   return IBLB_OK;
