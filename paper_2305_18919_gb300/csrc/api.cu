@@ -62,15 +62,12 @@ int check_mesh_id(Ctx &c, int mesh_id) {
   return 0;
 }
 
-// The vertex positions were replaced: refresh the displacements, and empty the tile map if it was
-// marked for the old ones (a step's face pass marks it).
-int positions_changed(Ctx &c) {
-  if (c.marked) {
-    CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[c.map], 0xff, c.ntiles * sizeof(int), c.stream));
-    CUDA_TRY(c, cudaMemsetAsync(c.counters + c.map, 0, sizeof(int), c.stream));
-    c.marked = 0;
-  }
-  CUDA_TRY(c, iblb::launch_displacement(c));
+// Empty tile map `which`. Between calls the map of the current positions is empty (a step's face
+// pass marks it, the next step clears it again); the other one is the last step's. No flag of the
+// host's says so: the steps of a captured graph run without it.
+int empty_map(Ctx &c, int which) {
+  CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[which], 0xff, c.ntiles * sizeof(int), c.stream));
+  CUDA_TRY(c, cudaMemsetAsync(c.counters + which, 0, sizeof(int), c.stream));
   return 0;
 }
 
@@ -95,12 +92,11 @@ int read_health(Ctx &c, int *h) {
 int empty_maps(Ctx &c) {
   if (c.nv == 0) return 0;
   for (int b = 0; b < 2; b++)
-    CUDA_TRY(c, cudaMemsetAsync(c.tile_slot[b], 0xff, c.ntiles * sizeof(int), c.stream));
-  CUDA_TRY(c, cudaMemsetAsync(c.counters, 0, 3 * sizeof(int), c.stream));      // [3]: health
+    if (int rc = empty_map(c, b)) return rc;
+  CUDA_TRY(c, cudaMemsetAsync(c.counters + 2, 0, sizeof(int), c.stream));      // ([3]: health)
   CUDA_TRY(c, cudaMemsetAsync(c.counters + 4, 0, 2 * sizeof(int), c.stream));
   CUDA_TRY(c, cudaMemsetAsync(c.slot_count, 0, (size_t)c.max_slots * sizeof(int), c.stream));
   CUDA_TRY(c, cudaMemsetAsync(c.spill_bits, 0, (size_t)c.spill_words * sizeof(unsigned), c.stream));
-  c.marked = 0;
   c.have_force = 0;
   return 0;
 }
@@ -554,9 +550,7 @@ int iblb_add_mesh(iblb_ctx *h, const double *verts, int32_t nv, const int32_t *f
   c.map = 0;
   c.config_gen++;
   c.have_force = 0;
-  c.marked = 0;
-  int rc = positions_changed(c);
-  if (rc) return rc;
+  CUDA_TRY(c, iblb::launch_displacement(c));
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
   if (mesh_id) *mesh_id = 0;
   return IBLB_OK;
@@ -581,7 +575,8 @@ int iblb_set_vertices(iblb_ctx *h, int32_t mesh_id, const double *q) {
   if (int rc = check_mesh_id(c, mesh_id)) return rc;
   CUDA_TRY(c, cudaMemcpyAsync(c.q, q, (size_t)3 * c.nv * sizeof(double), cudaMemcpyHostToDevice, c.stream));
   // the map of the last spreading step (map ^ 1) stays: read_fields still uses its force
-  return positions_changed(c);
+  CUDA_TRY(c, iblb::launch_displacement(c));
+  return IBLB_OK;
 }
 
 int iblb_init_equilibrium(iblb_ctx *h, const double *rho, const double *u) {
@@ -692,7 +687,6 @@ int enqueue_fused(Ctx &c, int nsteps, int *left) {
     c.cur ^= n & 1;
     if (c.nv) {
       c.map ^= n & 1;
-      c.marked = 0;
       c.have_force = 1;
     }
     c.steps_done += n;
@@ -759,7 +753,6 @@ int enqueue_steps(Ctx &c, int nsteps) {
       CUDA_TRY(c, iblb::launch_interpolate_advect(c, tail));
       c.kernel_launches += 2;
       c.map ^= 1;
-      c.marked = 0;
       c.have_force = 1;
     }
     c.steps_done++;
@@ -802,7 +795,8 @@ int restore_positions(Ctx &c, const double *q, int fresh) {
   CUDA_TRY(c, cudaMemcpyAsync(c.q, q, (size_t)3 * c.nv * sizeof(double), cudaMemcpyDeviceToDevice,
                               c.stream));
   c.fresh = fresh;
-  return positions_changed(c);
+  CUDA_TRY(c, launch_displacement(c));
+  return 0;
 }
 
 int restore_state(Ctx &c, const void *P, const double *q, int fresh) {
@@ -896,13 +890,12 @@ int iblb_read_force_field(iblb_ctx *h, double *F) {
   CUDA_TRY(c, cudaMemsetAsync(c.dscratch, 0, 3 * c.ncell * sizeof(double), c.stream));
   if (c.nv) {
     CUDA_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
-    if (!c.marked) CUDA_TRY(c, iblb::launch_mark(c));
-    c.marked = 1;
+    CUDA_TRY(c, iblb::launch_mark(c));
     CUDA_TRY(c, iblb::launch_face_forces(c, 0, c.stream));
     CUDA_TRY(c, iblb::launch_vertex_forces(c, 1, c.stream));
     CUDA_TRY(c, iblb::launch_spread(c, c.stream));
     CUDA_TRY(c, iblb::launch_expand_force(c, c.dscratch));
-    CUDA_TRY(c, iblb::launch_clear_counts(c));
+    if (int rc = empty_map(c, c.map)) return rc;
   }
   CUDA_TRY(c, cudaMemcpyAsync(F, c.dscratch, 3 * c.ncell * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
@@ -1032,7 +1025,7 @@ int iblb_load_state(iblb_ctx *h, const char *path) {
     CUDA_TRY(c, cudaMemcpyAsync(c.q, qbuf.data(), qbuf.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
     CUDA_TRY(c, cudaMemcpyAsync(c.qdot, qdbuf.data(), qdbuf.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
     c.have_force = 0;
-    if (int rc = positions_changed(c)) return rc;
+    CUDA_TRY(c, iblb::launch_displacement(c));
   }
   CUDA_TRY(c, cudaStreamSynchronize(c.stream));
   return IBLB_OK;

@@ -478,7 +478,6 @@ int iblb_batch_step(iblb_batch *b, int32_t nsteps) {
         Ctx &c = b->inst[i]->c;
         c.steps_done += kPairSteps;
         if (c.nv) c.have_force = 1;
-        c.marked = 0;
         c.fresh = 0;
       }
     }

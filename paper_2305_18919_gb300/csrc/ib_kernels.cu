@@ -10,18 +10,6 @@ __global__ void mark_kernel(int nv, const double *IBLB_RO q, Dims D, TileMap M) 
   mark_vertices(q, nv, kMarkVertices * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5), D, M);
 }
 
-__global__ void clear_counts_kernel(const int *__restrict__ nslots, int *__restrict__ slot_count,
-                                    int *__restrict__ ovf_count, int max_slots) {
-  const int n = min(*nslots, max_slots);
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
-    slot_count[s] = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    ovf_count[0] = 0;
-    ovf_count[2] = 0;
-    ovf_count[3] = 0;
-  }
-}
-
 __global__ void volume_sum_kernel(const double *__restrict__ part, int n, double V0,
                                   double *__restrict__ out) {
   double V;
@@ -165,14 +153,6 @@ cudaError_t launch_displacement(Ctx &c) {
     displacement_kernel<double><<<blocks, 128, 0, c.stream>>>(c.nv, c.q, c.xref, (Vec4<double> *)c.disp);
   else
     displacement_kernel<float><<<blocks, 128, 0, c.stream>>>(c.nv, c.q, c.xref, (Vec4<float> *)c.disp);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_clear_counts(Ctx &c) {
-  int grid = (c.max_slots + 255) / 256;
-  if (grid > 1024) grid = 1024;
-  clear_counts_kernel<<<grid, 256, 0, c.stream>>>(c.counters + c.map, c.slot_count, c.counters + 2,
-                                                  c.max_slots);
   return cudaGetLastError();
 }
 

@@ -179,9 +179,8 @@ struct Ctx {
   void *Uslot = nullptr;                   // [max_slots][64] Vec4 velocity
   int *pair_list = nullptr;                // [32 max_slots] slot * 32 + pair: the node pairs with
                                            //   a non-zero force (K4b appends, K1t reads)
-  int map = 0;                             // tile map of the current vertex positions
-  int marked = 0;                          // that map holds their tiles (else it is empty and
-                                           //   the next step's face pass marks it)
+  int map = 0;                             // tile map of the current vertex positions: empty
+                                           //   between calls, the next step's face pass marks it
   // mesh
   int nv = 0, nf = 0;
   double *q = nullptr;       // [nv][3] positions (double in every precision)
@@ -292,7 +291,6 @@ cudaError_t launch_interpolate_advect(Ctx &c, cudaStream_t s);
 // Mark the (empty) tile map of the current positions; refresh the displacements from them.
 cudaError_t launch_mark(Ctx &c);
 cudaError_t launch_displacement(Ctx &c);
-cudaError_t launch_clear_counts(Ctx &c);
 cudaError_t launch_expand_force(Ctx &c, double *F_dev);
 cudaError_t launch_phi_to_double(Ctx &c, double *phi_dev);
 cudaError_t launch_volume(Ctx &c, double *V_dev);
