@@ -628,7 +628,8 @@ int iblb_step_async(iblb_ctx *h, int32_t nsteps) {
   if (nsteps == 0) return IBLB_OK;
   // a failure still unread stays in the health word; otherwise it starts clear (as it is where the
   // last steps' word was read and none has run since: a loop that exchanges data every step)
-  if (!c.health_pending && (!c.health_clear || capturing(c.stream)))
+  c.captured |= capturing(c.stream);
+  if (!c.health_pending && (!c.health_clear || c.captured))
     CUDA_TRY(c, cudaMemsetAsync(c.counters + 3, 0, sizeof(int), c.stream));
   if (int rc = iblb::enqueue_steps(c, nsteps)) return rc;
   c.health_pending = 1;

@@ -229,6 +229,7 @@ struct Ctx {
   int health_every = 1000;  // iblb_step reads the health word every this many steps (0: at its end)
   int health_pending = 0;   // steps queued by iblb_step_async whose health word is unread
   int health_clear = 0;     // the health word is known to be 0 (read so, and nothing run since)
+  int captured = 0;         // steps were captured: replays write the health word unseen by the host
   int *health_host = nullptr;  // pinned: the health word read with a call's own transfers
   int fused = 0;               // iblb_step's steps may run as one kernel (fused.cu)
   void *fused_ctl = nullptr;   // control words of the fused kernel (kFusedControlBytes, zeroed)

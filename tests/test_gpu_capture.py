@@ -78,3 +78,22 @@ def test_replayed_steps_and_the_force_field(precision, force_field_first):
     c.replay()
     _same(c.both(lambda lat: lat.vertex_velocities()))
     c.close()
+
+
+def test_failure_of_replayed_steps_is_not_that_of_later_ones():
+    import torch
+    c = Case("fp32")
+    lat, ref = c.lats
+    for x in c.lats:
+        x.step_async(2)
+        x.vertices()  # reads the health word: clear
+    lat.set_vertices(c.v.mean(0) + 0.9 * (c.v - c.v.mean(0)))  # beyond the volume check
+    with torch.cuda.stream(c.stream):
+        c.graph.replay()
+    torch.cuda.synchronize()
+    for x in c.lats:
+        x.init_equilibrium(c.rho, c.u)
+        x.set_vertices(inputs.perturb(c.v, 0.02, seed=3))
+        x.step_async(2)
+    _same(c.both(lambda x: x.vertices()))
+    c.close()
