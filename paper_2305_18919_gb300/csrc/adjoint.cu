@@ -1116,9 +1116,15 @@ int iblb_adjoint_gradient(iblb_ctx *h, const double *dJdq, double *dJdtheta) {
       rc = c.pop_size == sizeof(double) ? iblb::reverse_segment<double>(c, a, len, first_fresh)
                                         : iblb::reverse_segment<float>(c, a, len, first_fresh);
   }
-  // back to the end of the recorded run
-  if (rc == 0) rc = iblb::restore_state(c, a->ck_P[nseg], a->ck_q[nseg], 0);
-  if (rc) return rc;
+  // back to the end of the recorded run, also after a failure: the recomputed states were lent to the
+  // context, whose own arrays hold older ones
+  const std::string why = c.err;
+  const int back = iblb::restore_state(c, a->ck_P[nseg], a->ck_q[nseg], 0);
+  if (rc) {
+    c.err = why;
+    return rc;
+  }
+  if (back) return back;
   ADJ_TRY(c, cudaMemcpyAsync(dJdtheta, a->grad, 4 * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
   ADJ_TRY(c, cudaStreamSynchronize(c.stream));
   return IBLB_OK;
