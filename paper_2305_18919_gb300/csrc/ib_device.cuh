@@ -599,6 +599,9 @@ __device__ __forceinline__ void add_plane(Vec4<real> *region, int plane, int l, 
   o = v;
 }
 
+// Words of the spill bitmap that a warp scans per round (at most 8: list entries are a byte).
+constexpr int kScanWords = 8;
+
 // Shared memory of one group of kSourceThreads threads of K4a.
 template <typename real>
 struct SourceShared {
@@ -607,6 +610,8 @@ struct SourceShared {
   real w[BUCKET_CAP][12];
   int b[BUCKET_CAP];
   int v[BUCKET_CAP];
+  unsigned char list[kSourceThreads / 32][32 * kScanWords];  // of a spilled tile: see below
+  int listed[kSourceThreads / 32];
 };
 
 // Barrier of the kSourceThreads threads of group `g` of a block.
@@ -658,6 +663,32 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, So
         if (slot_t >= 0) out_src[8 * (size_t)slot_t + e] = reg;
       }
     }
+    // vertex v's record, completed with the volume term, to place r of the stage. Its base is relative
+    // to S_lo (x, y wrapped into [0, n) by the vertex kernel): x, y in 0..3, z in -4..3 (below 0 only
+    // at a wall), in a byte each
+    auto stage = [&](int r, const StencilRec<real> &rec, const Vec4<real> &pv, const Vec4<real> &gv) {
+      for (int k = 0; k < 4; k++) {
+        sh.w[r][k] = rec.w[0][k];
+        sh.w[r][4 + k] = rec.w[1][k];
+        sh.w[r][8 + k] = rec.w[2][k];
+      }
+      sh.f[r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
+      const int bz = max(rec.base[2] - Sz, -4);
+      sh.b[r] = (rec.base[0] - Sx) | (rec.base[1] - Sy) << 8 | (bz + 4) << 16;
+    };
+    // add the n staged vertices, the tile's rank-th and following: even ranks by the lower half warp
+    auto add_staged = [&](int n, int rank) {
+      for (int c0 = 0; c0 < n; c0 += 2) {
+        const int c = c0 + ((half ^ rank) & 1);
+        if (c < n) {
+          const int b = sh.b[c];
+          const Vec4<real> f = sh.f[c];
+          add_plane(sh.region[half], warp, l16, b & 255, (b >> 8) & 255, (b >> 16) - 4, sh.w[c],
+                    sh.w[c] + 4, sh.w[c] + 8, f.x, f.y, f.z);
+        }
+        __syncwarp();
+      }
+    };
     if (cnt <= BUCKET_CAP) {
       // sort the bucket by vertex index and stage the records in that order
       StencilRec<real> rec;
@@ -672,64 +703,66 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, So
       if (tid < cnt) {
         int r = 0;
         for (int m = 0; m < cnt; m++) r += sh.v[m] < v;
-        for (int k = 0; k < 4; k++) {
-          sh.w[r][k] = rec.w[0][k];
-          sh.w[r][4 + k] = rec.w[1][k];
-          sh.w[r][8 + k] = rec.w[2][k];
-        }
-        sh.f[r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
-        // base relative to S_lo (x, y wrapped into [0, n) by the vertex kernel): x, y in 0..3,
-        // z in -4..3 (below 0 only at a wall), in a byte each
-        const int bz = max(rec.base[2] - Sz, -4);
-        sh.b[r] = (rec.base[0] - Sx) | (rec.base[1] - Sy) << 8 | (bz + 4) << 16;
+        stage(r, rec, pv, gv);
       }
       group_barrier(g);
-      for (int c0 = 0; c0 < cnt; c0 += 2) {
-        const int c = c0 + half;
-        if (c < cnt) {
-          const int b = sh.b[c];
-          const Vec4<real> f = sh.f[c];
-          add_plane(sh.region[half], warp, l16, b & 255, (b >> 8) & 255, (b >> 16) - 4, sh.w[c],
-                    sh.w[c] + 4, sh.w[c] + 8, f.x, f.y, f.z);
-        }
-        __syncwarp();
-      }
+      add_staged(cnt, 0);
     } else {
       // the tile spilled: mark its bucket's vertices too, then add every vertex of the tile in
-      // increasing index (bitmap words read through L2, where the atomics are performed); every
-      // warp scans for itself and adds the planes it owns
+      // increasing index (bitmap words read through L2, where the atomics are performed). A round
+      // scans the next kScanWords words of each of the four warps, which list the tile's vertices
+      // among them in a row each; the rows, one after the other, are staged and added like a bucket.
+      // (With every warp scanning all words, and a vertex's record read when its turn came, a tile
+      // was a chain of memory latencies. 96^3 FP32 with 40962 vertices on a sphere of radius 20, whose
+      // tiles nearly all spill: 377 us per step against 1026, by the separate kernels 232 against 606;
+      // radius 16, 262 against 762.)
       atomicOr(&spill_bits[v >> 5], 1u << (v & 31));
       group_barrier(g);
       int rank = 0;
-      for (int wb = 0; wb < A.spill_words; wb += 32) {
-        const unsigned word_l = wb + lane < A.spill_words ? __ldcg(&spill_bits[wb + lane]) : 0u;
-        unsigned nonzero = __ballot_sync(0xffffffffu, word_l != 0u);
-        while (nonzero) {
-          const int l = __ffs(nonzero) - 1;
-          nonzero &= nonzero - 1;
-          const unsigned word = __shfl_sync(0xffffffffu, word_l, l);
-          const int vl = (wb + l) * 32 + lane;  // this lane's vertex of the word
-          bool mine = false;
-          if ((word >> lane) & 1u) {
-            const StencilRec<real> &rl = stencil[vl];
-            const int bzc = min(max(rl.base[2], 0), D.nz - 1);
-            mine = (rl.base[0] >> 2) == tsx && (rl.base[1] >> 2) == tsy && (bzc >> 2) == tsz;
-          }
-          unsigned members = __ballot_sync(0xffffffffu, mine);
-          while (members) {  // the tile's vertices of this word, in index order
-            const int b = __ffs(members) - 1;
-            members &= members - 1;
-            if ((rank++ & 1) == half) {
-              const int vm = (wb + l) * 32 + b;
-              const StencilRec<real> &rec = stencil[vm];
-              const Vec4<real> pv = phi[vm], gv = gvol[vm];
-              add_plane(sh.region[half], warp, l16, rec.base[0] - Sx, rec.base[1] - Sy,
-                        max(rec.base[2] - Sz, -4), rec.w[0], rec.w[1], rec.w[2],
-                        pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z);
+      for (int wb = 0; wb < A.spill_words; wb += kScanWords * (kSourceThreads / 32)) {
+        const int w0 = wb + kScanWords * warp;
+        const unsigned words =
+            lane < kScanWords && w0 + lane < A.spill_words ? __ldcg(&spill_bits[w0 + lane]) : 0u;
+        int n = 0;
+#pragma unroll 1
+        for (int k0 = 0; k0 < kScanWords; k0 += 2) {  // (two words' loads in flight: few registers)
+          bool mine[2];
+#pragma unroll
+          for (int k = 0; k < 2; k++) {
+            mine[k] = (__shfl_sync(0xffffffffu, words, k0 + k) >> lane) & 1u;
+            if (mine[k]) {
+              const StencilRec<real> &rl = stencil[(w0 + k0 + k) * 32 + lane];
+              mine[k] = (rl.base[0] >> 2) == tsx && (rl.base[1] >> 2) == tsy &&
+                        (min(max(rl.base[2], 0), D.nz - 1) >> 2) == tsz;
             }
-            __syncwarp();
+          }
+#pragma unroll
+          for (int k = 0; k < 2; k++) {
+            const unsigned members = __ballot_sync(0xffffffffu, mine[k]);
+            if (mine[k])
+              sh.list[warp][n + __popc(members & ((1u << lane) - 1u))] =
+                  (unsigned char)(32 * (k0 + k) + lane);
+            n += __popc(members);
           }
         }
+        if (lane == 0) sh.listed[warp] = n;
+        group_barrier(g);
+        const int e1 = sh.listed[0], e2 = e1 + sh.listed[1], e3 = e2 + sh.listed[2];
+        const int total = e3 + sh.listed[3];
+        for (int c0 = 0; c0 < total; c0 += kSourceThreads) {
+          const int e = c0 + tid, m = min(total - c0, kSourceThreads);
+          if (tid < m) {
+            const int row = (e >= e1) + (e >= e2) + (e >= e3);
+            const int at = e - (row == 0 ? 0 : row == 1 ? e1 : row == 2 ? e2 : e3);
+            const int vm = 32 * (wb + kScanWords * row) + sh.list[row][at];
+            stage(tid, stencil[vm], phi[vm], gvol[vm]);
+          }
+          group_barrier(g);
+          add_staged(m, rank);
+          rank += m;
+          group_barrier(g);  // the stage and the lists are written again
+        }
+        if (total == 0) group_barrier(g);
       }
     }
     group_barrier(g);
@@ -748,8 +781,9 @@ __global__ void __launch_bounds__(kSourceThreads) spread_source_kernel(const Sou
   spread_source_body(A, sh, blockIdx.x, gridDim.x, 0, threadIdx.x);
 }
 
+// (float: seven blocks per SM, a few registers fewer than it would take)
 template <typename real>
-__global__ void __launch_bounds__(kSourceThreads) spread_source_kernel_multi(
+__global__ void __launch_bounds__(kSourceThreads, sizeof(real) == 4 ? 7 : 1) spread_source_kernel_multi(
     const SourceArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   __shared__ SourceShared<real> sh;
