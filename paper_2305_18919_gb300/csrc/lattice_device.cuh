@@ -39,6 +39,7 @@ struct CollideCoef {
   real Fh[3];         // g/2:            u = (j + g/2)/rho
   real Kc[3];         // (2 tau - 1/2) g: K = j + (2 tau - 1/2) g
   real Lc[3];         // g/omega:        L = j + g/omega
+  real ga[3], gd[3];  // 3 w g of the axis and diagonal directions (FP32, see collide)
 };
 
 // Coefficients of the active-tile correction (in the arithmetic's units, see Correction).
@@ -105,6 +106,8 @@ CollideCoef<real> collide_coef(const Ctx &c, double scale) {
     k.Fh[a] = (real)(0.5 * c.g[a]);
     k.Kc[a] = (real)((2.0 * tau - 0.5) * c.g[a]);
     k.Lc[a] = (real)(c.g[a] / om);
+    k.ga[a] = (real)(c.g[a] / 6.0);
+    k.gd[a] = (real)(c.g[a] / 12.0);
   }
   return k;
 }
@@ -471,15 +474,20 @@ __device__ __forceinline__ float relaxed(float f, float P, const CollideCoef<flo
 // copy bandwidth (256^3: 366 us); 16-bit storage, 256^3 BF16 on 112 SMs 223 us against 229.
 // The rounding of u enters at second order only, where a form with rho u rounds it into the
 // linear term: u of the 256^3 FP32 run is 1.2e-7 off 64 bits after 40 steps, against 3.6e-7.
+// FP32 with a force keeps 3 w c.g out of the momentum part and adds it beside the smaller
+// equilibrium part: rounding j + g/omega, the same way at a node step after step, would change the
+// force by as much as the last place of j (24x20x18, g = 2e-6, u about 1e-3: u after 500 steps 8e-8
+// off 64 bits against 5.6e-6, and 3.6e-6 with the source added to each population by itself).
 template <bool FORCE, typename real>
 __device__ __forceinline__ void collide(real f[Q], real drho, const real j[3], real ir,
                                         const CollideCoef<real> &k) {
+  constexpr bool apart = FORCE && sizeof(real) == 4;
   real u[3], K[3], L[3];
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     u[a] = mul_(FORCE ? add_(j[a], k.Fh[a]) : j[a], ir);
     K[a] = FORCE ? add_(j[a], k.Kc[a]) : j[a];
-    L[a] = FORCE ? add_(j[a], k.Lc[a]) : j[a];
+    L[a] = FORCE && !apart ? add_(j[a], k.Lc[a]) : j[a];
   }
   const real qxx = mul_(u[0], K[0]), qyy = mul_(u[1], K[1]), qzz = mul_(u[2], K[2]);
   const real s = fma_(real(-1.5), add_(add_(qxx, qyy), qzz), drho);
@@ -489,8 +497,8 @@ __device__ __forceinline__ void collide(real f[Q], real drho, const real j[3], r
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     const real P = fma_(k.qa, qk[a], pa);
-    f[2 * a + 1] = relaxed(f[2 * a + 1], P, k.la, L[a], k);
-    f[2 * a + 2] = relaxed(f[2 * a + 2], P, -k.la, L[a], k);
+    f[2 * a + 1] = relaxed(f[2 * a + 1], apart ? add_(P, k.ga[a]) : P, k.la, L[a], k);
+    f[2 * a + 2] = relaxed(f[2 * a + 2], apart ? add_(P, -k.ga[a]) : P, -k.la, L[a], k);
   }
 #pragma unroll
   for (int p = 0; p < 3; p++) {  // planes xy, xz, yz: directions 7 + 4 p .. 10 + 4 p
@@ -501,10 +509,11 @@ __device__ __forceinline__ void collide(real f[Q], real drho, const real j[3], r
     const real qm = FORCE ? k.qd : k.qa;
     const real Pp = fma_(qm, m, P), Pm = fma_(-qm, m, P);
     const real lp = add_(L[a], L[b]), lm = add_(L[a], -L[b]);
-    f[i] = relaxed(f[i], Pp, k.ld, lp, k);
-    f[i + 1] = relaxed(f[i + 1], Pp, -k.ld, lp, k);
-    f[i + 2] = relaxed(f[i + 2], Pm, k.ld, lm, k);
-    f[i + 3] = relaxed(f[i + 3], Pm, -k.ld, lm, k);
+    const real gp = add_(k.gd[a], k.gd[b]), gm = add_(k.gd[a], -k.gd[b]);
+    f[i] = relaxed(f[i], apart ? add_(Pp, gp) : Pp, k.ld, lp, k);
+    f[i + 1] = relaxed(f[i + 1], apart ? add_(Pp, -gp) : Pp, -k.ld, lp, k);
+    f[i + 2] = relaxed(f[i + 2], apart ? add_(Pm, gm) : Pm, k.ld, lm, k);
+    f[i + 3] = relaxed(f[i + 3], apart ? add_(Pm, -gm) : Pm, -k.ld, lm, k);
   }
 }
 
