@@ -63,16 +63,18 @@ typedef struct {
   int32_t precision;       /* IBLB_FP64, IBLB_FP32, IBLB_FP16 or IBLB_BF16 */
   int32_t z_periodic;      /* 0: bounce-back walls at both z ends; 1: periodic z (tests) */
   int32_t ib_sms;          /* SMs given to the interface chain of iblb_step as a partition of
-                              the GPU (green context); the stream-collide passes get the rest.
+                              the GPU (green context); the stream-collide passes get the rest
+                              and, of more than 16, eight of these as well.
                               0: by the bytes that the stream-collide pass moves
-                              (2 x 19 x nx ny nz x storage bytes), 64 below 1 GiB, 40 below
-                              1.5 GiB, then 32 with 16-bit storage or below 2 GiB, else 24
-                              (rounded to the device's partition granularity); none with
-                              FP64 from 192 MiB up. < 0: no
+                              (2 x 19 x nx ny nz x storage bytes), 64 below 768 MiB, 48 below
+                              1 GiB, 40 below 1.5 GiB, then 32 with 16-bit storage or below
+                              2 GiB, else 24 (rounded to the device's partition granularity);
+                              none with FP64 from 192 MiB up. < 0: no
                               partition (both share all SMs, interface stream at top priority).
                               If the device or driver cannot partition, no partition is used.
-                              With 0, a mesh and less than 1 GiB a step runs as one kernel on
-                              all SMs, and the partition serves the steps that cannot. */
+                              With 0, a mesh and less than 320 MiB (1 GiB with FP64, and with
+                              16-bit storage where nx is no multiple of 8) a step runs as one
+                              kernel on all SMs, and the partition serves the steps that cannot. */
   double tau;              /* BGK relaxation time, > 1/2 (viscosity (tau - 1/2)/3) */
   double rho0;             /* reference density (initial state and moving-wall term) */
   double wall_u_bottom[3]; /* wall velocity at z = 0.5 (tangential components only) */

@@ -174,15 +174,25 @@ bool green_api(GreenApi &g) {
 }
 
 // Whether the steps of a default context run as one kernel (fused.cu), by the bytes that its
-// stream-collide pass reads and writes. With a mesh: below 1 GiB (us per step, fused against the
-// separate kernels: 24^3 FP32 28 / 46, 64^3 35 / 52, 128x128x96 65 / 69, 128^3 FP32 77 / 78 and
-// FP16 60 / 72, 192^3 FP32 189 / 187). Without one, where the separate passes are launched early
-// (except the staged one): below 20 MB in FP32 and 8 MB in 16 bits, 80 MB where the staged pass
-// would be taken, never in FP64 (32^3 FP32 3.2 / 3.4, 48^3 4.8 / 6.0, 64^3 9.3 / 6.5; FP16 staged
-// 64^3 5.3 / 8.4, 128^3 30.6 / 29.8, not staged 84x68x64 7.9 / 5.5; FP64 48^3 37.5 / 32.4).
+// stream-collide pass reads and writes (us per step, one kernel / separate kernels).
+//
+// With a mesh, FP32: below 320 MiB (24^3 24 / 42, 64^3 28 / 45, 96^3 41 / 56, 128x128x96 55 / 61, 128^3,
+// 304 MiB, 71 / 74; from there the two are equal and a finer mesh is faster by the separate kernels,
+// 144^3 with 10242 vertices 102 / 93). 16 bits: below 320 MiB as well where the separate kernels have the
+// staged pass (128^3 52 / 59, 144^3 70 / 77, 160^3, 297 MiB, 92 / 92; 192^3 141 / 129, 240^3 251 / 198),
+// below 1 GiB where rows are no whole number of 16-byte blocks (188^3 130 / 142, 236^3 235 / 274). FP64:
+// below 1 GiB (96^3 241 / 250, 150^3 800 / 833).
+//
+// Without a mesh, where the separate passes are launched early (except the staged one): below 20 MB in
+// FP32 and 8 MB in 16 bits, 80 MB where the staged pass would be taken, never in FP64 (32^3 FP32 3.2 /
+// 3.4, 48^3 4.8 / 6.0, 64^3 9.3 / 6.5; FP16 staged 64^3 5.3 / 8.4, 128^3 30.6 / 29.8, not staged
+// 84x68x64 7.9 / 5.5; FP64 48^3 37.5 / 32.4).
 bool fused_by_size(const Ctx &c) {
   const size_t pass = (size_t)2 * iblb::Q * c.ncell * c.pop_size;
-  if (c.nv) return pass < ((size_t)1 << 30);
+  if (c.nv) {
+    const bool most = c.pop_size == 8 || (c.pop_size == 2 && !iblb::stream_collide_staged(c));
+    return pass < (size_t)(most ? 1024 : 320) << 20;
+  }
   if (c.pop_size == 2) return pass < (iblb::stream_collide_staged(c) ? 80000000u : 8000000u);
   return c.pop_size == 4 && pass < 20000000;
 }
@@ -379,16 +389,19 @@ int iblb_create(const iblb_lattice_desc *d, void *cuda_stream, iblb_ctx **out) {
   // 240^3 (2.10 GB) 401 / 357 / 340; 256^3 (2.55 GB) 408 / 414 / 423, 390 / 397 / 406. 16 bits, whose
   // pass has twice the arithmetic per byte: 256^3 (1.28 GB) 348 / 292 / 248; 288^3 (1.82 GB) 385 /
   // 385 / 408, 371 / 378 / 403; 320^3 (2.49 GB) 498 / 471 / 500; 384^3 (4.30 GB) 780 / 726 / 720.
-  // A pass below 1 GiB leaves the chain as the critical path, which then takes 64 SMs where the
-  // separate kernels run (128x128x96 FP32 wetting, 1.5 M nodes: 0.090 ms against 0.115 ms on 32
-  // SMs). An FP64 pass is bound by the FP64 units (1/64 of the FP32 rate),
+  // A pass below 768 MiB leaves the chain as the critical path, which then takes 64 SMs where the
+  // separate kernels run (160^3 FP32 with 2562 / 10242 / 40962 vertices on 48: 115 / 118 / 164, on 64:
+  // 123 / 123 / 140; 128^3 78 / 86 / 196 and 71 / 77 / 184); from there to 1 GiB 48 (188^3 FP32 on 40 /
+  // 48 / 64: 175 / 178 / 190, 177 / 180 / 192, 216 / 196 / 199; 224^3 FP16 165 / 176 / 200, 178 / 178 /
+  // 201, 235 / 212 / 202). An FP64 pass is bound by the FP64 units (1/64 of the FP32 rate),
   // not by memory, and from 192 MiB (about 650k nodes) up the interface chain is short beside
   // it: no partition (96^3 FP64: 0.301 ms per step against 0.407 on 64 interface SMs and 0.309
   // on 24; 128^3: 0.583 against 0.899 and 0.632; below it, 64^3: 0.147 against 0.137 on 64).
   const size_t pass_bytes = (size_t)2 * iblb::Q * c.ncell * c.pop_size;
   const int want = d->ib_sms != 0 ? d->ib_sms
                    : c.pop_size == 8 && pass_bytes >= ((size_t)192 << 20) ? -1
-                   : pass_bytes < ((size_t)1 << 30) ? 64
+                   : pass_bytes < ((size_t)3 << 28) ? 64
+                   : pass_bytes < ((size_t)1 << 30) ? 48
                    : pass_bytes < ((size_t)3 << 29) ? 40
                    : pass_bytes < ((size_t)2 << 30) || c.pop_size == 2 ? 32
                    : 24;
