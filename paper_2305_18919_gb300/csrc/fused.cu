@@ -200,8 +200,8 @@ __device__ __forceinline__ void fused_steps(const FusedArgs<real, S> &P, SourceS
       for (int g = chain_first; g - lane < 4 * A.vertex.nv; g += chain_stride) vertex_body(A.vertex, g);
       CHAIN_BARRIER();
       const int g = tid / kSourceThreads, ng = nt / kSourceThreads;
-      spread_source_body(A.source, sh[g], blockIdx.x + g * nchain, ng * nchain, g,
-                         tid % kSourceThreads);
+      spread_source_body<sizeof(S) != 2>(A.source, sh[g], blockIdx.x + g * nchain, ng * nchain, g,
+                                         tid % kSourceThreads);
       CHAIN_BARRIER();
       const int h = tid / TILE_CELLS, nh = nt / TILE_CELLS;
       spread_gather_body(A.gather, blockIdx.x + h * nchain, nh * nchain, tid % TILE_CELLS);

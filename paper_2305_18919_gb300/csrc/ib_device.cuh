@@ -619,8 +619,117 @@ __device__ __forceinline__ void group_barrier(int g) {
   asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + g), "n"(kSourceThreads) : "memory");
 }
 
-// K4a for the source tiles bid, bid + nb, ..., by group `g` of its block (thread tid of it).
+// A vertex's record, completed with the volume term, to place r of the stage of source tile S. Its base
+// is relative to S_lo (x, y wrapped into [0, n) by the vertex kernel): x, y in 0..3, z in -4..3 (below 0
+// only at a wall), in a byte each.
 template <typename real>
+__device__ __forceinline__ void stage_record(SourceShared<real> &sh, int r, const StencilRec<real> &rec,
+                                             const Vec4<real> &pv, const Vec4<real> &gv, real coef,
+                                             int Sx, int Sy, int Sz) {
+  for (int k = 0; k < 4; k++) {
+    sh.w[r][k] = rec.w[0][k];
+    sh.w[r][4 + k] = rec.w[1][k];
+    sh.w[r][8 + k] = rec.w[2][k];
+  }
+  sh.f[r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
+  const int bz = max(rec.base[2] - Sz, -4);
+  sh.b[r] = (rec.base[0] - Sx) | (rec.base[1] - Sy) << 8 | (bz + 4) << 16;
+}
+// Add the n staged vertices, the tile's rank-th and following: even ranks by the lower half warp.
+template <typename real>
+__device__ __forceinline__ void add_staged(SourceShared<real> &sh, int n, int rank, int warp, int half,
+                                           int l16) {
+  for (int c0 = 0; c0 < n; c0 += 2) {
+    const int c = c0 + ((half ^ rank) & 1);
+    if (c < n) {
+      const int b = sh.b[c];
+      const Vec4<real> f = sh.f[c];
+      add_plane(sh.region[half], warp, l16, b & 255, (b >> 8) & 255, (b >> 16) - 4, sh.w[c],
+                sh.w[c] + 4, sh.w[c] + 8, f.x, f.y, f.z);
+    }
+    __syncwarp();
+  }
+}
+
+// A tile that spilled: mark its bucket's vertices too, then add every vertex of the tile in
+// increasing index (bitmap words read through L2, where the atomics are performed). A round
+// scans the next kScanWords words of each of the four warps, which list the tile's vertices
+// among them in a row each; the rows, one after the other, are staged and added like a bucket.
+// (With every warp scanning all words, and a vertex's record read when its turn came, a tile
+// was a chain of memory latencies. 96^3 FP32 with 40962 vertices on a sphere of radius 20, whose
+// tiles nearly all spill: 411 us per step against 1026, by the separate kernels 232 against 606;
+// radius 16, 275 against 762.)
+template <typename real>
+__device__ __forceinline__ void spread_spilled(const SourceArgs<real> &A, SourceShared<real> &sh, int g,
+                                               int tid, int v, int t) {
+  unsigned *spill_bits = A.spill_bits;
+  const StencilRec<real> *stencil = A.stencil;
+  const Dims &D = A.D;
+  const real coef = *A.vcoef;
+  const int lane = tid & 31, warp = tid >> 5, half = lane >> 4, l16 = lane & 15;
+  const int tsx = t % D.ntx, tsy = (t / D.ntx) % D.nty, tsz = t / (D.ntx * D.nty);
+  atomicOr(&spill_bits[v >> 5], 1u << (v & 31));
+  group_barrier(g);
+  int rank = 0;
+  for (int wb = 0; wb < A.spill_words; wb += kScanWords * (kSourceThreads / 32)) {
+    const int w0 = wb + kScanWords * warp;
+    const unsigned words =
+        lane < kScanWords && w0 + lane < A.spill_words ? __ldcg(&spill_bits[w0 + lane]) : 0u;
+    int n = 0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < kScanWords; k0 += 2) {  // (two words' loads in flight: few registers)
+      bool mine[2];
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        mine[k] = (__shfl_sync(0xffffffffu, words, k0 + k) >> lane) & 1u;
+        if (mine[k]) {
+          const StencilRec<real> &rl = stencil[(w0 + k0 + k) * 32 + lane];
+          mine[k] = (rl.base[0] >> 2) == tsx && (rl.base[1] >> 2) == tsy &&
+                    (min(max(rl.base[2], 0), D.nz - 1) >> 2) == tsz;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        const unsigned members = __ballot_sync(0xffffffffu, mine[k]);
+        if (mine[k])
+          sh.list[warp][n + __popc(members & ((1u << lane) - 1u))] =
+              (unsigned char)(32 * (k0 + k) + lane);
+        n += __popc(members);
+      }
+    }
+    if (lane == 0) sh.listed[warp] = n;
+    group_barrier(g);
+    const int e1 = sh.listed[0], e2 = e1 + sh.listed[1], e3 = e2 + sh.listed[2];
+    const int total = e3 + sh.listed[3];
+    for (int c0 = 0; c0 < total; c0 += kSourceThreads) {
+      const int e = c0 + tid, m = min(total - c0, kSourceThreads);
+      if (tid < m) {
+        const int row = (e >= e1) + (e >= e2) + (e >= e3);
+        const int at = e - (row == 0 ? 0 : row == 1 ? e1 : row == 2 ? e2 : e3);
+        const int vm = 32 * (wb + kScanWords * row) + sh.list[row][at];
+        stage_record(sh, tid, stencil[vm], A.phi[vm], A.gvol[vm], coef, tsx * TILE, tsy * TILE,
+                     tsz * TILE);
+      }
+      group_barrier(g);
+      add_staged(sh, m, rank, warp, half, l16);
+      rank += m;
+      group_barrier(g);  // the stage and the lists are written again
+    }
+    if (total == 0) group_barrier(g);
+  }
+}
+// The same as a function of its own, where inlining it slows code that it does not touch: the kernel of
+// a whole step in FP64 (128^3 562 us per step inlined, 552 so) and FP32 (112^3 63.3, 61.3), but not
+// in 16 bits (128^3 57.5 inlined, 60.3 so).
+template <typename real>
+__device__ __noinline__ void spread_spilled_call(const SourceArgs<real> &A, SourceShared<real> &sh, int g,
+                                                 int tid, int v, int t) {
+  spread_spilled(A, sh, g, tid, v, t);
+}
+
+// K4a for the source tiles bid, bid + nb, ..., by group `g` of its block (thread tid of it).
+// CALL: spilled tiles by a call.
+template <bool CALL, typename real>
 __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, SourceShared<real> &sh,
                                                    int bid, int nb, int g, int tid) {
   const int *IBLB_RO tile_slot = A.tile_slot;
@@ -663,32 +772,6 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, So
         if (slot_t >= 0) out_src[8 * (size_t)slot_t + e] = reg;
       }
     }
-    // vertex v's record, completed with the volume term, to place r of the stage. Its base is relative
-    // to S_lo (x, y wrapped into [0, n) by the vertex kernel): x, y in 0..3, z in -4..3 (below 0 only
-    // at a wall), in a byte each
-    auto stage = [&](int r, const StencilRec<real> &rec, const Vec4<real> &pv, const Vec4<real> &gv) {
-      for (int k = 0; k < 4; k++) {
-        sh.w[r][k] = rec.w[0][k];
-        sh.w[r][4 + k] = rec.w[1][k];
-        sh.w[r][8 + k] = rec.w[2][k];
-      }
-      sh.f[r] = Vec4<real>{pv.x - coef * gv.x, pv.y - coef * gv.y, pv.z - coef * gv.z, real(0)};
-      const int bz = max(rec.base[2] - Sz, -4);
-      sh.b[r] = (rec.base[0] - Sx) | (rec.base[1] - Sy) << 8 | (bz + 4) << 16;
-    };
-    // add the n staged vertices, the tile's rank-th and following: even ranks by the lower half warp
-    auto add_staged = [&](int n, int rank) {
-      for (int c0 = 0; c0 < n; c0 += 2) {
-        const int c = c0 + ((half ^ rank) & 1);
-        if (c < n) {
-          const int b = sh.b[c];
-          const Vec4<real> f = sh.f[c];
-          add_plane(sh.region[half], warp, l16, b & 255, (b >> 8) & 255, (b >> 16) - 4, sh.w[c],
-                    sh.w[c] + 4, sh.w[c] + 8, f.x, f.y, f.z);
-        }
-        __syncwarp();
-      }
-    };
     if (cnt <= BUCKET_CAP) {
       // sort the bucket by vertex index and stage the records in that order
       StencilRec<real> rec;
@@ -703,67 +786,14 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, So
       if (tid < cnt) {
         int r = 0;
         for (int m = 0; m < cnt; m++) r += sh.v[m] < v;
-        stage(r, rec, pv, gv);
+        stage_record(sh, r, rec, pv, gv, coef, Sx, Sy, Sz);
       }
       group_barrier(g);
-      add_staged(cnt, 0);
+      add_staged(sh, cnt, 0, warp, half, l16);
+    } else if constexpr (CALL) {
+      spread_spilled_call(A, sh, g, tid, v, t);
     } else {
-      // the tile spilled: mark its bucket's vertices too, then add every vertex of the tile in
-      // increasing index (bitmap words read through L2, where the atomics are performed). A round
-      // scans the next kScanWords words of each of the four warps, which list the tile's vertices
-      // among them in a row each; the rows, one after the other, are staged and added like a bucket.
-      // (With every warp scanning all words, and a vertex's record read when its turn came, a tile
-      // was a chain of memory latencies. 96^3 FP32 with 40962 vertices on a sphere of radius 20, whose
-      // tiles nearly all spill: 377 us per step against 1026, by the separate kernels 232 against 606;
-      // radius 16, 262 against 762.)
-      atomicOr(&spill_bits[v >> 5], 1u << (v & 31));
-      group_barrier(g);
-      int rank = 0;
-      for (int wb = 0; wb < A.spill_words; wb += kScanWords * (kSourceThreads / 32)) {
-        const int w0 = wb + kScanWords * warp;
-        const unsigned words =
-            lane < kScanWords && w0 + lane < A.spill_words ? __ldcg(&spill_bits[w0 + lane]) : 0u;
-        int n = 0;
-#pragma unroll 1
-        for (int k0 = 0; k0 < kScanWords; k0 += 2) {  // (two words' loads in flight: few registers)
-          bool mine[2];
-#pragma unroll
-          for (int k = 0; k < 2; k++) {
-            mine[k] = (__shfl_sync(0xffffffffu, words, k0 + k) >> lane) & 1u;
-            if (mine[k]) {
-              const StencilRec<real> &rl = stencil[(w0 + k0 + k) * 32 + lane];
-              mine[k] = (rl.base[0] >> 2) == tsx && (rl.base[1] >> 2) == tsy &&
-                        (min(max(rl.base[2], 0), D.nz - 1) >> 2) == tsz;
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < 2; k++) {
-            const unsigned members = __ballot_sync(0xffffffffu, mine[k]);
-            if (mine[k])
-              sh.list[warp][n + __popc(members & ((1u << lane) - 1u))] =
-                  (unsigned char)(32 * (k0 + k) + lane);
-            n += __popc(members);
-          }
-        }
-        if (lane == 0) sh.listed[warp] = n;
-        group_barrier(g);
-        const int e1 = sh.listed[0], e2 = e1 + sh.listed[1], e3 = e2 + sh.listed[2];
-        const int total = e3 + sh.listed[3];
-        for (int c0 = 0; c0 < total; c0 += kSourceThreads) {
-          const int e = c0 + tid, m = min(total - c0, kSourceThreads);
-          if (tid < m) {
-            const int row = (e >= e1) + (e >= e2) + (e >= e3);
-            const int at = e - (row == 0 ? 0 : row == 1 ? e1 : row == 2 ? e2 : e3);
-            const int vm = 32 * (wb + kScanWords * row) + sh.list[row][at];
-            stage(tid, stencil[vm], phi[vm], gvol[vm]);
-          }
-          group_barrier(g);
-          add_staged(m, rank);
-          rank += m;
-          group_barrier(g);  // the stage and the lists are written again
-        }
-        if (total == 0) group_barrier(g);
-      }
+      spread_spilled(A, sh, g, tid, v, t);
     }
     group_barrier(g);
     Vec4<real> *out = A.Rslot + (size_t)reg * REGION_NODES;
@@ -776,18 +806,19 @@ __device__ __forceinline__ void spread_source_body(const SourceArgs<real> &A, So
 }
 
 template <typename real>
-__global__ void __launch_bounds__(kSourceThreads) spread_source_kernel(const SourceArgs<real> A) {
+__global__ void __launch_bounds__(kSourceThreads)
+    spread_source_kernel(const __grid_constant__ SourceArgs<real> A) {
   __shared__ SourceShared<real> sh;
-  spread_source_body(A, sh, blockIdx.x, gridDim.x, 0, threadIdx.x);
+  spread_source_body<sizeof(real) == 8>(A, sh, blockIdx.x, gridDim.x, 0, threadIdx.x);
 }
 
-// (float: seven blocks per SM, a few registers fewer than it would take)
+// (seven blocks per SM, in FP64 four: a few registers fewer than it would take)
 template <typename real>
-__global__ void __launch_bounds__(kSourceThreads, sizeof(real) == 4 ? 7 : 1) spread_source_kernel_multi(
+__global__ void __launch_bounds__(kSourceThreads, sizeof(real) == 4 ? 7 : 4) spread_source_kernel_multi(
     const SourceArgs<real> *__restrict__ all, const int *__restrict__ start, int n) {
   const MultiBlock m = multi_block(start, n);
   __shared__ SourceShared<real> sh;
-  spread_source_body(all[m.inst], sh, m.block, m.nblocks, 0, threadIdx.x);
+  spread_source_body<sizeof(real) == 8>(all[m.inst], sh, m.block, m.nblocks, 0, threadIdx.x);
 }
 
 // K4b: spreading, second pass. One 64-thread block per active tile T (grid-stride), thread =
