@@ -74,7 +74,11 @@ typedef struct {
                               If the device or driver cannot partition, no partition is used.
                               With 0, a mesh and less than 320 MiB (1 GiB with FP64, and with
                               16-bit storage where nx is no multiple of 8) a step runs as one
-                              kernel on all SMs, and the partition serves the steps that cannot. */
+                              kernel on all SMs, up to about 16 ms of steps per launch, which
+                              work on other streams waits for; the partition serves the steps
+                              that cannot. (To step several contexts at once, or beside long
+                              kernels of the caller's, ask for no partition: the separate
+                              kernels of a step share the GPU.) */
   double tau;              /* BGK relaxation time, > 1/2 (viscosity (tau - 1/2)/3) */
   double rho0;             /* reference density (initial state and moving-wall term) */
   double wall_u_bottom[3]; /* wall velocity at z = 0.5 (tangential components only) */

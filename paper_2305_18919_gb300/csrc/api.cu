@@ -678,16 +678,26 @@ bool takes_fused(const Ctx &c) {
          !c.stage_wait_set && !capturing(c.stream);
 }
 
-// Steps of one fused launch: the GPU is the launch's own while it runs, so work of other streams
-// waits this long at most (some milliseconds).
-constexpr int kFusedSteps = 64;
+// Steps of one fused launch. The GPU is the launch's own while it runs, and work of other streams waits
+// for its end; 64 steps of 128^3 in FP64 would be 35 ms. A launch is kept to 16 ms by an estimate of the
+// step (128^3 FP64 650 us for 540, 236^3 BF16 380 for 260; a mesh so fine that its tiles spill takes two
+// to four times its estimate). Shorter launches cost more than they give: at the end of one the next
+// lattice pass does not run beside the interpolation (4 ms: 128^3 FP64 552 us per step against 540,
+// 128x128x96 FP32 64.5 against 62.5).
+int fused_launch_steps(const Ctx &c) {
+  const double per_node = c.pop_size == 8 ? 0.28 : c.pop_size == 4 ? 0.035 : 0.025;  // ns
+  const double ns = 3e4 + per_node * (double)c.ncell + (c.pop_size == 8 ? 3.0 : 1.0) * c.nv;
+  const int n = (int)(16e6 / ns);
+  return n < 1 ? 1 : n > 64 ? 64 : n;
+}
 
 // `left` returns the steps that the separate kernels have to take: those of a launch that the
 // caller's context has too few SMs for (the context then keeps to them).
 int enqueue_fused(Ctx &c, int nsteps, int *left) {
   *left = 0;
+  const int most = fused_launch_steps(c);
   for (int done = 0; done < nsteps;) {
-    const int n = nsteps - done < kFusedSteps ? nsteps - done : kFusedSteps;
+    const int n = nsteps - done < most ? nsteps - done : most;
     const cudaError_t e = launch_fused_steps(c, n, c.stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       cudaGetLastError();
