@@ -74,7 +74,8 @@ typedef struct {
                               If the device or driver cannot partition, no partition is used.
                               With 0, a mesh and less than 320 MiB (1 GiB with FP64, and with
                               16-bit storage where nx is no multiple of 8) a step runs as one
-                              kernel on all SMs, up to about 16 ms of steps per launch, which
+                              kernel on all SMs (on half of them up to 2^18 nodes, in FP64
+                              2^16, with up to 4096 vertices), up to about 16 ms of steps per launch, which
                               work on other streams waits for; the partition serves the steps
                               that cannot. (To step several contexts at once, or beside long
                               kernels of the caller's, ask for no partition: the separate

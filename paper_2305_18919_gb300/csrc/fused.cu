@@ -9,7 +9,7 @@
 // advances many steps. The device code of the phases is that of the separate kernels, so the
 // results are the same bit for bit.
 //
-// Half of the blocks (one per SM) run the interface phases. The other half run the lattice pass of
+// Half of the blocks (one per SM of those that the grid is sized for, fused_sms) run the interface phases. The other half run the lattice pass of
 // the same step meanwhile (it needs the previous step's populations only); a block of the first
 // half that is done with the spreading helps with what is left of the lattice pass. Both halves
 // then correct the active tiles, after which the second half starts the next step's lattice pass
@@ -285,6 +285,17 @@ cudaError_t launch_lattice_steps_t(Ctx &c, int nsteps, cudaStream_t st) {
                                      dim3(need < room ? need : room), dim3(128), params, 0, st);
 }
 
+// SMs that a step's grid is sized for. A small lattice has too little work for all of them, and its
+// barriers are the cheaper the fewer blocks meet there: half of the SMs, from 40^3 (FP64) and 64^3 nodes
+// down, with up to 4096 vertices. What that leaves free serves other contexts: us per step and context
+// on half / on all SMs, one context alone and two at once, 24^3 FP32 24.4 / 24.5 and 12.5 / 24.2, 48^3
+// 26.6 / 27.5 and 13.7 / 27.2, 64^3 26.7 / 28.7 and 15.2 / 29.0, 32^3 FP64 38.2 / 42.7 and 20.6 / 42.6;
+// above the line 96^3 FP32 49.9 / 41.8, 48^3 FP64 61.4 / 52.1, 64^3 FP32 with 10242 vertices 53.5 / 46.5.
+int fused_sms(const Ctx &c) {
+  const size_t nodes = (size_t)1 << (c.pop_size == 8 ? 16 : 18);
+  return c.ncell <= nodes && c.nv <= 4096 ? (c.sm_count + 1) / 2 : c.sm_count;
+}
+
 template <typename real, typename S>
 cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
   if (c.nv == 0) return launch_lattice_steps_t<real, S>(c, nsteps, st);
@@ -309,12 +320,12 @@ cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
   a.health = c.counters + 3;
   a.wait_ns = c.barrier_wait_ns;
   a.nsteps = nsteps;
-  a.nchain = c.sm_count;
+  a.nchain = fused_sms(c);
   void *params[] = {&a};
   // (two blocks per SM always fit: the launch bound limits their registers, and each has 40 KB of
   // shared memory; a caller's context with fewer SMs than the device refuses the launch)
   return cudaLaunchCooperativeKernel((const void *)fused_step_kernel<real, S>,
-                                     dim3(FusedShape<real>::per_sm * c.sm_count),
+                                     dim3(FusedShape<real>::per_sm * a.nchain),
                                      dim3(FusedShape<real>::threads), params, 0, st);
 }
 
