@@ -83,7 +83,8 @@ CollideCoef<real> collide_coef(const Ctx &c, double scale) {
   k.nom = (real)(-1.0 / tau);
   k.omc = (real)(1.0 - 1.0 / tau);
   const bool delta = sizeof(real) == 4 && scale == 0.0;  // f - om f (see collide)
-  const double om = delta ? -(double)k.nom : 1.0 - (double)k.omc;
+  double om = delta ? -(double)k.nom : 1.0 - (double)k.omc;
+  if (!(om > 0.0)) om = 1.0 / tau;  // 1/tau below the last place of 1: the f term keeps all of f
   if (scale != 0.0) {
     k.la = k.ld = (real)(3.0 * scale * om);
     k.ba = k.bd = k.b0 = (real)(scale * om);
