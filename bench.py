@@ -219,7 +219,7 @@ def k1_source_hash():
     for f in ("lattice_kernels.cu", "iblb_internal.cuh", "lattice_device.cuh"):
         path = os.path.join(ROOT, "paper_2305_18919_gb300", "csrc", f)
         if f == "lattice_device.cuh" and not os.path.exists(path):
-            continue  # sources from before the device code had a file of its own
+            continue  # a copy of the two kernel files alone hashes as well
         with open(path, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()

@@ -608,8 +608,8 @@ int iblb_init_equilibrium(iblb_ctx *h, const double *rho, const double *u) {
 }
 
 // One step in the order of Sec. III on two streams. The interface chain (forces, spreading;
-// after the collision: velocity gather, interpolation, update, marking) runs on the library
-// stream `ib`. The stream-collide of every node with the body force only runs on the
+// after the collision: velocity gather, interpolation, update; the active tiles are marked beside the
+// face forces) runs on the library stream `ib`. The stream-collide of every node with the body force only runs on the
 // caller's stream without waiting for it, so it overlaps the interface chain of the same
 // step and the tail of the previous one; then the nodes of the active tiles are collided
 // again once the spread force is ready.

@@ -245,14 +245,15 @@ struct LatticeSteps {
   unsigned long long wait_ns;
   int nsteps;
 };
-// Blocks of 128 threads per SM: what the pass's registers allow.
-template <typename real, typename S>
+// (FP32 and 16-bit storage: FP64 is faster by the separate passes.) Blocks of 128 threads per SM: what
+// the pass's registers allow.
+template <typename S>
 struct LatticeShape {
-  static constexpr int per_sm = sizeof(S) == 2 ? 4 : sizeof(real) == 4 ? 7 : 3;
+  static constexpr int per_sm = sizeof(S) == 2 ? 4 : 7;
 };
 
 template <typename real, typename S>
-__global__ void __launch_bounds__(128, (LatticeShape<real, S>::per_sm))
+__global__ void __launch_bounds__(128, LatticeShape<S>::per_sm)
     lattice_steps_kernel(const __grid_constant__ LatticeSteps<real, S> P) {
   unsigned n_all = 0;
   const int nsteps = gave_up(P.health) ? 0 : P.nsteps;
@@ -279,7 +280,7 @@ cudaError_t launch_lattice_steps_t(Ctx &c, int nsteps, cudaStream_t st) {
   a.health = c.counters + 3;
   a.wait_ns = c.barrier_wait_ns;
   a.nsteps = nsteps;
-  const int need = (a.step[0].G.n + 127) / 128, room = LatticeShape<real, S>::per_sm * c.sm_count;
+  const int need = (a.step[0].G.n + 127) / 128, room = LatticeShape<S>::per_sm * c.sm_count;
   void *params[] = {&a};
   return cudaLaunchCooperativeKernel((const void *)lattice_steps_kernel<real, S>,
                                      dim3(need < room ? need : room), dim3(128), params, 0, st);
@@ -298,7 +299,10 @@ int fused_sms(const Ctx &c) {
 
 template <typename real, typename S>
 cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
-  if (c.nv == 0) return launch_lattice_steps_t<real, S>(c, nsteps, st);
+  if (c.nv == 0) {
+    if constexpr (sizeof(real) == 4) return launch_lattice_steps_t<real, S>(c, nsteps, st);
+    return cudaErrorInvalidValue;  // (no FP64 lattice without a mesh comes here)
+  }
   FusedArgs<real, S> a;
   const int cur = c.cur, map = c.map;
   for (int p = 0; p < 2; p++) {
@@ -322,7 +326,7 @@ cudaError_t launch_fused_t(Ctx &c, int nsteps, cudaStream_t st) {
   a.nsteps = nsteps;
   a.nchain = fused_sms(c);
   void *params[] = {&a};
-  // (two blocks per SM always fit: the launch bound limits their registers, and each has 40 KB of
+  // (two blocks per SM always fit: the launch bound limits their registers, and each has 42 KB of
   // shared memory; a caller's context with fewer SMs than the device refuses the launch)
   return cudaLaunchCooperativeKernel((const void *)fused_step_kernel<real, S>,
                                      dim3(FusedShape<real>::per_sm * a.nchain),

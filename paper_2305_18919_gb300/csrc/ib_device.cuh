@@ -1,7 +1,7 @@
 // Interface passes, device code: per-face forces (Eqs. 2, 17-19) with the double-precision volume sum,
 // per-vertex gathering into nodal forces (Eq. 16) and binning by 4x4x4 source tile,
 // spreading by owner-computes gather over the binned vertices (Eq. 13), interpolation and
-// the Euler update (Eqs. 11-12), and the marking of active tiles for the next step.
+// the Euler update (Eqs. 11-12). The active tiles of a step are marked beside its face forces.
 //
 // Arithmetic runs in the population type `real` (float or double); vertex positions, the
 // enclosed volume V and V - V0 are always double.
@@ -403,7 +403,7 @@ __device__ __forceinline__ void peskin_weights(real r, real w[4]) {
 // Faces around a vertex gathered with all loads in flight (icosphere valences are 5 and 6).
 constexpr int GATHER_UNROLL = 8;
 
-// K3b: one thread per vertex. Gathers, in face order, the strain + wall force of the vertex's
+// K3b: four lanes per vertex. Gathers, in face order, the strain + wall force of the vertex's
 // corners (phi, Eq. 16 without the volume term) and its volume gradient g = dV/dq_i; the
 // volume term -kV (V - V0)/V0 g is added where the force is used (spreading, read-back),
 // after V is complete. Then the delta stencil of the vertex and its binning into the source
@@ -425,7 +425,7 @@ struct VertexArgs {
   const int *tile_slot;
   int *slot_count, *bucket, *ovf_count, *src_slot, *nsources, *health, *zero_counter;
   unsigned *spill_bits;  // bit i: vertex i did not fit in its tile's bucket
-  const double *vol_partial;  // per-block V_j - V0_j partials of the face kernel
+  const double *vol_partial;  // per-warp V_j - V0_j partials of the face kernel
   VolumeParams vp;
   real *vcoef;                // out: kV (V - V0)/V0 for the spreading pass
   Dims D;

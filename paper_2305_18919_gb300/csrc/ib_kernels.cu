@@ -87,18 +87,6 @@ cudaError_t ib_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStream_t 
   }
 }
 
-template <typename real>
-size_t ib_record_align(MultiKernel k) {
-  switch (k) {
-    case MK_FACE: return alignof(FaceArgs<real>);
-    case MK_VERTEX: return alignof(VertexArgs<real>);
-    case MK_SOURCE: return alignof(SourceArgs<real>);
-    case MK_GATHER: return alignof(GatherArgs<real>);
-    case MK_INTERP: return alignof(InterpArgs<real>);
-    default: return 0;
-  }
-}
-
 }  // namespace
 
 int ib_multi_record(const Ctx &c, MultiKernel k, std::vector<unsigned char> &bytes) {
@@ -109,10 +97,6 @@ int ib_multi_record(const Ctx &c, MultiKernel k, std::vector<unsigned char> &byt
 cudaError_t ib_launch_multi(int precision, MultiKernel k, const MultiLaunch &m, cudaStream_t s) {
   return precision == IBLB_FP64 ? ib_launch_multi_t<double>(k, m, s)
                                 : ib_launch_multi_t<float>(k, m, s);
-}
-
-size_t ib_multi_record_align(int precision, MultiKernel k) {
-  return precision == IBLB_FP64 ? ib_record_align<double>(k) : ib_record_align<float>(k);
 }
 
 size_t stencil_record_bytes(const Ctx &c) {

@@ -85,7 +85,6 @@ struct MultiBlock {
   int nblocks;  // blocks of the instance
 };
 
-// Instance and local block of this block (every thread of the block must call it).
 // Instance and block of virtual block b, from the block offsets staged in shared memory.
 __device__ __forceinline__ MultiBlock multi_block_of(const int *s_start, int n, int b) {
   int lo = 0, hi = n;  // the largest lo with start[lo] <= b
@@ -101,24 +100,14 @@ __device__ __forceinline__ MultiBlock multi_block_of(const int *s_start, int n, 
   return m;
 }
 
+// Instance and local block of this block (every thread of the block must call it).
 __device__ __forceinline__ MultiBlock multi_block(const int *__restrict__ start, int n) {
   __shared__ int s_start[kMultiMax + 1];
   pdl_let_next();
   for (int k = threadIdx.x; k <= n; k += blockDim.x) s_start[k] = start[k];
   __syncthreads();
   pdl_wait();  // (the block table is no predecessor's output)
-  const int b = blockIdx.x;
-  int lo = 0, hi = n;  // the largest lo with start[lo] <= b
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (s_start[mid] <= b) lo = mid;
-    else hi = mid;
-  }
-  MultiBlock m;
-  m.inst = lo;
-  m.block = b - s_start[lo];
-  m.nblocks = s_start[lo + 1] - s_start[lo];
-  return m;
+  return multi_block_of(s_start, n, blockIdx.x);
 }
 
 // Force and velocity blocks of the active tiles are [slot][64 nodes] of these: x, y, z and one
@@ -320,10 +309,6 @@ struct MultiLaunch {
 // 1), or -1 where k does not belong to this file.
 int ib_multi_record(const Ctx &c, MultiKernel k, std::vector<unsigned char> &bytes);
 int lattice_multi_record(const Ctx &c, MultiKernel k, std::vector<unsigned char> &bytes);
-// Alignment of the records of kernel k for this precision (records are packed at their size);
-// 0 where k does not belong to the file.
-size_t ib_multi_record_align(int precision, MultiKernel k);
-size_t lattice_multi_record_align(int precision, MultiKernel k);
 // Launch kernel k over the records of m (contexts of precision `precision`) on stream s.
 cudaError_t ib_launch_multi(int precision, MultiKernel k, const MultiLaunch &m, cudaStream_t s);
 cudaError_t lattice_launch_multi(int precision, MultiKernel k, const MultiLaunch &m,

@@ -57,8 +57,6 @@ struct LatParams {
   int nx, ny, nz, has_walls;
   int ntx, nty;
   size_t ncell;
-  real omega;        // 1/tau
-  real guo;          // 1 - 1/(2 tau)
   real rho0;
   real g[3];         // uniform body force
   real wb[19];       // 6 w_i rho0 (c_i . u_bottom): moving-wall term, bottom wall
@@ -138,8 +136,6 @@ LatParams<real> lat_params(const Ctx &c) {
   p.nx = c.nx; p.ny = c.ny; p.nz = c.nz; p.has_walls = c.has_walls;
   p.ntx = c.ntx; p.nty = c.nty;
   p.ncell = c.ncell;
-  p.omega = (real)(1.0 / c.tau);
-  p.guo = (real)(1.0 - 0.5 / c.tau);
   p.rho0 = (real)c.rho0;
   for (int k = 0; k < 3; k++) p.g[k] = (real)c.g[k];
   for (int i = 0; i < Q; i++) {

@@ -990,17 +990,6 @@ cudaError_t lattice_launch_multi_t(MultiKernel k, const MultiLaunch &m, cudaStre
 }
 
 template <typename real, typename S>
-size_t lattice_record_align_t(MultiKernel k) {
-  switch (k) {
-    case MK_FORCED:
-    case MK_STREAM_COLLIDE: return alignof(StreamArgs<real, S>);
-    case MK_TILES: return alignof(TilesArgs<real, S>);
-    case MK_SHELL: return alignof(ShellArgs<real, S>);
-    default: return 0;
-  }
-}
-
-template <typename real, typename S>
 cudaError_t fields_t(Ctx &c, double *rho_dev, double *u_dev) {
   const FlatGroups G = flat_groups(c.nx / 2, c.ny, c.nz);
   const int block = 128, grid = (G.n + block - 1) / block;
@@ -1071,15 +1060,6 @@ cudaError_t lattice_launch_multi(int precision, MultiKernel k, const MultiLaunch
     case IBLB_FP16: return lattice_launch_multi_t<float, __half>(k, m, s);
     case IBLB_BF16: return lattice_launch_multi_t<float, __nv_bfloat16>(k, m, s);
     default: return lattice_launch_multi_t<float, float>(k, m, s);
-  }
-}
-
-size_t lattice_multi_record_align(int precision, MultiKernel k) {
-  switch (precision) {
-    case IBLB_FP64: return lattice_record_align_t<double, double>(k);
-    case IBLB_FP16: return lattice_record_align_t<float, __half>(k);
-    case IBLB_BF16: return lattice_record_align_t<float, __nv_bfloat16>(k);
-    default: return lattice_record_align_t<float, float>(k);
   }
 }
 
